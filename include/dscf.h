@@ -215,9 +215,10 @@ int64_t dscf_launches_per_step(const dscf_ctx* ctx);
  * kfuse <= 2 (rows of 256 sites have contour kernels of their own), and kfuse <= N), or kfuse = 0 for
  * persistent sweeps (FP32; every replica with nx in {32, 48, 64, 96, 128} and ny a multiple of 8;
  * bricks of nx x 8 x 16 sites (nx x 16 x 16 for rows of at most 64 sites where ny allows), one
- * CTA of 16 warps per SM, or of nx x 8 x 8 (nx x 16 x 8) sites, two CTAs of 8 warps per SM; nz a
- * multiple of the brick depth; one warp per plane; replicas share cooperative launches while
- * their bricks fit the SMs together, so a batch takes a few launches per sweep direction).  With
+ * CTA of 16 compute warps per SM, or of nx x 8 x 8 (nx x 16 x 8) sites, two CTAs of 8 per SM; nz a
+ * multiple of the brick depth; one warp per plane; both sweep directions in one launch; replicas
+ * share cooperative launches while their bricks fit the SMs together, so a batch takes a few
+ * launches per density evaluation).  With
  * kfuse = 0, zc = 16 or 8 selects the brick depth (DSCF_ERR_ARG if the grids do not allow it),
  * any other zc keeps the current depth.  Synchronises the stream; the
  * next dscf_step re-captures its graph.  Results do not depend on either value beyond rounding. */

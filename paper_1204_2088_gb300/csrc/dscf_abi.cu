@@ -244,7 +244,7 @@ struct dscf_ctx {
     int kfuse = 1;          // contour steps per propagator launch (1 = single-step kernels, 0 = persistent)
     int pers_bz = 0;        // brick depth of the persistent sweeps (0 = not available)
     int pers_nw = 16;       // warps per CTA of the persistent sweeps
-    struct PersGroup { int width, pby, first, nbricks; };   // one cooperative launch per sweep direction
+    struct PersGroup { int width, pby, first, nbricks; };   // one cooperative launch
     std::vector<PersGroup> pgroups;                    // brick table entries [first, first + nbricks)
     int wait_limit = kPersSpinLimit;   // polls before a persistent sweep gives up on a neighbour
     double ncg_tol = 0.0;   // > 0: residual stop of the inversion (conditional graph nodes)
@@ -381,10 +381,10 @@ int place_bricks(dscf_ctx* c) {
     return rc;
 }
 
-// One direction of the persistent sweeps of every replica: one cooperative launch per group.
-int64_t launch_pers_sweeps(dscf_ctx* c, const Launch& L, bool bwd, int limit) {
+// The persistent sweeps of every replica, both chains: one cooperative launch per group.
+int64_t launch_pers_sweeps(dscf_ctx* c, const Launch& L, int limit) {
     for (const auto& g : c->pgroups)
-        launch_prop_pers(L, bwd, g.width, g.pby, c->pers_bz, c->pers_nw, g.nbricks, pers_table(c) + g.first,
+        launch_prop_pers(L, g.width, g.pby, c->pers_bz, c->pers_nw, g.nbricks, pers_table(c) + g.first,
                          pers_flags(c), c->d_status + 2, limit);
     return (int64_t)c->pgroups.size();
 }
@@ -395,8 +395,7 @@ int64_t enqueue_sweeps(dscf_ctx* c, const Launch& L) {
     int64_t n = 0;
     const int K = c->kfuse;
     if (K == 0) {
-        n += launch_pers_sweeps(c, L, false, c->wait_limit);
-        n += launch_pers_sweeps(c, L, true, c->wait_limit);
+        n += launch_pers_sweeps(c, L, c->wait_limit);
         return n;
     }
     if (K > 1) {
@@ -756,8 +755,7 @@ int autotune_zc(dscf_ctx* c) {
                 cudaEventCreate(&e1);
                 auto run = [&]() {
                     if (K == 0) {
-                        launch_pers_sweeps(c, L, false, kPersSpinLimit);
-                        launch_pers_sweeps(c, L, true, kPersSpinLimit);
+                        launch_pers_sweeps(c, L, kPersSpinLimit);
                     } else if (c->prec == DSCF_FP64) {
                         enqueue_sweeps<double>(c, L);
                     } else {

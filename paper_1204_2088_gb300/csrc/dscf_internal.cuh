@@ -55,7 +55,8 @@ enum { ST_NONFINITE = 1, ST_TIMEOUT = 2 };
 // persistent sweeps, [3] change flag of the solvent-component labelling, [kFlagBase..] one step
 // counter per persistent brick.
 constexpr int kFlagBase = 64;
-constexpr int kFlagStride = 32;   // ints between brick step counters: one 128-byte line each
+constexpr int kFlagStride = 32;   // ints between bricks' step counters: one 128-byte line each
+constexpr int kFlagChain = 16;    // the backward chain's counter in that line (the forward's is first)
 constexpr int kMaxBricks = 4096;
 // status block: the words above, kMaxBricks counters, then the int4 brick table of the sweeps
 constexpr size_t kStatusInts = (size_t)kFlagBase + (size_t)kMaxBricks * kFlagStride + 4 * (size_t)kMaxBricks;
@@ -397,7 +398,7 @@ bool pers_supported(const Rep& R, int bz, int nw, int nsm);   // nw: warps per C
 int pers_bricks(const Rep& R, int bz);
 int pers_prepare(int width, int pby, int bz, int nw);   // cudaError_t; width 0: the mixed-width kernel
 // width 0: bricks of several widths in one launch (bricks of 16 planes)
-int launch_prop_pers(const Launch& L, bool bwd, int width, int pby, int bz, int nw, int nbricks, const int4* table,
+int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, int nbricks, const int4* table,
                      int* flags, int* abortf, int limit);  // cudaError_t
 // SM id of each CTA of a sweep-shaped cooperative launch (cudaError_t)
 int pers_placement(int bz, int nw, int nbricks, int* d_smid, cudaStream_t stream);

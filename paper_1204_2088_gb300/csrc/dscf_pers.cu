@@ -1,53 +1,93 @@
 // Persistent contour sweeps (Eq. 16-17) in the whole-row layout (FP32), for one replica or a
 // batch of replicas.
 //
-// One launch runs a whole forward (or backward) sweep of N contour steps.  The lattice is cut
-// into bricks of nx x 8 x BZ sites, one brick per CTA (one CTA per SM for BZ = 16, two for
-// BZ = 8; the launch is cooperative, so all CTAs are resident together), one warp per plane of
-// the brick.  Rows of 96 or 128 sites are held by a whole warp (3 or 4 sites per lane), rows of
-// 32, 48 or 64 sites by half a warp (2, 3 or 4 sites per lane), two rows side by side; bricks of
-// these narrow rows have 16 rows instead of 8 where ny allows it.  A CTA takes its brick from a
-// table (replica, brick, flag base), so replicas of one row width share a launch; a brick waits
-// only on the bricks of its own replica.  A warp keeps its plane's x-filtered rows in registers
-// from one contour step to the next; per step the CTA only reads the halo rows and planes of its
-// eight y/z neighbours from L2, after checking with an acquire load that they have published that
-// step.  Per step:
-//   halo rows of the previous step -> x pass -> shared XH (y-halo rows) and ZH (z-halo planes);
-//   barrier; each warp y-filters its plane in registers (two halo rows from XH) into shared YS,
-//   and one row of a z-halo plane;
-//   barrier; z pass (the neighbouring planes from YS) -> sig;
-//   forward:  G_s = exp(-U_{I_s}) sig; brick-boundary values stored to the contour stack;
-//   backward: q_{I_s} += G_s sig in registers (G_s prefetched a step ahead by bulk copies that
-//             complete on an mbarrier, so the halo wait never waits for them),
-//             G+_s = exp(-U_{I_s}) sig, boundary values stored to a ping-pong exchange buffer;
-//   barrier, release store of the brick's step counter; then the forward interior stores and the
-//   x pass of the new values, in registers.
-// q is accumulated in registers over a whole block of beads and written once; nothing is
-// read-modify-written per step.  Each 1-D pass of the separable stencil is one add and one fma
-// per site, as packed f32x2 pairs (a scalar tail for three sites per lane), with the centre weight
-// folded into the Boltzmann factors.  Every wait is bounded: on timeout the CTA sets a status bit
-// and a global abort flag that makes every other CTA stop waiting, so the launch always finishes.
+// One launch runs both chains of a density evaluation: the forward propagator G_s (s = 1 .. N) and
+// the backward one G+_s (s = N .. 1) do not depend on each other until the quadrature, so every
+// CTA advances them in turn, one contour step of each (a "unit") at a time, and they meet in the
+// middle, h = ceil(N / 2): the forward chain stores G_s for s <= h and the backward chain G+_s for
+// s > h in the contour stack; past the middle each chain multiplies sigma of its own field with the
+// stored value of the other, q_{I_s} += sigma[G_{s-1}] G+_s = G_s sigma[G+_{s+1}].  The HBM bytes
+// are those of one chain after the other (each stack level written once and read once, and the
+// levels near the middle are read back while still in L2), but a chain's halo exchange (release,
+// neighbours' counters, copies: L2 round trips of 5 to 6 thousand cycles) runs while the SM
+// computes the other chain's unit.  128^3, N = 64: 540 us for the two sweeps one after the other
+// (4.2 us a contour step, the exchange in the open), 345 us so (2.7 us).
+//
+// The lattice is cut into bricks of nx x PBY x BZ sites, one brick per CTA (one CTA per SM for
+// BZ = 16, two for BZ = 8; the launch is cooperative, so all CTAs are resident together), one
+// compute warp per plane of the brick and four warps for the exchange.  Rows of 96 or 128 sites
+// are held by a whole warp (3 or 4 sites per lane), rows of 32, 48 or 64 sites by half a warp (2,
+// 3 or 4 sites per lane), two rows side by side; bricks of these narrow rows have 16 rows instead
+// of 8 where ny allows it.  A CTA takes its brick from a table (replica, brick, flag base), so
+// replicas share a launch; a brick waits only on the bricks of its own replica.
+//
+// Per unit a compute warp
+//   takes the halo rows of the previous step from shared memory (x pass in registers), y-filters
+//   its plane in registers (the x-filtered rows of both chains stay in registers from step to
+//   step) into shared YS, and one row of a z-halo plane;
+//   barrier; z pass (the neighbouring planes from YS), times the Boltzmann factor; boundary stores
+//   and, past the middle, the quadrature; arrives on the unit's `pub` mbarrier;
+//   stores the interior of a stack level or fetches the next unit's one; x pass in registers.
+// The exchange warps (two per chain) wait for `pub`, publish the brick's step counter of that chain
+// with a release store, wait for its eight y/z neighbours' counters and copy the next step's raw
+// halo rows into shared memory (cp.async, completing on the chain's `full` mbarrier).  `pub` is also
+// what keeps YS from being overwritten before every warp's z pass has read it, so a unit has one
+// CTA barrier.
+//
+// The Boltzmann factors of both species and both quadrature accumulators (each as large as the
+// brick) live in tensor memory, one 32-bit column per thread and value (tcgen05.ld / st): beside
+// the two chains' rows they do not fit in the registers.  The allocation never waits for another
+// sweep: the registers let one CTA of 16 compute warps (all 512 columns) or two of 8 (256 each)
+// on an SM, whatever context or stream they belong to.
+// Each 1-D pass of the separable stencil is one add and one fma per site, as packed f32x2 pairs
+// (a scalar tail for three sites per lane), with the centre weight folded into the Boltzmann
+// factors.  Every wait is bounded: on timeout the CTA sets a status bit and a global abort flag
+// that makes every other CTA stop waiting, so the launch always finishes.
 #include "dscf_internal.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace dscf {
 
 namespace {
 
-// Polls of the backward G_s prefetch's mbarrier before giving up.  The copies depend on no other
-// CTA, so this bound is fixed and far above any real copy time (a shorter neighbour-wait limit set
-// for failure tests must not abandon a copy that is still landing in this CTA's shared memory).
-constexpr long long kGsSpinLimit = 1LL << 26;
-// Warps per CTA: 16 for bricks of 16 planes (one CTA per SM), 8 for bricks of 8 planes, which
-// fit two CTAs per SM so that one brick computes while the other waits on its neighbours.
+// Polls of a shared-memory mbarrier before giving up.  What completes them (this CTA's copies, its
+// compute warps, its exchange warp, whose own waits on neighbours are bounded by the context's
+// limit) depends on no unbounded wait, so this bound is fixed and far above any real time (a
+// shorter neighbour-wait limit set for failure tests must not abandon a copy that is still landing
+// in this CTA's shared memory).
+constexpr long long kBarSpinLimit = 1LL << 28;
+// Compute warps per CTA: 16 for bricks of 16 planes (one CTA per SM), 8 for bricks of 8 planes, two
+// CTAs per SM.  Beside them one warpgroup of four warps, of which two do the exchange (one per
+// chain): a whole warpgroup, so that it can hand most of its registers to the compute warps
+// (setmaxnreg).  Launched registers a thread (what the launch bounds leave): 96 for 640 threads,
+// 80 for 384 threads twice; the shares 512 x 112 + 128 x 32 = 640 x 96 and
+// 256 x 104 + 128 x 24 <= 384 x 80 stay within them.
+constexpr int kXWarps = 4;
+template <int NW>
+struct PersRegs {
+    static constexpr int compute = NW == 16 ? 112 : 104;
+    static constexpr int exchange = NW == 16 ? 32 : 24;
+};
 
 __device__ __forceinline__ unsigned saddr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp16(void* s, const void* g) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(saddr(s)), "l"(g));
 }
-__device__ __forceinline__ void cpc() { asm volatile("cp.async.commit_group;\n" ::); }
-__device__ __forceinline__ void cpw0() { asm volatile("cp.async.wait_group 0;\n" ::); }
+template <int VEC>
+__device__ __forceinline__ void cpv(float* s, const float* g) {   // VEC values of a lane: 16, 8 or 3 x 4 bytes
+    if constexpr (VEC == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(saddr(s)), "l"(g));
+    else if constexpr (VEC == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(saddr(s)), "l"(g));
+    else
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(saddr(s + k)), "l"(g + k));
+}
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+// arrive on bar (one of its expected arrivals) when all earlier cp.async of this thread have landed
+__device__ __forceinline__ void cp_arrive(unsigned long long* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(saddr(bar)) : "memory");
+}
 __device__ __forceinline__ int ld_acquire(const int* p) {
     int v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
@@ -56,19 +96,11 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 __device__ __forceinline__ void st_release(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ void bar_init(unsigned long long* bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(saddr(bar)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+__device__ __forceinline__ void bar_init(unsigned long long* bar, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(saddr(bar)), "r"(count) : "memory");
 }
-__device__ __forceinline__ void bar_expect(unsigned long long* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(saddr(bar)), "r"(bytes) : "memory");
-}
-// bulk copy global -> shared (both 16-byte aligned, bytes a multiple of 16) completing on bar
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                     saddr(dst)),
-                 "l"(src), "r"(bytes), "r"(saddr(bar))
-                 : "memory");
+__device__ __forceinline__ void bar_arrive(unsigned long long* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(saddr(bar)) : "memory");
 }
 __device__ __forceinline__ bool bar_test(unsigned long long* bar, unsigned parity) {
     unsigned done;
@@ -107,43 +139,57 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
     return r;
 }
 
+// Tensor memory: N (2 or 4) consecutive 32-bit columns of the warp's 32 lanes, one lane per thread.
+// A load's values are valid after the wait that names them (which also keeps their uses behind it).
+template <int N>
+__device__ __forceinline__ void tm_ld(unsigned a, float (&v)[N]) {
+    if constexpr (N == 4)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                     : "r"(a));
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];\n" : "=f"(v[0]), "=f"(v[1]) : "r"(a));
+}
+template <int N>
+__device__ __forceinline__ void tm_wait_ld(float (&v)[N], float (&u)[N]) {
+    if constexpr (N == 4)
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+                     : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(u[0]), "+f"(u[1]), "+f"(u[2]), "+f"(u[3]));
+    else
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" : "+f"(v[0]), "+f"(v[1]), "+f"(u[0]), "+f"(u[1]));
+}
+template <int N>
+__device__ __forceinline__ void tm_wait_ld(float (&v)[N]) {
+    if constexpr (N == 4)
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]));
+    else
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" : "+f"(v[0]), "+f"(v[1]));
+}
+template <int N>
+__device__ __forceinline__ void tm_st(unsigned a, const float (&v)[N]) {
+    if constexpr (N == 4)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(a), "f"(v[0]), "f"(v[1]),
+                     "f"(v[2]), "f"(v[3]));
+    else
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};\n" ::"r"(a), "f"(v[0]), "f"(v[1]));
+}
+__device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
+
+template <int N>
+__device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(N)); }
+// Barrier of the compute warps.
+__device__ __forceinline__ void compute_sync(int threads) {
+    asm volatile("bar.sync 1, %0;\n" ::"r"(threads) : "memory");
+}
+
 struct PersCtl {
-    int* flags;          // one step counter per brick, kFlagStride ints apart
+    int* flags;          // two step counters (chains) per brick, kFlagStride ints apart
     int* abort;          // set by a CTA that gave up waiting
     int* status;         // device status word
     const int4* table;   // per CTA: replica, brick in the replica, flag index of the replica's brick 0
     int limit;           // polls before giving up
-};
-
-// Wait until every neighbour brick has published `target`; threads 0..7 poll one neighbour each
-// (each counter on its own cache line).  Only the pollers look at the shared abort flag, and only
-// every 32 polls, so that the waits of all CTAs do not contend on one line.
-__device__ __forceinline__ void wait_nb(const PersCtl& c, const int* nb, unsigned target, bool& aborted) {
-    if (threadIdx.x < 8 && !aborted) {
-        const int* f = c.flags + (size_t)nb[threadIdx.x] * kFlagStride;
-        int spins = 0;
-        while ((int)((unsigned)ld_acquire(f) - target) < 0) {   // wrap-safe: counters only grow
-            if ((++spins & 31) == 0) {
-                if (ld_acquire(c.abort) != 0) {
-                    aborted = true;
-                    break;
-                }
-                if (spins > c.limit) {
-                    atomicOr(c.status, (int)ST_TIMEOUT);
-                    atomicExch(c.abort, 1);
-                    aborted = true;
-                    break;
-                }
-            }
-            __nanosleep(32);
-        }
-    }
-    __syncthreads();
-}
-
-template <int BZ, int PBY>
-struct PersGeom {
-    static constexpr int NH = 2 * (BZ + 2) + 2 * PBY;   // halo rows per step
 };
 
 // Row geometry of a brick of width W and PBY rows: a row is held by LPR lanes, VEC consecutive
@@ -156,9 +202,7 @@ struct PRow {
     static constexpr int VEC = W / LPR;
     static constexpr int HALVES = 32 / LPR;
     static constexpr int RPL = PBY / HALVES;
-    static constexpr int CH = W / 4;   // 16-byte chunks per row
     static_assert(LPR * VEC == W && VEC >= 2 && VEC <= 4, "row width");
-    static_assert(HALVES * CH <= 32, "one 16-byte chunk per lane for the rows a warp copies");
 };
 
 // VEC consecutive FP32 values: one vector access for 2 and 4, three scalar ones for 3
@@ -185,6 +229,18 @@ __device__ __forceinline__ void stv(float* p, const float (&v)[VEC]) {
 #pragma unroll
         for (int k = 0; k < VEC; ++k) p[k] = v[k];
     }
+}
+// Global stores as asm without a memory clobber: the compiler may move the shared-memory loads of the
+// next rows over them (it cannot tell that they do not alias).
+template <int VEC>
+__device__ __forceinline__ void stg(float* p, const float (&v)[VEC]) {
+    if constexpr (VEC == 4)
+        asm volatile("st.global.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]));
+    else if constexpr (VEC == 2)
+        asm volatile("st.global.v2.f32 [%0], {%1, %2};\n" ::"l"(p), "f"(v[0]), "f"(v[1]));
+    else
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) asm volatile("st.global.f32 [%0], %1;\n" ::"l"(p + k), "f"(v[k]));
 }
 // o = c + r (a + d) per site: packed pairs, a scalar tail for odd VEC (same rounding: one add, one
 // fma per site either way)
@@ -219,47 +275,258 @@ __device__ __forceinline__ void scalev(float c, unsigned long long c2, float (&v
     if constexpr (VEC & 1) v[VEC - 1] = __fmul_rn(c, v[VEC - 1]);
 }
 
+// Arrays of a replica as the sweep uses them, in shared memory (the descriptor itself is in device
+// memory, whose cached copy the acquire loads keep invalidating).
+struct PersArrays {
+    float* exch[2][2];   // exchange buffers per chain
+    float* stack;
+    size_t V;
+};
+
+// What a compute warp keeps through the sweep.
+struct PersWarp {
+    const PersArrays& A;
+    const PersCtl& ctl;
+    unsigned long long *full, *pub;
+    float *YS, *HS, *GS;   // GS: the lane's first value of the stack level
+    size_t own;            // lane's first site of its first row in a field
+    size_t slab;           // lane's 128-byte line of the plane's run in a field (past its end: none)
+    int N, nA, hm, w, lane, hf, xo, lsrc, rsrc;
+    bool face_plane;
+    float rr;
+    unsigned long long rr2;
+    unsigned tbase;
+    float qsum;
+    bool dead;
+};
+
+// Level j of chain C (contour step s = j + 1 forward, s = N - j backward): the contour stack before
+// the chains meet, the chain's exchange buffers (boundary rows only) past it.
+__device__ __forceinline__ float* level_of(const PersArrays& A, int c, int N, int hm, int j) {
+    return (c ? j < N - hm : j < hm) ? A.stack + (size_t)(c ? N - j - 1 : j) * A.V : A.exch[c][j & 1];
+}
+
+// Bounded wait on an mbarrier phase; a thread that gives up reports it and waits no more.
+__device__ __forceinline__ void bar_wait(unsigned long long* bar, unsigned parity, const PersCtl& ctl, bool& dead) {
+    if (dead) return;
+    for (long long spins = 0; !bar_test(bar, parity); ++spins)
+        if (spins > kBarSpinLimit) {
+            atomicOr(ctl.status, (int)ST_TIMEOUT);
+            atomicExch(ctl.abort, 1);
+            dead = true;
+            return;
+        }
+}
+
+// x pass of a periodic row: v + r (left + right)
+template <int VEC>
+__device__ __forceinline__ void xpassv(const PersWarp& k, const float (&v)[VEC], float (&o)[VEC]) {
+    const float lv = __shfl_sync(0xffffffffu, v[VEC - 1], k.lsrc);
+    const float rv = __shfl_sync(0xffffffffu, v[0], k.rsrc);
+    float a[VEC], d[VEC];
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+        a[i] = i ? v[i - 1] : lv;
+        d[i] = (i + 1 < VEC) ? v[i + 1] : rv;
+    }
+    mixv<VEC>(a, v, d, k.rr, k.rr2, o);
+}
+
+// Halo rows (row r, plane pl of the brick's frame, r in -1..PBY, pl in -1..BZ) in HS: rows -1, then rows
+// 0..PBY-1 of plane -1; rows PBY of planes -1..BZ, then rows 0..PBY-1 of plane BZ.
+template <int PBY, int BZ>
+__device__ __forceinline__ int halo_row(int r, int pl) {
+    constexpr int P = BZ + 2 + PBY;
+    if (r < 0) return pl + 1;
+    if (r >= PBY) return P + pl + 1;
+    return (pl < 0 ? BZ + 2 : P + BZ + 2) + r;
+}
+
+// One unit: contour step j of chain C (0 forward, s = j + 1; 1 backward, s = N - j).
+template <int W, int PBY, int BZ, int NW, int C>
+__device__ __forceinline__ void pers_unit(PersWarp& k, float (&xf)[PRow<W, PBY>::RPL][PRow<W, PBY>::VEC], const int j) {
+    using RG = PRow<W, PBY>;
+    constexpr int VEC = RG::VEC, LPR = RG::LPR, RPL = RG::RPL;
+    constexpr int VS = VEC == 3 ? 4 : VEC;   // tensor-memory columns of a row's sites
+    constexpr int NH = 2 * (BZ + 2 + PBY);
+    const int N = k.N, hm = k.hm, w = k.w, xo = k.xo;
+    const float rr = k.rr;
+    const unsigned long long rr2 = k.rr2;
+    float* ysl = k.YS + (w * PBY + k.hf * RPL) * W + xo;   // plane w - 1 (YS holds planes -1..BZ)
+    const float* hs = k.HS + C * NH * W + xo;
+    const int s = C ? N - j : j + 1;
+    const int sp = s <= k.nA ? 0 : 1;
+    const bool acc = C ? j >= N - hm : j >= hm;
+    if (j > 0) bar_wait(k.full + C, (unsigned)((j - 1) & 1), k.ctl, k.dead);
+    // the rows next to the lane's first and last row: y-halo rows, or across the lane halves
+    float up[VEC], dn[VEC];
+    if constexpr (RG::HALVES == 2) {
+        float v[VEC], o[VEC];
+        ldv<VEC>(hs + halo_row<PBY, BZ>(k.hf ? PBY : -1, w) * W, v);
+        xpassv<VEC>(k, v, o);
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            const float last = __shfl_xor_sync(0xffffffffu, xf[RPL - 1][i], LPR);
+            const float first = __shfl_xor_sync(0xffffffffu, xf[0][i], LPR);
+            up[i] = k.hf ? last : o[i];
+            dn[i] = k.hf ? o[i] : first;
+        }
+    } else {
+        float v[VEC], u[VEC];
+        ldv<VEC>(hs + halo_row<PBY, BZ>(-1, w) * W, v);
+        ldv<VEC>(hs + halo_row<PBY, BZ>(PBY, w) * W, u);
+        xpassv<VEC>(k, v, up);
+        xpassv<VEC>(k, u, dn);
+    }
+    // every warp has read YS of the previous unit
+    if (C) bar_wait(k.pub, (unsigned)(j & 1), k.ctl, k.dead);
+    else if (j > 0) bar_wait(k.pub + 1, (unsigned)((j - 1) & 1), k.ctl, k.dead);
+    // z-halo planes, one row per lane half: y pass of the raw rows, then the x pass
+#pragma unroll
+    for (int t0 = w * RG::HALVES; t0 < 2 * PBY; t0 += NW * RG::HALVES) {
+        const int t = t0 + k.hf;
+        const int side = t / PBY, r = t % PBY, pl = side ? BZ : -1;
+        float a[VEC], c[VEC], d[VEC], m[VEC], o[VEC];
+        ldv<VEC>(hs + halo_row<PBY, BZ>(r - 1, pl) * W, a);
+        ldv<VEC>(hs + halo_row<PBY, BZ>(r, pl) * W, c);
+        ldv<VEC>(hs + halo_row<PBY, BZ>(r + 1, pl) * W, d);
+        mixv<VEC>(a, c, d, rr, rr2, m);
+        xpassv<VEC>(k, m, o);
+        stv<VEC>(k.YS + ((pl + 1) * PBY + r) * W + xo, o);
+    }
+    {
+        float* yw = ysl + PBY * W;
+        float prev[VEC];
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) prev[i] = up[i];
+#pragma unroll
+        for (int p = 0; p < RPL; ++p) {
+            float yv[VEC], cur[VEC];
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) cur[i] = xf[p][i];
+            if (p + 1 < RPL) mixv<VEC>(prev, cur, xf[p + 1 < RPL ? p + 1 : p], rr, rr2, yv);
+            else mixv<VEC>(prev, cur, dn, rr, rr2, yv);
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) {
+                prev[i] = cur[i];
+                xf[p][i] = yv[i];   // xf now holds the y-filtered rows
+            }
+            stv<VEC>(yw + p * W, yv);
+        }
+    }
+    compute_sync(32 * NW);
+    if (acc) cp_wait_all();   // the thread's own stack values of this unit
+    // z pass and step output.  The boundary rows go first and are published; the interior of a stored
+    // level (no interior is stored past the middle) follows with the x pass.
+    const bool last = j + 1 == N;
+    float* dst = level_of(k.A, C, N, hm, j) + k.own;
+    const unsigned te = k.tbase + (unsigned)(sp * 32), ta = te + 64u;
+    const int hf = k.hf;
+    auto edge_row = [&](int p) { return k.face_plane || (p == 0 && hf == 0) || (p == RPL - 1 && hf == RG::HALVES - 1); };
+    float e2[2][VS], q2[2][VS];   // Boltzmann factors and quadrature of this row and the next
+#pragma unroll
+    for (int i = 0; i < VS; ++i) q2[0][i] = q2[1][i] = 0.f;
+    tm_ld<VS>(te, e2[0]);
+    if (acc) tm_ld<VS>(ta, q2[0]);
+#pragma unroll
+    for (int p = 0; p < RPL; ++p) {
+        tm_wait_ld<VS>(e2[p & 1], q2[p & 1]);
+        if (p + 1 < RPL) {
+            tm_ld<VS>(te + (p + 1) * VS, e2[(p + 1) & 1]);
+            if (acc) tm_ld<VS>(ta + (p + 1) * VS, q2[(p + 1) & 1]);
+        }
+        float a[VEC], d[VEC], sg[VEC], e[VEC], out[VEC];
+        ldv<VEC>(ysl + p * W, a);
+        ldv<VEC>(ysl + (2 * PBY + p) * W, d);
+        mixv<VEC>(a, xf[p], d, rr, rr2, sg);
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) e[i] = e2[p & 1][i];
+        mulv<VEC>(e, sg, out);
+        if (acc) {   // q_I += sigma[own chain] x (the other chain's stored value)
+            float st[VEC], q[VEC];
+            ldv<VEC>(k.GS + p * W, st);
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) q[i] = q2[p & 1][i];
+            fmav<VEC>(st, sg, q);
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) q2[p & 1][i] = q[i];
+            tm_st<VS>(ta + p * VS, q2[p & 1]);
+        }
+        if (edge_row(p) && !last) stg<VEC>(dst + p * W, out);
+        if (C == 0 && last) {
+            float t = out[0] + out[1];
+            if constexpr (VEC == 3) t = t + out[2];
+            if constexpr (VEC == 4) t = t + (out[2] + out[3]);
+            k.qsum += t;
+        }
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) xf[p][i] = out[i];
+    }
+    if (acc) tm_wait_st();
+    __syncwarp();
+    if (k.lane == 0) bar_arrive(k.pub + C);
+    if (!acc) {
+#pragma unroll
+        for (int p = 0; p < RPL; ++p)
+            if (!edge_row(p)) stg<VEC>(dst + p * W, xf[p]);
+    }
+    // The next unit's stack level (the other chain's), if that unit accumulates: every thread copies
+    // the values of its own sites, which it stored itself, and brings the line that the chain after
+    // it takes next into L2 meanwhile.
+    {
+        const int jn = C ? j + 1 : j;
+        if ((C ? jn >= hm : jn >= N - hm) && jn < N) {
+            const float* src = k.A.stack + (size_t)(C ? jn : N - jn - 1) * k.A.V;
+#pragma unroll
+            for (int p = 0; p < RPL; ++p) cpv<VEC>(k.GS + p * W, src + k.own + p * W);
+            if (k.lane * 32 < PBY * W && jn + 1 < N)
+                asm volatile("prefetch.global.L2 [%0];\n" ::"l"(C ? src + k.A.V + k.slab : src - k.A.V + k.slab));
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < RPL; ++p) {
+        float o[VEC];
+        xpassv<VEC>(k, xf[p], o);
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) xf[p][i] = o[i];
+    }
+}
+
 }  // namespace
 
 size_t pers_smem_bytes(int width, int pby, int bz) {
     const size_t PBY = (size_t)pby;
-    // YS (y-filtered level, planes -1..bz) + XH (x-filtered y-halo rows of the own planes) + ZH
-    // (x-filtered z-halo planes, rows -1..pby) + halo staging + backward G_s of the brick
-    const size_t rows = (size_t)(bz + 2) * PBY + 2 * (size_t)bz + 2 * (PBY + 2) + (2 * (bz + 2) + 2 * PBY) +
-                        (size_t)bz * PBY;
+    // YS (y-filtered level, planes -1..bz) + raw halo rows of both chains + stack values
+    const size_t rows = (size_t)(bz + 2) * PBY + 2 * 2 * (bz + 2 + PBY) + (size_t)bz * PBY;
     return rows * (size_t)width * sizeof(float);
 }
 
-// Warp w owns plane w of the brick, all PBY rows (HALVES rows side by side), VEC sites of each
-// row per lane; the x-filtered rows of the previous level stay in its registers, so the y pass
-// runs in registers (the rows across the lane halves by one shuffle, the two y-halo rows of the
-// plane from shared memory) and only the y-filtered rows go through shared memory, for the z pass
-// of the neighbouring planes.  The z-halo planes are y-filtered one row per lane half.  Brick-
-// boundary values are stored and published first; the rest of the forward G_s follows without a
-// fence (the backward G+ interior is never stored: it stays in registers).
-// Each CTA takes its brick from the table, so several replicas run in one launch (of one row
-// width here; the mixed-width kernel below calls this per CTA), each brick waiting only on the
-// bricks of its own replica.
-template <int W, int PBY, int BZ, bool BWD, int NW>
+// Warp w < NW owns plane w of the brick, all PBY rows (HALVES rows side by side), VEC sites of each
+// row per lane, of both chains.  What bounds a unit (clock64 per phase, 128 x 8 x 16 bricks, about
+// 6000 cycles): the shared-memory pipe (y-filtered rows written once and read twice, halo and stack
+// rows, shuffles: about 2500 cycles of it before the middle and 3700 past it) and the latencies
+// between the barriers.
+template <int W, int PBY, int BZ, int NW>
 __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const PersCtl& ctl) {
     static_assert(NW == BZ, "one warp per plane");
     using RG = PRow<W, PBY>;
-    constexpr int VEC = RG::VEC, LPR = RG::LPR, HALVES = RG::HALVES, RPL = RG::RPL, CH = RG::CH;
-    constexpr int PWARPS = NW;
-    using G = PersGeom<BZ, PBY>;
-    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int VEC = RG::VEC, LPR = RG::LPR, RPL = RG::RPL;
+    constexpr int VS = VEC == 3 ? 4 : VEC;   // tensor-memory columns of a row's sites
+    constexpr int NH = 2 * (BZ + 2 + PBY), CH = W / 4;   // halo rows; 16-byte chunks per row
+    constexpr int TCOLS = 128 * (NW / 4);    // 4 regions of 32 columns per warp, 4 warps side by side
+    static_assert(RPL * VS <= 32, "tensor-memory columns");
+    extern __shared__ __align__(128) unsigned char smem[];
     float* YS = (float*)smem;                                  // [BZ+2][PBY][W]
-    float* XH = YS + (BZ + 2) * PBY * W;                       // [2][BZ][W]   rows -1 and PBY
-    float* ZH = XH + 2 * BZ * W;                               // [2][PBY+2][W] planes -1 and BZ
-    float* HS = ZH + 2 * (PBY + 2) * W;                        // [NH][W]
-    float* GS = HS + G::NH * W;                                // [BZ][PBY][W] backward G_s
+    float* HS = YS + (BZ + 2) * PBY * W;                       // [2][NH][W] raw halo rows of each chain
+    float* GS = HS + 2 * NH * W;                               // [BZ][PBY][W] stack values
     __shared__ double sh[33];
     __shared__ int nbs[8];
-    __shared__ __align__(8) unsigned long long gs_bar;   // backward: completion of the G_s prefetch
+    __shared__ PersArrays arr;
+    __shared__ __align__(8) unsigned long long full[2], pub[2];
+    __shared__ unsigned tmem_slot;
     const int4 tb = ctl.table[blockIdx.x];
     const Rep& R = reps[tb.x];
     const int b = tb.y;
-    const int fown = tb.z + tb.y;   // own step counter
     const int ny = R.ny, nz = R.nz, N = R.N, nA = R.nA;
     const int plane = W * ny;
     const size_t V = (size_t)R.V;
@@ -267,293 +534,198 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
     const int by = b % nby, bz = b / nby;
     const int y0 = by * PBY, z0 = bz * BZ;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int hf = lane / LPR, li = lane - hf * LPR;   // lane half (row group) and lane within the row
-    const int xo = VEC * li;
-    const int seg = lane - li;
-    const int lsrc = seg + ((li + LPR - 1) & (LPR - 1)), rsrc = seg + ((li + 1) & (LPR - 1));
-    // Each 1-D pass is applied as c + r (a + d) with r = alpha / (1 - 2 alpha), i.e. the
-    // stencil's pass divided by its centre weight be = 1 - 2 alpha; the three passes then give
-    // sigma / be^3, and be^3 is folded into the Boltzmann factors (and into q at its write-out).
-    const double be_d = 1.0 - 2.0 * R.alpha;
-    const float rr = (float)(R.alpha / be_d), be3 = (float)(be_d * be_d * be_d);
-    const unsigned long long rr2 = pk2(rr, rr), be32 = pk2(be3, be3);
+    int* fown = ctl.flags + (size_t)(tb.z + tb.y) * kFlagStride;   // own step counters: +0 forward, +kFlagChain
     if (threadIdx.x < 8) {
         const int k = threadIdx.x < 4 ? threadIdx.x : threadIdx.x + 1;   // skip the centre
         const int dy = k % 3 - 1, dz = k / 3 - 1;
         nbs[threadIdx.x] = tb.z + (by + dy + nby) % nby + nby * ((bz + dz + nbz) % nbz);
     }
-    // halo row h -> (row r, plane pl) of the brick's frame, r in -1..PBY, pl in -1..BZ
-    auto halo_rp = [&](int h, int& r, int& pl) {
-        if (h < 2 * (BZ + 2)) { r = (h < BZ + 2) ? -1 : PBY; pl = h % (BZ + 2) - 1; }
-        else { const int h2 = h - 2 * (BZ + 2); pl = (h2 < PBY) ? -1 : BZ; r = h2 % PBY; }
-    };
-    // where the x-filtered halo row lives: a y-halo row of an own plane, or a z-halo plane row
-    auto halo_dst = [&](int r, int pl) -> float* {
-        if (pl >= 0 && pl < BZ) return XH + ((r < 0 ? 0 : 1) * BZ + pl) * W;
-        return ZH + ((pl < 0 ? 0 : 1) * (PBY + 2) + (r + 1)) * W;
-    };
-    __shared__ int hoff[2 * (BZ + 2) + 2 * PBY];   // global row offsets of the halo rows
-    for (int h = threadIdx.x; h < G::NH; h += 32 * PWARPS) {
-        int r, pl;
-        halo_rp(h, r, pl);
-        const int y = (y0 + r + ny) % ny, z = (z0 + pl + nz) % nz;
-        hoff[h] = z * plane + y * W;
+    if (threadIdx.x < 4)
+        arr.exch[threadIdx.x >> 1][threadIdx.x & 1] =
+            (float*)(threadIdx.x == 0 ? R.del0 : threadIdx.x == 1 ? R.del1 : threadIdx.x == 2 ? R.Gp0 : R.Gp1);
+    if (threadIdx.x == 4) arr.stack = (float*)R.G;
+    if (threadIdx.x == 5) arr.V = V;
+    // the first inputs: G_0 = 1 and G+_{N+1} = 1
+    for (int i = threadIdx.x; i < 2 * NH * W; i += 32 * (NW + kXWarps)) HS[i] = 1.0f;
+    if (w == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(saddr(&tmem_slot)), "r"(TCOLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
-    // step counters of a replica's bricks are equal at launch (unsigned: they may wrap in long runs)
-    const unsigned c0 = (unsigned)ctl.flags[(size_t)fown * kFlagStride];
-    bool aborted = ld_acquire(ctl.abort) != 0;
-
-    auto xpass = [&](const float (&v)[VEC], float (&o)[VEC]) {   // x pass of a periodic row: v + r (left + right)
-        const float lv = __shfl_sync(0xffffffffu, v[VEC - 1], lsrc);
-        const float rv = __shfl_sync(0xffffffffu, v[0], rsrc);
-        float a[VEC], d[VEC];
-#pragma unroll
-        for (int k = 0; k < VEC; ++k) {
-            a[k] = k ? v[k - 1] : lv;
-            d[k] = (k + 1 < VEC) ? v[k + 1] : rv;
+    if (threadIdx.x == 0) {
+        for (int c = 0; c < 2; ++c) {
+            bar_init(&full[c], 64);
+            bar_init(&pub[c], NW);
         }
-        mixv<VEC>(a, v, d, rr, rr2, o);
-    };
-    auto ys = [&](int pl, int r) { return YS + ((pl + 1) * PBY + r) * W + xo; };
-    const bool face_plane = (w == 0 || w == BZ - 1);
-    auto is_boundary = [&](int r) { return face_plane || r == 0 || r == PBY - 1; };
-    // own plane never wraps: offset of (row r, plane w) is own0 + r * W
-    const size_t own0 = (size_t)(z0 + w) * plane + (size_t)y0 * W + xo;
-    auto row_of = [&](int p) { return hf * RPL + p; };
-
-    float e[RPL][VEC];
-    auto load_e = [&](int species) {
-        const float* E = (const float*)R.E + (size_t)species * V;
-#pragma unroll
-        for (int p = 0; p < RPL; ++p) {
-            ldv<VEC>(E + own0 + (size_t)row_of(p) * W, e[p]);
-            scalev<VEC>(be3, be32, e[p]);
-        }
-    };
-    // backward: G_s of the brick into GS, issued by thread 0 as one bulk copy per plane (the
-    // plane's PBY rows are contiguous in memory and in GS); the copies complete on gs_bar
-    unsigned gs_phase = 0;
-    bool gs_pending = false, gs_dead = false;
-    auto prefetch_gs = [&](int s) {
-        if (gs_dead) return;   // a copy that never completed: issue no more
-        if (threadIdx.x == 0) {
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // after the generic reads of GS
-            const float* Gs = (const float*)R.G + (size_t)(s - 1) * V + (size_t)z0 * plane + (size_t)y0 * W;
-            bar_expect(&gs_bar, (unsigned)(BZ * PBY * W * sizeof(float)));
-            for (int pl = 0; pl < BZ; ++pl)
-                bulk_g2s(GS + pl * PBY * W, Gs + (size_t)pl * plane, (unsigned)(PBY * W * sizeof(float)), &gs_bar);
-        }
-        gs_pending = true;
-    };
-    // bounded wait for the pending prefetch; on timeout the CTA reports it, raises the abort and
-    // stops prefetching (the copy stays pending for the last wait at the end of the sweep)
-    auto wait_gs = [&]() {
-        if (!gs_pending || gs_dead) return;
-        for (long long spins = 0; !bar_test(&gs_bar, gs_phase); ++spins) {
-            if (spins > kGsSpinLimit) {
-                atomicOr(ctl.status, (int)ST_TIMEOUT);
-                atomicExch(ctl.abort, 1);
-                aborted = true;
-                gs_dead = true;
-                return;
-            }
-        }
-        gs_phase ^= 1u;
-        gs_pending = false;
-    };
-
-    // the first input (G_0 = 1, or G+_{N+1} = 1): its x pass is 1 + 2 r everywhere
-    const float one = 1.0f + 2.0f * rr;
-    float xf[RPL][VEC];
-#pragma unroll
-    for (int p = 0; p < RPL; ++p)
-#pragma unroll
-        for (int k = 0; k < VEC; ++k) xf[p][k] = one;
-    for (int i = threadIdx.x; i < (2 * BZ + 2 * (PBY + 2)) * W; i += 32 * PWARPS) XH[i] = one;   // XH and ZH
-    float qacc[BWD ? RPL : 1][VEC];
-#pragma unroll
-    for (int p = 0; p < (BWD ? RPL : 1); ++p)
-#pragma unroll
-        for (int k = 0; k < VEC; ++k) qacc[p][k] = 0.f;
-    float qsum = 0.f;
-    int species = BWD ? (N <= nA ? 0 : 1) : (1 <= nA ? 0 : 1);
-    load_e(species);
-    if (BWD) {
-        if (threadIdx.x == 0) bar_init(&gs_bar);
-        __syncthreads();
-        prefetch_gs(N);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    // step counters of a replica's bricks are equal at launch (unsigned: they may wrap in long runs);
+    // read by both of a chain's exchange warps before either publishes
+    const unsigned c0 = w >= NW ? (unsigned)fown[((w - NW) >> 1) * kFlagChain] : 0u;
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 
-    auto write_q = [&](int sp) {   // a block's quadrature, scaled back by be^3
-        float* q = (float*)R.q + (size_t)sp * V;
-#pragma unroll
-        for (int p = 0; p < (BWD ? RPL : 1); ++p) {
-            float o[VEC];
-#pragma unroll
-            for (int k = 0; k < VEC; ++k) o[k] = qacc[p][k];
-            scalev<VEC>(be3, be32, o);
-            stv<VEC>(q + own0 + (size_t)row_of(p) * W, o);
-#pragma unroll
-            for (int k = 0; k < VEC; ++k) qacc[p][k] = 0.f;
-        }
-    };
-
-    for (int j = 0; j < N; ++j) {
-        const int s = BWD ? N - j : j + 1;
-        const int sp = (s <= nA) ? 0 : 1;
-        if (sp != species) {
-            if (BWD) write_q(species);   // leaving the B block: its quadrature is complete
-            species = sp;
-            load_e(species);
-        }
-        // halo of the previous step, x-filtered into XH / ZH; each warp copies and filters the
-        // rows of its own lane halves (a __syncwarp makes every lane's copied chunk visible)
-        if (j > 0) {
-            wait_nb(ctl, nbs, c0 + (unsigned)j, aborted);
-            const float* src = BWD ? (const float*)(((j - 1) & 1) ? R.Gp1 : R.Gp0)
-                                   : (const float*)R.G + (size_t)(s - 2) * V;
-            {
-                const int i = lane / CH, ch = lane - i * CH;
-                for (int h0 = w * HALVES; h0 < G::NH; h0 += PWARPS * HALVES)
-                    if (i < HALVES) cp16(HS + (h0 + i) * W + 4 * ch, src + hoff[h0 + i] + 4 * ch);
-            }
-            cpc();
-            cpw0();
-            __syncwarp();
-            for (int h0 = w * HALVES; h0 < G::NH; h0 += PWARPS * HALVES) {
-                const int h = h0 + hf;
-                float v[VEC], o[VEC];
-                ldv<VEC>(HS + h * W + xo, v);
-                xpass(v, o);
-                int r, pl;
-                halo_rp(h, r, pl);
-                stv<VEC>(halo_dst(r, pl) + xo, o);
-            }
-        }
-        __syncthreads();
-        // y pass of the own plane in registers (its two y-halo rows from XH), into YS
-        {
-            float up[VEC], dn[VEC];   // the row above the lane's first row, below its last
-            ldv<VEC>(XH + w * W + xo, up);           // row -1
-            ldv<VEC>(XH + (BZ + w) * W + xo, dn);    // row PBY
-            if constexpr (HALVES == 2) {   // rows across the two lane halves
-#pragma unroll
-                for (int k = 0; k < VEC; ++k) {
-                    const float last = __shfl_xor_sync(0xffffffffu, xf[RPL - 1][k], LPR);
-                    const float first = __shfl_xor_sync(0xffffffffu, xf[0][k], LPR);
-                    if (hf == 1) up[k] = last;
-                    else dn[k] = first;
+    if (w >= NW) {
+        // ---- exchange warps, two per chain: per step publish, wait for the neighbours, copy halo rows ----
+        regs_dec<PersRegs<NW>::exchange>();
+        const int c = (w - NW) >> 1, part = (w - NW) & 1;   // part 0: rows -1 and plane -1, 1: rows PBY and plane BZ
+        fown += c * kFlagChain;
+        bool aborted = ld_acquire(ctl.abort) != 0, dead = false;
+        const int* nbf = ctl.flags + (size_t)nbs[lane & 7] * kFlagStride + c * kFlagChain;
+        constexpr int RPI = 32 / CH;                        // rows a warp copies at once
+        const int lr = lane / CH, lc = 4 * (lane - lr * CH);
+        float* hdst = HS + (c * NH + part * (NH / 2) + lr) * W + lc;
+        const int yrow = (part ? (y0 + PBY == ny ? 0 : y0 + PBY) : (y0 == 0 ? ny - 1 : y0 - 1)) * W + lc;
+        const int zpl = (part ? (z0 + BZ == nz ? 0 : z0 + BZ) : (z0 == 0 ? nz - 1 : z0 - 1)) * plane + y0 * W + lc;
+        for (int j = 0; j < N; ++j) {
+            bar_wait(&pub[c], (unsigned)(j & 1), ctl, dead);
+            // pub orders every warp's boundary stores before this release store, and release is
+            // cumulative, so a CTA whose acquire load reads the new counter sees them
+            const unsigned target = c0 + (unsigned)j + 1u;
+            if (part == 0 && lane == 0) st_release(fown, (int)target);
+            if (j + 1 >= N) break;
+            // lanes 0..7 poll one neighbour each; every 32 polls they look at the abort flag
+            if (lane < 8 && !aborted) {
+                int spins = 0;
+                while ((int)((unsigned)ld_acquire(nbf) - target) < 0) {   // wrap-safe: counters only grow
+                    if ((++spins & 31) == 0) {
+                        if (ld_acquire(ctl.abort) != 0) {
+                            aborted = true;
+                            break;
+                        }
+                        if (spins > ctl.limit) {
+                            atomicOr(ctl.status, (int)ST_TIMEOUT);
+                            atomicExch(ctl.abort, 1);
+                            aborted = true;
+                            break;
+                        }
+                    }
+                    __nanosleep(32);
                 }
             }
-            float prev[VEC];
+            aborted = __any_sync(0xffffffffu, aborted);
+            const float* src = level_of(arr, c, N, (N + 1) / 2, j);
+            if (lr < RPI) {
+#pragma unroll 3
+                for (int i0 = 0; i0 < BZ + 2; i0 += RPI) {   // row -1 (PBY) of planes -1..BZ
+                    const int i = i0 + lr;
+                    int z = z0 - 1 + i;
+                    z = z < 0 ? z + nz : (z >= nz ? z - nz : z);
+                    if ((BZ + 2) % RPI == 0 || i < BZ + 2) cp16(hdst + i0 * W, src + z * plane + yrow);
+                }
+#pragma unroll 2
+                for (int i0 = 0; i0 < PBY; i0 += RPI)        // the own rows of plane -1 (BZ)
+                    cp16(hdst + (BZ + 2 + i0) * W, src + zpl + (i0 + lr) * W);
+            }
+            cp_arrive(&full[c]);
+        }
+    } else {
+        // ---- compute warps ----
+        regs_inc<PersRegs<NW>::compute>();
+        const int hf = lane / LPR, li = lane - hf * LPR;   // lane half (row group) and lane within the row
+        const int xo = VEC * li;
+        const int seg = lane - li;
+        const int lsrc = seg + ((li + LPR - 1) & (LPR - 1)), rsrc = seg + ((li + 1) & (LPR - 1));
+        // Each 1-D pass is applied as c + r (a + d) with r = alpha / (1 - 2 alpha), i.e. the
+        // stencil's pass divided by its centre weight be = 1 - 2 alpha; the three passes then give
+        // sigma / be^3, and be^3 is folded into the Boltzmann factors (and into q at its write-out).
+        const double be_d = 1.0 - 2.0 * R.alpha;
+        const float rr = (float)(R.alpha / be_d), be3 = (float)(be_d * be_d * be_d);
+        const unsigned long long be32 = pk2(be3, be3);
+        // own plane never wraps: (row r, plane w) is own0 + r * W
+        const size_t own0 = (size_t)(z0 + w) * plane + (size_t)(y0 + hf * RPL) * W + xo;
+        PersWarp k = {arr, ctl, full, pub, YS, HS, GS + (w * PBY + hf * RPL) * W + xo, own0,
+                      (size_t)(z0 + w) * plane + (size_t)y0 * W + 32 * lane,
+                      N, nA, (N + 1) / 2, w, lane, hf, xo, lsrc, rsrc, w == 0 || w == BZ - 1, rr, pk2(rr, rr),
+                      tmem_slot + ((unsigned)((w & 3) * 32) << 16) + (unsigned)((w >> 2) * 128), 0.f, false};
+        const unsigned tbase = k.tbase;
+
+        // tensor memory regions: 0, 1 Boltzmann factors of A, B (scaled by be^3); 2, 3 quadratures
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) prev[k] = up[k];
+        for (int I = 0; I < 2; ++I) {
+            const float* E = (const float*)R.E + (size_t)I * V;
 #pragma unroll
             for (int p = 0; p < RPL; ++p) {
-                float yv[VEC], cur[VEC];
+                float t[VS], zero[VS], e[VEC];
+                ldv<VEC>(E + own0 + (size_t)p * W, e);
+                scalev<VEC>(be3, be32, e);
 #pragma unroll
-                for (int k = 0; k < VEC; ++k) cur[k] = xf[p][k];
-                if (p + 1 < RPL) mixv<VEC>(prev, cur, xf[p + 1 < RPL ? p + 1 : p], rr, rr2, yv);
-                else mixv<VEC>(prev, cur, dn, rr, rr2, yv);
-#pragma unroll
-                for (int k = 0; k < VEC; ++k) {
-                    prev[k] = cur[k];
-                    xf[p][k] = yv[k];   // xf now holds the y-filtered rows
+                for (int i = 0; i < VS; ++i) {
+                    t[i] = i < VEC ? e[i < VEC ? i : 0] : 0.f;
+                    zero[i] = 0.f;
                 }
-                stv<VEC>(ys(w, row_of(p)), yv);
+                tm_st<VS>(tbase + I * 32 + p * VS, t);
+                tm_st<VS>(tbase + (2 + I) * 32 + p * VS, zero);
             }
         }
-        // y pass of the z-halo planes, one row per lane half (PBY rows of each of the two planes)
-        for (int t0 = w * HALVES; t0 < 2 * PBY; t0 += PWARPS * HALVES) {
-            const int t = t0 + hf;
-            const int side = t / PBY, r = t % PBY;
-            const float* zr = ZH + (side * (PBY + 2) + r + 1) * W + xo;
-            float a[VEC], c[VEC], d[VEC], o[VEC];
-            ldv<VEC>(zr - W, a);
-            ldv<VEC>(zr, c);
-            ldv<VEC>(zr + W, d);
-            mixv<VEC>(a, c, d, rr, rr2, o);
-            stv<VEC>(ys(side ? BZ : -1, r), o);
-        }
-        __syncthreads();
-        // z pass and step output
-        float* dst = BWD ? (float*)((j & 1) ? R.Gp1 : R.Gp0) : (float*)R.G + (size_t)(s - 1) * V;
-        if (BWD) wait_gs();
-        float out[RPL][VEC];
+        tm_wait_st();
+
+        const float one = 1.0f + 2.0f * rr;   // the x pass of G_0 = 1 and of G+_{N+1} = 1
+        float xF[RPL][VEC], xB[RPL][VEC];
 #pragma unroll
-        for (int p = 0; p < RPL; ++p) {
-            const int r = row_of(p);
-            float a[VEC], d[VEC], sg[VEC];
-            ldv<VEC>(ys(w - 1, r), a);
-            ldv<VEC>(ys(w + 1, r), d);
-            mixv<VEC>(a, xf[p], d, rr, rr2, sg);
-            mulv<VEC>(e[p], sg, out[p]);
-            if constexpr (BWD) {
-                float g[VEC];
-                ldv<VEC>(GS + (w * PBY + r) * W + xo, g);
-                fmav<VEC>(g, sg, qacc[p]);
-            } else {
-                if (s == N) {
-                    float t = out[p][0] + out[p][1];
-                    if constexpr (VEC == 3) t = t + out[p][2];
-                    if constexpr (VEC == 4) t = t + (out[p][2] + out[p][3]);
-                    qsum += t;
-                }
-            }
-            if (is_boundary(r) && (!BWD || s > 1)) stv<VEC>(dst + own0 + (size_t)r * W, out[p]);
-        }
-        // publish the boundary of this step: the CTA barrier orders every thread's boundary stores
-        // before thread 0's release store, and release is cumulative, so a CTA whose acquire load
-        // reads the new counter sees them.  The barrier also ends every warp's reads of YS, XH
-        // and ZH for this step.
-        __syncthreads();
-        if (threadIdx.x == 0) st_release(ctl.flags + (size_t)fown * kFlagStride, (int)(c0 + (unsigned)j + 1u));
-        if (BWD && s > 1) prefetch_gs(s - 1);   // GS slots of this thread were read above
+        for (int p = 0; p < RPL; ++p)
 #pragma unroll
-        for (int p = 0; p < RPL; ++p) {
-            if (!BWD && !is_boundary(row_of(p))) stv<VEC>(dst + own0 + (size_t)row_of(p) * W, out[p]);
-            xpass(out[p], xf[p]);
+            for (int i = 0; i < VEC; ++i) xF[p][i] = xB[p][i] = one;
+
+#pragma unroll 1
+        for (int j = 0; j < N; ++j) {
+            pers_unit<W, PBY, BZ, NW, 0>(k, xF, j);
+            pers_unit<W, PBY, BZ, NW, 1>(k, xB, j);
         }
-    }
-    if (BWD) {   // the A block ends at s = 1
-        if (gs_dead) {   // one more bounded wait for a copy still in flight
-            for (long long spins = 0; spins <= kGsSpinLimit && !bar_test(&gs_bar, gs_phase); ++spins) {
+        // both quadratures, scaled back by be^3
+#pragma unroll
+        for (int I = 0; I < 2; ++I) {
+            float* q = (float*)R.q + (size_t)I * V;
+#pragma unroll
+            for (int p = 0; p < RPL; ++p) {
+                float t[VS], o[VEC];
+                tm_ld<VS>(tbase + (2 + I) * 32 + p * VS, t);
+                tm_wait_ld<VS>(t);
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) o[i] = t[i];
+                scalev<VEC>(be3, be32, o);
+                stv<VEC>(q + own0 + (size_t)p * W, o);
             }
         }
-        write_q(species);
-    } else {
-        const double t = block_sum((double)qsum, sh);
-        const int bl = ctl.table[blockIdx.x].y;   // reloaded: not kept live through the sweep
-        if (threadIdx.x == 0) slot(R, P_Q)[bl] = t;
-        if (bl == 0) {   // slots past the replica's bricks (the propagator tiling may have more)
-            const int nb = nby * nbz;
-            for (int i = threadIdx.x + nb; i < R.ntiles; i += 32 * PWARPS) slot(R, P_Q)[i] = 0.0;
+        // the brick's share of Q, the end of the tensor memory's use (compute warps only: the
+        // exchange warps hold too few registers to join code that follows both branches)
+        const double t = warp_sum((double)k.qsum);
+        if (lane == 0) sh[w] = t;
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        compute_sync(32 * NW);
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        if (w == 0) {
+            const double q = warp_sum(lane < NW ? sh[lane] : 0.0);
+            if (lane == 0) slot(R, P_Q)[b] = q;
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_slot), "r"(TCOLS) : "memory");
+        }
+        if (b == 0) {   // slots past the replica's bricks (the propagator tiling may have more)
+            for (int i = threadIdx.x + nby * nbz; i < R.ntiles; i += 32 * NW) slot(R, P_Q)[i] = 0.0;
         }
     }
 }
 
-
-template <int W, int PBY, int BZ, bool BWD, int NW>
-__global__ void __launch_bounds__(32 * NW, 16 / NW) k_prop_pers(const Rep* __restrict__ reps, PersCtl ctl) {
-    pers_sweep<W, PBY, BZ, BWD, NW>(reps, ctl);
+template <int W, int PBY, int BZ, int NW>
+__global__ void __launch_bounds__(32 * (NW + kXWarps), 16 / NW) k_prop_pers(const Rep* __restrict__ reps, PersCtl ctl) {
+    pers_sweep<W, PBY, BZ, NW>(reps, ctl);
 }
 
 // Bricks of several row widths (32 to 96 sites) in one launch (batches): each CTA runs the sweep of
 // its replica's width; the launch's dynamic shared memory covers the largest.  128-wide replicas
 // keep launches of their own (with them in the same function the registers would spill).
-template <int BZ, bool BWD, int NW>
-__global__ void __launch_bounds__(32 * NW, 16 / NW) k_prop_pers_mix(const Rep* __restrict__ reps, PersCtl ctl) {
+template <int BZ, int NW>
+__global__ void __launch_bounds__(32 * (NW + kXWarps), 16 / NW) k_prop_pers_mix(const Rep* __restrict__ reps, PersCtl ctl) {
     const Rep& R = reps[ctl.table[blockIdx.x].x];
     const int pby = pers_pby_of(R.nx, R.ny);
     switch (R.nx * 32 + pby) {
-        case 32 * 32 + 8: pers_sweep<32, 8, BZ, BWD, NW>(reps, ctl); break;
-        case 32 * 32 + 16: pers_sweep<32, 16, BZ, BWD, NW>(reps, ctl); break;
-        case 48 * 32 + 8: pers_sweep<48, 8, BZ, BWD, NW>(reps, ctl); break;
-        case 48 * 32 + 16: pers_sweep<48, 16, BZ, BWD, NW>(reps, ctl); break;
-        case 64 * 32 + 8: pers_sweep<64, 8, BZ, BWD, NW>(reps, ctl); break;
-        case 64 * 32 + 16: pers_sweep<64, 16, BZ, BWD, NW>(reps, ctl); break;
-        case 96 * 32 + 8: pers_sweep<96, 8, BZ, BWD, NW>(reps, ctl); break;
+        case 32 * 32 + 8: pers_sweep<32, 8, BZ, NW>(reps, ctl); break;
+        case 32 * 32 + 16: pers_sweep<32, 16, BZ, NW>(reps, ctl); break;
+        case 48 * 32 + 8: pers_sweep<48, 8, BZ, NW>(reps, ctl); break;
+        case 48 * 32 + 16: pers_sweep<48, 16, BZ, NW>(reps, ctl); break;
+        case 64 * 32 + 8: pers_sweep<64, 8, BZ, NW>(reps, ctl); break;
+        case 64 * 32 + 16: pers_sweep<64, 16, BZ, NW>(reps, ctl); break;
+        case 96 * 32 + 8: pers_sweep<96, 8, BZ, NW>(reps, ctl); break;
         default: break;   // not reached: the host builds mixed launches of these widths only
     }
 }
@@ -582,29 +754,26 @@ bool pers_supported(const Rep& R, int bz, int nw, int nsm) {
 int pers_bricks(const Rep& R, int bz) { return (R.ny / pers_pby(R)) * (R.nz / bz); }
 
 namespace {
+// Also checks that the registers the kernel launches with cover the shares its warps take
+// (setmaxnreg would wait for ever if they did not).
+template <int NW, typename K>
+cudaError_t pers_attr_of(K kernel, size_t smem) {
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess &&
+        fa.numRegs * (NW + kXWarps) < PersRegs<NW>::compute * NW + PersRegs<NW>::exchange * kXWarps)
+        e = cudaErrorInvalidConfiguration;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    return e;
+}
 template <int W, int PBY, int BZ, int NW>
 cudaError_t pers_attr() {
-    const int sm = (int)pers_smem_bytes(W, PBY, BZ);
-    cudaError_t e = cudaFuncSetAttribute(k_prop_pers<W, PBY, BZ, false, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_prop_pers<W, PBY, BZ, true, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_prop_pers<W, PBY, BZ, false, NW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_prop_pers<W, PBY, BZ, true, NW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    return e;
+    return pers_attr_of<NW>(k_prop_pers<W, PBY, BZ, NW>, pers_smem_bytes(W, PBY, BZ));
 }
 template <int BZ, int NW>
 cudaError_t pers_mix_attr() {
-    const int sm = (int)pers_mix_smem_bytes(BZ);
-    cudaError_t e = cudaFuncSetAttribute(k_prop_pers_mix<BZ, false, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_prop_pers_mix<BZ, true, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_prop_pers_mix<BZ, false, NW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_prop_pers_mix<BZ, true, NW>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    return e;
+    return pers_attr_of<NW>(k_prop_pers_mix<BZ, NW>, pers_mix_smem_bytes(BZ));
 }
 }  // namespace
 
@@ -640,7 +809,7 @@ namespace {
 // The SM that runs each CTA of a launch shaped like the sweep (same block size, shared memory
 // and cooperative attribute), for the placement of bricks on SMs.
 template <int NW>
-__global__ void __launch_bounds__(32 * NW, 16 / NW) k_pers_place(int* smid) {
+__global__ void __launch_bounds__(32 * (NW + kXWarps), 16 / NW) k_pers_place(int* smid) {
     if (threadIdx.x == 0) {
         unsigned id;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
@@ -652,7 +821,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) k_pers_place(int* smid) {
 int pers_placement(int bz, int nw, int nbricks, int* d_smid, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nbricks);
-    cfg.blockDim = dim3(32 * nw);
+    cfg.blockDim = dim3(32 * (nw + kXWarps));
     cfg.dynamicSmemBytes = pers_smem_bytes(128, 8, bz);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -672,7 +841,7 @@ int pers_placement(int bz, int nw, int nbricks, int* d_smid, cudaStream_t stream
     return (int)e;
 }
 
-int launch_prop_pers(const Launch& L, bool bwd, int width, int pby, int bz, int nw, int nbricks, const int4* table,
+int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, int nbricks, const int4* table,
                      int* flags, int* abortf, int limit) {
     PersCtl ctl;
     ctl.flags = flags;
@@ -682,7 +851,7 @@ int launch_prop_pers(const Launch& L, bool bwd, int width, int pby, int bz, int 
     ctl.limit = limit;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nbricks);
-    cfg.blockDim = dim3(32 * nw);
+    cfg.blockDim = dim3(32 * (nw + kXWarps));
     cfg.dynamicSmemBytes = width ? pers_smem_bytes(width, pby, bz) : pers_mix_smem_bytes(bz);
     cfg.stream = L.stream;
     cudaLaunchAttribute attr[1];
@@ -691,18 +860,12 @@ int launch_prop_pers(const Launch& L, bool bwd, int width, int pby, int bz, int 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaError_t e = cudaErrorInvalidValue;
-#define DSCF_PERS_LAUNCH(WW, PP, BB, NN)                                                                  \
-    e = bwd ? cudaLaunchKernelEx(&cfg, k_prop_pers<WW, PP, BB, true, NN>, L.reps, ctl)                    \
-            : cudaLaunchKernelEx(&cfg, k_prop_pers<WW, PP, BB, false, NN>, L.reps, ctl)
+#define DSCF_PERS_LAUNCH(WW, PP, BB, NN) e = cudaLaunchKernelEx(&cfg, k_prop_pers<WW, PP, BB, NN>, L.reps, ctl)
     if (bz == 16 && nw == 16) {
-        if (width == 0)
-            e = bwd ? cudaLaunchKernelEx(&cfg, k_prop_pers_mix<16, true, 16>, L.reps, ctl)
-                    : cudaLaunchKernelEx(&cfg, k_prop_pers_mix<16, false, 16>, L.reps, ctl);
+        if (width == 0) e = cudaLaunchKernelEx(&cfg, k_prop_pers_mix<16, 16>, L.reps, ctl);
         else DSCF_PERS_SWITCH(16, 16, DSCF_PERS_LAUNCH)
     } else if (bz == 8 && nw == 8) {
-        if (width == 0)
-            e = bwd ? cudaLaunchKernelEx(&cfg, k_prop_pers_mix<8, true, 8>, L.reps, ctl)
-                    : cudaLaunchKernelEx(&cfg, k_prop_pers_mix<8, false, 8>, L.reps, ctl);
+        if (width == 0) e = cudaLaunchKernelEx(&cfg, k_prop_pers_mix<8, 8>, L.reps, ctl);
         else DSCF_PERS_SWITCH(8, 8, DSCF_PERS_LAUNCH)
     }
 #undef DSCF_PERS_LAUNCH
