@@ -7,7 +7,8 @@
 // implicit GEMM over (offset, input channel) in BF16 with FP32 accumulation; weight gradients are
 // per-offset GEMMs over sites.  The forward convolutions run on tcgen05 (operands in shared
 // memory, accumulators in tensor memory; dscf_tc.cu) when nx is a multiple of 128 and ny of 8,
-// and with warp-level mma.sync m16n8k16 otherwise (and for the backward pass).  Activations are stored
+// and with warp-level mma.sync m16n8k16 on input blocks staged in shared memory otherwise (and for
+// the backward pass).  Activations are stored
 // channel-last in BF16 with channel counts padded to multiples of 16 (zero weights in the pad);
 // the tcgen05 forward keeps its own copies in a padded channel-group layout (x16f, h1p, h2p) from
 // which it stages rows by bulk copies, and the backward pass reads channel-last copies of them.
@@ -19,6 +20,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/dscf.h"
@@ -34,14 +36,12 @@ constexpr int NL = 3;
 constexpr int KVOL = 125;
 constexpr int CIN[NL] = {2, 32, 32}, COUT[NL] = {32, 32, 2};
 constexpr int CINP[NL] = {16, 32, 32}, COUTP[NL] = {32, 32, 16};
+constexpr int NTF[NL] = {4, 4, 1};   // n-tiles of 8 output channels of the mma.sync forward
 constexpr size_t wcount(int l) { return (size_t)COUT[l] * CIN[l] * KVOL; }
 constexpr size_t NPARAM = wcount(0) + 32 + wcount(1) + 32 + wcount(2) + 2;
 
 enum { EPI_TANH = 0, EPI_LIN_F32 = 1, EPI_DTANH = 2 };
 
-__device__ __forceinline__ int wrapd(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
-
-__device__ __forceinline__ unsigned ld32(const bf16* p) { return *(const unsigned*)p; }
 __device__ __forceinline__ unsigned pack2(bf16 lo, bf16 hi) {
     return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
 }
@@ -52,88 +52,177 @@ __device__ __forceinline__ void mma16816(float* c, const unsigned* a, const unsi
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
+__device__ __forceinline__ unsigned sm_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void ldsm4(unsigned addr, unsigned (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldsm4t(unsigned addr, unsigned (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src));
+}
+// the same, zeros instead of the source where !ok
+__device__ __forceinline__ void cp_async16z(unsigned dst, const void* src, bool ok) {
+    const int n = ok ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(n));
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Implicit-GEMM circular 5^3 convolution, one warp per 16 consecutive sites of an x row:
+// Byte offset of 16-byte chunk c (8 channels) of staged site i, C channels per site: chunks are
+// permuted within 128-byte lines so that the 8 consecutive sites of an ldmatrix row group fall
+// into different banks.
+template <int C>
+__device__ __forceinline__ unsigned swz(int i, int c) {
+    if constexpr (C == 32) return (unsigned)(i * 64 + ((c ^ ((i >> 1) & 3)) << 4));
+    else return (unsigned)(i * 32 + ((c ^ ((i >> 2) & 1)) << 4));
+}
+
+// Implicit-GEMM circular 5^3 convolution on mma.sync:
 //   out[r][co] = sum_o sum_ci in[r + o][ci] W[o][co][ci]  (+ epilogue)
-// in: [B][V][CI] bf16, W: [125][CO][CI] bf16.  Epilogues: tanh(acc + bias) -> bf16;
-// acc + bias -> f32; acc * (1 - h^2) with h the forward activation -> bf16.
-// With EPI_DTANH and bgrad != NULL, the FP32 values (before rounding to BF16) are also summed per
-// channel into bgrad: the bias gradient of the layer whose activation is hact.
-template <int CI, int CO, int EPI>
-__global__ void __launch_bounds__(128) k_conv(const bf16* __restrict__ in, const bf16* __restrict__ W,
-                                              const float* __restrict__ bias, int cout, const bf16* __restrict__ hact,
-                                              void* __restrict__ out, int nx, int ny, int nz, int ntiles,
-                                              float* __restrict__ bgrad) {
-    const int lane = threadIdx.x & 31;
-    const int mt = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (mt >= ntiles) return;
+// in: [B][V][CI] bf16; W: fragments (k_prep_w).  A CTA of four warps computes a block of 16 MX x 4 x
+// (4 / MX) sites whose input, two sites larger on every side, it stages once in shared memory; a
+// warp holds four m-tiles of 16 sites, so an offset's weight fragments (16-byte loads in fragment
+// order, fetched an offset ahead) serve four tiles and an input fragment is one ldmatrix.  Blocks of
+// two tiles in x for rows of a multiple of 32 sites (fewest halo sites), of one otherwise; two CTAs
+// per SM (32 input channels: 110 KB each), so one stages while the other computes.
+// Tensor-pipe bound: per offset a warp issues 4 x 2 x 4 MMAs against 8 ldmatrix (32 -> 32 channels:
+// 8 x 32^3 sites in 240 us = 280 TFLOP/s; 32 -> 8: 167 us, ldmatrix bound; before, with 4-byte
+// gathers from global memory and no reuse of weights, a gradient's five convolutions took 2.4 ms).
+// Each accumulator takes its products in the order (offset, channel group).
+// Epilogues: tanh(acc + bias) -> bf16; acc + bias -> f32 (channels 0 and 1 of 16 stored per site);
+// acc * (1 - h^2) with h the forward activation -> bf16, with bgrad != NULL also summed per channel
+// into bgrad in FP32: the bias gradient of the layer whose activation is hact.
+constexpr int CV_TY = 4;
+template <int MX>
+struct ConvTile {
+    static constexpr int TZ = 4 / MX, HX = 16 * MX + 4, HY = CV_TY + 4, HZ = TZ + 4, SITES = HX * HY * HZ;
+};
+template <int CI, int NT, int EPI, int MX>
+__global__ void __launch_bounds__(128, CI == 32 ? 2 : 3) k_conv(const bf16* __restrict__ in, const uint4* __restrict__ W,
+                                                                const float* __restrict__ bias, int cout,
+                                                                const bf16* __restrict__ hact, void* __restrict__ out,
+                                                                int nx, int ny, int nz, float* __restrict__ bgrad) {
+    using CT = ConvTile<MX>;
+    constexpr int HX = CT::HX, HY = CT::HY, KC = CI / 16, CO = NT == 1 ? 16 : NT * 8;
+    constexpr int WV = KC * NT / 2;            // 16-byte weight vectors per lane and offset
+    extern __shared__ __align__(128) unsigned char smem[];
+    const unsigned sm0 = sm_addr(smem);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int V = nx * ny * nz;
-    const int tpv = V / 16;
-    const int b = mt / tpv;
-    const int s0 = (mt - b * tpv) * 16;
-    const int x0 = s0 % nx, y = (s0 / nx) % ny, z = s0 / (nx * ny);
-    const int g = lane >> 2, t = lane & 3;
+    // block -> sample, origin
+    int t = blockIdx.x;
+    const int nbx = nx / (16 * MX), nby = (ny + CV_TY - 1) / CV_TY, nbz = (nz + CT::TZ - 1) / CT::TZ;
+    const int x0 = (t % nbx) * 16 * MX;
+    t /= nbx;
+    const int y0 = (t % nby) * CV_TY;
+    t /= nby;
+    const int z0 = (t % nbz) * CT::TZ, b = t / nbz;
     const bf16* inb = in + (size_t)b * V * CI;
-    float acc[CO / 8][4];
+    constexpr int CPS = CI / 8;                // 16-byte chunks per site
+    for (int i = tid; i < CT::SITES * CPS; i += 128) {
+        const int site = i / CPS, c = i - site * CPS;
+        const int hx = site % HX, hyz = site / HX, hy = hyz % HY, hz = hyz / HY;
+        int x = x0 + hx - 2, y = y0 + hy - 2, z = z0 + hz - 2;
+        x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+        y = (y % ny + ny) % ny;                // ragged blocks reach further than one wrap
+        z = (z % nz + nz) % nz;
+        cp_async16(sm0 + swz<CI>(site, c), inb + (size_t)((z * ny + y) * nx + x) * CI + c * 8);
+    }
+    cp_async_commit();
+    const uint4* wl = W + lane * WV;
+    uint4 wn[WV];
 #pragma unroll
-    for (int j = 0; j < CO / 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-    for (int o = 0; o < KVOL; ++o) {
-        const int oz = o / 25 - 2, oy = (o / 5) % 5 - 2, ox = o % 5 - 2;
-        const int rowoff = (wrapd(z + oz, nz) * ny + wrapd(y + oy, ny)) * nx;
-        const int sa = rowoff + wrapd(x0 + g + ox, nx);       // site of A row g
-        const int sb = rowoff + wrapd(x0 + g + 8 + ox, nx);   // site of A row g + 8
-        const bf16* Wo = W + (size_t)o * CO * CI;
+    for (int v = 0; v < WV; ++v) wn[v] = __ldg(wl + v);
+    float acc[4][NT][4];
 #pragma unroll
-        for (int kc = 0; kc < CI / 16; ++kc) {
-            unsigned a[4];
-            const int c0 = kc * 16 + 2 * t;
-            a[0] = ld32(inb + (size_t)sa * CI + c0);
-            a[1] = ld32(inb + (size_t)sb * CI + c0);
-            a[2] = ld32(inb + (size_t)sa * CI + c0 + 8);
-            a[3] = ld32(inb + (size_t)sb * CI + c0 + 8);
+    for (int m = 0; m < 4; ++m)
 #pragma unroll
-            for (int j = 0; j < CO / 8; ++j) {
-                unsigned bb[2];
-                const bf16* wr = Wo + (size_t)(j * 8 + g) * CI + c0;
-                bb[0] = ld32(wr);
-                bb[1] = ld32(wr + 8);
-                mma16816(acc[j], a, bb);
+        for (int j = 0; j < NT; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
+    cp_async_wait<0>();
+    __syncthreads();
+    // this warp's tiles: MX = 2: plane w / 2, rows 2 (w % 2) + m / 2, x half m % 2; MX = 1: plane w, row m
+    const int wz = MX == 2 ? w >> 1 : w, wy = MX == 2 ? 2 * (w & 1) : 0;
+    const int row = (lane & 7) + ((lane >> 3) & 1) * 8, ch = lane >> 4;
+    int o = 0;
+#pragma unroll 1
+    for (int ozy = 0; ozy < 25; ++ozy) {
+        const int i0 = ((wz + ozy / 5) * HY + wy + ozy % 5) * HX + row;
+#pragma unroll
+        for (int ox = 0; ox < 5; ++ox, ++o) {
+            unsigned wf[WV * 4];
+#pragma unroll
+            for (int v = 0; v < WV; ++v) {
+                wf[4 * v] = wn[v].x; wf[4 * v + 1] = wn[v].y; wf[4 * v + 2] = wn[v].z; wf[4 * v + 3] = wn[v].w;
+            }
+            if (o + 1 < KVOL) {
+#pragma unroll
+                for (int v = 0; v < WV; ++v) wn[v] = __ldg(wl + (size_t)(o + 1) * 32 * WV + v);
+            }
+            const unsigned base = swz<CI>(i0 + ox, ch);   // tile 0
+#pragma unroll
+            for (int kc = 0; kc < KC; ++kc) {
+                // the other tiles lie a constant number of sites on; a row (HX sites) later the chunk
+                // permutation differs by one fixed bit (HX = 36 or 20), 16 sites later it is the same
+                unsigned a[4][4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int dr = MX == 2 ? m >> 1 : m, di = dr * HX + (MX == 2 ? 16 * (m & 1) : 0);
+                    const unsigned flip = (dr & 1) ? (CI == 32 ? 32u : 16u) : 0u;
+                    ldsm4(sm0 + ((base + di * CI * 2) ^ flip ^ (kc ? 32u : 0u)), a[m]);
+                }
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) mma16816(acc[m][j], a[m], wf + (kc * NT + j) * 2);
             }
         }
     }
-    // epilogue: rows g, g + 8 (sites s0 + g, s0 + g + 8), columns co = 8 j + 2 t, +1
+    // epilogue: rows g, g + 8 of each tile, columns co = 8 j + 2 t, + 1
+    const int g = lane >> 2, tq = lane & 3;
 #pragma unroll
-    for (int j = 0; j < CO / 8; ++j) {
-        const int co = j * 8 + 2 * t;
+    for (int j = 0; j < NT; ++j) {
+        const int co = j * 8 + 2 * tq;
+        const float b0 = (EPI != EPI_DTANH && co < cout) ? bias[co] : 0.f;
+        const float b1 = (EPI != EPI_DTANH && co + 1 < cout) ? bias[co + 1] : 0.f;
         float bs0 = 0.f, bs1 = 0.f;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const size_t site = (size_t)b * V + s0 + g + 8 * h;
-            float v0 = acc[j][2 * h], v1 = acc[j][2 * h + 1];
-            if (EPI == EPI_TANH || EPI == EPI_LIN_F32) {
-                v0 += (co < cout) ? bias[co] : 0.f;
-                v1 += (co + 1 < cout) ? bias[co + 1] : 0.f;
-            }
-            if (EPI == EPI_TANH) {
-                v0 = tanhf(v0);
-                v1 = tanhf(v1);
-                *(unsigned*)((bf16*)out + site * CO + co) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
-            } else if (EPI == EPI_LIN_F32) {
-                *(float2*)((float*)out + site * CO + co) = make_float2(v0, v1);
-            } else {
-                const float h0 = __bfloat162float(hact[site * CO + co]), h1 = __bfloat162float(hact[site * CO + co + 1]);
-                v0 *= 1.f - h0 * h0;
-                v1 *= 1.f - h1 * h1;
-                bs0 += v0;
-                bs1 += v1;
-                *(unsigned*)((bf16*)out + site * CO + co) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+        for (int m = 0; m < 4; ++m) {
+            const int y = y0 + wy + (MX == 2 ? m >> 1 : m), z = z0 + wz;
+            if (y >= ny || z >= nz) continue;
+            const size_t s0 = (size_t)b * V + (size_t)(z * ny + y) * nx + x0 + (MX == 2 ? 16 * (m & 1) : 0) + g;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const size_t site = s0 + 8 * h;
+                float v0 = acc[m][j][2 * h] + b0, v1 = acc[m][j][2 * h + 1] + b1;
+                if (EPI == EPI_TANH) {
+                    v0 = tanhf(v0);
+                    v1 = tanhf(v1);
+                    *(unsigned*)((bf16*)out + site * CO + co) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+                } else if (EPI == EPI_LIN_F32) {
+                    if (tq == 0) *(float2*)((float*)out + site * CO) = make_float2(v0, v1);
+                } else {
+                    v0 = acc[m][j][2 * h];
+                    v1 = acc[m][j][2 * h + 1];
+                    const __nv_bfloat162 hh = *(const __nv_bfloat162*)(hact + site * CO + co);
+                    const float h0 = __low2float(hh), h1 = __high2float(hh);
+                    v0 *= 1.f - h0 * h0;
+                    v1 *= 1.f - h1 * h1;
+                    bs0 += v0;
+                    bs1 += v1;
+                    *(unsigned*)((bf16*)out + site * CO + co) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+                }
             }
         }
         if (EPI == EPI_DTANH && bgrad) {   // sum over the 8 row groups (lane bits 2..4)
 #pragma unroll
-            for (int m = 4; m < 32; m <<= 1) {
-                bs0 += __shfl_xor_sync(0xffffffffu, bs0, m);
-                bs1 += __shfl_xor_sync(0xffffffffu, bs1, m);
+            for (int s = 4; s < 32; s <<= 1) {
+                bs0 += __shfl_xor_sync(0xffffffffu, bs0, s);
+                bs1 += __shfl_xor_sync(0xffffffffu, bs1, s);
             }
             if (g == 0) {
                 if (co < cout) atomicAdd(&bgrad[co], bs0);
@@ -143,86 +232,189 @@ __global__ void __launch_bounds__(128) k_conv(const bf16* __restrict__ in, const
     }
 }
 
-// Weight gradient of one layer: dW[co][ci][o] += sum_r in[r + o][ci] dout[r][co]; a GEMM per
-// offset (M = input channels, N = output channels, K = sites) on tensor cores; each warp covers
-// `chunk` consecutive m-tiles of sites and adds its FP32 partial with atomics.
-template <int CI, int CO>
-__global__ void __launch_bounds__(128) k_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dout,
-                                               float* __restrict__ dW, int cin, int cout, int nx, int ny, int nz,
-                                               int ntiles, int chunk) {
-    const int lane = threadIdx.x & 31;
-    const int o = blockIdx.y;
-    const int w0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * chunk;
-    const int g = lane >> 2, t = lane & 3;
-    const int oz = o / 25 - 2, oy = (o / 5) % 5 - 2, ox = o % 5 - 2;
-    const int V = nx * ny * nz;
-    const int tpv = V / 16;
-    float acc[CI / 16][CO / 8][4];
-#pragma unroll
-    for (int i = 0; i < CI / 16; ++i)
-#pragma unroll
-        for (int j = 0; j < CO / 8; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
-    for (int mt = w0; mt < min(w0 + chunk, ntiles); ++mt) {
-        const int b = mt / tpv;
-        const int s0 = (mt - b * tpv) * 16;
-        const int x0 = s0 % nx, y = (s0 / nx) % ny, z = s0 / (nx * ny);
-        const int rowoff = (wrapd(z + oz, nz) * ny + wrapd(y + oy, ny)) * nx;
-        const bf16* inb = in + (size_t)b * V * CI;
-        const bf16* db = dout + ((size_t)b * V + s0) * CO;
-        // k index = site within the tile: pairs (2t, 2t+1) and (2t+8, 2t+9)
-        int sk[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = 2 * t + (q & 1) + 8 * (q >> 1);
-            sk[q] = rowoff + wrapd(x0 + k + ox, nx);
+// Weight gradient of one layer: dW[co][ci][o] = sum_r in[r + o][ci] dout[r][co], a GEMM per offset
+// (M = input channels, N = output channels, K = sites) on mma.sync.  A CTA keeps the 25 offsets of one
+// dz in registers, spread over 12 warps (three per tensor core: 2 offsets each, the last warp 3; CI x
+// 8 NT accumulators per offset over the lanes), and goes over every nsplit-th tile of 8 rows x 16 MX
+// sites: per tile it stages the rows of dout and the rows of in at plane z + dz, two larger in y
+// and x, in one of two shared-memory buffers while it computes from the other, so a staged site is
+// used by 25 offsets and a dout fragment by a warp's two.  Per 16 sites a warp issues 2 x 2 x 4 MMAs
+// against 6 ldmatrix (32 x 32 channels): tensor-pipe bound.  The tensor core truncates its sums, so
+// a long chain of MMAs drifts (560 of them: 2e-5 of the gradient); every second tile the accumulators
+// are added, rounded, to the CTA's totals in shared memory and start again (32 MMAs: 1e-6).  The
+// totals of a CTA go to part[split][o][CI][8 NT]; k_wgrad_sum adds the splits in order.  8 x 32^3
+// sites: 230 us (32 x 32), 147 and 142 us (32 x 2, 2 x 32); 3.9 ms together with 2-byte gathers and
+// atomics per 128 sites.
+constexpr int WG_TY = 8, WG_WARPS = 12, WG_OFF = 3;   // rows per tile; warps; most offsets per warp
+constexpr int WG_FLUSH = 2;                             // tiles between additions to the totals
+template <int CI, int NT, int CD, int MX>
+struct WgTile {
+    static constexpr int HX = 16 * MX + 4, HY = WG_TY + 4;
+    static constexpr int INB = HX * HY * CI * 2, DB = 16 * MX * WG_TY * CD * 2;   // bytes staged of in and dout
+    static constexpr int SMEM = 2 * (INB + DB) + 25 * CI * 8 * NT * 4;
+};
+template <int CI, int NT, int CD, int MX>   // CD: channels per site of dout
+__global__ void __launch_bounds__(32 * WG_WARPS, 1) k_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dout,
+                                                            float* __restrict__ part, int nx, int ny, int nz, int B) {
+    using WT = WgTile<CI, NT, CD, MX>;
+    constexpr int HX = WT::HX, HY = WT::HY, TX = 16 * MX, MI = CI / 16, T = 32 * WG_WARPS;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const unsigned sm0 = sm_addr(smem);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int split = blockIdx.x, nsplit = gridDim.x, dz = blockIdx.y;
+    const int nbx = nx / TX, nby = (ny + WG_TY - 1) / WG_TY;
+    const int ntile = B * nz * nby * nbx;
+    const size_t V = (size_t)nx * ny * nz;
+    auto stage = [&](int tile, int buf) {
+        int t = tile;
+        const int x0 = (t % nbx) * TX;
+        t /= nbx;
+        const int y0 = (t % nby) * WG_TY;
+        t /= nby;
+        const int z = t % nz, b = t / nz;
+        const int zi = ((z + dz - 2) % nz + nz) % nz;
+        const unsigned si = sm0 + buf * (WT::INB + WT::DB), sd = si + WT::INB;
+        const bf16* inb = in + ((size_t)b * V + (size_t)zi * ny * nx) * CI;
+        for (int i = tid; i < HX * HY * (CI / 8); i += T) {
+            const int site = i / (CI / 8), c = i - site * (CI / 8);
+            const int hx = site % HX, hy = site / HX;
+            int x = x0 + hx - 2;
+            x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+            const int y = ((y0 + hy - 2) % ny + ny) % ny;
+            cp_async16(si + swz<CI>(site, c), inb + (size_t)(y * nx + x) * CI + c * 8);
         }
+        const bf16* db = dout + ((size_t)b * V + (size_t)z * ny * nx) * CD;
+        for (int i = tid; i < TX * WG_TY * (CD / 8); i += T) {
+            const int site = i / (CD / 8), c = i - site * (CD / 8);
+            const int x = x0 + site % TX, y = y0 + site / TX;
+            cp_async16z(sd + swz<CD>(site, c), db + (size_t)((y < ny ? y : 0) * nx + x) * CD + c * 8, y < ny);   // rows past ny add nothing
+        }
+        cp_async_commit();
+    };
+    float acc[WG_OFF][MI][NT][4];
 #pragma unroll
-        for (int i = 0; i < CI / 16; ++i) {
-            unsigned a[4];
-            const int ci0 = i * 16 + g;
-            a[0] = pack2(inb[(size_t)sk[0] * CI + ci0], inb[(size_t)sk[1] * CI + ci0]);
-            a[1] = pack2(inb[(size_t)sk[0] * CI + ci0 + 8], inb[(size_t)sk[1] * CI + ci0 + 8]);
-            a[2] = pack2(inb[(size_t)sk[2] * CI + ci0], inb[(size_t)sk[3] * CI + ci0]);
-            a[3] = pack2(inb[(size_t)sk[2] * CI + ci0 + 8], inb[(size_t)sk[3] * CI + ci0 + 8]);
+    for (int o = 0; o < WG_OFF; ++o)
 #pragma unroll
-            for (int j = 0; j < CO / 8; ++j) {
-                const int co = j * 8 + g;
-                unsigned bb[2];
-                bb[0] = pack2(db[(size_t)(2 * t) * CO + co], db[(size_t)(2 * t + 1) * CO + co]);
-                bb[1] = pack2(db[(size_t)(2 * t + 8) * CO + co], db[(size_t)(2 * t + 9) * CO + co]);
-                mma16816(acc[i][j], a, bb);
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < NT; ++j) acc[o][i][j][0] = acc[o][i][j][1] = acc[o][i][j][2] = acc[o][i][j][3] = 0.f;
+    const int o0 = 2 * w, no = w == WG_WARPS - 1 ? 3 : 2;   // offsets o0 .. o0 + no - 1 of the plane's 25
+    // ldmatrix rows: in: sites k (lane & 7, + 8 for the upper lane half), channel chunk by lane bit 3;
+    // dout: sites k by lane bits 0-3, chunk by lane bit 4
+    const int ka = (lane & 7) + ((lane >> 4) << 3), ca = (lane >> 3) & 1;
+    const int kb = lane & 15, cb = lane >> 4;
+    int doff[WG_OFF];   // site shift of each offset
+#pragma unroll
+    for (int o = 0; o < WG_OFF; ++o) doff[o] = (o0 + o) / 5 * HX + (o0 + o) % 5 + ka;
+    // the thread's totals: value pairs (offset, m-tile, n-tile, row half), 32 lanes side by side
+    float2* tot = (float2*)(smem + 2 * (WT::INB + WT::DB)) + o0 * (CI * 4 * NT) + lane;
+    int left = WG_FLUSH;
+    bool first = true;
+    auto flush = [&]() {
+#pragma unroll
+        for (int o = 0; o < WG_OFF; ++o) {
+            if (o >= no) break;
+#pragma unroll
+            for (int i = 0; i < MI; ++i)
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float2* q = tot + (((o * MI + i) * NT + j) * 2 + h) * 32;
+                        float2 v = make_float2(acc[o][i][j][2 * h], acc[o][i][j][2 * h + 1]);
+                        if (!first) {
+                            const float2 u = *q;
+                            v.x += u.x;
+                            v.y += u.y;
+                        }
+                        *q = v;
+                        acc[o][i][j][2 * h] = acc[o][i][j][2 * h + 1] = 0.f;
+                    }
+        }
+        first = false;
+        left = WG_FLUSH;
+    };
+    int buf = 0;
+    if (split < ntile) stage(split, 0);
+    for (int tile = split; tile < ntile; tile += nsplit, buf ^= 1) {
+        if (tile + nsplit < ntile) {
+            stage(tile + nsplit, buf ^ 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
+        }
+        __syncthreads();
+        const unsigned si = sm0 + buf * (WT::INB + WT::DB), sd = si + WT::INB;
+#pragma unroll 2
+        for (int ks = 0; ks < WG_TY * MX; ++ks) {
+            const int r = ks / MX, xs = (ks % MX) * 16;
+            unsigned bf[(NT + 1) / 2][4];
+#pragma unroll
+            for (int jp = 0; jp < (NT + 1) / 2; ++jp) ldsm4t(sd + swz<CD>(r * TX + xs + kb, jp * 2 + cb), bf[jp]);
+#pragma unroll
+            for (int o = 0; o < WG_OFF; ++o) {
+                if (o == 2 && no < 3) break;   // uniform in the warp
+                const int site = r * HX + xs + doff[o];
+#pragma unroll
+                for (int i = 0; i < MI; ++i) {
+                    unsigned a[4];
+                    ldsm4t(si + swz<CI>(site, 2 * i + ca), a);
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) mma16816(acc[o][i][j], a, &bf[j >> 1][(j & 1) * 2]);
+                }
             }
         }
+        if (--left == 0) flush();
+        __syncthreads();   // the buffer is staged over after the next tile
     }
-    // C rows = input channel (g, g + 8 within the m-tile), columns = output channel (2t, 2t+1)
+    flush();
+    // rows = input channel (g, g + 8 within the m-tile), columns = output channel (2 t, 2 t + 1)
+    const int g = lane >> 2, tq = lane & 3;
+    float* p = part + ((size_t)split * KVOL + dz * 25 + o0) * (CI * 8 * NT);
+    for (int o = 0; o < no; ++o)
 #pragma unroll
-    for (int i = 0; i < CI / 16; ++i)
+        for (int i = 0; i < MI; ++i)
 #pragma unroll
-        for (int j = 0; j < CO / 8; ++j)
+            for (int j = 0; j < NT; ++j)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int ci = i * 16 + g + 8 * (q >> 1);
-                const int co = j * 8 + 2 * t + (q & 1);
-                if (ci < cin && co < cout) atomicAdd(&dW[((size_t)co * cin + ci) * KVOL + o], acc[i][j][q]);
-            }
+                for (int h = 0; h < 2; ++h)
+                    *(float2*)(p + (size_t)o * (CI * 8 * NT) + (i * 16 + g + 8 * h) * (8 * NT) + j * 8 + 2 * tq) =
+                        tot[(((o * MI + i) * NT + j) * 2 + h) * 32];
+}
+// dW[co][ci][o] = sum over the splits of part[split][o][CI][CO8], in order; one thread per (o, ci, co).
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, int nsplit, int CI, int CO8, int cin,
+                                                   int cout, float* __restrict__ dW) {
+    const int n = KVOL * CI * CO8;
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const int co = i % CO8, ci = i / CO8 % CI, o = i / (CO8 * CI);
+    if (co >= cout || ci >= cin) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < nsplit; ++k) s += part[(size_t)k * n + i];
+    dW[((size_t)co * cin + ci) * KVOL + o] = s;
 }
 
-// Per-sample, per-channel FP64 partial sums of a [B][C][V] float field (grid: blocks x C x B).
+// Per-sample, per-channel FP64 partial sums of a [B][C][V] float field (grid: blocks x C x B).  WIDE: a
+// thread takes several sites and sums them in FP64 (grids of few sites, where a block per 256 sites
+// would be mostly launch cost: 27 us for 8 x 32^3, 4 us with 4096 sites per block).
+template <bool WIDE>
 __global__ void k_chan_parts(const float* __restrict__ f, int C, int V, double* __restrict__ part) {
     __shared__ double sh[33];
     const int c = blockIdx.y, b = blockIdx.z;
     const float* p = f + ((size_t)b * C + c) * V;
-    float acc = 0.f;
+    std::conditional_t<WIDE, double, float> acc = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) acc += p[i];
     const double t = block_sum((double)acc, sh);
     if (threadIdx.x == 0) part[((size_t)b * C + c) * gridDim.x + blockIdx.x] = t;
 }
 // Same for a channel-last [B][V][CS] float field (channels 0..C-1).
+template <bool WIDE>
 __global__ void k_chan_parts_cl(const float* __restrict__ f, int C, int CS, int V, double* __restrict__ part) {
     __shared__ double sh[33];
     const int c = blockIdx.y, b = blockIdx.z;
     const float* p = f + (size_t)b * V * CS + c;
-    float acc = 0.f;
+    std::conditional_t<WIDE, double, float> acc = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) acc += p[(size_t)i * CS];
     const double t = block_sum((double)acc, sh);
     if (threadIdx.x == 0) part[((size_t)b * C + c) * gridDim.x + blockIdx.x] = t;
@@ -349,43 +541,38 @@ __global__ void k_dy(const float* __restrict__ g, const double* __restrict__ mea
     dst[1] = *(const uint4*)&v[8];
 }
 
-// BF16 weight copies of layer l: forward Wf[o][co][ci] and input-gradient Wb[o'][ci][co] with
-// Wb[o'][ci][co] = W[co][ci][-o'] (zero in padded channels).
-__global__ void k_prep_w(const float* __restrict__ W, int cin, int cout, int cinp, int coutp, bf16* __restrict__ Wf,
-                         bf16* __restrict__ Wb) {
-    const int n = KVOL * coutp * cinp;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int o = i / (coutp * cinp), rem = i % (coutp * cinp);
-        {
-            const int co = rem / cinp, ci = rem % cinp;
-            const float v = (co < cout && ci < cin) ? W[((size_t)co * cin + ci) * KVOL + o] : 0.f;
-            Wf[i] = __float2bfloat16(v);
-        }
-        if (Wb) {
-            const int ci = rem / coutp, co = rem % coutp;
-            const int oz = o / 25 - 2, oy = (o / 5) % 5 - 2, ox = o % 5 - 2;
-            const int of = (-oz + 2) * 25 + (-oy + 2) * 5 + (-ox + 2);
-            const float v = (co < cout && ci < cin) ? W[((size_t)co * cin + ci) * KVOL + of] : 0.f;
-            Wb[(size_t)o * cinp * coutp + (size_t)ci * coutp + co] = __float2bfloat16(v);
-        }
+// BF16 weights of layer l as mma.sync fragments (the B operand of k_conv): forward Wf with N = output
+// and K = input channels (cinp, NT n-tiles of 8), and for the input gradient Wb with N = input and
+// K = output channels (coutp, NTb n-tiles) and the offsets reversed; zero in padded channels.  Layout
+// [o][lane][k group of 16][n-tile][register][half]: n = 8 j + lane / 4, k = 16 kc + 2 (lane % 4) + 8 r + h.
+__global__ void k_prep_w(const float* __restrict__ W, int cin, int cout, int cinp, int coutp, int NT, int NTb,
+                         bf16* __restrict__ Wf, bf16* __restrict__ Wb) {
+    auto frag = [&](int i, int KC, int nt, int& o, int& n, int& k) {
+        const int h = i & 1, r = (i >> 1) & 1;
+        int t = i >> 2;
+        const int j = t % nt;
+        t /= nt;
+        const int kc = t % KC;
+        t /= KC;
+        const int lane = t & 31;
+        o = t >> 5;
+        n = 8 * j + (lane >> 2);
+        k = 16 * kc + 2 * (lane & 3) + 8 * r + h;
+    };
+    const int step = gridDim.x * blockDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    int o, n, k;
+    for (int i = i0; i < KVOL * NT * 8 * cinp; i += step) {
+        frag(i, cinp / 16, NT, o, n, k);
+        Wf[i] = __float2bfloat16((n < cout && k < cin) ? W[((size_t)n * cin + k) * KVOL + o] : 0.f);
+    }
+    if (!Wb) return;
+    for (int i = i0; i < KVOL * NTb * 8 * coutp; i += step) {
+        frag(i, coutp / 16, NTb, o, n, k);
+        Wb[i] = __float2bfloat16((k < cout && n < cin) ? W[((size_t)k * cin + n) * KVOL + (KVOL - 1 - o)] : 0.f);
     }
 }
 
-// BF16 weights of layer l in the tcgen05 operand layout Wt[o][ci / 8][co][ci % 8] (zero in
-// padded channels): for each offset and group of 8 input channels, 8 output channels x 16 bytes
-// form one contiguous core matrix.
-__global__ void k_prep_wt(const float* __restrict__ W, int cin, int cout, int cinp, int coutp, bf16* __restrict__ Wt) {
-    const int n = KVOL * coutp * cinp;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int o = i / (coutp * cinp), rem = i % (coutp * cinp);
-        const int kc = rem / (coutp * 8), r2 = rem % (coutp * 8);
-        const int co = r2 / 8, ci = kc * 8 + r2 % 8;
-        const float v = (co < cout && ci < cin) ? W[((size_t)co * cin + ci) * KVOL + o] : 0.f;
-        Wt[i] = __float2bfloat16(v);
-    }
-}
-
-// Weights of a stacked tcgen05 layer: Wt[dz][dx][ci / 8][4 - dy][co][ci % 8] (zero in padded
+// BF16 weights of a stacked tcgen05 layer: Wt[dz][dx][ci / 8][4 - dy][co][ci % 8] (zero in padded
 // channels): per (dz, dx, 8 input channels) the five dy offsets' output channels, last dy first,
 // form the rows of one N = 5 CO operand.
 __global__ void k_prep_wt_stk(const float* __restrict__ W, int cin, int cout, int cinp, int coutp, bf16* __restrict__ Wt) {
@@ -438,10 +625,20 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct NetLayout {
-    size_t params, grads, m, v, wf[NL], wb[NL], wt[NL], x16, x16f, h1, h2, h1p, h2p, y16, dy16, dz2, dz1, gtmp, part,
+    size_t params, grads, m, v, wf[NL], wb[NL], wt[NL], x16, x16f, h1, h2, h1p, h2p, y16, dy16, dz2, dz1, gtmp, wpart, part,
         means, lpart, err, bytes;
 };
 constexpr int kPartBlocks = 512;   // partial sums per channel and sample
+
+// CTAs per dz of a weight gradient: one CTA per SM over the five dz (152 SMs), at most one per tile.
+constexpr int kWgradSplits = 30;
+int wgrad_tiles(int nx, int ny, int nz, int B) {
+    return B * nz * ((ny + WG_TY - 1) / WG_TY) * (nx / (nx % 32 == 0 ? 32 : 16));
+}
+int wgrad_splits(int nx, int ny, int nz, int B) {
+    const int t = wgrad_tiles(nx, ny, nz, B);
+    return t < kWgradSplits ? t : kWgradSplits;
+}
 
 NetLayout net_layout(int nx, int ny, int nz, int B) {
     NetLayout L;
@@ -469,6 +666,7 @@ NetLayout net_layout(int nx, int ny, int nz, int B) {
     L.dz2 = take(S * 32 * 2);
     L.dz1 = take(S * 32 * 2);
     L.gtmp = take(S * 2 * 4);
+    L.wpart = take((size_t)wgrad_splits(nx, ny, nz, B) * KVOL * 32 * 32 * 4);
     const size_t ntc = tc_conv_supported(nx, ny) ? (size_t)tc_conv_blocks(nx, ny, nz) : 0;
     L.part = take((size_t)B * 2 * (ntc > (size_t)kPartBlocks ? ntc : (size_t)kPartBlocks) * 8);
     L.means = take((size_t)B * 2 * 8);
@@ -516,8 +714,9 @@ int ncheck(dscf_net* n, cudaError_t e, const char* what) {
 
 void prep_weights(dscf_net* n) {
     for (int l = 0; l < NL; ++l)
-        k_prep_w<<<64, 256, 0, n->stream>>>(n->at<float>(n->L.params) + poff(l), CIN[l], COUT[l], CINP[l], COUTP[l],
-                                              n->at<bf16>(n->L.wf[l]), l > 0 ? n->at<bf16>(n->L.wb[l]) : nullptr);
+        k_prep_w<<<128, 256, 0, n->stream>>>(n->at<float>(n->L.params) + poff(l), CIN[l], COUT[l], CINP[l], COUTP[l],
+                                               NTF[l], CINP[l] / 8, n->at<bf16>(n->L.wf[l]),
+                                               l > 0 ? n->at<bf16>(n->L.wb[l]) : nullptr);
     if (n->tc_ok) {
         k_prep_wt_fold<<<64, 256, 0, n->stream>>>(n->at<float>(n->L.params) + poff(0), n->at<bf16>(n->L.wt[0]));
         for (int l = 1; l < NL; ++l)
@@ -526,18 +725,72 @@ void prep_weights(dscf_net* n) {
     }
 }
 
+// Blocks of a channel sum: up to kPartBlocks x 256 sites every thread would have at most one site, so
+// the wide form takes 16 per thread instead.
+bool chan_wide(const dscf_net* n) { return n->V <= (size_t)kPartBlocks * 256; }
+int chan_blocks(const dscf_net* n) { return chan_wide(n) ? (int)((n->V + 4095) / 4096) : kPartBlocks; }
 // means of C = 2 channels of a [B][C][V] field into L.means
 void chan_means(dscf_net* n, const float* f, int C) {
-    k_chan_parts<<<dim3(kPartBlocks, C, n->B), 256, 0, n->stream>>>(f, C, (int)n->V, n->at<double>(n->L.part));
-    k_chan_final<<<C * n->B, 256, 0, n->stream>>>(n->at<double>(n->L.part), kPartBlocks, (int)n->V,
-                                                  n->at<double>(n->L.means));
+    const int nb = chan_blocks(n);
+    const dim3 grid(nb, C, n->B);
+    if (chan_wide(n)) k_chan_parts<true><<<grid, 256, 0, n->stream>>>(f, C, (int)n->V, n->at<double>(n->L.part));
+    else k_chan_parts<false><<<grid, 256, 0, n->stream>>>(f, C, (int)n->V, n->at<double>(n->L.part));
+    k_chan_final<<<C * n->B, 256, 0, n->stream>>>(n->at<double>(n->L.part), nb, (int)n->V, n->at<double>(n->L.means));
+}
+
+// mma.sync convolution and weight gradient of the network's grid
+template <int CI, int NT, int EPI, int MX>
+void conv_mx(dscf_net* n, const bf16* in, const bf16* W, const float* bias, int cout, const bf16* hact, void* out, float* bgrad) {
+    using CT = ConvTile<MX>;
+    constexpr int smem = CT::SITES * CI * 2;
+    const int blocks = n->B * (n->nx / (16 * MX)) * ((n->ny + CV_TY - 1) / CV_TY) * ((n->nz + CT::TZ - 1) / CT::TZ);
+    k_conv<CI, NT, EPI, MX><<<blocks, 128, smem, n->stream>>>(in, (const uint4*)W, bias, cout, hact, out, n->nx, n->ny, n->nz, bgrad);
+}
+template <int CI, int NT, int EPI>
+void conv(dscf_net* n, const bf16* in, const bf16* W, const float* bias, int cout, const bf16* hact, void* out, float* bgrad) {
+    if (n->nx % 32 == 0) conv_mx<CI, NT, EPI, 2>(n, in, W, bias, cout, hact, out, bgrad);
+    else conv_mx<CI, NT, EPI, 1>(n, in, W, bias, cout, hact, out, bgrad);
+}
+template <int CI, int NT, int CD, int MX>
+void wgrad_mx(dscf_net* n, const bf16* in, const bf16* dout, int nsplit) {
+    using WT = WgTile<CI, NT, CD, MX>;
+    constexpr int smem = WT::SMEM;
+    k_wgrad<CI, NT, CD, MX><<<dim3(nsplit, 5), 32 * WG_WARPS, smem, n->stream>>>(in, dout, n->at<float>(n->L.wpart), n->nx, n->ny, n->nz, n->B);
+}
+template <int CI, int NT, int CD>
+void wgrad(dscf_net* n, int l, const bf16* in, const bf16* dout, float* dW) {
+    const int nsplit = wgrad_splits(n->nx, n->ny, n->nz, n->B);
+    if (n->nx % 32 == 0) wgrad_mx<CI, NT, CD, 2>(n, in, dout, nsplit);
+    else wgrad_mx<CI, NT, CD, 1>(n, in, dout, nsplit);
+    k_wgrad_sum<<<(KVOL * CI * 8 * NT + 255) / 256, 256, 0, n->stream>>>(n->at<float>(n->L.wpart), nsplit, CI, 8 * NT, CIN[l], COUT[l], dW);
+}
+
+// Dynamic shared memory of the kernels above, once per network (cudaError_t of the first failure).
+template <int CI, int NT, int EPI, int MX>
+cudaError_t conv_smem() {
+    return cudaFuncSetAttribute(k_conv<CI, NT, EPI, MX>, cudaFuncAttributeMaxDynamicSharedMemorySize, ConvTile<MX>::SITES * CI * 2);
+}
+template <int CI, int NT, int CD, int MX>
+cudaError_t wgrad_smem() {
+    using WT = WgTile<CI, NT, CD, MX>;
+    return cudaFuncSetAttribute(k_wgrad<CI, NT, CD, MX>, cudaFuncAttributeMaxDynamicSharedMemorySize, WT::SMEM);
+}
+template <int MX>
+cudaError_t mma_prepare() {
+    cudaError_t e = conv_smem<16, 4, EPI_TANH, MX>();
+    if (e == cudaSuccess) e = conv_smem<32, 4, EPI_TANH, MX>();
+    if (e == cudaSuccess) e = conv_smem<32, 1, EPI_LIN_F32, MX>();
+    if (e == cudaSuccess) e = conv_smem<16, 4, EPI_DTANH, MX>();
+    if (e == cudaSuccess) e = conv_smem<32, 4, EPI_DTANH, MX>();
+    if (e == cudaSuccess) e = wgrad_smem<32, 1, 16, MX>();
+    if (e == cudaSuccess) e = wgrad_smem<32, 4, 32, MX>();
+    if (e == cudaSuccess) e = wgrad_smem<16, 4, 32, MX>();
+    return e;
 }
 
 // forward pass from U ([B][2][V] float, device) to phi ([B][2][V] float, device)
 void forward(dscf_net* n, const float* U, double pb0, double pb1, float* phi) {
     const int V = (int)n->V, B = n->B;
-    const int ntiles = (int)(n->V * B / 16);
-    const int blocks = (ntiles + 3) / 4;
     const int eb = (int)((n->V * B + 255) / 256);
     chan_means(n, U, 2);
     k_net_in<<<eb, 256, 0, n->stream>>>(U, n->at<double>(n->L.means), V, B, n->at<bf16>(n->L.x16));
@@ -552,18 +805,18 @@ void forward(dscf_net* n, const float* U, double pb0, double pb1, float* phi) {
         k_chan_final<<<2 * B, 256, 0, n->stream>>>(n->at<double>(n->L.part), tc_conv_blocks(n->nx, n->ny, n->nz), V,
                                                    n->at<double>(n->L.means));
     } else {
-        k_conv<16, 32, EPI_TANH><<<blocks, 128, 0, n->stream>>>(n->at<bf16>(n->L.x16), n->at<bf16>(n->L.wf[0]),
-            n->at<float>(n->L.params) + poff(0) + wcount(0), 32, nullptr, n->at<bf16>(n->L.h1), n->nx, n->ny, n->nz, ntiles,
-            nullptr);
-        k_conv<32, 32, EPI_TANH><<<blocks, 128, 0, n->stream>>>(n->at<bf16>(n->L.h1), n->at<bf16>(n->L.wf[1]),
-            n->at<float>(n->L.params) + poff(1) + wcount(1), 32, nullptr, n->at<bf16>(n->L.h2), n->nx, n->ny, n->nz, ntiles,
-            nullptr);
-        k_conv<32, 16, EPI_LIN_F32><<<blocks, 128, 0, n->stream>>>(n->at<bf16>(n->L.h2), n->at<bf16>(n->L.wf[2]),
-            n->at<float>(n->L.params) + poff(2) + wcount(2), 2, nullptr, n->at<float>(n->L.y16), n->nx, n->ny, n->nz, ntiles,
-            nullptr);
-        k_chan_parts_cl<<<dim3(kPartBlocks, 2, B), 256, 0, n->stream>>>(n->at<float>(n->L.y16), 2, 16, V,
-                                                                         n->at<double>(n->L.part));
-        k_chan_final<<<2 * B, 256, 0, n->stream>>>(n->at<double>(n->L.part), kPartBlocks, V, n->at<double>(n->L.means));
+        const float* prm = n->at<float>(n->L.params);
+        conv<16, 4, EPI_TANH>(n, n->at<bf16>(n->L.x16), n->at<bf16>(n->L.wf[0]), prm + poff(0) + wcount(0), 32, nullptr,
+                              n->at<bf16>(n->L.h1), nullptr);
+        conv<32, 4, EPI_TANH>(n, n->at<bf16>(n->L.h1), n->at<bf16>(n->L.wf[1]), prm + poff(1) + wcount(1), 32, nullptr,
+                              n->at<bf16>(n->L.h2), nullptr);
+        conv<32, 1, EPI_LIN_F32>(n, n->at<bf16>(n->L.h2), n->at<bf16>(n->L.wf[2]), prm + poff(2) + wcount(2), 2, nullptr,
+                                 n->at<float>(n->L.y16), nullptr);
+        const int nb = chan_blocks(n);
+        const dim3 grid(nb, 2, B);
+        if (chan_wide(n)) k_chan_parts_cl<true><<<grid, 256, 0, n->stream>>>(n->at<float>(n->L.y16), 2, 16, V, n->at<double>(n->L.part));
+        else k_chan_parts_cl<false><<<grid, 256, 0, n->stream>>>(n->at<float>(n->L.y16), 2, 16, V, n->at<double>(n->L.part));
+        k_chan_final<<<2 * B, 256, 0, n->stream>>>(n->at<double>(n->L.part), nb, V, n->at<double>(n->L.means));
     }
     k_net_out<<<eb, 256, 0, n->stream>>>(n->at<float>(n->L.y16), n->at<double>(n->L.means), V, B, pb0, pb1, phi);
 }
@@ -572,8 +825,6 @@ void forward(dscf_net* n, const float* U, double pb0, double pb1, float* phi) {
 void backward(dscf_net* n, const float* phi, const float* tgt) {
     const int V = (int)n->V, B = n->B;
     const size_t S = n->V * B;
-    const int ntiles = (int)(S / 16);
-    const int blocks = (ntiles + 3) / 4;
     const int eb = (int)((S + 255) / 256);
     float* grads = n->at<float>(n->L.grads);
     if (n->use_tc()) {   // the forward pass left its activations in the padded layout
@@ -584,22 +835,17 @@ void backward(dscf_net* n, const float* phi, const float* tgt) {
     k_loss_g<<<1024, 256, 0, n->stream>>>(phi, tgt, S * 2, n->at<float>(n->L.gtmp), n->at<double>(n->L.lpart));
     chan_means(n, n->at<float>(n->L.gtmp), 2);
     k_dy<<<eb, 256, 0, n->stream>>>(n->at<float>(n->L.gtmp), n->at<double>(n->L.means), V, B, n->at<bf16>(n->L.dy16));
-    const int chunk = 8;
-    const int wblocks = (ntiles + 4 * chunk - 1) / (4 * chunk);
     // layer 3
-    k_wgrad<32, 16><<<dim3(wblocks, KVOL), 128, 0, n->stream>>>(n->at<bf16>(n->L.h2), n->at<bf16>(n->L.dy16),
-        grads + poff(2), 32, 2, n->nx, n->ny, n->nz, ntiles, chunk);
+    wgrad<32, 1, 16>(n, 2, n->at<bf16>(n->L.h2), n->at<bf16>(n->L.dy16), grads + poff(2));
     // the output bias cannot change phi_hat (its per-sample mean is removed): its gradient is zero
-    k_conv<16, 32, EPI_DTANH><<<blocks, 128, 0, n->stream>>>(n->at<bf16>(n->L.dy16), n->at<bf16>(n->L.wb[2]), nullptr,
-        32, n->at<bf16>(n->L.h2), n->at<bf16>(n->L.dz2), n->nx, n->ny, n->nz, ntiles, grads + poff(1) + wcount(1));
+    conv<16, 4, EPI_DTANH>(n, n->at<bf16>(n->L.dy16), n->at<bf16>(n->L.wb[2]), nullptr, 32, n->at<bf16>(n->L.h2),
+                           n->at<bf16>(n->L.dz2), grads + poff(1) + wcount(1));
     // layer 2
-    k_wgrad<32, 32><<<dim3(wblocks, KVOL), 128, 0, n->stream>>>(n->at<bf16>(n->L.h1), n->at<bf16>(n->L.dz2),
-        grads + poff(1), 32, 32, n->nx, n->ny, n->nz, ntiles, chunk);
-    k_conv<32, 32, EPI_DTANH><<<blocks, 128, 0, n->stream>>>(n->at<bf16>(n->L.dz2), n->at<bf16>(n->L.wb[1]), nullptr,
-        32, n->at<bf16>(n->L.h1), n->at<bf16>(n->L.dz1), n->nx, n->ny, n->nz, ntiles, grads + poff(0) + wcount(0));
+    wgrad<32, 4, 32>(n, 1, n->at<bf16>(n->L.h1), n->at<bf16>(n->L.dz2), grads + poff(1));
+    conv<32, 4, EPI_DTANH>(n, n->at<bf16>(n->L.dz2), n->at<bf16>(n->L.wb[1]), nullptr, 32, n->at<bf16>(n->L.h1),
+                           n->at<bf16>(n->L.dz1), grads + poff(0) + wcount(0));
     // layer 1
-    k_wgrad<16, 32><<<dim3(wblocks, KVOL), 128, 0, n->stream>>>(n->at<bf16>(n->L.x16), n->at<bf16>(n->L.dz1),
-        grads + poff(0), 2, 32, n->nx, n->ny, n->nz, ntiles, chunk);
+    wgrad<16, 4, 32>(n, 0, n->at<bf16>(n->L.x16), n->at<bf16>(n->L.dz1), grads + poff(0));
 }
 
 // splitmix64-based normal deviates for the initial weights (Box-Muller)
@@ -670,7 +916,8 @@ int dscf_net_init(int32_t nx, int32_t ny, int32_t nz, int32_t batch, uint64_t se
             w[i] = (float)(sd * std::sqrt(-2.0 * std::log(u1)) * std::cos(6.283185307179586 * u2));
         }
     }
-    int rc = ncheck(n, cudaMemcpy(n->at<float>(n->L.params), p.data(), NPARAM * 4, cudaMemcpyHostToDevice), "params");
+    int rc = ncheck(n, nx % 32 == 0 ? mma_prepare<2>() : mma_prepare<1>(), "shared-memory limit");
+    if (!rc) rc = ncheck(n, cudaMemcpy(n->at<float>(n->L.params), p.data(), NPARAM * 4, cudaMemcpyHostToDevice), "params");
     if (!rc) rc = ncheck(n, cudaMemset(n->at<float>(n->L.m), 0, NPARAM * 4), "m");
     if (!rc) rc = ncheck(n, cudaMemset(n->at<float>(n->L.v), 0, NPARAM * 4), "v");
     if (!rc) rc = ncheck(n, cudaMemset(n->at<int>(n->L.err), 0, sizeof(int)), "error word");
