@@ -157,9 +157,9 @@ int dscf_set_fields(dscf_ctx* ctx, int32_t which, const void* src, int32_t on_ho
  *  (6..10 are reduced from the current populations and velocity when this is called),
  *  11 Q of the last gradient evaluation, 12 <exp(-U_S)>, 13 NCG iterations per step,
  *  14 <g,g> and 15 max|g| at the start of the last inversion, 16 <g,g> and 17 max|g|
- *  at its end, 18 steps done, 19 z-chunk of the propagator tiles (the brick depth when 20 is 0)
- *  and 20 contour steps fused per propagator launch (0: persistent sweeps), as chosen at
- *  dscf_init or by dscf_set_tuning, 21 steps taken with the
+ *  at its end, 18 steps done, 19 and 20 the contour sweeps, zc and kfuse
+ *  of dscf_set_tuning (20: 0 persistent brick sweeps, with their depth in 19; 1 general sweeps), as
+ *  chosen at dscf_init or by dscf_set_tuning, 21 steps taken with the
  *  learned predictor and 22 exact steps since dscf_set_predictor, 23 the predictor's last
  *  judged error (see dscf_set_predictor; -1 before the first judgement).  Slots 13, 16 and 17
  *  follow the inversion of the last step taken (a predictor step may use fewer iterations). */
@@ -210,15 +210,16 @@ const char* dscf_last_error(const dscf_ctx* ctx);
 int64_t dscf_launches_per_step(const dscf_ctx* ctx);
 
 /* Override the autotuner's choice (for instance with a value cached from an earlier run):
- * zc = z planes per propagator tile (>= 1), kfuse = contour steps per propagator launch (1..4;
- * > 1 needs FP32 and nx in {32, 64, 128} for every replica, or nx = 256 for every replica with
- * kfuse <= 2 (rows of 256 sites have contour kernels of their own), and kfuse <= N), or kfuse = 0 for
- * persistent sweeps (FP32; every replica with nx in {32, 48, 64, 96, 128} and ny a multiple of 8;
- * bricks of nx x 8 x 16 sites (nx x 16 x 16 for rows of at most 64 sites where ny allows), one
- * CTA of 16 compute warps per SM, or of nx x 8 x 8 (nx x 16 x 8) sites, two CTAs of 8 per SM; nz a
- * multiple of the brick depth; one warp per plane; both sweep directions in one launch; replicas
- * share cooperative launches while their bricks fit the SMs together, so a batch takes a few
- * launches per density evaluation).  With
+ * zc (>= 1) and kfuse name the contour sweeps.  kfuse = 1: the general sweeps (any grid and precision;
+ * both sweep directions of every replica in one launch; zc is kept but has no effect).  kfuse = 2..4:
+ * the same; accepted where contour steps used to be fused per launch (FP32 and nx in {32, 64, 128} for
+ * every replica, or nx = 256 for every replica with kfuse <= 2; kfuse <= N).  kfuse = 0: persistent
+ * brick sweeps (FP32; every replica with nx in {32, 48, 64, 96, 128} and ny a multiple of 8;
+ * bricks of nx x 8 x 16 sites (nx x 16 x 16 for rows of at most 64 sites where ny allows) on 16 compute
+ * warps, or of nx x 8 x 8 (nx x 16 x 8) on 8, one CTA per SM; nz a multiple of the brick depth; at
+ * most one brick of 16 planes, or two of 8, of a replica per SM; replicas share cooperative launches
+ * while their bricks fit the SMs together, so a batch takes a few launches per density evaluation;
+ * a context whose shallow bricks do not run together, one per SM, takes the general sweeps).  With
  * kfuse = 0, zc = 16 or 8 selects the brick depth (DSCF_ERR_ARG if the grids do not allow it),
  * any other zc keeps the current depth.  Synchronises the stream; the
  * next dscf_step re-captures its graph.  Results do not depend on either value beyond rounding. */

@@ -23,15 +23,14 @@ thread_local std::string g_init_error;
 
 struct Layout {
     std::vector<Rep> reps;          // host copy, pointers filled by place()
-    std::vector<int> tile2rep, blk2rep;
-    std::vector<int> fwd_grid;      // [s] for s = 1..Nmax (index s), tiles of replicas with N >= s
-    std::vector<size_t> fwd_smem, bwd_smem;   // [s] dynamic shared memory of the contour launches
-    size_t es = 8;
-    int ntiles = 0, nblk = 0, nlb = 0, Nmax = 0;
-    bool w8 = false;                // every replica in whole rows of 256 sites
+    std::vector<int> blk2rep;
+    std::vector<CoopRep> coop;      // general sweeps: replicas by decreasing N
+    long long units = 0;            // their row planes
+    int kk = 0;                     // row layout if all replicas have the same, else 0
+    int nblk = 0, nlb = 0, Nmax = 0;
     size_t bytes = 0;
     // offsets of the shared blocks
-    size_t off_reps = 0, off_t2r = 0, off_b2r = 0, off_status = 0;
+    size_t off_reps = 0, off_b2r = 0, off_coop = 0, off_status = 0;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -66,9 +65,8 @@ bool validate(const dscf_params* p, int n, std::string& why) {
     return true;
 }
 
-// Assign tiles (replicas in order of decreasing chain length own the first tiles, so the
-// replicas still active at contour step s are a prefix) and per-step grid sizes, for the
-// current z-chunk of every replica.
+// Flat blocks of the replicas and the general sweeps' table (replicas by decreasing chain length, so that
+// those still active at a contour step are a prefix).
 void assign_tiles(Layout& L, const dscf_params* p, int n) {
     // Flat kernels: about kMaxFlatBlocks blocks over the whole batch (one wave of four per SM).  A
     // replica whose own tiling would give it smaller chunks takes the batch's common chunk, so a
@@ -91,9 +89,7 @@ void assign_tiles(Layout& L, const dscf_params* p, int n) {
     std::vector<int> order(n);
     for (int r = 0; r < n; ++r) order[r] = r;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return p[a].N > p[b].N; });
-    L.tile2rep.clear();
     L.blk2rep.clear();
-    L.ntiles = 0;
     L.nblk = 0;
     L.nlb = 0;
     for (int r = 0; r < n; ++r) {
@@ -102,40 +98,32 @@ void assign_tiles(Layout& L, const dscf_params* p, int n) {
     }
     for (int k = 0; k < n; ++k) {
         Rep& R = L.reps[order[k]];
-        R.tile0 = L.ntiles;
-        for (int t = 0; t < R.ntiles; ++t) L.tile2rep.push_back(order[k]);
-        L.ntiles += R.ntiles;
         R.blk0 = L.nblk;
         for (int b = 0; b < R.nblk; ++b) L.blk2rep.push_back(order[k]);
         L.nblk += R.nblk;
     }
-    L.fwd_grid.assign(L.Nmax + 2, 0);
-    L.fwd_smem.assign(L.Nmax + 2, 0);
-    L.bwd_smem.assign(L.Nmax + 2, 0);
-    for (int s = 1; s <= L.Nmax; ++s)
-        for (int r = 0; r < n; ++r)
-            if (L.reps[r].N >= s) {
-                L.fwd_grid[s] += L.reps[r].ntiles;
-                L.fwd_smem[s] = std::max(L.fwd_smem[s], prop_smem_bytes(L.reps[r].vec, false, L.es));
-                L.bwd_smem[s] = std::max(L.bwd_smem[s], prop_smem_bytes(L.reps[r].vec, true, L.es));
-            }
+    L.coop.clear();
+    L.units = 0;
+    L.kk = coop_layout(L.reps[0].nx);
+    int cost = 0;
+    for (int k = 0; k < n; ++k) {
+        const Rep& R = L.reps[order[k]];
+        L.coop.push_back(coop_rep(R, cost));
+        L.units += L.coop.back().units;
+        cost += L.coop.back().units * coop_sites(R.nx);
+        if (L.coop.back().layout != L.kk) L.kk = 0;
+    }
 }
 
-int default_zc(int nz) { return std::min(nz, 8); }
 constexpr int kPersSpinLimit = 1 << 22;   // polls (~64 ns sleep each) before a persistent sweep gives up
 
-// Tiling and workspace layout.  With base == nullptr only sizes are computed.  Tile maps and
-// partial-sum slots are sized for the smallest z-chunk the autotuner may choose, so re-tiling
-// never moves anything.
+// Tiling and workspace layout.  With base == nullptr only sizes are computed.
 Layout make_layout(const dscf_params* p, int n, int prec, char* base) {
     Layout L;
     const size_t es = (prec == DSCF_FP64) ? sizeof(double) : sizeof(float);
-    L.es = es;
     L.reps.resize(n);
     long long ext = 0, vb = 0;
-    int max_tiles_total = 0, max_blk_total = 0;
-    L.w8 = true;
-    for (int r = 0; r < n; ++r) L.w8 = L.w8 && p[r].nx == 256;
+    int max_blk_total = 0;
     for (int r = 0; r < n; ++r) {
         Rep& R = L.reps[r];
         std::memset(&R, 0, sizeof(Rep));
@@ -143,12 +131,11 @@ Layout make_layout(const dscf_params* p, int n, int prec, char* base) {
         const dscf_params& q = p[r];
         R.nx = q.nx; R.ny = q.ny; R.nz = q.nz; R.ns = q.ns; R.N = q.N; R.nA = q.nA;
         R.V = (long long)q.nx * q.ny * q.nz;
-        tile_replica(R, kMinZc, L.w8);
-        const int max_tiles = R.ntiles;
-        max_tiles_total += max_tiles;
+        tile_replica(R);
         max_blk_total += R.nblk;
-        R.part_stride = std::max(std::max(max_tiles, R.nblk), R.lb_nblk);
-        tile_replica(R, default_zc(q.nz), L.w8);
+        R.part_stride = std::max(R.nblk, R.lb_nblk);
+        R.nq_units = (int)coop_units(R);
+        R.part_stride = std::max(R.part_stride, (R.nq_units + 31) / 32);
         R.hydro = q.hydro;
         R.cn_sweeps = q.cn_sweeps;
         R.phi_p = q.phi_p; R.kappa = q.kappa; R.alpha = q.a * q.a / 6.0; R.dt = q.dt; R.M = q.M;
@@ -192,12 +179,13 @@ Layout make_layout(const dscf_params* p, int n, int prec, char* base) {
         R.del1 = take(ns * V * es);
         R.rhs = take(ns * V * es);
         R.Uprev = take(ns * V * es);
+        R.qrow = (double*)take((size_t)R.nq_units * sizeof(double));
         R.part = (double*)take((size_t)NPART * R.part_stride * sizeof(double));
         R.scal = (double*)take((size_t)kScalStride * sizeof(double));
     }
     L.off_reps = off; take(sizeof(Rep) * n);
-    L.off_t2r = off; take(sizeof(int) * max_tiles_total);
     L.off_b2r = off; take(sizeof(int) * max_blk_total);
+    L.off_coop = off; take(sizeof(CoopRep) * n);
     L.off_status = off; take(sizeof(int) * kStatusInts);
     L.bytes = off;
     return L;
@@ -224,8 +212,8 @@ struct dscf_ctx {
     char* ws = nullptr;
     cudaStream_t stream = nullptr, cap = nullptr, cap_body = nullptr;   // graph capture; conditional bodies
     Rep* d_reps = nullptr;
-    int* d_t2r = nullptr;
     int* d_b2r = nullptr;
+    CoopRep* d_coop = nullptr;   // table of the general sweeps
     int* d_status = nullptr;
     int* d_counter = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -241,7 +229,8 @@ struct dscf_ctx {
     long long pred_counter = 0, n_pred = 0, n_exact = 0;
     double pred_err = -1.0;
     cudaGraphExec_t exec_pred = nullptr;
-    int kfuse = 1;          // contour steps per propagator launch (1 = single-step kernels, 0 = persistent)
+    int kfuse = 1;          // as chosen or asked for: 0 persistent brick sweeps, 1..4 general sweeps
+    bool bricks = false;    // the brick sweeps run (kfuse 0, and all bricks of a replica fit the SMs together)
     int pers_bz = 0;        // brick depth of the persistent sweeps (0 = not available)
     int pers_nw = 16;       // warps per CTA of the persistent sweeps
     struct PersGroup { int width, pby, first, nbricks; };   // one cooperative launch
@@ -253,7 +242,6 @@ struct dscf_ctx {
     cudaError_t cap_err = cudaSuccess;   // first graph-construction error of a capture
     const char* cap_what = "";
     int nsm = 0;
-    bool fusable = false;   // FP32 and every replica in the whole-row layout
     long long steps = 0;
     int64_t launches = 0;
     std::string err;
@@ -279,7 +267,6 @@ int cuda_check(dscf_ctx* c, cudaError_t e, const char* what) {
 Launch launch_of(dscf_ctx* c, cudaStream_t s) {
     Launch L;
     L.reps = c->d_reps;
-    L.tile2rep = c->d_t2r;
     L.blk2rep = c->d_b2r;
     L.status = c->d_status;
     L.counter = c->d_counter;
@@ -288,7 +275,6 @@ Launch launch_of(dscf_ctx* c, cudaStream_t s) {
     L.nrep = c->nrep;
     L.noise = c->noise;
     L.stream = s;
-    L.w8 = c->L.w8 ? 1 : 0;
     return L;
 }
 
@@ -308,8 +294,7 @@ int pers_total_bricks(const dscf_ctx* c) {
 }
 
 // Launch groups and brick table of the persistent sweeps.  The replicas are packed into
-// cooperative launches of at most as many bricks as can be co-resident (one per SM for bricks of
-// 16 planes, two for 8), every replica's bricks in one launch (they wait on one another): first
+// cooperative launches of at most as many bricks as can be co-resident (one per SM), every replica's bricks in one launch (they wait on one another): first
 // fit, replicas taken by decreasing chain length and then decreasing brick count, so that a launch
 // (which lasts as long as its longest chain) mostly holds chains of equal length.  A launch whose
 // replicas share one row width and brick height runs that width's kernel, any other the
@@ -324,7 +309,7 @@ int pers_total_bricks(const dscf_ctx* c) {
 int place_bricks(dscf_ctx* c) {
     c->pgroups.clear();
     const int n = c->nrep, bz = c->pers_bz;
-    const int cap = std::min(c->nsm * (c->pers_nw == 8 ? 2 : 1), kMaxBricks);
+    const int cap = std::min(c->nsm, kMaxBricks);
     std::vector<int> fbase(n), nbr(n), order(n);
     int tot = 0;
     for (int r = 0; r < n; ++r) {
@@ -389,27 +374,32 @@ int64_t launch_pers_sweeps(dscf_ctx* c, const Launch& L, int limit) {
     return (int64_t)c->pgroups.size();
 }
 
+// CTAs of the general sweeps.
+int coop_grid(const dscf_ctx* c) {
+    const int nsm = std::min(c->nsm, kCoopMaxCtas);
+    return coop_ctas(c->L.units, nsm);
+}
+CoopPlan coop_plan(const dscf_ctx* c) {
+    CoopPlan p;
+    p.reps = c->d_coop;
+    p.nrep = c->nrep;
+    p.cnt = c->d_status + kCoopBase;
+    p.abort = c->d_status + 2;
+    p.kk = c->L.kk;
+    p.ncta = coop_grid(c);
+    return p;
+}
+
 // Forward and backward contour sweeps of one gradient evaluation.
 template <typename T>
 int64_t enqueue_sweeps(dscf_ctx* c, const Launch& L) {
     int64_t n = 0;
-    const int K = c->kfuse;
-    if (K == 0) {
+    if (c->bricks) {
         n += launch_pers_sweeps(c, L, c->wait_limit);
         return n;
     }
-    if (K > 1) {
-        int vmax = 0;
-        for (const Rep& R : c->L.reps) vmax = std::max(vmax, R.vec);
-        const size_t sm = prop_fused_smem_bytes(vmax, K);
-        const int ng = (c->L.Nmax + K - 1) / K;
-        for (int g = 0; g < ng; ++g) { launch_prop_fused(L, false, K, g, c->L.fwd_grid[g * K + 1], sm); ++n; }
-        for (int g = 0; g < ng; ++g) { launch_prop_fused(L, true, K, g, c->L.fwd_grid[g * K + 1], sm); ++n; }
-        return n;
-    }
-    for (int s = 1; s <= c->L.Nmax; ++s) { launch_prop_fwd<T>(L, s, c->L.fwd_grid[s], c->L.fwd_smem[s]); ++n; }
-    for (int j = 0; j < c->L.Nmax; ++j) { launch_prop_bwd<T>(L, j, c->L.fwd_grid[j + 1], c->L.bwd_smem[j + 1]); ++n; }
-    return n;
+    launch_prop_coop<T>(L, coop_plan(c), 0, c->L.Nmax, c->wait_limit);
+    return n + 1;
 }
 
 // One gradient evaluation: Boltzmann factors, forward and backward contour sweeps.
@@ -627,11 +617,10 @@ int check_predictor(dscf_ctx* c, bool after_pred) {
 int set_dev(dscf_ctx* c) { return cuda_check(c, cudaSetDevice(c->device), "cudaSetDevice"); }
 
 int upload_tiles(dscf_ctx* c) {
+    // partial sums of Q that the sweeps in use leave
+    for (Rep& R : c->L.reps) R.nq = c->bricks ? pers_bricks(R, c->pers_bz) : (R.nq_units + 31) / 32;
     int rc = cuda_check(c, cudaMemcpyAsync(c->d_reps, c->L.reps.data(), sizeof(Rep) * c->nrep, cudaMemcpyHostToDevice,
                                            c->stream), "reps");
-    if (rc) return rc;
-    rc = cuda_check(c, cudaMemcpyAsync(c->d_t2r, c->L.tile2rep.data(), sizeof(int) * c->L.ntiles, cudaMemcpyHostToDevice,
-                                       c->stream), "tile map");
     if (rc) return rc;
     rc = cuda_check(c, cudaMemcpyAsync(c->d_b2r, c->L.blk2rep.data(), sizeof(int) * c->L.nblk, cudaMemcpyHostToDevice,
                                        c->stream), "block map");
@@ -639,14 +628,8 @@ int upload_tiles(dscf_ctx* c) {
     return cuda_check(c, cudaStreamSynchronize(c->stream), "tile upload");
 }
 
-void set_zc(dscf_ctx* c, int zc) {
-    for (int r = 0; r < c->nrep; ++r) tile_replica(c->L.reps[r], std::min(zc, c->L.reps[r].nz), c->L.w8);
-    assign_tiles(c->L, c->params.data(), c->nrep);
-}
-
-// Persistent-sweep candidates (one warp per plane of the brick): bricks of 16 planes (one CTA per
-// SM) and bricks of 8 planes (two CTAs per SM).  The first becomes the context's persistent
-// configuration.
+// Persistent-sweep candidates (one warp per plane of the brick): bricks of 16 planes and bricks of 8
+// planes.  The first becomes the context's persistent configuration.
 bool pers_all_supported(const dscf_ctx* c, int bz, int nw) {
     if (c->prec != DSCF_FP32) return false;
     const int nsm = std::min(c->nsm, kMaxBricks / 2);
@@ -656,6 +639,13 @@ bool pers_all_supported(const dscf_ctx* c, int bz, int nw) {
         tot += pers_bricks(R, bz);
     }
     return tot <= kMaxBricks;
+}
+
+// Every replica's bricks at the context's depth run together, one per SM.
+bool pers_fit(const dscf_ctx* c) {
+    for (const Rep& R : c->L.reps)
+        if (pers_bricks(R, c->pers_bz) > c->nsm) return false;
+    return true;
 }
 
 int pers_select(dscf_ctx* c, std::vector<std::pair<int, int>>& pcand) {
@@ -678,138 +668,82 @@ int pers_select(dscf_ctx* c, std::vector<std::pair<int, int>>& pcand) {
     return DSCF_OK;
 }
 
-// Fusion support and its shared-memory limit (needed before any fused launch).
-int fusion_setup(dscf_ctx* c) {
-    c->fusable = (c->prec == DSCF_FP32);
-    for (const Rep& R : c->L.reps) c->fusable = c->fusable && (R.vec > 0);
-    if (c->fusable) {
-        const size_t lim = prop_fused_smem_bytes(4, 4);
-        return cuda_check(c, (cudaError_t)prop_fused_set_smem_limit(lim), "fused shared-memory limit");
+// Grids for which contour fusion can be asked for (kfuse 2..4).  Those kernels are gone (the general
+// sweeps take 0.92 ms against 1.52 at 128^3 with N = 64, 0.31 against 0.87 at 64^3, 7.9 against 8.1 at
+// 256^3), but the request stays valid and runs the general sweeps.
+bool fusable(const dscf_ctx* c, int kfuse) {
+    if (c->prec != DSCF_FP32) return false;
+    bool all256 = true, rows = true;
+    for (const Rep& R : c->L.reps) {
+        all256 = all256 && R.nx == 256;
+        rows = rows && (R.nx == 32 || R.nx == 64 || R.nx == 128);
     }
-    return DSCF_OK;
+    return rows || (all256 && kfuse <= 2);
 }
 
-// Autotuner: pick the z-chunk of the propagator tiles and the number of contour steps fused per
-// launch (one pair for all replicas) by timing forward contour launches on the context's own
-// buffers; the figure of merit is time per contour step.  Small problems keep the defaults.
+// Autotuner: one density evaluation of each kind of sweeps, timed on the context's own buffers: the
+// general sweeps, and the persistent brick sweeps where the grids allow them (both brick depths).  Small
+// problems and grids without bricks take the general sweeps untimed.
 int autotune_zc(dscf_ctx* c) {
     long long Vtot = 0;
-    int Nmin = 1 << 30;
-    for (const Rep& R : c->L.reps) { Vtot += R.V; Nmin = std::min(Nmin, R.N); }
-    int best = default_zc(c->L.reps[0].nz), bestK = 1;
-    if (int rc = fusion_setup(c)) return rc;
-    if (Vtot >= 32 * 32 * 32) {
+    for (const Rep& R : c->L.reps) Vtot += R.V;
+    std::vector<std::pair<int, int>> pcand;
+    if (int rc = pers_select(c, pcand)) return rc;
+    c->kfuse = 1;
+    c->bricks = false;
+    if (Vtot >= 32 * 32 * 32 && !pcand.empty()) {
         cudaEvent_t e0, e1;
         if (int rc = cuda_check(c, cudaEventCreate(&e0), "tune event")) return rc;
         if (int rc = cuda_check(c, cudaEventCreate(&e1), "tune event")) { cudaEventDestroy(e0); return rc; }
-        float best_ms = 1e30f;
-        const int cands[] = {4, 5, 6, 8, 11, 16, 22, 32};
-        const int kmax = c->fusable ? std::min(c->L.w8 ? 2 : 4, Nmin) : 1;   // rows of 256 sites: two steps
-        for (int zc : cands) {
-            set_zc(c, zc);
-            if (int rc = upload_tiles(c)) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
+        auto leave = [&](int rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; };
+        auto sweep_ms = [&]() -> float {   // (bricks exist in FP32 only)
+            if (upload_tiles(c)) return 1e30f;
             const Launch L = launch_of(c, c->stream);
-            for (int K = 1; K <= kmax; ++K) {
-                int vmax = 0;
-                for (const Rep& R : c->L.reps) vmax = std::max(vmax, R.vec);
-                auto run = [&]() {
-                    if (K == 1) {
-                        if (c->prec == DSCF_FP64) launch_prop_fwd<double>(L, 2, c->L.fwd_grid[2], c->L.fwd_smem[2]);
-                        else launch_prop_fwd<float>(L, 2, c->L.fwd_grid[2], c->L.fwd_smem[2]);
-                    } else {
-                        launch_prop_fused(L, false, K, 0, c->L.fwd_grid[1], prop_fused_smem_bytes(vmax, K));
-                    }
-                };
-                for (int i = 0; i < 3; ++i) run();
-                cudaEventRecord(e0, c->stream);
-                for (int i = 0; i < 8; ++i) run();
-                cudaEventRecord(e1, c->stream);
-                float ms = 0.f;
-                cudaError_t e = cudaEventSynchronize(e1);
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                if (e == cudaSuccess) e = cudaGetLastError();
-                if (e != cudaSuccess) { cudaEventDestroy(e0); cudaEventDestroy(e1); return cuda_check(c, e, "tune timing"); }
-                ms /= (float)K;
-                if (ms < best_ms) { best_ms = ms; best = zc; bestK = K; }
-            }
+            enqueue_sweeps<float>(c, L);
+            cudaEventRecord(e0, c->stream);
+            enqueue_sweeps<float>(c, L);
+            enqueue_sweeps<float>(c, L);
+            cudaEventRecord(e1, c->stream);
+            float ms = 1e30f;
+            if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+            return cudaGetLastError() == cudaSuccess ? ms : 1e30f;
+        };
+        const float t = sweep_ms();
+        float tp = 1e30f;
+        std::pair<int, int> pbest = pcand[0];
+        for (auto& pc : pcand) {   // the first candidate (bricks of 16 planes) unless another is 2% faster
+            c->pers_bz = pc.first;
+            c->pers_nw = pc.second;
+            if (!pers_fit(c)) continue;
+            int rc = reset_pers_flags(c);
+            if (!rc) rc = place_bricks(c);
+            if (rc) return leave(rc);
+            c->bricks = true;
+            const float ti = sweep_ms();
+            if (ti < (tp < 1e29f ? 0.98f * tp : tp)) { tp = ti; pbest = pc; }
         }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-    }
-    // persistent sweeps (FP32, supported row widths; both brick depths): a forward and a backward
-    // sweep of the whole batch per candidate, per sweep against the best above
-    std::vector<std::pair<int, int>> pcand;
-    if (int rc = pers_select(c, pcand)) return rc;
-    if (!pcand.empty()) {
-        c->pers_bz = pcand[0].first;
-        c->pers_nw = pcand[0].second;
-        if (Vtot >= 32 * 32 * 32 && Nmin >= 2) {
-            // per contour step of the best multi-launch configuration, measured on a forward sweep
-            auto sweep_ms = [&](int K, int zc) -> float {
-                c->kfuse = K;
-                set_zc(c, K == 0 ? c->pers_bz : zc);
-                if (upload_tiles(c)) return 1e30f;
-                const Launch L = launch_of(c, c->stream);
-                cudaEvent_t e0, e1;
-                cudaEventCreate(&e0);
-                cudaEventCreate(&e1);
-                auto run = [&]() {
-                    if (K == 0) {
-                        launch_pers_sweeps(c, L, kPersSpinLimit);
-                    } else if (c->prec == DSCF_FP64) {
-                        enqueue_sweeps<double>(c, L);
-                    } else {
-                        enqueue_sweeps<float>(c, L);
-                    }
-                };
-                run();
-                cudaEventRecord(e0, c->stream);
-                run();
-                run();
-                cudaEventRecord(e1, c->stream);
-                float ms = 1e30f;
-                if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-                if (cudaGetLastError() != cudaSuccess) return 1e30f;
-                return ms / 2.0f / 2.0f;   // per sweep, forward and backward
-            };
-            float tp = 1e30f;
-            std::pair<int, int> pbest = pcand[0];
-            for (auto& pc : pcand) {   // the first candidate (bricks of 16 planes) unless another is 2% faster
-                c->pers_bz = pc.first;
-                c->pers_nw = pc.second;
-                if (int rc = reset_pers_flags(c)) return rc;
-                if (int rc = place_bricks(c)) return rc;
-                const float t = sweep_ms(0, 0);
-                if (t < (tp < 1e29f ? 0.98f * tp : tp)) { tp = t; pbest = pc; }
-            }
-            c->pers_bz = pbest.first;
-            c->pers_nw = pbest.second;
-            if (int rc = reset_pers_flags(c)) return rc;
-            if (int rc = place_bricks(c)) return rc;
-            const float tm = sweep_ms(bestK, best);
-            int st = 0;
-            cudaMemcpy(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost);
-            if (st & ST_TIMEOUT) return fail(c, DSCF_ERR_TIMEOUT, "persistent sweep timed out during tuning");
-            if (tp < tm) bestK = 0;
+        c->pers_bz = pbest.first;
+        c->pers_nw = pbest.second;
+        c->bricks = tp < t;
+        if (c->bricks) {
+            c->kfuse = 0;
+            int rc = reset_pers_flags(c);
+            if (!rc) rc = place_bricks(c);
+            if (rc) return leave(rc);
         }
+        leave(0);
+        int st = 0;
+        cudaMemcpy(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost);
+        if (st & ST_TIMEOUT) return fail(c, DSCF_ERR_TIMEOUT, "a contour sweep timed out during tuning");
     }
-    c->zc = bestK == 0 ? c->pers_bz : best;   // with persistent sweeps the brick depth
-    c->kfuse = bestK;
-    set_zc(c, bestK == 0 ? c->pers_bz : best);
+    c->zc = c->bricks ? c->pers_bz : std::min(c->L.reps[0].nz, 8);
     return upload_tiles(c);
 }
 // A tuning chosen earlier (for instance cached from an autotuner run) instead of the autotuner.
 int apply_tuning(dscf_ctx* c, int zc, int kfuse) {
     std::vector<std::pair<int, int>> pcand;
     if (int rc = pers_select(c, pcand)) return rc;
-    if (int rc = fusion_setup(c)) return rc;
     if (int rc = dscf_set_tuning(c, zc, kfuse)) return rc;
-    if (kfuse == 0) {
-        if (int rc = reset_pers_flags(c)) return rc;
-        if (int rc = place_bricks(c)) return rc;
-    }
     return DSCF_OK;
 }
 }  // namespace
@@ -858,8 +792,8 @@ int dscf_init_tuned(const dscf_params* p, int32_t n, int32_t precision, void* wo
         return fail(nullptr, DSCF_ERR_OOM, "workspace has %zu bytes, needs %zu", wbytes, c->L.bytes);
     }
     c->d_reps = (Rep*)(c->ws + c->L.off_reps);
-    c->d_t2r = (int*)(c->ws + c->L.off_t2r);
     c->d_b2r = (int*)(c->ws + c->L.off_b2r);
+    c->d_coop = (CoopRep*)(c->ws + c->L.off_coop);
     c->d_status = (int*)(c->ws + c->L.off_status);
     c->d_counter = c->d_status + 1;
     auto chk = [&](cudaError_t e, const char* w) { return cuda_check(c, e, w); };
@@ -867,8 +801,9 @@ int dscf_init_tuned(const dscf_params* p, int32_t n, int32_t precision, void* wo
     rc = rc ? rc : chk(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking), "capture stream");
     rc = rc ? rc : chk(cudaStreamCreateWithFlags(&c->cap_body, cudaStreamNonBlocking), "capture stream");
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_reps, c->L.reps.data(), sizeof(Rep) * n, cudaMemcpyHostToDevice, c->stream), "reps");
-    rc = rc ? rc : chk(cudaMemcpyAsync(c->d_t2r, c->L.tile2rep.data(), sizeof(int) * c->L.ntiles, cudaMemcpyHostToDevice, c->stream), "t2r");
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_b2r, c->L.blk2rep.data(), sizeof(int) * c->L.nblk, cudaMemcpyHostToDevice, c->stream), "b2r");
+    assign_tiles(c->L, c->params.data(), n);   // (the sweeps' table with the final pointers)
+    rc = rc ? rc : chk(cudaMemcpyAsync(c->d_coop, c->L.coop.data(), sizeof(CoopRep) * n, cudaMemcpyHostToDevice, c->stream), "sweep table");
     rc = rc ? rc : chk(cudaMemsetAsync(c->d_status, 0, sizeof(int) * kStatusInts, c->stream), "status");
     const size_t es = precision == DSCF_FP64 ? 8 : 4;
     for (int r = 0; r < n && !rc; ++r) {
@@ -893,11 +828,7 @@ int dscf_init_tuned(const dscf_params* p, int32_t n, int32_t precision, void* wo
     }
     rc = rc ? rc : chk(cudaGetLastError(), "fill");
     rc = rc ? rc : chk(cudaStreamSynchronize(c->stream), "init sync");
-    if (!rc) {
-        const size_t lim = std::max(prop_smem_bytes(4, true, c->L.es), prop_smem_bytes(0, true, c->L.es));
-        const int e = precision == DSCF_FP64 ? prop_set_smem_limit<double>(lim) : prop_set_smem_limit<float>(lim);
-        rc = cuda_check(c, (cudaError_t)e, "propagator shared-memory limit");
-    }
+    rc = rc ? rc : chk((cudaError_t)(precision == DSCF_FP64 ? coop_prepare<double>(c->L.kk) : coop_prepare<float>(c->L.kk)), "contour sweeps");
     if (!rc) rc = (zc < 0) ? autotune_zc(c) : apply_tuning(c, zc, kfuse);
     if (rc) {
         g_init_error = c->err;
@@ -1239,7 +1170,7 @@ int dscf_status(dscf_ctx* c) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_status, &clear, sizeof(int), cudaMemcpyHostToDevice, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (int rc = cuda_check(c, e, "re-arming after a timeout")) return rc;
-        return fail(c, DSCF_ERR_TIMEOUT, "a persistent contour sweep gave up waiting for a neighbour");
+        return fail(c, DSCF_ERR_TIMEOUT, "a contour sweep gave up waiting for its neighbours");
     }
     if (st & ST_NONFINITE) return fail(c, DSCF_ERR_NUMERIC, "non-finite value in a reduction");
     return DSCF_OK;
@@ -1318,7 +1249,7 @@ int dscf_set_wait_limit(dscf_ctx* c, int32_t polls) {
 
 int dscf_inject_lag(dscf_ctx* c, int32_t brick) {
     if (!c) return DSCF_ERR_ARG;
-    if (!c->pers_bz || c->kfuse != 0) return fail(c, DSCF_ERR_STATE, "the context does not run persistent sweeps");
+    if (!c->bricks) return fail(c, DSCF_ERR_STATE, "the context does not run persistent sweeps");
     const int nb = pers_total_bricks(c);
     if (brick < 0 || brick >= nb) return fail(c, DSCF_ERR_ARG, "brick index out of range");
     if (int rc = set_dev(c)) return rc;
@@ -1396,9 +1327,8 @@ int dscf_set_predictor(dscf_ctx* c, dscf_net* net, int32_t corrector_every, doub
 int dscf_set_tuning(dscf_ctx* c, int32_t zc, int32_t kfuse) {
     if (!c) return DSCF_ERR_ARG;
     if (zc < 1 || kfuse < 0 || kfuse > 4) return fail(c, DSCF_ERR_ARG, "need zc >= 1 and 0 <= kfuse <= 4");
-    if (kfuse > 1 && !c->fusable)
-        return fail(c, DSCF_ERR_ARG, "contour fusion needs FP32 and nx in {32, 64, 128} (or 256 for every replica)");
-    if (kfuse > 2 && c->L.w8) return fail(c, DSCF_ERR_ARG, "rows of 256 sites fuse at most two contour steps");
+    if (kfuse > 1 && !fusable(c, kfuse))
+        return fail(c, DSCF_ERR_ARG, "contour fusion needs FP32 and nx in {32, 64, 128} (or 256 for every replica and at most two steps)");
     if (kfuse == 0 && !c->pers_bz)
         return fail(c, DSCF_ERR_ARG,
                     "persistent sweeps need FP32 replicas with nx in {32, 48, 64, 96, 128}, ny %% 8 = 0 and nz a "
@@ -1421,19 +1351,22 @@ int dscf_set_tuning(dscf_ctx* c, int32_t zc, int32_t kfuse) {
         cudaGraphExecDestroy(c->exec_pred);
         c->exec_pred = nullptr;
     }
-    if (kfuse == 0 && (pbz != c->pers_bz || pnw != c->pers_nw || c->pgroups.empty())) {
+    c->bricks = false;
+    if (kfuse == 0) {
         for (const Rep& R : c->L.reps)
             if (int rc = cuda_check(c, (cudaError_t)pers_prepare(R.nx, pers_pby(R), pbz, pnw), "persistent sweep set-up"))
                 return rc;
         if (int rc = cuda_check(c, (cudaError_t)pers_prepare(0, 0, pbz, pnw), "persistent sweep set-up")) return rc;
         c->pers_bz = pbz;
         c->pers_nw = pnw;
-        if (int rc = reset_pers_flags(c)) return rc;
-        if (int rc = place_bricks(c)) return rc;
+        if (pers_fit(c)) {   // otherwise the general sweeps
+            if (int rc = reset_pers_flags(c)) return rc;
+            if (int rc = place_bricks(c)) return rc;
+            c->bricks = true;
+        }
     }
     c->zc = kfuse == 0 ? c->pers_bz : zc;
     c->kfuse = kfuse;
-    set_zc(c, c->zc);
     return upload_tiles(c);
 }
 

@@ -1,0 +1,584 @@
+// General contour sweeps (Eq. 16-17): any grid, both precisions, one replica or a batch of unlike
+// ones, in one launch.
+//
+// A cooperative launch of one CTA per SM runs both chains of a density evaluation level by level.
+// Like the brick kernel's (dscf_pers.cu), the forward chain G_s and the backward one G+_s meet in the
+// middle, h = ceil(N / 2): each stores its levels up to there in the contour stack (G_s, s <= h;
+// G+_s, s > h) and past it multiplies sigma of its own field with the stored value of the other,
+// q_{I_s} += sigma[G_{s-1}] G+_s = G_s sigma[G+_{s+1}].  A chain's level needs the whole previous
+// level, so a counter per chain is the grid's barrier between levels; a CTA arrives at one chain's
+// barrier, computes its share of the other chain's level and only then waits, so that the barrier's
+// L2 round trips overlap with work (a warp per chain arrives and polls; the compute warps only meet
+// it in shared memory).
+//
+// Work is cut into runs of consecutive z planes of one x row (or one x tile of a row of more than 256
+// sites), spread evenly over all warps of the launch.  A warp marches its run: per plane it loads the
+// row and its two y neighbours, applies the y pass, then the x pass by shuffles (lane L holds sites L,
+// L + 32, ... of the row, so any row length and alignment has coalesced accesses), and combines three
+// planes in registers.  No pass is computed twice but the y and x passes of the two planes beside a
+// run, no shared memory and no barrier inside a level, and each pass is one add and one fma
+// (c + r (a + d), r = alpha / (1 - 2 alpha), the centre weights folded into the Boltzmann factors and the
+// normalisation): 7 operations a site and contour step forward, 8 with the quadrature.
+//
+// FP64 at 128^3 is bound by the FP64 pipe (32 us of operations in a level's 33 us); small or odd
+// grids by the latency of a level (loads, the barrier).  A density evaluation, before (one launch per
+// contour step and direction, rows staged through shared memory, 9 operations on 10/8 of the rows)
+// and so: 32^3, N = 32, FP64 539 -> 192 us; 100 x 90 x 75, N = 48, FP32 1010 -> 424 us; 128^3, N = 64,
+// FP64 8.9 -> 4.2 ms; 256^3, N = 64, FP32 8.1 (fused pairs of steps) -> 7.9 ms.  Against the brick
+// sweeps: 48^3, N = 16 80 us (bricks 137), 64^3, N = 64 306 (361), 128^3, N = 64 924 (392).
+//
+// Every wait is bounded as in dscf_pers.cu: a CTA that runs out sets the status bit and the abort flag
+// and waits no more; arrivals do not depend on waits, so the launch always finishes and leaves its
+// counters at zero.
+// Included by dscf_coop32.cu and dscf_coop64.cu, one per precision (they compile in parallel).
+#pragma once
+#include "dscf_internal.cuh"
+
+#include <cstring>
+
+// the row layouts that coop_layout() gives: (sites per lane, mode)
+#define DSCF_COOP_LAYOUTS(X)                                                                                \
+    X(1, BLOCKED) X(2, BLOCKED) X(3, BLOCKED) X(4, BLOCKED) X(6, BLOCKED) X(8, BLOCKED) X(1, STRIDED) X(2, STRIDED) \
+    X(3, STRIDED) X(4, STRIDED) X(5, STRIDED) X(6, STRIDED) X(7, STRIDED) X(8, STRIDED) X(8, TILE)
+
+namespace dscf {
+
+namespace {
+
+struct CoopCtl {
+    const CoopRep* reps;         // replicas by decreasing chain length
+    int nrep;
+    int j0, j1;                  // levels of this launch
+    int* cnt;                    // barrier counters: chain c at c * kFlagStride, exits at 2 * kFlagStride
+    int* abort;
+    int* status;
+    int limit;                   // polls before giving up
+};
+
+__device__ __forceinline__ int cld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cred_release(int* p) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;\n" ::"l"(p) : "memory");
+}
+
+// One chain's level on one replica.
+template <typename T>
+struct CoopOps {
+    const T* src;   // previous level; nullptr: the constant field 1
+    T* dst;         // nullptr: the level is not needed
+    const T* E;
+    const T* st;    // stored level of the other chain (quadrature), nullptr before the middle
+    T* q;           // quadrature
+    bool first;     // q starts here
+    bool lastQ;     // sum the level (G_N)
+    double* qrow;   // its sums per row plane, or nullptr: one sum per warp
+};
+
+// Level i of chain C (contour step s = i + 1 forward, s = N - i backward).  Before the chains meet it is
+// stored at its bead's place in the stack.  Past the middle a chain overwrites the place of its bead,
+// whose value of the other chain it has just used at the same site (and thread), except at its
+// first level there: that place is still the other chain's input, so the level goes to a field of its
+// own.  (A later place was last read as a neighbour at least one full level of both chains earlier.)
+template <typename T, int C>
+__device__ __forceinline__ CoopOps<T> coop_ops(const CoopRep& R, int j) {
+    CoopOps<T> o;
+    const size_t V = (size_t)R.V;
+    const int N = R.N, nA = R.nA, h = (N + 1) / 2;
+    const int s = C ? N - j : j + 1, sp = s <= nA ? 0 : 1;
+    T* stack = (T*)R.G;
+    const int mid = C ? N - h : h;
+    auto level = [&](int i) -> T* {
+        if (i == mid) return (T*)(C ? R.Gp1 : R.Gp0);
+        return stack + (size_t)(C ? N - i - 1 : i) * V;
+    };
+    o.src = j == 0 ? nullptr : level(j - 1);
+    o.dst = j == N - 1 ? nullptr : level(j);   // the last level of a chain is not read again (Q is summed in registers)
+    o.E = (const T*)R.E + (sp ? V : 0);
+    o.st = j >= mid ? stack + (size_t)(s - 1) * V : nullptr;
+    o.q = (T*)R.q + (sp ? V : 0);
+    // A block's quadrature starts at its first bead past the middle on either side.  Where beads of
+    // one block lie on both sides both chains add to it: the same thread, in the order of the units
+    // (backward first for odd N).
+    const bool both = nA != h;   // the block of beads h and h + 1
+    o.first = C ? ((j == mid && !(both && (N & 1) == 0)) || s == nA) : ((j == mid && !(both && (N & 1))) || s == nA + 1);
+    o.lastQ = !C && j == N - 1;
+    o.qrow = R.qrow;
+    return o;
+}
+
+// Layout of a row over a warp's lanes, from its length (coop_layout):
+//   blocked: lane L holds sites K L .. K L + K - 1 (K divides nx, nx / K <= 32 lanes): vector
+//            accesses, two shuffles for the x pass;
+//   strided: lane L holds sites L, L + 32, ... (any nx <= 256): scalar accesses, 2 K + 2 shuffles;
+//   tile:    like strided, of columns x0 - 1 .. x0 + 254 of which the outer two are halo (nx > 256).
+enum { BLOCKED = 0, STRIDED = 1, TILE = 2 };
+
+// K values of a lane at p: one access of 16, 8 or 4 bytes each where their size allows.
+template <typename T, int K>
+__device__ __forceinline__ void ldk(const T* p, T (&v)[K]) {
+    constexpr int B = K * (int)sizeof(T);
+    if constexpr (B % 16 == 0) {
+#pragma unroll
+        for (int i = 0; i < B / 16; ++i) {
+            const int4 t = ((const int4*)p)[i];
+            memcpy((char*)&v[0] + 16 * i, &t, 16);
+        }
+    } else if constexpr (B % 8 == 0 && sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i < B / 8; ++i) {
+            const float2 t = ((const float2*)p)[i];
+            v[2 * i] = t.x;
+            v[2 * i + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) v[i] = p[i];
+    }
+}
+template <typename T, int K>
+__device__ __forceinline__ void stk(T* p, const T (&v)[K]) {
+    constexpr int B = K * (int)sizeof(T);
+    if constexpr (B % 16 == 0) {
+#pragma unroll
+        for (int i = 0; i < B / 16; ++i) {
+            int4 t;
+            memcpy(&t, (const char*)&v[0] + 16 * i, 16);
+            ((int4*)p)[i] = t;
+        }
+    } else if constexpr (B % 8 == 0 && sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i < B / 8; ++i) ((float2*)p)[i] = make_float2(v[2 * i], v[2 * i + 1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) p[i] = v[i];
+    }
+}
+
+// n planes from za of x row (or x tile at x0) y.
+template <typename T, int K, int MODE>
+__device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, int x0, int y, int za, int n, T rr, int unit,
+                                         double& qs) {
+    // planes loaded ahead of their use: rows, and operands of the output plane
+    constexpr bool FEW = K * sizeof(T) <= 16;
+    constexpr int D = FEW ? 3 : 1, DE = FEW ? 2 : 1, U = D + 1;
+    const int lane = threadIdx.x & 31;
+    const int nx = R.nx, ny = R.ny, nz = R.nz;
+    const int plane = nx * ny;
+    const int r0 = y * nx;
+    const int dm = (y == 0 ? ny - 1 : -1) * nx, dp = (y == ny - 1 ? 1 - ny : 1) * nx;   // to the y neighbours
+    // lane's first column, its other columns, which of them exist
+    const int LL = MODE == BLOCKED ? nx / K - 1 : 31;   // blocked: last lane
+    const int xl = MODE == BLOCKED ? K * min(lane, LL) : lane;
+    auto col = [&](int k) {
+        if (MODE == BLOCKED) return xl + k;
+        if (MODE == STRIDED) return 32 * k + lane;
+        int x = x0 - 1 + 32 * k + lane;
+        return x < 0 ? x + nx : (x >= nx ? x - nx : x);
+    };
+    auto there = [&](int k) {   // loads: columns of the row (tile: up to the halo column of a ragged last tile)
+        if (MODE == BLOCKED) return true;
+        if (MODE == STRIDED) return k < K - 1 || 32 * (K - 1) + lane < nx;
+        return x0 - 1 + 32 * k + lane <= nx;
+    };
+    auto mine = [&](int k) {    // outputs
+        if (MODE == BLOCKED) return lane <= LL;
+        if (MODE == STRIDED) return k < K - 1 || 32 * (K - 1) + lane < nx;
+        const int c = 32 * k + lane;
+        return c >= 1 && c <= 32 * K - 2 && x0 - 1 + c < nx;
+    };
+    auto get = [&](const T* p, T (&v)[K], bool outs) {
+        if constexpr (MODE == BLOCKED) {
+            ldk<T, K>(p + xl, v);
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (outs ? mine(k) : there(k)) v[k] = p[col(k)];
+        }
+    };
+    auto put = [&](T* p, const T (&v)[K]) {
+        if constexpr (MODE == BLOCKED) {
+            if (lane <= LL) stk<T, K>(p + xl, v);
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (mine(k)) p[col(k)] = v[k];
+        }
+    };
+    T raw[U][3][K], e[U][K], st[U][K], q[U][K];
+#pragma unroll
+    for (int d = 0; d < U; ++d)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            raw[d][0][k] = raw[d][1][k] = raw[d][2][k] = T(1);
+            e[d][k] = st[d][k] = q[d][k] = T(0);
+        }
+    int zl = za == 0 ? nz - 1 : za - 1;                       // next plane to load
+    const T* sp = o.src + (size_t)zl * plane + r0;
+    int left = n + 2;
+    auto load = [&](T (&v)[3][K]) {
+        if (left <= 0) return;
+        --left;
+        if (o.src) {
+            get(sp + dm, v[0], false);
+            get(sp, v[1], false);
+            get(sp + dp, v[2], false);
+        }
+        sp += plane;
+        if (++zl == nz) {
+            zl = 0;
+            sp -= (size_t)nz * plane;
+        }
+    };
+    const size_t at0 = (size_t)za * plane + r0;
+    const T *pe = o.E + at0, *ps = o.st + at0;
+    T *pq = o.q + at0, *pd = o.dst + at0;                     // pq: to load; the plane being written is DE planes back
+    int eleft = n;
+    auto loade = [&](int d) {
+        if (eleft <= 0) return;
+        --eleft;
+        get(pe, e[d], true);
+        pe += plane;
+        if (o.st) {
+            get(ps, st[d], true);
+            if (!o.first) get(pq, q[d], true);
+            ps += plane;
+            pq += plane;
+        }
+    };
+    T* pw = o.q + at0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) load(raw[d]);
+    // operands of output plane i - 2 are loaded at step i - DE
+#pragma unroll
+    for (int d = 2 - DE; d < 0; ++d) loade((d + DE) % U);
+    T pm[K], p0[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) pm[k] = p0[k] = T(0);
+    const int lsrc = MODE == BLOCKED ? (lane == 0 ? LL : lane - 1) : ((lane + 31) & 31);
+    const int rsrc = MODE == BLOCKED ? (lane >= LL ? 0 : lane + 1) : ((lane + 1) & 31);
+    for (int i0 = 0; i0 < n + 2; i0 += U) {
+#pragma unroll
+        for (int d = 0; d < U; ++d) {
+            const int i = i0 + d;
+            if (i >= n + 2) break;
+            load(raw[(d + D) % U]);
+            if (i + DE >= 2) loade((d + DE) % U);
+            // y pass, then the x pass
+            T t[K], u[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) t[k] = fma(rr, raw[d][0][k] + raw[d][2][k], raw[d][1][k]);
+            if constexpr (MODE == BLOCKED) {
+                const T lv = __shfl_sync(0xffffffffu, t[K - 1], lsrc), rv = __shfl_sync(0xffffffffu, t[0], rsrc);
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    u[k] = fma(rr, (k ? t[k ? k - 1 : 0] : lv) + (k + 1 < K ? t[k + 1 < K ? k + 1 : k] : rv), t[k]);
+            } else {
+                T lf[K], rg[K];
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    lf[k] = __shfl_sync(0xffffffffu, t[k], lsrc);
+                    rg[k] = __shfl_sync(0xffffffffu, t[k], rsrc);
+                }
+                T lastv = lf[0], firstv = rg[0];
+                const int ll = (nx - 1) & 31;              // lane of the row's last site (register K - 1)
+                if constexpr (MODE == STRIDED) {
+                    lastv = __shfl_sync(0xffffffffu, t[K - 1], ll);
+                    firstv = __shfl_sync(0xffffffffu, t[0], 0);
+                }
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const T l = lane > 0 ? lf[k] : (k > 0 ? lf[k > 0 ? k - 1 : 0] : lastv);
+                    T r = lane < 31 ? rg[k] : rg[k < K - 1 ? k + 1 : k];
+                    if (MODE == STRIDED && k == K - 1) r = lane == ll ? firstv : r;
+                    u[k] = fma(rr, l + r, t[k]);
+                }
+            }
+            if (i >= 2) {
+                T g[K], v[K];
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const T sg = fma(rr, pm[k] + u[k], p0[k]);
+                    g[k] = e[d][k] * sg;
+                    v[k] = fma(st[d][k], sg, q[d][k]);
+                }
+                if (o.st) {
+                    put(pw, v);
+                    pw += plane;
+                }
+                if (o.dst) {
+                    put(pd, g);
+                    pd += plane;
+                }
+                if (o.lastQ) {
+                    double qp = 0.0;
+#pragma unroll
+                    for (int k = 0; k < K; ++k)
+                        if (mine(k)) qp += (double)g[k];
+                    if (o.qrow) {
+                        qp = warp_sum(qp);
+                        if (lane == 0) o.qrow[unit + i - 2] = qp;
+                    } else {
+                        qs += qp;
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                pm[k] = p0[k];
+                p0[k] = u[k];
+            }
+        }
+    }
+}
+
+// Rows of the x tiling: one whole row up to 256 sites, tiles of 254 columns beyond.
+constexpr int kCoopTile = 32 * 8 - 2;
+
+template <typename T, int K, int MODE, int C>
+__device__ __forceinline__ void coop_segment(const CoopRep& R, int j, int u0, int u1, double& qs) {
+    const CoopOps<T> o = coop_ops<T, C>(R, j);
+    const T rr = (T)R.rr;
+    const int nz = R.nz;
+    for (int u = u0; u < u1;) {
+        const int row = u / nz;
+        const int z = u - row * nz;
+        const int n = min(nz - z, u1 - u);
+        const int xt = MODE == TILE ? row / R.ny : 0, y = row - xt * R.ny;
+        coop_run<T, K, MODE>(R, o, xt * kCoopTile, y, z, n, rr, u, qs);
+        u += n;
+    }
+}
+
+// KK: row layout of every replica of the launch, or 0: a switch per replica.
+template <typename T, int KK, int C>
+__device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int j, int p, int b0, int b1) {
+    for (int i = 0; i < nact; ++i) {
+        const CoopRep& R = reps[i];
+        const int lay = KK > 0 ? KK : R.layout, w = lay & 15;
+        const int c0 = R.cost0, c1 = c0 + R.units * w;
+        if (c1 <= b0) continue;
+        if (c0 >= b1) break;
+        // this warp's units (row planes) of the replica: cost bounds rounded up to whole units
+        const int u0 = b0 > c0 ? (b0 - c0 + w - 1) / w : 0;
+        const int u1 = b1 < c1 ? (b1 - c0 + w - 1) / w : R.units;
+        double qs = 0.0;
+        if constexpr (KK > 0) {
+            coop_segment<T, (KK & 15), (KK >> 4) - 1, C>(R, j, u0, u1, qs);
+        } else {
+#define DSCF_COOP_CASE(KV, MV) case KV + 16 * (MV + 1): coop_segment<T, KV, MV, C>(R, j, u0, u1, qs); break;
+            switch (lay) {
+                DSCF_COOP_LAYOUTS(DSCF_COOP_CASE)
+                default: break;
+            }
+#undef DSCF_COOP_CASE
+        }
+        if (C == 0 && j == R.N - 1 && !R.qrow) {   // s = N: this warp's share of Q
+            const double t = warp_sum(qs);
+            if ((threadIdx.x & 31) == 0) R.pq[p] = t;
+        }
+    }
+}
+
+// Warps of a CTA, one CTA per SM: eight compute warps of up to 232 registers a thread (for the planes in
+// flight), and one warpgroup for the barriers, one warp per chain (the launch has 168 a thread:
+// 8 x 232 + 4 x 24 <= 12 x 168).
+constexpr int kCoopWarps = 8, kCoopSync = 4, kCoopRegs = 232, kCoopSyncRegs = 24;
+constexpr int kCoopShared = 128;   // largest table kept in shared memory
+constexpr long long kCoopSpinLimit = 1LL << 28;   // polls of a shared-memory mbarrier (see kBarSpinLimit in dscf_pers.cu)
+
+__device__ __forceinline__ unsigned csaddr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cbar_init(unsigned long long* bar, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(csaddr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void cbar_arrive(unsigned long long* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(csaddr(bar)) : "memory");
+}
+__device__ __forceinline__ bool cbar_test(unsigned long long* bar, unsigned parity) {
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred P1;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, P1;\n\t}\n"
+        : "=r"(done)
+        : "r"(csaddr(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+__device__ __forceinline__ void cbar_wait(unsigned long long* bar, unsigned parity, const CoopCtl& ctl, bool& dead) {
+    if (dead) return;
+    for (long long spins = 0; !cbar_test(bar, parity); ++spins)
+        if (spins > kCoopSpinLimit) {
+            atomicOr(ctl.status, (int)ST_TIMEOUT);
+            atomicExch(ctl.abort, 1);
+            dead = true;
+            return;
+        }
+}
+
+template <typename T, int KK>
+__global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(const CoopCtl ctl) {
+    constexpr int NW = kCoopWarps;
+    // the table in shared memory: the levels' acquire loads keep invalidating its cached copy
+    __shared__ CoopRep tab[kCoopShared];
+    __shared__ __align__(8) unsigned long long done[2], go[2];   // per chain: level computed here; computed everywhere
+    const int ncta = (int)gridDim.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool sync = ctl.j1 - ctl.j0 > 1;   // one level per launch: the launches are the barriers
+    const CoopRep* reps = ctl.nrep <= kCoopShared ? tab : ctl.reps;
+    if (ctl.nrep <= kCoopShared) {
+        constexpr int WORDS = sizeof(CoopRep) / sizeof(int);
+        for (int i = threadIdx.x; i < ctl.nrep * WORDS; i += blockDim.x) ((int*)tab)[i] = ((const int*)ctl.reps)[i];
+    }
+    if (threadIdx.x == 0) {
+        for (int c = 0; c < 2; ++c) {
+            cbar_init(&done[c], NW);
+            cbar_init(&go[c], 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncthreads();
+    bool dead = false;
+    if (w >= NW) {
+        // ---- barrier warps, one per chain: the compute warps go on with the other chain meanwhile ----
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kCoopSyncRegs));
+        const int c = w - NW;
+        if (!sync || c >= 2 || lane != 0) return;
+        bool aborted = cld_acquire(ctl.abort) != 0;
+        int* f = ctl.cnt + c * kFlagStride;
+        for (int d = 0; d < ctl.j1 - ctl.j0; ++d) {
+            cbar_wait(&done[c], (unsigned)(d & 1), ctl, dead);
+            // `done` orders the compute warps' stores before this release; release is cumulative
+            cred_release(f);
+            const int target = (d + 1) * ncta;
+            int spins = 0;
+            while (!aborted && cld_acquire(f) < target) {
+                if ((++spins & 31) == 0) {
+                    if (cld_acquire(ctl.abort) != 0) {
+                        aborted = true;
+                    } else if (spins > ctl.limit) {
+                        atomicOr(ctl.status, (int)ST_TIMEOUT);
+                        atomicExch(ctl.abort, 1);
+                        aborted = true;
+                    }
+                }
+                __nanosleep(20);
+            }
+            cbar_arrive(&go[c]);
+        }
+        // the last of all barrier warps leaves the counters at zero
+        __threadfence();
+        if (atomicInc((unsigned*)ctl.cnt + 2 * kFlagStride, 2u * (unsigned)ncta - 1u) == 2u * (unsigned)ncta - 1u) {
+            ctl.cnt[0] = 0;
+            ctl.cnt[kFlagStride] = 0;
+        }
+        return;
+    }
+    // ---- compute warps ----
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kCoopRegs));
+    // neighbouring runs (the same row, then the next rows) go to one CTA: their rows meet in its L1
+    const int p = blockIdx.x * NW + w, P = ncta * NW;
+    int nact = ctl.nrep + 1, b0 = 0, b1 = 0;   // active replicas; this warp's share of their cost
+    if (ctl.j0 == 0) {   // shares of Q of replicas this warp has none of
+        for (int r = lane; r < ctl.nrep; r += 32)
+            if (!reps[r].qrow) reps[r].pq[p] = 0.0;
+        __syncwarp();
+    }
+    for (int j = ctl.j0; j < ctl.j1; ++j) {
+        const int before = nact;
+        nact = min(nact, ctl.nrep);
+        while (nact > 0 && reps[nact - 1].N <= j) --nact;
+        if (nact != before) {
+            const CoopRep& last = reps[nact - 1];
+            const long long total = last.cost0 + last.units * (last.layout & 15);
+            b0 = (int)(total * p / P);
+            b1 = (int)(total * (p + 1) / P);
+        }
+        const int d = j - ctl.j0;            // levels of this launch before this one
+        const unsigned par = (unsigned)((d - 1) & 1);
+        if (sync && d > 0) {
+            cbar_wait(&go[0], par, ctl, dead);
+            // another cut of the work when chains end: what a warp has written itself so far may now
+            // be another warp's, so both chains' levels must be complete
+            if (nact != before) cbar_wait(&go[1], par, ctl, dead);
+            __syncwarp();
+        }
+        coop_level<T, KK, 0>(reps, nact, j, p, b0, b1);
+        if (sync) {
+            __syncwarp();
+            if (lane == 0) cbar_arrive(&done[0]);
+            if (d > 0) cbar_wait(&go[1], par, ctl, dead);
+            __syncwarp();
+        }
+        coop_level<T, KK, 1>(reps, nact, j, p, b0, b1);
+        if (sync) {
+            __syncwarp();
+            if (lane == 0) cbar_arrive(&done[1]);
+        }
+    }
+    if (sync) {
+        // Q: every 32 row planes of a replica make one partial sum, whatever the cut of the work, so a
+        // replica's Q is the same alone and in any batch
+        cbar_wait(&go[0], (unsigned)((ctl.j1 - ctl.j0 - 1) & 1), ctl, dead);
+        __syncwarp();
+        for (int r = 0; r < ctl.nrep; ++r) {
+            const CoopRep& R = reps[r];
+            const int units = R.units;
+            for (int g = p; 32 * g < units; g += P) {
+                const int u = 32 * g + lane;
+                const double t = warp_sum(u < units ? R.qrow[u] : 0.0);
+                if (lane == 0) R.pq[g] = t;
+            }
+        }
+    }
+}
+
+template <typename T>
+const void* coop_kernel(int kk) {
+#define DSCF_COOP_KERNEL(KV, MV) case KV + 16 * (MV + 1): return (const void*)k_prop_coop<T, KV + 16 * (MV + 1)>;
+    switch (kk) {
+        DSCF_COOP_LAYOUTS(DSCF_COOP_KERNEL)
+        default: return (const void*)k_prop_coop<T, 0>;
+    }
+#undef DSCF_COOP_KERNEL
+}
+
+}  // namespace
+
+// Checks that the kernels launch with the registers their warps share out (setmaxnreg would wait for
+// ever if they did not).
+template <typename T>
+int coop_prepare(int kk) {
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, coop_kernel<T>(kk));
+    if (e == cudaSuccess && fa.numRegs * (kCoopWarps + kCoopSync) < kCoopRegs * kCoopWarps + kCoopSyncRegs * kCoopSync)
+        e = cudaErrorInvalidConfiguration;
+    return (int)e;
+}
+
+template <typename T>
+int launch_prop_coop(const Launch& L, const CoopPlan& c, int j0, int j1, int limit) {
+    CoopCtl ctl;
+    ctl.reps = c.reps;
+    ctl.nrep = c.nrep;
+    ctl.j0 = j0;
+    ctl.j1 = j1;
+    ctl.cnt = c.cnt;
+    ctl.abort = c.abort;
+    ctl.status = L.status;
+    ctl.limit = limit;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c.ncta);
+    cfg.blockDim = dim3(32 * (kCoopWarps + kCoopSync));
+    cfg.stream = L.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = j1 - j0 > 1 ? 1 : 0;
+    void* args[] = {(void*)&ctl};
+    return (int)cudaLaunchKernelExC(&cfg, coop_kernel<T>(c.kk), args);
+}
+
+}  // namespace dscf

@@ -10,16 +10,12 @@ constexpr int kFlatThreads = 256;     // threads of every site-parallel ("flat")
 constexpr int kMaxFlatBlocks = 608;   // flat blocks per replica (= partial sums per replica): 4 per SM, one wave
 constexpr int kMaxNcg = 32;           // Fletcher-Reeves iterations per step, upper bound
 constexpr int kScalStride = 192;      // FP64 scalar slots per replica
-constexpr int kPropCols = 30;         // output x columns per propagator CTA (a warp minus 2 halo lanes)
-constexpr int kPropRows = 8;          // output y rows per propagator CTA
-// cp.async ring depth of the propagator kernels for an element size
-__host__ __device__ constexpr int prop_depth(size_t es) { return es == 8 ? 2 : 4; }
 
 // Partial-sum slots: one array of per-block FP64 partials per slot and replica.  Reducing a
 // slot is done redundantly, in a fixed order, by every block that needs the total, so the
 // result is bit-identical in all blocks and from run to run.
 enum PartSlot {
-    P_Q = 0,     // sum_r G_N(r)            (written by the last forward contour step)
+    P_Q = 0,     // sum_r G_N(r)            (written by the last forward contour step; nq entries)
     P_ES,        // sum_r exp(-U_S)         (written by the Boltzmann-factor kernel)
     P_H0,        // <g, d>
     P_CD,        // <d, phi_m d>
@@ -52,9 +48,11 @@ enum ScalSlot {
 // Device status bits.
 enum { ST_NONFINITE = 1, ST_TIMEOUT = 2 };
 // Layout of the status block: [0] status word, [1] LB step counter, [2] abort flag of the
-// persistent sweeps, [3] change flag of the solvent-component labelling, [kFlagBase..] one step
-// counter per persistent brick.
-constexpr int kFlagBase = 64;
+// persistent sweeps, [3] change flag of the solvent-component labelling, [kCoopBase..] the barrier
+// counters of the general sweeps (three lines), [kFlagBase..] the step counters of the persistent
+// bricks.
+constexpr int kCoopBase = 32;
+constexpr int kFlagBase = 128;
 constexpr int kFlagStride = 32;   // ints between bricks' step counters: one 128-byte line each
 constexpr int kFlagChain = 16;    // the backward chain's counter in that line (the forward's is first)
 constexpr int kMaxBricks = 4096;
@@ -66,9 +64,8 @@ constexpr size_t kStatusInts = (size_t)kFlagBase + (size_t)kMaxBricks * kFlagStr
 struct Rep {
     int nx, ny, nz, ns, N, nA;
     long long V;
-    int tiles_x, tiles_y, tiles_z, zc;     // propagator tiling
-    int vec;                               // 1, 2, 4: whole-row layout with nx = 32 vec; 0: tiled
-    int tile0, ntiles;
+    int nq;                                // P_Q partials of the sweep kernel in use
+    int nq_units;                          // general sweeps: row planes, entries of qrow
     int blk0, nblk, chunk;                 // flat tiling: nblk blocks of `chunk` sites
     int lb_blk0, lb_nblk;                  // LB grid: one site per thread, lb_nblk blocks
     int hydro, cn_sweeps;
@@ -99,22 +96,14 @@ struct Rep {
     double noise_amp2, noise_kT;
     unsigned long long noise_seed;
     int rep_index;                         // counter word 3 of the noise (replica in the batch)
+    double* qrow;   // general sweeps: sums of G_N per row plane
     double* part;   // [NPART][part_stride]
     int part_stride;
     double* scal;   // [kScalStride]
 };
 
-// Propagator and flat tiling of one replica for a given z-chunk; the context path and the
-// allocation-free path both use it.
-// rows256: every replica of the launch has rows of 256 sites, which then take the whole-row
-// contour kernels of their own (8 sites per lane); otherwise such rows take the tiled layout.
-inline void tile_replica(Rep& R, int zc, bool rows256 = false) {
-    R.vec = (R.nx == 32 || R.nx == 64 || R.nx == 128) ? R.nx / 32 : ((rows256 && R.nx == 256) ? 8 : 0);
-    R.tiles_x = R.vec ? 1 : (R.nx + kPropCols - 1) / kPropCols;
-    R.tiles_y = (R.ny + kPropRows - 1) / kPropRows;
-    R.zc = zc < 1 ? 1 : (zc > R.nz ? R.nz : zc);
-    R.tiles_z = (R.nz + R.zc - 1) / R.zc;
-    R.ntiles = R.tiles_x * R.tiles_y * R.tiles_z;
+// Flat tiling of one replica; the context path and the allocation-free path both use it.
+inline void tile_replica(Rep& R) {
     long long nb = (R.V + kFlatThreads - 1) / kFlatThreads;
     if (nb > kMaxFlatBlocks) nb = kMaxFlatBlocks;
     long long chunk = (R.V + nb - 1) / nb;
@@ -123,12 +112,10 @@ inline void tile_replica(Rep& R, int zc, bool rows256 = false) {
     R.nblk = (int)((R.V + chunk - 1) / chunk);
     R.lb_nblk = (int)((R.V + kFlatThreads - 1) / kFlatThreads);
 }
-constexpr int kMinZc = 4;             // smallest z-chunk the autotuner tries (most tiles)
 
 // Launch description shared by the host launchers.
 struct Launch {
     const Rep* reps;         // device table
-    const int* tile2rep;     // device map: propagator tile -> replica
     const int* blk2rep;      // device map: flat block -> replica
     int* status;             // device status word
     int* counter;            // device step counter (selects the LB buffer parity)
@@ -137,7 +124,6 @@ struct Launch {
     int nrep;
     int noise;               // thermal noise: 1 compositions, 2 LB modes
     cudaStream_t stream;
-    int w8 = 0;              // every replica in whole rows of 256 sites (their own contour kernels)
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -341,14 +327,44 @@ __device__ __forceinline__ float bexp(float x) { return expf(-x); }
 // ---------------------------------------------------------------------------------------------
 // Host launchers (defined in the kernel translation units, explicit per precision).
 // ---------------------------------------------------------------------------------------------
-template <typename T> void launch_prop_fwd(const Launch& L, int s, int grid, size_t smem);
-template <typename T> void launch_prop_bwd(const Launch& L, int j, int grid, size_t smem);
-template <typename T> int prop_set_smem_limit(size_t bytes);   // returns a cudaError_t
-size_t prop_smem_bytes(int vec, bool bwd, size_t es);           // dynamic shared memory of one CTA
-// fused contour groups of K steps (FP32, whole-row layout only)
-size_t prop_fused_smem_bytes(int vec, int K);
-void launch_prop_fused(const Launch& L, bool bwd, int K, int g, int grid, size_t smem);
-int prop_fused_set_smem_limit(size_t bytes);                    // returns a cudaError_t
+// General sweeps of both chains (dscf_coop.cu), levels j0 .. j1 - 1: a cooperative launch for several
+// levels, a plain one for one.  kk: row layout of every replica, 0 if they differ.
+// A replica as the general sweeps see it; their table holds the replicas by decreasing chain length.
+struct CoopRep {
+    int nx, ny, nz, N, nA;
+    int layout;          // coop_layout(nx)
+    int cost0;           // cost (row planes x sites per lane) of the entries before
+    int units;           // row planes
+    long long V;
+    void *E, *G, *Gp0, *Gp1, *q;
+    double *qrow, *pq;   // sums of G_N per row plane (or nullptr), the P_Q slot
+    double rr;           // alpha / (1 - 2 alpha)
+};
+struct CoopPlan {
+    const CoopRep* reps; // device table
+    int nrep;
+    int* cnt;            // device: barrier counters (3 lines), zero between launches
+    int* abort;
+    int kk, ncta;
+};
+// Row layout of a grid: sites per lane + 16 (1 + mode), mode 0 blocked, 1 strided, 2 tiled.  Blocked
+// where some K of 1, 2, 3, 4, 6, 8 divides nx into at most 32 lanes without leaving more than about
+// a third of them idle.
+__host__ __device__ constexpr int coop_layout(int nx) {
+    if (nx > 256) return 8 + 48;
+    const int k = (nx + 31) / 32;
+    for (int K = k; K <= 8 && 2 * K <= 3 * k + 1; ++K)
+        if (K != 5 && K != 7 && nx % K == 0) return K + 16;
+    return k + 32;
+}
+__host__ __device__ constexpr int coop_sites(int nx) { return coop_layout(nx) & 15; }
+constexpr int kCoopMaxCtas = 152;
+long long coop_units(const Rep& R);   // row planes (of x tiles beyond 256 sites)
+int coop_ctas(long long units, int nsm);
+int coop_warps_per_cta();
+CoopRep coop_rep(const Rep& R, int cost0);
+template <typename T> int coop_prepare(int kk);   // cudaError_t
+template <typename T> int launch_prop_coop(const Launch& L, const CoopPlan& c, int j0, int j1, int limit);   // cudaError_t
 // mode: 0 exp(-U), 1 trial exp(-(U + a1 d)), 2 commit U += a d then exp(-U), 3 exp(-Uext)
 template <typename T> void launch_exp(const Launch& L, int mode, int k, const void* Uext, int write_u = 0);
 // net != 0: the density at the evaluated potential is the learned predictor's output, stored in q

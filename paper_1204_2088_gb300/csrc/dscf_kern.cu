@@ -33,27 +33,51 @@ __device__ __forceinline__ void site_xyz(int i, int nx, int ny, int& x, int& y, 
 // phi_S = phi_s exp(-U_S)/<exp(-U_S)>.
 // ---------------------------------------------------------------------------------------------
 struct Norm {
-    double coef, qs, phis;
+    double coef, qs, phis, Q;
 };
+template <typename T>
 __device__ __forceinline__ Norm norm_of(const Rep& R, double* sh, int net = 0) {
     Norm n;
     if (net) {   // the learned predictor's output is already normalised
         n.coef = 1.0;
+        n.Q = 0.0;
         n.qs = 1.0;
         n.phis = 1.0 - R.phi_p;
         return n;
     }
-    const double Q = reduce_parts(slot(R, P_Q), R.ntiles, sh) / (double)R.V;
-    n.coef = R.phi_p / ((double)R.N * Q);
+    // the sweeps apply each pass of the stencil divided by its centre weight, c + r (a + d), and the
+    // Boltzmann factors of the copolymer carry the weight's cube; a quadrature has one stencil more than
+    // Boltzmann factors, so it lacks 1 / (1 + 2 r)^3, with r as rounded in the sweeps: only so do the
+    // densities keep their means (with be^3 instead they are off by up to 4e-8 in FP32)
+    const double Q = reduce_parts(slot(R, P_Q), R.nq, sh) / (double)R.V;
+    const double w = 1.0 + 2.0 * (double)(T)(R.alpha / (1.0 - 2.0 * R.alpha));
+    n.Q = Q;
+    n.coef = R.phi_p / ((double)R.N * Q) / (w * w * w);
     n.qs = (R.ns == 3) ? reduce_parts(slot(R, P_ES), R.nblk, sh) / (double)R.V : 1.0;
     n.phis = 1.0 - R.phi_p;
     return n;
 }
+// A factor of the model densities in the field precision: two parts for FP32, whose rounded factor alone
+// would shift every density the same way (up to 6e-8 of it, which the inversion turns into a shift of
+// the potentials).
+template <typename T>
+struct Fac {
+    T hi, lo;
+    __device__ __forceinline__ T operator()(T q) const {
+        if constexpr (sizeof(T) == 8) return hi * q;
+        else return fma(hi, q, lo * q);
+    }
+};
+template <typename T>
+__device__ __forceinline__ Fac<T> fac(double v) {
+    const T hi = (T)v;
+    return {hi, (T)(v - (double)hi)};
+}
 // phi_I[U] at one site in the field precision (FP64 only in the normalisation constants).
 template <typename T>
 __device__ __forceinline__ T model_phi(const Rep& R, const Norm& n, int I, int i) {
-    if (I < 2) return (T)n.coef * ((const T*)R.q)[(size_t)I * R.V + i];
-    return (T)n.phis * ((const T*)R.E)[2 * (size_t)R.V + i] / (T)n.qs;
+    if (I < 2) return fac<T>(n.coef)(((const T*)R.q)[(size_t)I * R.V + i]);
+    return fac<T>(n.phis / n.qs)(((const T*)R.E)[2 * (size_t)R.V + i]);
 }
 
 // FP32 fields with V a multiple of 4 are also walked as float4 (4 consecutive sites per thread and
@@ -64,14 +88,14 @@ __device__ __forceinline__ bool flat_vec(int V) {
     return false;
 }
 __device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
-// Scale and source of the model density of species I as a float4 stream: coef q_I, or for the
+// Factor and source of the model density of species I as a float4 stream: coef q_I, or for the
 // solvent phis E_S / qs.
-__device__ __forceinline__ const float* model_src(const Rep& R, const Norm& n, int I, float& sc) {
+__device__ __forceinline__ const float* model_src(const Rep& R, const Norm& n, int I, Fac<float>& sc) {
     if (I < 2) {
-        sc = (float)n.coef;
+        sc = fac<float>(n.coef);
         return (const float*)R.q + (size_t)I * R.V;
     }
-    sc = (float)(n.phis / n.qs);
+    sc = fac<float>(n.phis / n.qs);
     return (const float*)R.E + 2 * (size_t)R.V;
 }
 
@@ -81,13 +105,13 @@ __global__ void __launch_bounds__(kFlatThreads) k_trial(const Rep* __restrict__ 
                                                         int net) {
     __shared__ double sh[33];
     FLAT_PROLOGUE
-    const Norm n = norm_of(R, sh, net);
+    const Norm n = norm_of<T>(R, sh, net);
     const T* phi = (const T*)R.phi;
     const T* d = (const T*)R.d;
     T h1 = T(0);
     if (flat_vec<T>(V)) {
         const int ns = R.ns;
-        float sc[3];
+        Fac<float> sc[3];
         const float* src[3];
 #pragma unroll
         for (int I = 0; I < 3; ++I) src[I] = I < ns ? model_src(R, n, I, sc[I]) : nullptr;
@@ -98,8 +122,8 @@ __global__ void __launch_bounds__(kFlatThreads) k_trial(const Rep* __restrict__ 
                 if (I >= ns) break;
                 const size_t o = (size_t)I * V + i;
                 const float4 p = ld4((const float*)phi + o), dd = ld4((const float*)d + o), q = ld4(src[I] + i);
-                h1 += (T)((p.x - sc[I] * q.x) * dd.x + (p.y - sc[I] * q.y) * dd.y + (p.z - sc[I] * q.z) * dd.z +
-                          (p.w - sc[I] * q.w) * dd.w);
+                h1 += (T)((p.x - sc[I](q.x)) * dd.x + (p.y - sc[I](q.y)) * dd.y + (p.z - sc[I](q.z)) * dd.z +
+                          (p.w - sc[I](q.w)) * dd.w);
             }
         }
     } else {
@@ -125,9 +149,9 @@ __global__ void __launch_bounds__(kFlatThreads) k_grad(const Rep* __restrict__ r
                                                        int k, int net) {
     __shared__ double sh[33];
     FLAT_PROLOGUE
-    const Norm n = norm_of(R, sh, net);
+    const Norm n = norm_of<T>(R, sh, net);
     if (lb == 0 && threadIdx.x == 0 && !net) {
-        R.scal[S_Q] = n.coef > 0.0 ? R.phi_p / ((double)R.N * n.coef) : 0.0;
+        R.scal[S_Q] = n.coef > 0.0 ? n.Q : 0.0;
         R.scal[S_QS] = n.qs;
     }
     const T* __restrict__ phi = (const T*)R.phi;
@@ -135,7 +159,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_grad(const Rep* __restrict__ r
     T gg = T(0), gmax = T(0);
     if (flat_vec<T>(V)) {
         const int ns = R.ns;
-        float scs[3];
+        Fac<float> scs[3];
         const float* srcs[3];
 #pragma unroll
         for (int I = 0; I < 3; ++I) srcs[I] = I < ns ? model_src(R, n, I, scs[I]) : nullptr;
@@ -144,11 +168,11 @@ __global__ void __launch_bounds__(kFlatThreads) k_grad(const Rep* __restrict__ r
 #pragma unroll
             for (int I = 0; I < 3; ++I) {
                 if (I >= ns) break;
-                const float sc = scs[I];
+                const Fac<float> sc = scs[I];
                 const float* src = srcs[I];
                 const size_t o = (size_t)I * V + i;
                 const float4 q = ld4(src + i), p = ld4((const float*)phi + o);
-                const float4 m = make_float4(sc * q.x, sc * q.y, sc * q.z, sc * q.w);
+                const float4 m = make_float4(sc(q.x), sc(q.y), sc(q.z), sc(q.w));
                 *(float4*)((float*)pm + o) = m;
                 const float g0 = p.x - m.x, g1 = p.y - m.y, g2 = p.z - m.z, g3 = p.w - m.w;
                 gg += (T)(g0 * g0 + g1 * g1 + g2 * g2 + g3 * g3);
@@ -1130,7 +1154,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_dens_out(const Rep* __restrict
                                                            T* __restrict__ out) {
     __shared__ double sh[33];
     FLAT_PROLOGUE
-    const Norm n = norm_of(R, sh);
+    const Norm n = norm_of<T>(R, sh);
     for (int I = 0; I < R.ns; ++I)
         _Pragma("unroll 4") for (int i = i0 + threadIdx.x; i < i1; i += kFlatThreads)
             out[R.ext_off + (size_t)I * V + i] = model_phi<T>(R, n, I, i);

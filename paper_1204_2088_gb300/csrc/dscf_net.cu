@@ -632,12 +632,9 @@ constexpr int kPartBlocks = 512;   // partial sums per channel and sample
 
 // CTAs per dz of a weight gradient: one CTA per SM over the five dz (152 SMs), at most one per tile.
 constexpr int kWgradSplits = 30;
-int wgrad_tiles(int nx, int ny, int nz, int B) {
-    return B * nz * ((ny + WG_TY - 1) / WG_TY) * (nx / (nx % 32 == 0 ? 32 : 16));
-}
 int wgrad_splits(int nx, int ny, int nz, int B) {
-    const int t = wgrad_tiles(nx, ny, nz, B);
-    return t < kWgradSplits ? t : kWgradSplits;
+    const long long t = (long long)B * nz * ((ny + WG_TY - 1) / WG_TY) * (nx / (nx % 32 == 0 ? 32 : 16));
+    return t < kWgradSplits ? (int)t : kWgradSplits;
 }
 
 NetLayout net_layout(int nx, int ny, int nz, int B) {
@@ -666,7 +663,7 @@ NetLayout net_layout(int nx, int ny, int nz, int B) {
     L.dz2 = take(S * 32 * 2);
     L.dz1 = take(S * 32 * 2);
     L.gtmp = take(S * 2 * 4);
-    L.wpart = take((size_t)wgrad_splits(nx, ny, nz, B) * KVOL * 32 * 32 * 4);
+    L.wpart = take((size_t)kWgradSplits * KVOL * 32 * 32 * 4);
     const size_t ntc = tc_conv_supported(nx, ny) ? (size_t)tc_conv_blocks(nx, ny, nz) : 0;
     L.part = take((size_t)B * 2 * (ntc > (size_t)kPartBlocks ? ntc : (size_t)kPartBlocks) * 8);
     L.means = take((size_t)B * 2 * 8);

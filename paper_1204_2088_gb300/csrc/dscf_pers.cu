@@ -13,9 +13,9 @@
 // computes the other chain's unit.  128^3, N = 64: 540 us for the two sweeps one after the other
 // (4.2 us a contour step, the exchange in the open), 345 us so (2.7 us).
 //
-// The lattice is cut into bricks of nx x PBY x BZ sites, one brick per CTA (one CTA per SM for
-// BZ = 16, two for BZ = 8; the launch is cooperative, so all CTAs are resident together), one
-// compute warp per plane of the brick and four warps for the exchange.  Rows of 96 or 128 sites
+// The lattice is cut into bricks of nx x PBY x BZ sites, one brick per CTA and one CTA per SM (the
+// launch is cooperative, so all CTAs are resident together), one compute warp per plane of the
+// brick and four warps for the exchange.  Rows of 96 or 128 sites
 // are held by a whole warp (3 or 4 sites per lane), rows of 32, 48 or 64 sites by half a warp (2,
 // 3 or 4 sites per lane), two rows side by side; bricks of these narrow rows have 16 rows instead
 // of 8 where ny allows it.  A CTA takes its brick from a table (replica, brick, flag base), so
@@ -37,8 +37,8 @@
 // The Boltzmann factors of both species and both quadrature accumulators (each as large as the
 // brick) live in tensor memory, one 32-bit column per thread and value (tcgen05.ld / st): beside
 // the two chains' rows they do not fit in the registers.  The allocation never waits for another
-// sweep: the registers let one CTA of 16 compute warps (all 512 columns) or two of 8 (256 each)
-// on an SM, whatever context or stream they belong to.
+// sweep: the registers let one CTA of 16 compute warps (all 512 columns) or one of 8 (256) on an
+// SM, whatever context or stream they belong to.
 // Each 1-D pass of the separable stencil is one add and one fma per site, as packed f32x2 pairs
 // (a scalar tail for three sites per lane), with the centre weight folded into the Boltzmann
 // factors.  Every wait is bounded: on timeout the CTA sets a status bit and a global abort flag
@@ -58,16 +58,15 @@ namespace {
 // shorter neighbour-wait limit set for failure tests must not abandon a copy that is still landing
 // in this CTA's shared memory).
 constexpr long long kBarSpinLimit = 1LL << 28;
-// Compute warps per CTA: 16 for bricks of 16 planes (one CTA per SM), 8 for bricks of 8 planes, two
-// CTAs per SM.  Beside them one warpgroup of four warps, of which two do the exchange (one per
-// chain): a whole warpgroup, so that it can hand most of its registers to the compute warps
-// (setmaxnreg).  Launched registers a thread (what the launch bounds leave): 96 for 640 threads,
-// 80 for 384 threads twice; the shares 512 x 112 + 128 x 32 = 640 x 96 and
-// 256 x 104 + 128 x 24 <= 384 x 80 stay within them.
+// Compute warps per CTA: 16 for bricks of 16 planes, 8 for bricks of 8 planes; one CTA per SM.
+// Beside them one warpgroup of four warps does the exchange (two per chain): a whole warpgroup, so that
+// it can hand most of its registers to the compute warps (setmaxnreg).  Launched registers a thread
+// (what the launch bounds leave): 96 for 640 threads, 168 for 384; the shares 512 x 112 + 128 x 32 =
+// 640 x 96 and 256 x 208 + 128 x 24 <= 384 x 168 stay within them.
 constexpr int kXWarps = 4;
 template <int NW>
 struct PersRegs {
-    static constexpr int compute = NW == 16 ? 112 : 104;
+    static constexpr int compute = NW == 16 ? 112 : 208;
     static constexpr int exchange = NW == 16 ? 32 : 24;
 };
 
@@ -267,13 +266,7 @@ __device__ __forceinline__ void fmav(const float (&g)[VEC], const float (&v)[VEC
         upk2(fma2(pk2(g[k], g[k + 1]), pk2(v[k], v[k + 1]), pk2(q[k], q[k + 1])), q[k], q[k + 1]);
     if constexpr (VEC & 1) q[VEC - 1] = __fmaf_rn(g[VEC - 1], v[VEC - 1], q[VEC - 1]);
 }
-// scalar c times each site
-template <int VEC>
-__device__ __forceinline__ void scalev(float c, unsigned long long c2, float (&v)[VEC]) {
-#pragma unroll
-    for (int k = 0; k + 1 < VEC; k += 2) upk2(mul2(c2, pk2(v[k], v[k + 1])), v[k], v[k + 1]);
-    if constexpr (VEC & 1) v[VEC - 1] = __fmul_rn(c, v[VEC - 1]);
-}
+
 
 // Arrays of a replica as the sweep uses them, in shared memory (the descriptor itself is in device
 // memory, whose cached copy the acquire loads keep invalidating).
@@ -629,10 +622,9 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
         const int lsrc = seg + ((li + LPR - 1) & (LPR - 1)), rsrc = seg + ((li + 1) & (LPR - 1));
         // Each 1-D pass is applied as c + r (a + d) with r = alpha / (1 - 2 alpha), i.e. the
         // stencil's pass divided by its centre weight be = 1 - 2 alpha; the three passes then give
-        // sigma / be^3, and be^3 is folded into the Boltzmann factors (and into q at its write-out).
+        // sigma / be^3; the Boltzmann factors carry be^3, the normalisation gives it back to q.
         const double be_d = 1.0 - 2.0 * R.alpha;
-        const float rr = (float)(R.alpha / be_d), be3 = (float)(be_d * be_d * be_d);
-        const unsigned long long be32 = pk2(be3, be3);
+        const float rr = (float)(R.alpha / be_d);
         // own plane never wraps: (row r, plane w) is own0 + r * W
         const size_t own0 = (size_t)(z0 + w) * plane + (size_t)(y0 + hf * RPL) * W + xo;
         PersWarp k = {arr, ctl, full, pub, YS, HS, GS + (w * PBY + hf * RPL) * W + xo, own0,
@@ -641,7 +633,7 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
                       tmem_slot + ((unsigned)((w & 3) * 32) << 16) + (unsigned)((w >> 2) * 128), 0.f, false};
         const unsigned tbase = k.tbase;
 
-        // tensor memory regions: 0, 1 Boltzmann factors of A, B (scaled by be^3); 2, 3 quadratures
+        // tensor memory regions: 0, 1 Boltzmann factors of A, B; 2, 3 quadratures
 #pragma unroll
         for (int I = 0; I < 2; ++I) {
             const float* E = (const float*)R.E + (size_t)I * V;
@@ -649,7 +641,6 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
             for (int p = 0; p < RPL; ++p) {
                 float t[VS], zero[VS], e[VEC];
                 ldv<VEC>(E + own0 + (size_t)p * W, e);
-                scalev<VEC>(be3, be32, e);
 #pragma unroll
                 for (int i = 0; i < VS; ++i) {
                     t[i] = i < VEC ? e[i < VEC ? i : 0] : 0.f;
@@ -673,7 +664,7 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
             pers_unit<W, PBY, BZ, NW, 0>(k, xF, j);
             pers_unit<W, PBY, BZ, NW, 1>(k, xB, j);
         }
-        // both quadratures, scaled back by be^3
+        // both quadratures
 #pragma unroll
         for (int I = 0; I < 2; ++I) {
             float* q = (float*)R.q + (size_t)I * V;
@@ -684,7 +675,6 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
                 tm_wait_ld<VS>(t);
 #pragma unroll
                 for (int i = 0; i < VEC; ++i) o[i] = t[i];
-                scalev<VEC>(be3, be32, o);
                 stv<VEC>(q + own0 + (size_t)p * W, o);
             }
         }
@@ -700,14 +690,11 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
             if (lane == 0) slot(R, P_Q)[b] = q;
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_slot), "r"(TCOLS) : "memory");
         }
-        if (b == 0) {   // slots past the replica's bricks (the propagator tiling may have more)
-            for (int i = threadIdx.x + nby * nbz; i < R.ntiles; i += 32 * NW) slot(R, P_Q)[i] = 0.0;
-        }
     }
 }
 
 template <int W, int PBY, int BZ, int NW>
-__global__ void __launch_bounds__(32 * (NW + kXWarps), 16 / NW) k_prop_pers(const Rep* __restrict__ reps, PersCtl ctl) {
+__global__ void __launch_bounds__(32 * (NW + kXWarps), 1) k_prop_pers(const Rep* __restrict__ reps, PersCtl ctl) {
     pers_sweep<W, PBY, BZ, NW>(reps, ctl);
 }
 
@@ -715,7 +702,7 @@ __global__ void __launch_bounds__(32 * (NW + kXWarps), 16 / NW) k_prop_pers(cons
 // its replica's width; the launch's dynamic shared memory covers the largest.  128-wide replicas
 // keep launches of their own (with them in the same function the registers would spill).
 template <int BZ, int NW>
-__global__ void __launch_bounds__(32 * (NW + kXWarps), 16 / NW) k_prop_pers_mix(const Rep* __restrict__ reps, PersCtl ctl) {
+__global__ void __launch_bounds__(32 * (NW + kXWarps), 1) k_prop_pers_mix(const Rep* __restrict__ reps, PersCtl ctl) {
     const Rep& R = reps[ctl.table[blockIdx.x].x];
     const int pby = pers_pby_of(R.nx, R.ny);
     switch (R.nx * 32 + pby) {
@@ -743,7 +730,8 @@ size_t pers_mix_smem_bytes(int bz) {
     return m;
 }
 
-// Brick depths: 16 planes on 16 warps (one CTA per SM) or 8 planes on 8 warps (two CTAs per SM).
+// Brick depths: 16 planes on 16 warps or 8 planes on 8 warps.  (Grids of up to two shallow bricks per SM
+// are accepted; more than one do not run together, and such grids take the general sweeps.)
 bool pers_supported(const Rep& R, int bz, int nw, int nsm) {
     if (!pers_width_ok(R.nx) || R.ny % 8 || R.nz % bz) return false;
     if (!((bz == 16 && nw == 16) || (bz == 8 && nw == 8))) return false;   // one warp per plane
@@ -809,7 +797,7 @@ namespace {
 // The SM that runs each CTA of a launch shaped like the sweep (same block size, shared memory
 // and cooperative attribute), for the placement of bricks on SMs.
 template <int NW>
-__global__ void __launch_bounds__(32 * (NW + kXWarps), 16 / NW) k_pers_place(int* smid) {
+__global__ void __launch_bounds__(32 * (NW + kXWarps), 1) k_pers_place(int* smid) {
     if (threadIdx.x == 0) {
         unsigned id;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(id));

@@ -32,9 +32,12 @@ unsigned char* g_scratch_dev[kMaxDevices] = {};   // device address of g_scratch
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Writes the replica descriptor into the scratch; passed by value so no host-to-device copy
-// (and no staging buffer) is needed.
-__global__ void k_put_rep(Rep* dst, Rep r) { *dst = r; }
+// Writes the replica descriptors into the scratch; passed by value so no host-to-device copy (and no
+// staging buffer) is needed.
+__global__ void k_put_rep(Rep* dst, Rep r, CoopRep* dstc, CoopRep c) {
+    *dst = r;
+    *dstc = c;
+}
 
 }  // namespace
 
@@ -96,24 +99,33 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     std::memset(&R, 0, sizeof R);
     R.nx = p->nx; R.ny = p->ny; R.nz = p->nz; R.ns = p->ns; R.N = p->N; R.nA = p->nA;
     R.V = (long long)p->nx * p->ny * p->nz;
-    tile_replica(R, 8);
+    tile_replica(R);
     R.phi_p = p->phi_p;
     R.alpha = p->a * p->a / 6.0;
-    R.part_stride = R.ntiles > R.nblk ? R.ntiles : R.nblk;
+    int nsm = 0;
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        set_thread_error("dscf_densities_static: device query failed");
+        return DSCF_ERR_CUDA;
+    }
+    if (nsm > kCoopMaxCtas) nsm = kCoopMaxCtas;
+    const long long units = coop_units(R);
+    const int ncta = coop_ctas(units, nsm);
+    R.nq = ncta * coop_warps_per_cta();
+    R.part_stride = R.nq > R.nblk ? R.nq : R.nblk;
 
     // Scratch layout: replica table, maps, Boltzmann factors, propagators, quadratures,
     // partial sums, scalars.
     const size_t V = (size_t)R.V;
     size_t off = 0;
     const size_t o_rep = off; off = up256(off + sizeof(Rep));
-    const size_t o_t2r = off; off = up256(off + sizeof(int) * R.ntiles);
+    const size_t o_coop = off; off = up256(off + sizeof(CoopRep));
     const size_t o_b2r = off; off = up256(off + sizeof(int) * R.nblk);
     const size_t o_E = off; off = up256(off + (size_t)R.ns * V * es);
     const size_t o_G = off; off = up256(off + (size_t)R.N * V * es);
     const size_t o_Gp0 = off; off = up256(off + V * es);
     const size_t o_Gp1 = off; off = up256(off + V * es);
     const size_t o_q = off; off = up256(off + 2 * V * es);
-    const size_t o_part = off; off = up256(off + sizeof(double) * NPART * (size_t)R.part_stride);
+    const size_t o_part = off; off = up256(off + sizeof(double) * 2 * (size_t)R.part_stride);   // P_Q, P_ES
     const size_t o_scal = off; off = up256(off + sizeof(double) * kScalStride);
     if (off > (size_t)DSCF_STATIC_SCRATCH_BYTES) {
         set_thread_error("dscf_densities_static: the problem needs more scratch than DSCF_STATIC_SCRATCH_BYTES");
@@ -133,13 +145,6 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
                 return DSCF_ERR_CUDA;
             }
             g_scratch_dev[dev] = (unsigned char*)ptr;
-            // dynamic shared memory of the propagator kernels, for the largest layout
-            if (prop_set_smem_limit<double>(prop_smem_bytes(4, true, 8)) != 0 ||
-                prop_set_smem_limit<float>(prop_smem_bytes(4, true, 4)) != 0) {
-                g_scratch_dev[dev] = nullptr;
-                set_thread_error("dscf_densities_static: cudaFuncSetAttribute failed");
-                return DSCF_ERR_CUDA;
-            }
         }
         base = g_scratch_dev[dev];
     }
@@ -150,15 +155,19 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     R.q = base + o_q;
     R.part = (double*)(base + o_part);
     R.scal = (double*)(base + o_scal);
-    R.tile0 = 0;
     R.blk0 = 0;
     R.ext_off = 0;
     R.vbase = 0;
 
+    const int kk = coop_layout(R.nx);
+    if ((precision == DSCF_FP64 ? coop_prepare<double>(kk) : coop_prepare<float>(kk)) != 0) {
+        set_thread_error("dscf_densities_static: the contour kernels do not load");
+        return DSCF_ERR_CUDA;
+    }
+
     cudaStream_t s = (cudaStream_t)stream;
     Launch L;
     L.reps = (const Rep*)(base + o_rep);
-    L.tile2rep = (const int*)(base + o_t2r);
     L.blk2rep = (const int*)(base + o_b2r);
     L.status = nullptr;
     L.counter = nullptr;
@@ -166,23 +175,26 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     L.nlb_total = R.lb_nblk;
     L.nrep = 1;
     L.stream = s;
-    // the only state that must start at zero: the tile and block maps (one replica, index 0)
-    cudaError_t e = cudaMemsetAsync(base + o_t2r, 0, sizeof(int) * R.ntiles, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + o_b2r, 0, sizeof(int) * R.nblk, s);
+    CoopPlan plan;
+    plan.reps = (const CoopRep*)(base + o_coop);
+    plan.nrep = 1;
+    plan.cnt = plan.abort = nullptr;   // one level per launch: no barrier inside a launch
+    plan.kk = kk;
+    plan.ncta = ncta;
+    // the only state that must start at zero: the block map (one replica, index 0)
+    cudaError_t e = cudaMemsetAsync(base + o_b2r, 0, sizeof(int) * R.nblk, s);
     if (e != cudaSuccess) {
         set_thread_error("dscf_densities_static: cudaMemsetAsync failed");
         return DSCF_ERR_CUDA;
     }
-    k_put_rep<<<1, 1, 0, s>>>((Rep*)(base + o_rep), R);
+    k_put_rep<<<1, 1, 0, s>>>((Rep*)(base + o_rep), R, (CoopRep*)(base + o_coop), coop_rep(R, 0));
     if (precision == DSCF_FP64) {
         launch_exp<double>(L, 3, 0, U_in);
-        for (int k = 1; k <= R.N; ++k) launch_prop_fwd<double>(L, k, R.ntiles, prop_smem_bytes(R.vec, false, 8));
-        for (int j = 0; j < R.N; ++j) launch_prop_bwd<double>(L, j, R.ntiles, prop_smem_bytes(R.vec, true, 8));
+        for (int j = 0; j < R.N; ++j) launch_prop_coop<double>(L, plan, j, j + 1, 1);
         launch_dens_out<double>(L, phi_out);
     } else {
         launch_exp<float>(L, 3, 0, U_in);
-        for (int k = 1; k <= R.N; ++k) launch_prop_fwd<float>(L, k, R.ntiles, prop_smem_bytes(R.vec, false, 4));
-        for (int j = 0; j < R.N; ++j) launch_prop_bwd<float>(L, j, R.ntiles, prop_smem_bytes(R.vec, true, 4));
+        for (int j = 0; j < R.N; ++j) launch_prop_coop<float>(L, plan, j, j + 1, 1);
         launch_dens_out<float>(L, phi_out);
     }
     e = cudaGetLastError();

@@ -1,0 +1,129 @@
+"""Edges of the sweep and network kernels against the FP64 oracle: every row layout of the general
+sweeps, chain lengths around the place where the two chains meet, batches of unlike replicas, and
+ragged blocks of the network's mma.sync kernels.  Tolerances as in test_gpu_parity.py (FP64 1e-12,
+FP32 1e-5 of the largest value) and test_gpu_net_exact.py (exact, or the FP32 accumulation bound)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1204_2088_gb300 import build, dscf, inputs
+from test_gpu_net_exact import B, bf16, emulate_forward, exact_problem, flat, paired_integers
+from test_gpu_parity import melt, ncomp_shape, random_state, rel, run_gpu, solution, t2n
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    dscf.load()
+
+
+def check_densities(cfg, precision, seed, tuning=None):
+    U = inputs.random_field(ncomp_shape(cfg), seed=seed, scale=0.5)
+    ref, _, _ = oracle.densities(cfg, U)
+    ctx = dscf.Context(cfg, precision, tuning=tuning)
+    for _ in range(2):      # twice: the counters carry over between launches
+        got = t2n(ctx.densities(torch.from_numpy(U)))
+        ctx.status()
+        assert rel(got, ref) < (1e-12 if precision == dscf.FP64 else 1e-5)
+
+
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("nx", [1, 2, 31, 32, 33, 45, 53, 66, 96, 97, 100, 128, 131, 160, 163, 192, 200, 211, 224, 255,
+                                256, 257, 300, 511])
+def test_general_sweeps_row_layouts(nx, precision):
+    check_densities(melt((nx, 3, 5), 5, 2), precision, 20, tuning=(8, 1))
+
+
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 8, 9])
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+def test_general_sweeps_where_the_chains_meet(N, precision):
+    for nA in range(1, N):
+        check_densities(melt((34, 7, 6), N, nA), precision, 30 + N, tuning=(8, 1))
+
+
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 8, 9])
+@pytest.mark.parametrize("grid,zc", [((128, 16, 16), 16), ((64, 8, 8), 8), ((48, 16, 32), 16)])
+def test_brick_sweeps_where_the_chains_meet(N, grid, zc):
+    for nA in range(1, N):
+        check_densities(melt(grid, N, nA), dscf.FP32, 40 + N, tuning=(zc, 0))
+
+
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+def test_general_sweeps_of_unlike_replicas_equal_solo_runs(precision):
+    """Row layouts, chain lengths (the cut of the work changes as chains end) and species mixed."""
+    cfgs = [melt((33, 9, 10), 9, 4, hydro=1, ncg_iters=2, cn_sweeps=4),
+            solution((100, 4, 6), 6, 3, hydro=1, ncg_iters=2, cn_sweeps=4),
+            melt((12, 10, 8), 2, 1, hydro=1, ncg_iters=2, cn_sweeps=4),
+            melt((300, 3, 4), 5, 3, hydro=1, ncg_iters=2, cn_sweeps=4)]
+    states = [random_state(c, 80 + 3 * i) for i, c in enumerate(cfgs)]
+    ctx = dscf.Context(cfgs, precision)
+    dt = ctx.dtype
+    for which, k in ((dscf.PHI, 0), (dscf.U, 1), (dscf.POP, 2)):
+        ctx.set(which, torch.from_numpy(np.concatenate([s[k].ravel() for s in states])).to(dt).cuda())
+    ctx.step(2)
+    ctx.status()
+    phi = t2n(ctx.get(dscf.PHI))
+    off = 0
+    for c, (p, U, dn) in zip(cfgs, states):
+        solo = run_gpu(c, precision, p, U, dn, 2)
+        assert np.array_equal(phi[off:off + p.size], solo["phi"].ravel())
+        off += p.size
+
+
+def test_bricks_that_do_not_run_together_take_the_general_sweeps():
+    """256 shallow bricks: the tuning stays valid, the densities are those of the deep bricks."""
+    cfg = melt((128, 128, 128), 3, 2)
+    U = torch.from_numpy(inputs.random_field(ncomp_shape(cfg), seed=50, scale=0.5)).float().cuda()
+    out = []
+    for zc in (8, 16):
+        ctx = dscf.Context(cfg, dscf.FP32, tuning=(zc, 0))
+        assert ctx.diagnostics()["kfuse"] == 0 and ctx.diagnostics()["zc"] == zc
+        out.append(t2n(ctx.densities(U)))
+        ctx.status()
+        ctx.close()
+    assert rel(out[0], out[1]) < 1e-5
+
+
+@pytest.mark.parametrize("grid", [(16, 3, 2), (48, 5, 3), (32, 1, 4), (112, 9, 1), (96, 4, 5)], ids=lambda g: "x".join(map(str, g)))
+def test_mma_forward_on_ragged_blocks(grid):
+    """Every convolution sum is exact; the means (sums / V, V not a power of two) are not: the kernel
+    rounds phibar - <y> and its sum with y to FP32."""
+    U, params = exact_problem(grid)
+    ref, (_, _, _, y) = emulate_forward(params, U, [0.5, 0.5], grid)
+    net = dscf.Net(grid, B, seed=1)
+    net.set_params(torch.from_numpy(flat(params)).float())
+    got = net.forward(torch.from_numpy(U).float(), [0.5, 0.5]).cpu().numpy().astype(np.float64)
+    shift = np.abs(0.5 - y.mean(axis=(2, 3, 4), keepdims=True))
+    assert np.all(np.abs(got - ref) <= 2.0 ** -24 * (shift + np.abs(ref)) * (1 + 2.0 ** -20))
+
+
+@pytest.mark.parametrize("grid", [(16, 4, 2), (32, 16, 8), (64, 2, 16), (16, 1, 64)], ids=lambda g: "x".join(map(str, g)))
+def test_weight_gradients_on_ragged_tiles(grid):
+    U, params = exact_problem(grid)
+    (W1, b1), (W2, b2), (W3, b3) = params
+    phi, (x, h1, h2, y) = emulate_forward(params, U, [0.5, 0.5], grid)
+    nx, ny, nz = grid
+    V = nx * ny * nz
+    t = np.stack([np.stack([paired_integers(V, 1, 7, 700 + 10 * b + c).reshape(nz, ny, nx) for c in range(2)])
+                  for b in range(B)])
+    t = (2 * t - np.sign(t)) / 16.0
+    n = phi.size                              # a power of two: dy is exact in BF16
+    dy = bf16(t / n)
+    dW3, _, dh2 = oracle.conv3d_bwd(grid, B, W3, h2, dy)
+    dz2 = bf16(dh2 * (1.0 - h2 * h2))
+    dW2, _, dh1 = oracle.conv3d_bwd(grid, B, W2, h1, dz2)
+    dz1 = bf16(dh1 * (1.0 - h1 * h1))
+    dW1, _, _ = oracle.conv3d_bwd(grid, B, W1, x, dz1, want_din=False)
+    aW2 = oracle.conv3d_bwd(grid, B, np.abs(W2), np.abs(h1), np.abs(dz2), want_din=False)[0]
+    aW1 = oracle.conv3d_bwd(grid, B, np.abs(W1), np.abs(x), np.abs(dz1), want_din=False)[0]
+    net = dscf.Net(grid, B, seed=1)
+    net.set_params(torch.from_numpy(flat(params)).float())
+    _, g = net.gradient(torch.from_numpy(U).float(), torch.from_numpy(phi - t).float(), [0.5, 0.5])
+    (gW1, _), (gW2, _), (gW3, _) = dscf.net_params_split(g.cpu().numpy())
+    assert np.array_equal(gW3, dW3) and np.abs(dW3).max() > 0
+    for got, ref, a in ((gW2, dW2, aW2), (gW1, dW1, aW1)):
+        assert np.all(np.abs(got - ref) <= B * V * 2.0 ** -22 * a)
+        assert np.abs(ref).max() > 0
