@@ -147,6 +147,7 @@ Layout make_layout(const dscf_params* p, int n, int prec, char* base) {
         R.mass0[2] = q.ns == 3 ? (double)R.V * (1.0 - q.phi_p) : 0.0;
         R.ext_off = ext;
         R.vbase = vb;
+        set_pars(R);
         ext += (long long)q.ns * R.V;
         vb += R.V;
         L.Nmax = std::max(L.Nmax, q.N);
@@ -617,8 +618,6 @@ int check_predictor(dscf_ctx* c, bool after_pred) {
 int set_dev(dscf_ctx* c) { return cuda_check(c, cudaSetDevice(c->device), "cudaSetDevice"); }
 
 int upload_tiles(dscf_ctx* c) {
-    // partial sums of Q that the sweeps in use leave
-    for (Rep& R : c->L.reps) R.nq = c->bricks ? pers_bricks(R, c->pers_bz) : (R.nq_units + 31) / 32;
     int rc = cuda_check(c, cudaMemcpyAsync(c->d_reps, c->L.reps.data(), sizeof(Rep) * c->nrep, cudaMemcpyHostToDevice,
                                            c->stream), "reps");
     if (rc) return rc;
@@ -1187,6 +1186,7 @@ int dscf_set_noise(dscf_ctx* c, double omega, int32_t lb_noise, uint64_t seed) {
         R.noise_amp2 = omega > 0.0 ? 2.0 * q.M * q.dt / omega : 0.0;
         R.noise_kT = (omega > 0.0 && lb_noise) ? q.dt * q.dt / omega : 0.0;
         R.noise_seed = seed;
+        set_pars(R);
     }
     if (int rc = cuda_check(c, cudaMemcpyAsync(c->d_reps, c->L.reps.data(), sizeof(Rep) * c->nrep,
                                                cudaMemcpyHostToDevice, c->stream), "noise parameters"))

@@ -424,6 +424,7 @@ __global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(
     // the table in shared memory: the levels' acquire loads keep invalidating its cached copy
     __shared__ CoopRep tab[kCoopShared];
     __shared__ __align__(8) unsigned long long done[2], go[2];   // per chain: level computed here; computed everywhere
+    __shared__ bool fin;
     const int ncta = (int)gridDim.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool sync = ctl.j1 - ctl.j0 > 1;   // one level per launch: the launches are the barriers
     const CoopRep* reps = ctl.nrep <= kCoopShared ? tab : ctl.reps;
@@ -529,6 +530,23 @@ __global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(
                 const int u = 32 * g + lane;
                 const double t = warp_sum(u < units ? R.qrow[u] : 0.0);
                 if (lane == 0) R.pq[g] = t;
+            }
+        }
+        // the last CTA adds up the partial sums, in order
+        asm volatile("bar.sync 1, %0;\n" ::"r"(32 * NW) : "memory");
+        if (threadIdx.x == 0) {
+            __threadfence();
+            fin = atomicInc((unsigned*)ctl.cnt + 2 * kFlagStride + 16, (unsigned)ncta - 1u) == (unsigned)ncta - 1u;
+        }
+        asm volatile("bar.sync 1, %0;\n" ::"r"(32 * NW) : "memory");
+        if (fin) {
+            __threadfence();
+            for (int r = w; r < ctl.nrep; r += NW) {
+                const CoopRep& R = reps[r];
+                double s = 0.0;
+                for (int g = lane; 32 * g < R.units; g += 32) s += __ldcg(R.pq + g);
+                s = warp_sum(s);
+                if (lane == 0) *R.qsum = s;
             }
         }
     }

@@ -23,6 +23,7 @@ CoopRep coop_rep(const Rep& R, int cost0) {
     c.E = R.E; c.G = R.G; c.Gp0 = R.Gp0; c.Gp1 = R.Gp1; c.q = R.q;
     c.qrow = R.qrow;
     c.pq = R.part + (size_t)P_Q * R.part_stride;
+    c.qsum = R.scal + S_QSUM;
     c.rr = R.alpha / (1.0 - 2.0 * R.alpha);
     return c;
 }

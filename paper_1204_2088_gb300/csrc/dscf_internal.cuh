@@ -41,6 +41,9 @@ enum ScalSlot {
     S_H0S, S_CDS, S_H1S,         // line search: <g,d>, <d, phi_m d>, h1
     S_GGS0, S_GGS1,              // <g,g> in the parity slots of the iterations
     S_TOT0, S_TOT1, S_TOT2,      // sum_r phi_I before the mass correction
+    S_QSUM, S_ESS,               // sum_r G_N(r) and sum_r exp(-U_S) of the last evaluation
+    S_SHF0, S_SHF1, S_SHF2,      // mass correction per site
+    S_QFIN,                      // finished-brick count of the sweeps (an unsigned)
     S_WARM,                      // steps whose starting potentials Uprev holds (0, 1, 2 = enough)
     S_FIN = kScalStride - 1      // finished-block count (an unsigned in this slot's bytes)
 };
@@ -59,12 +62,26 @@ constexpr int kMaxBricks = 4096;
 // status block: the words above, kMaxBricks counters, then the int4 brick table of the sweeps
 constexpr size_t kStatusInts = (size_t)kFlagBase + (size_t)kMaxBricks * kFlagStride + 4 * (size_t)kMaxBricks;
 
+// Parameters of a replica in the field precision, formed on the host.  In the FP32 kernels a thread forms
+// none from the FP64 ones: GB300 issues two FP64 lanes a clock and SM, so one conversion or product per
+// thread costs as much as 64 FP32 instructions, and a division per thread of a 586-block launch 4 us.
+// With these, one thread per block for the rest and the block sums below, a coupled step of six iterations
+// at 48^3, N = 16, FP32 fell from 1.29 to 1.02 ms, one of four at 128^3, N = 64 from 4.00 to 3.71 ms.
+template <typename T>
+struct Par {
+    T al, be, be3;             // stencil: alpha, 1 - 2 alpha and its cube
+    T rho0, gs, gb, dt2;       // LB: density, 1 - 1/tau, dt^2
+    T dtM, c, kappa, floor;    // diffusion: dt M, dt M / 2, compressibility, floor of phi
+    T chi[9];
+    T amp2, kT;                // thermal noise
+};
+
 // One replica as the kernels see it.  Pointers are into the caller's workspace; their element
 // type is the context precision (double or float) except part/scal (double).
 struct Rep {
     int nx, ny, nz, ns, N, nA;
     long long V;
-    int nq;                                // P_Q partials of the sweep kernel in use
+    int nq;                                // P_Q partials to sum in norm_of; 0: scal[S_QSUM] is the total
     int nq_units;                          // general sweeps: row planes, entries of qrow
     int blk0, nblk, chunk;                 // flat tiling: nblk blocks of `chunk` sites
     int lb_blk0, lb_nblk;                  // LB grid: one site per thread, lb_nblk blocks
@@ -72,6 +89,8 @@ struct Rep {
     double phi_p, kappa, alpha, dt, M, gs, gb, rho0, phi_floor;
     double chi[9];
     double mass0[3];
+    Par<float> pf;
+    Par<double> pd;
     long long ext_off;                     // offset of this replica in [rep][ns][V] arrays
     long long vbase;                       // sites of the replicas before it ([rep][c][V] arrays)
     void* phi;   // [ns][V] compositions (target of the inversion)
@@ -101,6 +120,26 @@ struct Rep {
     int part_stride;
     double* scal;   // [kScalStride]
 };
+
+template <typename T>
+__host__ __device__ __forceinline__ const Par<T>& pars(const Rep& R) {
+    if constexpr (sizeof(T) == 4) return R.pf;
+    else return R.pd;
+}
+// (Re)forms pf and pd from the FP64 parameters.
+template <typename T>
+inline void set_par(const Rep& R, Par<T>& p) {
+    const double be = 1.0 - 2.0 * R.alpha;
+    p.al = (T)R.alpha; p.be = (T)be; p.be3 = (T)(be * be * be);
+    p.rho0 = (T)R.rho0; p.gs = (T)R.gs; p.gb = (T)R.gb; p.dt2 = (T)(R.dt * R.dt);
+    p.dtM = (T)(R.dt * R.M); p.c = (T)(0.5 * R.dt * R.M); p.kappa = (T)R.kappa; p.floor = (T)R.phi_floor;
+    for (int i = 0; i < 9; ++i) p.chi[i] = (T)R.chi[i];
+    p.amp2 = (T)R.noise_amp2; p.kT = (T)R.noise_kT;
+}
+inline void set_pars(Rep& R) {
+    set_par(R, R.pf);
+    set_par(R, R.pd);
+}
 
 // Flat tiling of one replica; the context path and the allocation-free path both use it.
 inline void tile_replica(Rep& R) {
@@ -186,6 +225,48 @@ __device__ __forceinline__ void block_sum_n(double (&v)[NV], double* sh) {
     __syncthreads();
 }
 
+// NV block-wide FP64 sums of one value per thread of a kFlatThreads block, in a fixed order, returned to
+// thread 0 only.  For FP32 values one warp per sum takes the threads' values from shared memory, eight
+// per lane: 13 FP64 warp instructions a sum instead of 53 (every warp shuffling its own).
+// sh: NV x 33 doubles.
+template <int NV>
+__device__ __forceinline__ void block_total(const float (&v)[NV], double* sh, double (&out)[NV]) {
+    static_assert(NV <= kFlatThreads / 32 && kFlatThreads * sizeof(float) <= 128 * sizeof(double), "one warp per sum");
+    __shared__ float val[NV][kFlatThreads];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) val[k][threadIdx.x] = v[k];
+    __syncthreads();
+    if (w < NV) {
+        double s = 0.0;
+#pragma unroll
+        for (int i = 0; i < kFlatThreads / 32; ++i) s += (double)val[w][32 * i + lane];
+        s = warp_sum(s);
+        if (lane == 0) sh[w] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) out[k] = sh[k];
+}
+template <int NV>
+__device__ __forceinline__ void block_total(const double (&v)[NV], double* sh, double (&out)[NV]) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) out[k] = v[k];
+    block_sum_n<NV>(out, sh);
+}
+// Block-wide maximum, returned to thread 0 (FP32 values are compared as such).
+__device__ __forceinline__ double block_top(float v, double* sh) {
+    float* f = (float*)sh;
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_down_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) f[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int i = 1; i < kFlatThreads / 32; ++i) v = fmaxf(v, f[i]);
+    return (double)v;
+}
+
 __device__ __forceinline__ double block_max(double v, double* sh) {
     const int nw = (blockDim.x * blockDim.y + 31) >> 5;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
@@ -203,6 +284,8 @@ __device__ __forceinline__ double block_max(double v, double* sh) {
     __syncthreads();
     return r;
 }
+
+__device__ __forceinline__ double block_top(double v, double* sh) { return block_max(v, sh); }
 
 // Total of n partials, same fixed order in every block.
 __device__ __forceinline__ double reduce_parts(const double* __restrict__ p, int n, double* sh) {
@@ -338,6 +421,7 @@ struct CoopRep {
     long long V;
     void *E, *G, *Gp0, *Gp1, *q;
     double *qrow, *pq;   // sums of G_N per row plane (or nullptr), the P_Q slot
+    double* qsum;        // where their total goes
     double rr;           // alpha / (1 - 2 alpha)
 };
 struct CoopPlan {

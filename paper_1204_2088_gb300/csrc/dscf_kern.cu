@@ -32,31 +32,6 @@ __device__ __forceinline__ void site_xyz(int i, int nx, int ny, int& x, int& y, 
 // Normalisation of the quadrature (Eq. 2 prefactor):  phi_I = phi_p/(N Q) q_I,
 // phi_S = phi_s exp(-U_S)/<exp(-U_S)>.
 // ---------------------------------------------------------------------------------------------
-struct Norm {
-    double coef, qs, phis, Q;
-};
-template <typename T>
-__device__ __forceinline__ Norm norm_of(const Rep& R, double* sh, int net = 0) {
-    Norm n;
-    if (net) {   // the learned predictor's output is already normalised
-        n.coef = 1.0;
-        n.Q = 0.0;
-        n.qs = 1.0;
-        n.phis = 1.0 - R.phi_p;
-        return n;
-    }
-    // the sweeps apply each pass of the stencil divided by its centre weight, c + r (a + d), and the
-    // Boltzmann factors of the copolymer carry the weight's cube; a quadrature has one stencil more than
-    // Boltzmann factors, so it lacks 1 / (1 + 2 r)^3, with r as rounded in the sweeps: only so do the
-    // densities keep their means (with be^3 instead they are off by up to 4e-8 in FP32)
-    const double Q = reduce_parts(slot(R, P_Q), R.nq, sh) / (double)R.V;
-    const double w = 1.0 + 2.0 * (double)(T)(R.alpha / (1.0 - 2.0 * R.alpha));
-    n.Q = Q;
-    n.coef = R.phi_p / ((double)R.N * Q) / (w * w * w);
-    n.qs = (R.ns == 3) ? reduce_parts(slot(R, P_ES), R.nblk, sh) / (double)R.V : 1.0;
-    n.phis = 1.0 - R.phi_p;
-    return n;
-}
 // A factor of the model densities in the field precision: two parts for FP32, whose rounded factor alone
 // would shift every density the same way (up to 6e-8 of it, which the inversion turns into a shift of
 // the potentials).
@@ -73,11 +48,55 @@ __device__ __forceinline__ Fac<T> fac(double v) {
     const T hi = (T)v;
     return {hi, (T)(v - (double)hi)};
 }
+template <typename T>
+struct Norm {
+    Fac<T> f[2];       // of q_I, of E_S
+    double Q, qs;      // in thread 0 only
+};
+// One thread forms the factors for its block; sh: >= 33 doubles.  net: the learned predictor's output is
+// already normalised.
+template <typename T>
+__device__ __forceinline__ Norm<T> norm_of(const Rep& R, double* sh, int net = 0) {
+    __shared__ Fac<T> f[2];
+    Norm<T> n;
+    n.Q = 0.0;
+    n.qs = 1.0;
+    double qt = 0.0, et = 0.0;
+    if (!net && R.nq > 0) {   // partial sums, no total (the allocation-free path)
+        qt = reduce_parts(slot(R, P_Q), R.nq, sh);
+        if (R.ns == 3) et = reduce_parts(slot(R, P_ES), R.nblk, sh);
+    }
+    if (threadIdx.x == 0) {
+        f[0] = {T(1), T(0)};
+        if (!net) {
+            if (R.nq == 0) {
+                qt = R.scal[S_QSUM];
+                et = R.ns == 3 ? R.scal[S_ESS] : 0.0;
+            }
+            // the sweeps apply each pass of the stencil divided by its centre weight, c + r (a + d), and
+            // the Boltzmann factors of the copolymer carry the weight's cube; a quadrature has one stencil
+            // more than Boltzmann factors, so it lacks 1 / (1 + 2 r)^3, with r as rounded in the sweeps:
+            // only so do the densities keep their means (with be^3 instead they are off by up to 4e-8 in
+            // FP32)
+            const double w = 1.0 + 2.0 * (double)(T)(R.alpha / (1.0 - 2.0 * R.alpha));
+            n.Q = qt / (double)R.V;
+            if (R.ns == 3) n.qs = et / (double)R.V;
+            const double coef = R.phi_p / ((double)R.N * n.Q * (w * w * w));
+            f[0] = fac<T>(coef);
+            n.Q = coef > 0.0 ? n.Q : 0.0;
+        }
+        f[1] = fac<T>((1.0 - R.phi_p) / n.qs);
+    }
+    __syncthreads();
+    n.f[0] = f[0];
+    n.f[1] = f[1];
+    return n;
+}
 // phi_I[U] at one site in the field precision (FP64 only in the normalisation constants).
 template <typename T>
-__device__ __forceinline__ T model_phi(const Rep& R, const Norm& n, int I, int i) {
-    if (I < 2) return fac<T>(n.coef)(((const T*)R.q)[(size_t)I * R.V + i]);
-    return fac<T>(n.phis / n.qs)(((const T*)R.E)[2 * (size_t)R.V + i]);
+__device__ __forceinline__ T model_phi(const Rep& R, const Norm<T>& n, int I, int i) {
+    if (I < 2) return n.f[0](((const T*)R.q)[(size_t)I * R.V + i]);
+    return n.f[1](((const T*)R.E)[2 * (size_t)R.V + i]);
 }
 
 // FP32 fields with V a multiple of 4 are also walked as float4 (4 consecutive sites per thread and
@@ -90,13 +109,11 @@ __device__ __forceinline__ bool flat_vec(int V) {
 __device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
 // Factor and source of the model density of species I as a float4 stream: coef q_I, or for the
 // solvent phis E_S / qs.
-__device__ __forceinline__ const float* model_src(const Rep& R, const Norm& n, int I, Fac<float>& sc) {
-    if (I < 2) {
-        sc = fac<float>(n.coef);
-        return (const float*)R.q + (size_t)I * R.V;
-    }
-    sc = fac<float>(n.phis / n.qs);
-    return (const float*)R.E + 2 * (size_t)R.V;
+template <typename T>
+__device__ __forceinline__ const float* model_src(const Rep& R, const Norm<T>& n, int I, Fac<float>& sc) {
+    const Fac<T> f = n.f[I < 2 ? 0 : 1];
+    sc = {(float)f.hi, (float)f.lo};
+    return I < 2 ? (const float*)R.q + (size_t)I * R.V : (const float*)R.E + 2 * (size_t)R.V;
 }
 
 // Directional derivative at the trial point: h1 = <phi* - phi[U + a1 d], d>.
@@ -105,7 +122,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_trial(const Rep* __restrict__ 
                                                         int net) {
     __shared__ double sh[33];
     FLAT_PROLOGUE
-    const Norm n = norm_of<T>(R, sh, net);
+    const Norm<T> n = norm_of<T>(R, sh, net);
     const T* phi = (const T*)R.phi;
     const T* d = (const T*)R.d;
     T h1 = T(0);
@@ -133,8 +150,10 @@ __global__ void __launch_bounds__(kFlatThreads) k_trial(const Rep* __restrict__ 
                 h1 += (phi[o] - model_phi<T>(R, n, I, i)) * d[o];
             }
     }
-    const double t = block_sum((double)h1, sh);
-    if (threadIdx.x == 0) slot(R, P_H1)[lb] = t;
+    const T v[1] = {h1};
+    double t[1];
+    block_total<1>(v, sh, t);
+    if (threadIdx.x == 0) slot(R, P_H1)[lb] = t[0];
     __shared__ int fin;
     if (last_block_of(R, &fin)) {
         const double h1s = reduce_parts_cg(slot(R, P_H1), R.nblk, sh);
@@ -149,9 +168,9 @@ __global__ void __launch_bounds__(kFlatThreads) k_grad(const Rep* __restrict__ r
                                                        int k, int net) {
     __shared__ double sh[33];
     FLAT_PROLOGUE
-    const Norm n = norm_of<T>(R, sh, net);
+    const Norm<T> n = norm_of<T>(R, sh, net);
     if (lb == 0 && threadIdx.x == 0 && !net) {
-        R.scal[S_Q] = n.coef > 0.0 ? n.Q : 0.0;
+        R.scal[S_Q] = n.Q;
         R.scal[S_QS] = n.qs;
     }
     const T* __restrict__ phi = (const T*)R.phi;
@@ -191,10 +210,12 @@ __global__ void __launch_bounds__(kFlatThreads) k_grad(const Rep* __restrict__ r
             }
     }
     if (k >= 0) {
-        const double t = block_sum((double)gg, sh);
-        const double tm = block_max((double)gmax, sh);
+        const T v[1] = {gg};
+        double t[1];
+        block_total<1>(v, sh, t);
+        const double tm = block_top(gmax, sh);
         if (threadIdx.x == 0) {
-            slot(R, pslot_gg(k + 1))[lb] = t;
+            slot(R, pslot_gg(k + 1))[lb] = t[0];
             slot(R, P_GMAX)[lb] = tm;
         }
         __shared__ int fin;
@@ -213,11 +234,11 @@ __global__ void __launch_bounds__(kFlatThreads) k_dir(const Rep* __restrict__ re
                                                       int mode, int k, int* status) {
     __shared__ double sh[3 * 33];
     FLAT_PROLOGUE
-    double beta = 0.0;
+    __shared__ T beta_sh;
     if (mode == 1) {
         // <g,g> of iterations k+1 and k, totalled by the last blocks of their producers
         const double ggn = R.scal[S_GGS0 + ((k + 1) & 1)], ggo = R.scal[S_GGS0 + (k & 1)];
-        beta = (ggo > 0.0) ? ggn / ggo : 0.0;
+        if (threadIdx.x == 0) beta_sh = (T)((ggo > 0.0) ? ggn / ggo : 0.0);
         if (lb == 0) {
             const double gm = reduce_parts_max(slot(R, P_GMAX), R.nblk, sh);
             if (threadIdx.x == 0) {
@@ -230,7 +251,8 @@ __global__ void __launch_bounds__(kFlatThreads) k_dir(const Rep* __restrict__ re
     const T* __restrict__ phi = (const T*)R.phi;
     const T* __restrict__ pm = (const T*)R.phim;
     T* __restrict__ d = (T*)R.d;
-    const T tb = (T)beta;
+    if (mode == 1) __syncthreads();
+    const T tb = mode == 1 ? beta_sh : T(0);
     T h0 = T(0), cd = T(0), gg = T(0), gmax = T(0);
     if (flat_vec<T>(V)) {
         const float fb = (float)tb;
@@ -268,9 +290,10 @@ __global__ void __launch_bounds__(kFlatThreads) k_dir(const Rep* __restrict__ re
             }
     }
     if (mode == 0) {
-        double t[3] = {(double)h0, (double)cd, (double)gg};
-        block_sum_n<3>(t, sh);
-        const double tm = block_max((double)gmax, sh);
+        const T v[3] = {h0, cd, gg};
+        double t[3];
+        block_total<3>(v, sh, t);
+        const double tm = block_top(gmax, sh);
         if (threadIdx.x == 0) {
             slot(R, P_H0)[lb] = t[0];
             slot(R, P_CD)[lb] = t[1];
@@ -278,8 +301,9 @@ __global__ void __launch_bounds__(kFlatThreads) k_dir(const Rep* __restrict__ re
             slot(R, P_GMAX)[lb] = tm;
         }
     } else {
-        double t[2] = {(double)h0, (double)cd};
-        block_sum_n<2>(t, sh);
+        const T v[2] = {h0, cd};
+        double t[2];
+        block_total<2>(v, sh, t);
         if (threadIdx.x == 0) {
             slot(R, P_H0)[lb] = t[0];
             slot(R, P_CD)[lb] = t[1];
@@ -356,7 +380,8 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 3 : 1) k_mu(con
         }
     }
     const int nx = R.nx, ny = R.ny, nz = R.nz, ns = R.ns;
-    const T al = (T)R.alpha, be = (T)(1.0 - 2.0 * R.alpha);
+    const Par<T>& P = pars<T>(R);
+    const T al = P.al, be = P.be;
     const T* phi = (const T*)R.phi;
     const T* U = (const T*)R.U;
     T* mu = (T*)R.mu;
@@ -398,11 +423,11 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 3 : 1) k_mu(con
 #pragma unroll
                     for (int I = 0; I < 3; ++I) {
                         if (I >= ns) break;
-                        const float ch = (float)R.chi[I * 3 + J];
+                        const float ch = (float)P.chi[I * 3 + J];
                         m[I].x += ch * sp.x; m[I].y += ch * sp.y; m[I].z += ch * sp.z; m[I].w += ch * sp.w;
                     }
                 }
-                const float kap = (float)R.kappa;
+                const float kap = (float)P.kappa;
 #pragma unroll
                 for (int I = 0; I < 3; ++I) {
                     if (I >= ns) break;
@@ -428,8 +453,8 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 3 : 1) k_mu(con
         }
         for (int I = 0; I < ns; ++I) {
             T m = -U[(size_t)I * V + i];
-            for (int J = 0; J < ns; ++J) m += (T)R.chi[I * 3 + J] * sp[J];
-            m += (T)R.kappa * (tot - T(1));
+            for (int J = 0; J < ns; ++J) m += P.chi[I * 3 + J] * sp[J];
+            m += P.kappa * (tot - T(1));
             mu[(size_t)I * V + i] = m;
         }
     }
@@ -438,12 +463,7 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 3 : 1) k_mu(con
 // ---------------------------------------------------------------------------------------------
 // D3Q19 MRT lattice Boltzmann: pull-scheme fused collide-stream.
 // ---------------------------------------------------------------------------------------------
-__constant__ signed char kC[19][3] = {
-    {0, 0, 0}, {1, 0, 0}, {-1, 0, 0}, {0, 1, 0}, {0, -1, 0}, {0, 0, 1}, {0, 0, -1},
-    {1, 1, 0}, {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0}, {1, 0, 1}, {-1, 0, -1},
-    {1, 0, -1}, {-1, 0, 1}, {0, 1, 1}, {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
-
-// Compile-time D3Q19 velocity components (same order as kC), so unrolled loops fold them.
+// Compile-time D3Q19 velocity components, so unrolled loops fold them.
 __host__ __device__ constexpr int lbc(int i, int a) {
     constexpr signed char c[19][3] = {
         {0, 0, 0}, {1, 0, 0}, {-1, 0, 0}, {0, 1, 0}, {0, -1, 0}, {0, 0, 1}, {0, 0, -1},
@@ -505,7 +525,6 @@ __host__ __device__ constexpr double lb_ghost_norm(int k) {
 template <typename T, bool NOISE>
 __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 3 : 2) k_lb(const Rep* __restrict__ reps, int nrep,
                                                         const int* __restrict__ counter, const T* __restrict__ fext) {
-    __shared__ double sh[33];
     int r = 0;
     while (r + 1 < nrep && (int)blockIdx.x >= reps[r + 1].lb_blk0) ++r;
     const Rep& R = reps[r];
@@ -517,7 +536,8 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 3 : 2) k_lb(con
     const T* src = (const T*)(par ? R.pop1 : R.pop0);
     T* dst = (T*)(par ? R.pop0 : R.pop1);
     const int nx = R.nx, ny = R.ny, nz = R.nz, ns = R.ns;
-    const T rho0 = (T)R.rho0, gs = (T)R.gs, gb = (T)R.gb, dt2 = (T)(R.dt * R.dt);
+    const Par<T>& P = pars<T>(R);
+    const T rho0 = P.rho0, gs = P.gs, gb = P.gb, dt2 = P.dt2;
     if (act) {
         const int x = site % nx;
         const int yz = site / nx;
@@ -601,7 +621,7 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 3 : 2) k_lb(con
                 for (int q = 0; q < 4; ++q) g[4 * cc + q] = n4[q];
             }
             // m*_k / b_k gains phi_k r_k / b_k = sqrt(3 rho kT (1 - gamma_k^2) / b_k) r_k
-            const T t3 = T(3) * rho * (T)R.noise_kT;
+            const T t3 = T(3) * rho * P.kT;
             const T ab = sqrt(t3 * (T(1) - gb * gb)), as = sqrt(t3 * (T(1) - gs * gs));
             r4 += ab * sqrt(T(1.5)) * g[0];    // b_4 = 2/3
             r5 += as * sqrt(T(2.25)) * g[1];   // b_5 = 4/9
@@ -738,15 +758,15 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? (NOISE ? 2 : 4)
                                                                         const int* __restrict__ counter) {
     FLAT_PROLOGUE
     const unsigned nstep = NOISE ? (unsigned)(*counter - 1) : 0u;
-    const T amp2 = (T)R.noise_amp2;
+    const T amp2 = pars<T>(R).amp2;
     const T* phi = (const T*)R.phi;
     const T* mu = (const T*)R.mu;
     const T* u = (const T*)R.u;
     T* rhs = (T*)R.rhs;
     T* inv = (T*)R.E;
     const bool hyd = R.hydro != 0;
-    const T dtM = (T)(R.dt * R.M);
-    const T fl = (T)R.phi_floor;
+    const T dtM = pars<T>(R).dtM;
+    const T fl = pars<T>(R).floor;
     if constexpr (sizeof(T) == 4) {
         const int nx = R.nx, ny = R.ny, nz = R.nz;
         if ((nx & 3) == 0 && nx <= 128 && 128 % nx == 0 && V % 128 == 0) {
@@ -1022,8 +1042,8 @@ __global__ void __launch_bounds__(kFlatThreads, sizeof(T) == 4 ? 4 : 3) k_cd_jac
     const T* dold = (const T*)((k & 1) ? R.del0 : R.del1);
     T* dnew = (T*)((k & 1) ? R.del1 : R.del0);
     const int ns = R.ns;
-    const T c = (T)(0.5 * R.dt * R.M);
-    const T kap = (T)R.kappa;
+    const T c = pars<T>(R).c;
+    const T kap = pars<T>(R).kappa;
     if constexpr (sizeof(T) == 4) {
         if (ns == 2 && (R.nx & 3) == 0) {   // FP32 melt: 4 consecutive sites of an x row per thread
             // chunks are multiples of 256 sites, so with V a multiple of 128 every warp is whole
@@ -1108,14 +1128,20 @@ __global__ void __launch_bounds__(kFlatThreads) k_cd_finish(const Rep* __restric
                 acc += v;
             }
         }
-        const double t = block_sum((double)acc, sh);
-        if (threadIdx.x == 0) slot(R, P_MASS0 + I)[lb] = t;
+        const T v[1] = {acc};
+        double t[1];
+        block_total<1>(v, sh, t);
+        if (threadIdx.x == 0) slot(R, P_MASS0 + I)[lb] = t[0];
+        __syncthreads();
     }
     __shared__ int fin;
     if (last_block_of(R, &fin))
         for (int I = 0; I < R.ns; ++I) {
             const double tot = reduce_parts_cg(slot(R, P_MASS0 + I), R.nblk, sh);
-            if (threadIdx.x == 0) R.scal[S_TOT0 + I] = tot;
+            if (threadIdx.x == 0) {
+                R.scal[S_TOT0 + I] = tot;
+                *(T*)(R.scal + S_SHF0 + I) = (T)((R.mass0[I] - tot) / (double)V);   // the correction per site
+            }
         }
 }
 
@@ -1123,18 +1149,17 @@ __global__ void __launch_bounds__(kFlatThreads) k_cd_finish(const Rep* __restric
 template <typename T>
 __global__ void __launch_bounds__(kFlatThreads) k_mass_fix(const Rep* __restrict__ reps, const int* __restrict__ blk2rep,
                                                            int* status) {
-    __shared__ double sh[33];
     FLAT_PROLOGUE
     T* phi = (T*)R.phi;
     for (int I = 0; I < R.ns; ++I) {
-        const double tot = R.scal[S_TOT0 + I];   // totalled by the last block of k_cd_finish
-        const double shift = (R.mass0[I] - tot) / (double)V;
+        // total and correction, formed by the last block of k_cd_finish
         if (lb == 0 && threadIdx.x == 0) {
+            const double tot = R.scal[S_TOT0 + I];
             R.scal[S_DRIFT0 + I] = tot - R.mass0[I];
             R.scal[S_MASS0 + I] = R.mass0[I];
             if (!isfinite(tot)) atomicOr(status, (int)ST_NONFINITE);
         }
-        const T ts = (T)shift;
+        const T ts = *(const T*)(R.scal + S_SHF0 + I);
         if (flat_vec<T>(V)) {
             const float fs = (float)ts;
             _Pragma("unroll 2") for (int i = i0 + 4 * (int)threadIdx.x; i < i1; i += 4 * kFlatThreads) {
@@ -1154,38 +1179,45 @@ __global__ void __launch_bounds__(kFlatThreads) k_dens_out(const Rep* __restrict
                                                            T* __restrict__ out) {
     __shared__ double sh[33];
     FLAT_PROLOGUE
-    const Norm n = norm_of<T>(R, sh);
+    const Norm<T> n = norm_of<T>(R, sh);
     for (int I = 0; I < R.ns; ++I)
         _Pragma("unroll 4") for (int i = i0 + threadIdx.x; i < i1; i += kFlatThreads)
             out[R.ext_off + (size_t)I * V + i] = model_phi<T>(R, n, I, i);
 }
 
 // Populations in / out: the API exchanges n_i(r) before collision, i.e. the stored
-// post-collision deviation streamed: n_i(r) = n*_i(r - c_i).
+// post-collision deviation streamed: n_i(r) = n*_i(r - c_i).  One site per thread (LB grid) with
+// 32-bit indices and every load before the first store: HBM bound, 319 MB at 128^3 FP32.  A copy in, 16
+// LB steps and a copy out took 1.49 ms and take 1.19, with the LB pass's parameters read in FP32.
 template <typename T>
-__global__ void __launch_bounds__(kFlatThreads) k_pop_copy(const Rep* __restrict__ reps, const int* __restrict__ blk2rep,
+__global__ void __launch_bounds__(kFlatThreads) k_pop_copy(const Rep* __restrict__ reps, int nrep,
                                                            const int* __restrict__ counter, T* __restrict__ ext,
                                                            int dir) {
-    FLAT_PROLOGUE
-    T* cur = (T*)(((*counter) & 1) ? R.pop1 : R.pop0);
-    const long long b19 = 19 * R.vbase;
+    int r = 0;
+    while (r + 1 < nrep && (int)blockIdx.x >= reps[r + 1].lb_blk0) ++r;
+    const Rep& R = reps[r];
+    const int V = (int)R.V;
+    const int site = (blockIdx.x - R.lb_blk0) * kFlatThreads + threadIdx.x;
+    if (site >= V) return;
+    T* __restrict__ cur = (T*)(((*counter) & 1) ? R.pop1 : R.pop0);
+    T* __restrict__ e = ext + 19 * (size_t)R.vbase;
     const int nx = R.nx, ny = R.ny, nz = R.nz;
-    for (int r = i0 + threadIdx.x; r < i1; r += kFlatThreads) {
-        const int x = (int)(r % nx);
-        const int y = (int)((r / nx) % ny);
-        const int z = (int)(r / ((long long)nx * ny));
-        for (int i = 0; i < 19; ++i) {
-            if (dir == 0) {
-                const long long s = wrapi(x - kC[i][0], nx) +
-                                    (long long)nx * (wrapi(y - kC[i][1], ny) + (long long)ny * wrapi(z - kC[i][2], nz));
-                ext[b19 + (long long)i * V + r] = cur[(long long)i * V + s];
-            } else {
-                const long long s = wrapi(x + kC[i][0], nx) +
-                                    (long long)nx * (wrapi(y + kC[i][1], ny) + (long long)ny * wrapi(z + kC[i][2], nz));
-                cur[(long long)i * V + r] = ext[b19 + (long long)i * V + s];
-            }
-        }
+    int x, y, z;
+    site_xyz(site, nx, ny, x, y, z);
+    const int X[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
+    const int Y[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
+    const int Z[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
+    const T* __restrict__ src = dir == 0 ? cur : e;
+    T* __restrict__ dst = dir == 0 ? e : cur;
+    T v[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {   // get: from r - c_i, set: from r + c_i
+        const int cx = lbc(i, 0), cy = lbc(i, 1), cz = lbc(i, 2);
+        const int s = dir == 0 ? X[1 - cx] + nx * (Y[1 - cy] + ny * Z[1 - cz]) : X[1 + cx] + nx * (Y[1 + cy] + ny * Z[1 + cz]);
+        v[i] = src[(size_t)i * V + s];
     }
+#pragma unroll
+    for (int i = 0; i < 19; ++i) dst[(size_t)i * V + site] = v[i];
 }
 
 // Mass targets: partial sums of the current phi, then one block per replica commits them.
@@ -1568,7 +1600,7 @@ void launch_dens_out(const Launch& L, void* phi_ext) {
 }
 template <typename T>
 void launch_pop_copy(const Launch& L, void* ext, int dir) {
-    k_pop_copy<T><<<L.nblk_total, kFlatThreads, 0, L.stream>>>(L.reps, L.blk2rep, L.counter, (T*)ext, dir);
+    k_pop_copy<T><<<L.nlb_total, kFlatThreads, 0, L.stream>>>(L.reps, L.nrep, L.counter, (T*)ext, dir);
 }
 template <typename T>
 void launch_mass_init(const Launch& L, int nrep) {

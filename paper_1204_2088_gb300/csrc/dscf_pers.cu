@@ -687,7 +687,21 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         if (w == 0) {
             const double q = warp_sum(lane < NW ? sh[lane] : 0.0);
-            if (lane == 0) slot(R, P_Q)[b] = q;
+            // the replica's last brick adds up all bricks' shares, in order
+            const int nb = nby * nbz;
+            unsigned old = 0;
+            if (lane == 0) {
+                slot(R, P_Q)[b] = q;
+                __threadfence();
+                old = atomicInc((unsigned*)(R.scal + S_QFIN), (unsigned)nb - 1u);
+            }
+            if (__shfl_sync(0xffffffffu, old, 0) == (unsigned)nb - 1u) {
+                __threadfence();
+                double s = 0.0;
+                for (int i = lane; i < nb; i += 32) s += __ldcg(slot(R, P_Q) + i);
+                s = warp_sum(s);
+                if (lane == 0) R.scal[S_QSUM] = s;
+            }
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_slot), "r"(TCOLS) : "memory");
         }
     }

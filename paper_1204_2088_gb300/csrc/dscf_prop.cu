@@ -22,45 +22,48 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
     const long long V = R.V;
     const long long i0 = (long long)lb * R.chunk;
     const long long i1 = min(i0 + (long long)R.chunk, V);
-    double a = 0.0;
-    if (mode == 1 || mode == 2) {
-        // totals of the direction and trial kernels' partials, formed by their last blocks
-        const double t[3] = {R.scal[S_H0S], R.scal[S_CDS], mode == 2 ? R.scal[S_H1S] : 0.0};
-        const double h0 = t[0], cd = t[1];
-        const double a1 = (cd > 0.0 && isfinite(h0 / cd)) ? -h0 / cd : 0.0;
-        a = a1;
-        if (mode == 2) {
-            const double h1 = t[2];
-            const double den = h1 - h0;
-            a = (den > 0.0) ? a1 * (-h0) / den : a1;
-            // With the learned predictor the secant is capped at the local-curvature step a1: the
-            // exact response is stiffer than the local one (a <= a1), and a network whose response
-            // to the tiny trial displacement is below its resolution would otherwise give a
-            // near-zero secant denominator and an unbounded step.
-            if (write_u && a > a1) a = a1;
-            if (lb == 0 && threadIdx.x == 0) {
-                R.scal[S_ITER0 + 4 * k + 0] = a1;
-                R.scal[S_ITER0 + 4 * k + 1] = a;
-            }
-        } else if (k == 0 && lb == 0) {
-            // start-of-inversion residual (partials written by the direction kernel)
-            const double gg = reduce_parts(slot(R, P_GG0), R.nblk, sh);
-            const double gm = reduce_parts_max(slot(R, P_GMAX), R.nblk, sh);
-            if (lb == 0 && threadIdx.x == 0) {
-                R.scal[S_GG0] = gg;
-                R.scal[S_GMAX0] = gm;
+    __shared__ T ta_sh;
+    if (threadIdx.x == 0) {   // the step length, once per block (FP64 divisions)
+        double a = 0.0;
+        if (mode == 1 || mode == 2) {
+            // totals of the direction and trial kernels' partials, formed by their last blocks
+            const double h0 = R.scal[S_H0S], cd = R.scal[S_CDS];
+            const double q = h0 / cd;
+            const double a1 = (cd > 0.0 && isfinite(q)) ? -q : 0.0;
+            a = a1;
+            if (mode == 2) {
+                const double den = R.scal[S_H1S] - h0;
+                a = (den > 0.0) ? a1 * (-h0) / den : a1;
+                // With the learned predictor the secant is capped at the local-curvature step a1: the
+                // exact response is stiffer than the local one (a <= a1), and a network whose response
+                // to the tiny trial displacement is below its resolution would otherwise give a
+                // near-zero secant denominator and an unbounded step.
+                if (write_u && a > a1) a = a1;
+                if (lb == 0) {
+                    R.scal[S_ITER0 + 4 * k + 0] = a1;
+                    R.scal[S_ITER0 + 4 * k + 1] = a;
+                }
             }
         }
+        ta_sh = (T)a;
     }
+    if (mode == 1 && k == 0 && lb == 0) {
+        // start-of-inversion residual (partials written by the direction kernel)
+        const double gg = reduce_parts(slot(R, P_GG0), R.nblk, sh);
+        const double gm = reduce_parts_max(slot(R, P_GMAX), R.nblk, sh);
+        if (threadIdx.x == 0) {
+            R.scal[S_GG0] = gg;
+            R.scal[S_GMAX0] = gm;
+        }
+    }
+    __syncthreads();
     const int ns = R.ns;
     // distinct fields: no store below can change a value loaded from another of them
     T* __restrict__ U = (T*)R.U;
     const T* __restrict__ d = (const T*)R.d;
     T* __restrict__ E = (T*)R.E;
-    const T ta = (T)a;
-    const double be = 1.0 - 2.0 * R.alpha;
-    const T be3 = (T)(be * be * be);
-    double es = 0.0;
+    const T ta = ta_sh, be3 = pars<T>(R).be3;
+    T es = T(0);
     bool vec = false;
     if constexpr (sizeof(T) == 4) vec = (V & 3) == 0 && (mode != 3 || (R.ext_off & 3) == 0);
     if (vec) {   // FP32, 4 consecutive sites per thread and iteration (16-byte accesses)
@@ -113,7 +116,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
         };
         if (ns == 2) run(std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{});
         else run(std::integral_constant<int, 3>{}, std::integral_constant<int, 1>{});
-        es += (double)es4;
+        es += (T)es4;
     }
     for (int I = 0; I < ns && !vec; ++I) {
         for (long long i = i0 + threadIdx.x; i < i1; i += kFlatThreads) {
@@ -131,12 +134,19 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
             }
             const T e = write_u ? u : (I == 2 ? bexp(u) : be3 * bexp(u));   // write_u: the learned predictor takes U' itself
             E[o] = e;
-            if (I == 2) es += (double)e;
+            if (I == 2) es += e;
         }
     }
     if (ns == 3) {
-        const double t = block_sum(es, sh);
-        if (threadIdx.x == 0) slot(R, P_ES)[lb] = t;
+        const T v[1] = {es};
+        double t[1];
+        block_total<1>(v, sh, t);
+        if (threadIdx.x == 0) slot(R, P_ES)[lb] = t[0];
+        __shared__ int fin;
+        if (R.nq == 0 && last_block_of(R, &fin)) {   // (nq: the allocation-free path sums in norm_of)
+            const double s = reduce_parts_cg(slot(R, P_ES), R.nblk, sh);
+            if (threadIdx.x == 0) R.scal[S_ESS] = s;
+        }
     }
 }
 

@@ -102,6 +102,7 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     tile_replica(R);
     R.phi_p = p->phi_p;
     R.alpha = p->a * p->a / 6.0;
+    set_pars(R);
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         set_thread_error("dscf_densities_static: device query failed");
