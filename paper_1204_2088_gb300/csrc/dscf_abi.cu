@@ -25,7 +25,7 @@ struct Layout {
     std::vector<Rep> reps;          // host copy, pointers filled by place()
     std::vector<int> blk2rep;
     std::vector<CoopRep> coop;      // general sweeps: replicas by decreasing N
-    long long units = 0;            // their row planes
+    long long work = 0;             // their row planes
     int kk = 0;                     // row layout if all replicas have the same, else 0
     int nblk = 0, nlb = 0, Nmax = 0;
     size_t bytes = 0;
@@ -67,7 +67,7 @@ bool validate(const dscf_params* p, int n, std::string& why) {
 
 // Flat blocks of the replicas and the general sweeps' table (replicas by decreasing chain length, so that
 // those still active at a contour step are a prefix).
-void assign_tiles(Layout& L, const dscf_params* p, int n) {
+void assign_tiles(Layout& L, const dscf_params* p, int n, int prec) {
     // Flat kernels: about kMaxFlatBlocks blocks over the whole batch (one wave of four per SM).  A
     // replica whose own tiling would give it smaller chunks takes the batch's common chunk, so a
     // batch of many replicas does not launch tens of thousands of short blocks.  (A single
@@ -103,14 +103,17 @@ void assign_tiles(Layout& L, const dscf_params* p, int n) {
         L.nblk += R.nblk;
     }
     L.coop.clear();
-    L.units = 0;
+    L.work = 0;
     L.kk = coop_layout(L.reps[0].nx);
+    // costs in 32 bits: not weighted where they would not fit
+    long long all = 0;
+    for (const Rep& R : L.reps) all += coop_units(R) * coop_cost(R, prec == DSCF_FP64);
     int cost = 0;
     for (int k = 0; k < n; ++k) {
         const Rep& R = L.reps[order[k]];
-        L.coop.push_back(coop_rep(R, cost));
-        L.units += L.coop.back().units;
-        cost += L.coop.back().units * coop_sites(R.nx);
+        L.coop.push_back(coop_rep(R, all <= INT32_MAX ? coop_cost(R, prec == DSCF_FP64) : 1, cost));
+        L.work += L.coop.back().units;
+        cost += L.coop.back().units / L.coop.back().strip * L.coop.back().wgt;
         if (L.coop.back().layout != L.kk) L.kk = 0;
     }
 }
@@ -152,7 +155,7 @@ Layout make_layout(const dscf_params* p, int n, int prec, char* base) {
         vb += R.V;
         L.Nmax = std::max(L.Nmax, q.N);
     }
-    assign_tiles(L, p, n);
+    assign_tiles(L, p, n, prec);
     // workspace
     size_t off = 0;
     auto take = [&](size_t bytes) -> void* {
@@ -375,11 +378,6 @@ int64_t launch_pers_sweeps(dscf_ctx* c, const Launch& L, int limit) {
     return (int64_t)c->pgroups.size();
 }
 
-// CTAs of the general sweeps.
-int coop_grid(const dscf_ctx* c) {
-    const int nsm = std::min(c->nsm, kCoopMaxCtas);
-    return coop_ctas(c->L.units, nsm);
-}
 CoopPlan coop_plan(const dscf_ctx* c) {
     CoopPlan p;
     p.reps = c->d_coop;
@@ -387,7 +385,7 @@ CoopPlan coop_plan(const dscf_ctx* c) {
     p.cnt = c->d_status + kCoopBase;
     p.abort = c->d_status + 2;
     p.kk = c->L.kk;
-    p.ncta = coop_grid(c);
+    coop_cut(p, c->L.reps[0], c->L.work, c->prec == DSCF_FP64, std::min(c->nsm, kCoopMaxCtas));
     return p;
 }
 
@@ -668,7 +666,7 @@ int pers_select(dscf_ctx* c, std::vector<std::pair<int, int>>& pcand) {
 }
 
 // Grids for which contour fusion can be asked for (kfuse 2..4).  Those kernels are gone (the general
-// sweeps take 0.92 ms against 1.52 at 128^3 with N = 64, 0.31 against 0.87 at 64^3, 7.9 against 8.1 at
+// sweeps take 0.69 ms against 1.52 at 128^3 with N = 64, 0.24 against 0.87 at 64^3, 7.4 against 8.1 at
 // 256^3), but the request stays valid and runs the general sweeps.
 bool fusable(const dscf_ctx* c, int kfuse) {
     if (c->prec != DSCF_FP32) return false;
@@ -801,7 +799,7 @@ int dscf_init_tuned(const dscf_params* p, int32_t n, int32_t precision, void* wo
     rc = rc ? rc : chk(cudaStreamCreateWithFlags(&c->cap_body, cudaStreamNonBlocking), "capture stream");
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_reps, c->L.reps.data(), sizeof(Rep) * n, cudaMemcpyHostToDevice, c->stream), "reps");
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_b2r, c->L.blk2rep.data(), sizeof(int) * c->L.nblk, cudaMemcpyHostToDevice, c->stream), "b2r");
-    assign_tiles(c->L, c->params.data(), n);   // (the sweeps' table with the final pointers)
+    assign_tiles(c->L, c->params.data(), n, precision);   // (the sweeps' table with the final pointers)
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_coop, c->L.coop.data(), sizeof(CoopRep) * n, cudaMemcpyHostToDevice, c->stream), "sweep table");
     rc = rc ? rc : chk(cudaMemsetAsync(c->d_status, 0, sizeof(int) * kStatusInts, c->stream), "status");
     const size_t es = precision == DSCF_FP64 ? 8 : 4;

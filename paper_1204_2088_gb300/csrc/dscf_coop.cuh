@@ -12,7 +12,7 @@
 // it in shared memory).
 //
 // Work is cut into runs of consecutive z planes of one x row (or one x tile of a row of more than 256
-// sites), spread evenly over all warps of the launch.  A warp marches its run: per plane it loads the
+// sites), spread over all warps of the launch (coop_cut).  A warp marches its run: per plane it loads the
 // row and its two y neighbours, applies the y pass, then the x pass by shuffles (lane L holds sites L,
 // L + 32, ... of the row, so any row length and alignment has coalesced accesses), and combines three
 // planes in registers.  No pass is computed twice but the y and x passes of the two planes beside a
@@ -20,12 +20,13 @@
 // (c + r (a + d), r = alpha / (1 - 2 alpha), the centre weights folded into the Boltzmann factors and the
 // normalisation): 7 operations a site and contour step forward, 8 with the quadrature.
 //
-// FP64 at 128^3 is bound by the FP64 pipe (32 us of operations in a level's 33 us); small or odd
-// grids by the latency of a level (loads, the barrier).  A density evaluation, before (one launch per
-// contour step and direction, rows staged through shared memory, 9 operations on 10/8 of the rows)
-// and so: 32^3, N = 32, FP64 539 -> 192 us; 100 x 90 x 75, N = 48, FP32 1010 -> 424 us; 128^3, N = 64,
-// FP64 8.9 -> 4.2 ms; 256^3, N = 64, FP32 8.1 (fused pairs of steps) -> 7.9 ms.  Against the brick
-// sweeps: 48^3, N = 16 80 us (bricks 137), 64^3, N = 64 306 (361), 128^3, N = 64 924 (392).
+// FP64 at 128^3 is bound by the FP64 pipe (31 us of operations in a level's 33 us), 256^3 by HBM (13 fields
+// of 67 MB a pair of levels), the rest by the latency of loads and of the barrier: hence loads several planes
+// ahead, 12 warps where the registers allow it (128^3 FP32: 750 us with 8, 689 with 12) and one run per warp.
+// A density evaluation, one launch per contour step and direction, and so: 32^3, N = 32, FP64 539 -> 127 us;
+// 100 x 90 x 75, N = 48, FP32 1013 -> 276 us; 128^3, N = 64, FP64 8.9 -> 4.2 ms; 256^3, N = 64, FP32 8.07
+// (fused pairs of steps) -> 7.40 ms.  Against the brick sweeps (dscf_pers.cu): 48^3, N = 16 71 us (bricks 137),
+// 64^3, N = 64 241 (361), 96^3, N = 48 347 (227), 128^3, N = 64 689 (386).
 //
 // Every wait is bounded as in dscf_pers.cu: a CTA that runs out sets the status bit and the abort flag
 // and waits no more; arrivals do not depend on waits, so the launch always finishes and leaves its
@@ -53,6 +54,7 @@ struct CoopCtl {
     int* abort;
     int* status;
     int limit;                   // polls before giving up
+    int runs, per;               // runs > 0: one replica, one run of a row per warp, `per` warps of a CTA
 };
 
 __device__ __forceinline__ int cld_acquire(const int* p) {
@@ -157,26 +159,32 @@ __device__ __forceinline__ void stk(T* p, const T (&v)[K]) {
     }
 }
 
-// n planes from za of x row (or x tile at x0) y.
-template <typename T, int K, int MODE>
+// n planes from za of x row (or x tile at x0) y.  PAST: past the middle (stored levels of the other chain are
+// read and the quadrature grows).  The march is bound by the latency of its loads, so those of a plane are
+// issued D planes (rows) and two planes (operands of the output plane) ahead; rings are registers by name, the
+// loop is unrolled by their length.
+template <typename T, int K, int MODE, bool PAST>
 __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, int x0, int y, int za, int n, T rr, int unit,
                                          double& qs) {
-    // planes loaded ahead of their use: rows, and operands of the output plane
-    constexpr bool FEW = K * sizeof(T) <= 16;
-    constexpr int D = FEW ? 3 : 1, DE = FEW ? 2 : 1, U = D + 1;
+    constexpr int B = K * (int)sizeof(T);
+    // rings of rows and of operands (the widest FP64 rows have registers for one operand plane only); FP64, bound by
+    // its pipe, loses more to the instruction cache in a longer loop than it gains (128^3, N = 64: 4.46 ms
+    // unrolled by 6, 4.18 by 2)
+    constexpr int RU = sizeof(T) == 8 ? (B <= 16 ? 3 : 2) : B <= 8 ? 6 : B <= 12 ? 4 : 3, D = RU - 1;
+    constexpr int EU = RU == 6 ? 3 : RU > 2 ? RU : B < 48 + 16 * (MODE == BLOCKED) ? 2 : 1, DE = EU > 2 ? 2 : EU - 1;
+    constexpr int UN = RU;
+    constexpr bool SHIFT = UN % 3 != 0;   // the planes of the z pass move by copies
     const int lane = threadIdx.x & 31;
     const int nx = R.nx, ny = R.ny, nz = R.nz;
     const int plane = nx * ny;
-    const int r0 = y * nx;
     const int dm = (y == 0 ? ny - 1 : -1) * nx, dp = (y == ny - 1 ? 1 - ny : 1) * nx;   // to the y neighbours
     // lane's first column, its other columns, which of them exist
     const int LL = MODE == BLOCKED ? nx / K - 1 : 31;   // blocked: last lane
     const int xl = MODE == BLOCKED ? K * min(lane, LL) : lane;
-    auto col = [&](int k) {
-        if (MODE == BLOCKED) return xl + k;
-        if (MODE == STRIDED) return 32 * k + lane;
+    auto col = [&](int k) {   // relative to xl
+        if (MODE != TILE) return 32 * k;
         int x = x0 - 1 + 32 * k + lane;
-        return x < 0 ? x + nx : (x >= nx ? x - nx : x);
+        return (x < 0 ? x + nx : (x >= nx ? x - nx : x)) - xl;
     };
     auto there = [&](int k) {   // loads: columns of the row (tile: up to the halo column of a ragged last tile)
         if (MODE == BLOCKED) return true;
@@ -191,7 +199,7 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
     };
     auto get = [&](const T* p, T (&v)[K], bool outs) {
         if constexpr (MODE == BLOCKED) {
-            ldk<T, K>(p + xl, v);
+            ldk<T, K>(p, v);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k)
@@ -200,81 +208,68 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
     };
     auto put = [&](T* p, const T (&v)[K]) {
         if constexpr (MODE == BLOCKED) {
-            if (lane <= LL) stk<T, K>(p + xl, v);
+            if (lane <= LL) stk<T, K>(p, v);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k)
                 if (mine(k)) p[col(k)] = v[k];
         }
     };
-    T raw[U][3][K], e[U][K], st[U][K], q[U][K];
+    T raw[RU][3][K], e[EU][K], st[EU][K], q[EU][K], u[3][K];
 #pragma unroll
-    for (int d = 0; d < U; ++d)
+    for (int k = 0; k < K; ++k) {   // (columns that do not exist stay 0)
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            raw[d][0][k] = raw[d][1][k] = raw[d][2][k] = T(1);
-            e[d][k] = st[d][k] = q[d][k] = T(0);
-        }
-    int zl = za == 0 ? nz - 1 : za - 1;                       // next plane to load
-    const T* sp = o.src + (size_t)zl * plane + r0;
-    int left = n + 2;
+        for (int d = 0; d < RU; ++d) raw[d][0][k] = raw[d][1][k] = raw[d][2][k] = T(0);
+#pragma unroll
+        for (int d = 0; d < EU; ++d) e[d][k] = st[d][k] = q[d][k] = T(0);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) u[d][k] = T(0);
+    }
+    // sites (a field has fewer than 2^31) of the lane's first column: next plane to load, next output plane
+    // to load operands of, output plane
+    int zl = za == 0 ? nz - 1 : za - 1;
+    int ol = zl * plane + y * nx + xl, oe = za * plane + y * nx + xl, ow = oe;
     auto load = [&](T (&v)[3][K]) {
-        if (left <= 0) return;
-        --left;
-        if (o.src) {
-            get(sp + dm, v[0], false);
-            get(sp, v[1], false);
-            get(sp + dp, v[2], false);
-        }
-        sp += plane;
+        get(o.src + (ol + dm), v[0], false);
+        get(o.src + ol, v[1], false);
+        get(o.src + (ol + dp), v[2], false);
+        ol += plane;
         if (++zl == nz) {
             zl = 0;
-            sp -= (size_t)nz * plane;
+            ol -= nz * plane;
         }
     };
-    const size_t at0 = (size_t)za * plane + r0;
-    const T *pe = o.E + at0, *ps = o.st + at0;
-    T *pq = o.q + at0, *pd = o.dst + at0;                     // pq: to load; the plane being written is DE planes back
-    int eleft = n;
     auto loade = [&](int d) {
-        if (eleft <= 0) return;
-        --eleft;
-        get(pe, e[d], true);
-        pe += plane;
-        if (o.st) {
-            get(ps, st[d], true);
-            if (!o.first) get(pq, q[d], true);
-            ps += plane;
-            pq += plane;
+        get(o.E + oe, e[d], true);
+        if constexpr (PAST) {
+            get(o.st + oe, st[d], true);
+            if (!o.first) get(o.q + oe, q[d], true);
         }
+        oe += plane;
     };
-    T* pw = o.q + at0;
+    const int last = n + 2;
 #pragma unroll
-    for (int d = 0; d < D; ++d) load(raw[d]);
-    // operands of output plane i - 2 are loaded at step i - DE
-#pragma unroll
-    for (int d = 2 - DE; d < 0; ++d) loade((d + DE) % U);
-    T pm[K], p0[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) pm[k] = p0[k] = T(0);
+    for (int d = 0; d < D; ++d)
+        if (d < last) load(raw[d]);
     const int lsrc = MODE == BLOCKED ? (lane == 0 ? LL : lane - 1) : ((lane + 31) & 31);
     const int rsrc = MODE == BLOCKED ? (lane >= LL ? 0 : lane + 1) : ((lane + 1) & 31);
-    for (int i0 = 0; i0 < n + 2; i0 += U) {
+    for (int i0 = 0; i0 < last; i0 += UN) {
 #pragma unroll
-        for (int d = 0; d < U; ++d) {
+        for (int d = 0; d < UN; ++d) {
             const int i = i0 + d;
-            if (i >= n + 2) break;
-            load(raw[(d + D) % U]);
-            if (i + DE >= 2) loade((d + DE) % U);
+            if (i >= last) break;
+            if (i + D < last) load(raw[(d + D) % RU]);
+            if ((d + DE >= 2 || i0 > 0) && i + DE < last) loade((d + DE) % EU);
             // y pass, then the x pass
-            T t[K], u[K];
+            T t[K];
+            T(&uc)[K] = u[SHIFT ? 2 : d % 3];
 #pragma unroll
-            for (int k = 0; k < K; ++k) t[k] = fma(rr, raw[d][0][k] + raw[d][2][k], raw[d][1][k]);
+            for (int k = 0; k < K; ++k) t[k] = fma(rr, raw[d % RU][0][k] + raw[d % RU][2][k], raw[d % RU][1][k]);
             if constexpr (MODE == BLOCKED) {
                 const T lv = __shfl_sync(0xffffffffu, t[K - 1], lsrc), rv = __shfl_sync(0xffffffffu, t[0], rsrc);
 #pragma unroll
                 for (int k = 0; k < K; ++k)
-                    u[k] = fma(rr, (k ? t[k ? k - 1 : 0] : lv) + (k + 1 < K ? t[k + 1 < K ? k + 1 : k] : rv), t[k]);
+                    uc[k] = fma(rr, (k ? t[k ? k - 1 : 0] : lv) + (k + 1 < K ? t[k + 1 < K ? k + 1 : k] : rv), t[k]);
             } else {
                 T lf[K], rg[K];
 #pragma unroll
@@ -293,26 +288,23 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
                     const T l = lane > 0 ? lf[k] : (k > 0 ? lf[k > 0 ? k - 1 : 0] : lastv);
                     T r = lane < 31 ? rg[k] : rg[k < K - 1 ? k + 1 : k];
                     if (MODE == STRIDED && k == K - 1) r = lane == ll ? firstv : r;
-                    u[k] = fma(rr, l + r, t[k]);
+                    uc[k] = fma(rr, l + r, t[k]);
                 }
             }
-            if (i >= 2) {
+            if (d >= 2 || i0 > 0) {
+                constexpr int ring3 = 3;
+                const int de = d % EU, um = SHIFT ? 0 : (d + 1) % ring3, u0 = SHIFT ? 1 : (d + 2) % ring3;
                 T g[K], v[K];
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                    const T sg = fma(rr, pm[k] + u[k], p0[k]);
-                    g[k] = e[d][k] * sg;
-                    v[k] = fma(st[d][k], sg, q[d][k]);
+                    const T sg = fma(rr, u[um][k] + uc[k], u[u0][k]);
+                    g[k] = e[de][k] * sg;
+                    if constexpr (PAST) v[k] = fma(st[de][k], sg, q[de][k]);
                 }
-                if (o.st) {
-                    put(pw, v);
-                    pw += plane;
-                }
-                if (o.dst) {
-                    put(pd, g);
-                    pd += plane;
-                }
-                if (o.lastQ) {
+                if constexpr (PAST) put(o.q + ow, v);
+                if (o.dst) put(o.dst + ow, g);
+                ow += plane;
+                if (PAST && o.lastQ) {
                     double qp = 0.0;
 #pragma unroll
                     for (int k = 0; k < K; ++k)
@@ -325,67 +317,117 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
                     }
                 }
             }
+            if constexpr (SHIFT) {
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                pm[k] = p0[k];
-                p0[k] = u[k];
+                for (int k = 0; k < K; ++k) {
+                    u[0][k] = u[1][k];
+                    u[1][k] = u[2][k];
+                }
             }
         }
     }
 }
 
+// The first level of a chain, sigma[1] E (the passes' rounding included).
+template <typename T, int K, int MODE>
+__device__ __forceinline__ void coop_run_first(const CoopRep& R, const CoopOps<T>& o, int x0, int y, int za, int n, T rr) {
+    const int lane = threadIdx.x & 31, nx = R.nx, plane = nx * R.ny;
+    const T t = fma(rr, T(2), T(1)), u = fma(rr, t + t, t), sg = fma(rr, u + u, u);
+    const int xe = MODE == TILE ? min(nx, x0 + 32 * K - 2) : nx;
+    for (int z = za; z < za + n; ++z)
+        for (int x = x0 + lane; x < xe; x += 32) {
+            const int i = z * plane + y * nx + x;
+            o.dst[i] = o.E[i] * sg;
+        }
+}
+
 // Rows of the x tiling: one whole row up to 256 sites, tiles of 254 columns beyond.
 constexpr int kCoopTile = 32 * 8 - 2;
 
+// n planes from za of row y of x tile xt, at level j of chain C.
 template <typename T, int K, int MODE, int C>
-__device__ __forceinline__ void coop_segment(const CoopRep& R, int j, int u0, int u1, double& qs) {
-    const CoopOps<T> o = coop_ops<T, C>(R, j);
+__device__ __forceinline__ void coop_rows(const CoopRep& R, const CoopOps<T>& o, int j, int xt, int y, int za, int n, double& qs) {
     const T rr = (T)R.rr;
+    if (j == 0) coop_run_first<T, K, MODE>(R, o, xt * kCoopTile, y, za, n, rr);
+    else if (o.st) coop_run<T, K, MODE, true>(R, o, xt * kCoopTile, y, za, n, rr, (xt * R.ny + y) * R.nz + za, qs);
+    else coop_run<T, K, MODE, false>(R, o, xt * kCoopTile, y, za, n, rr, 0, qs);
+}
+
+// Planes u0 .. u1 - 1 of the strips (strip-major) of a replica; of strips of 8 rows this warp's row.
+template <typename T, int K, int MODE, int C>
+__device__ __forceinline__ void coop_segment(const CoopRep& R, int j, int u0, int u1, int w, double& qs) {
+    const CoopOps<T> o = coop_ops<T, C>(R, j);
     const int nz = R.nz;
     for (int u = u0; u < u1;) {
-        const int row = u / nz;
-        const int z = u - row * nz;
-        const int n = min(nz - z, u1 - u);
-        const int xt = MODE == TILE ? row / R.ny : 0, y = row - xt * R.ny;
-        coop_run<T, K, MODE>(R, o, xt * kCoopTile, y, z, n, rr, u, qs);
+        const int g = u / nz, z = u - g * nz, n = min(nz - z, u1 - u);
+        const int row = R.strip == 8 ? 8 * g + w : g;
+        const int xt = MODE == TILE ? row / R.ny : 0;
+        coop_rows<T, K, MODE, C>(R, o, j, xt, row - xt * R.ny, z, n, qs);
         u += n;
     }
 }
 
-// KK: row layout of every replica of the launch, or 0: a switch per replica.
+// This warp's share of a level.  KK: row layout of every replica of the launch, or 0: a switch per replica.
+// cut: its run of the one replica (row; first plane, end), or the cost bounds of the warp and of its CTA.
+struct CoopCut {
+    int row, za, ze;
+    int b0, b1, a0, a1;
+};
 template <typename T, int KK, int C>
-__device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int j, int p, int b0, int b1) {
+__device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int runs, int j, int p, const CoopCut& cut) {
+    if constexpr (KK > 0) {
+        if (runs > 0) {
+            const CoopRep& R = reps[0];
+            constexpr int MODE = (KK >> 4) - 1;
+            double qs = 0.0;
+            if (cut.za < cut.ze) {
+                const int xt = MODE == TILE ? cut.row / R.ny : 0;
+                coop_rows<T, (KK & 15), MODE, C>(R, coop_ops<T, C>(R, j), j, xt, cut.row - xt * R.ny, cut.za, cut.ze - cut.za, qs);
+            }
+            if (C == 0 && j == R.N - 1 && !R.qrow) {   // s = N: this warp's share of Q
+                const double t = warp_sum(qs);
+                if ((threadIdx.x & 31) == 0) R.pq[p] = t;
+            }
+            return;
+        }
+    }
+    const int w = threadIdx.x >> 5;
     for (int i = 0; i < nact; ++i) {
         const CoopRep& R = reps[i];
-        const int lay = KK > 0 ? KK : R.layout, w = lay & 15;
-        const int c0 = R.cost0, c1 = c0 + R.units * w;
-        if (c1 <= b0) continue;
-        if (c0 >= b1) break;
-        // this warp's units (row planes) of the replica: cost bounds rounded up to whole units
-        const int u0 = b0 > c0 ? (b0 - c0 + w - 1) / w : 0;
-        const int u1 = b1 < c1 ? (b1 - c0 + w - 1) / w : R.units;
+        const int lay = KK > 0 ? KK : R.layout, wgt = R.wgt, planes = R.units / R.strip;
+        const int b0 = R.strip == 8 ? cut.a0 : cut.b0, b1 = R.strip == 8 ? cut.a1 : cut.b1;
+        const int c0 = R.cost0, c1 = c0 + planes * wgt;
+        if (c1 <= cut.a0) continue;
+        if (c0 >= cut.a1) break;
+        // planes of the replica: cost bounds rounded up to whole planes
+        const int u0 = b0 > c0 ? (b0 - c0 + wgt - 1) / wgt : 0;
+        const int u1 = b1 < c1 ? (max(b1 - c0, 0) + wgt - 1) / wgt : planes;
         double qs = 0.0;
         if constexpr (KK > 0) {
-            coop_segment<T, (KK & 15), (KK >> 4) - 1, C>(R, j, u0, u1, qs);
+            coop_segment<T, (KK & 15), (KK >> 4) - 1, C>(R, j, u0, u1, w, qs);
         } else {
-#define DSCF_COOP_CASE(KV, MV) case KV + 16 * (MV + 1): coop_segment<T, KV, MV, C>(R, j, u0, u1, qs); break;
+#define DSCF_COOP_CASE(KV, MV) case KV + 16 * (MV + 1): coop_segment<T, KV, MV, C>(R, j, u0, u1, w, qs); break;
             switch (lay) {
                 DSCF_COOP_LAYOUTS(DSCF_COOP_CASE)
                 default: break;
             }
 #undef DSCF_COOP_CASE
         }
-        if (C == 0 && j == R.N - 1 && !R.qrow) {   // s = N: this warp's share of Q
+        if (C == 0 && j == R.N - 1 && !R.qrow) {
             const double t = warp_sum(qs);
             if ((threadIdx.x & 31) == 0) R.pq[p] = t;
         }
     }
 }
 
-// Warps of a CTA, one CTA per SM: eight compute warps of up to 232 registers a thread (for the planes in
-// flight), and one warpgroup for the barriers, one warp per chain (the launch has 168 a thread:
-// 8 x 232 + 4 x 24 <= 12 x 168).
-constexpr int kCoopWarps = 8, kCoopSync = 4, kCoopRegs = 232, kCoopSyncRegs = 24;
+// Warps of a CTA, one CTA per SM: compute warps, and one warpgroup for the barriers, one warp per chain.
+// Rows of at most 16 bytes a lane leave room for 12 compute warps of 160 registers a thread (the launch has 128: 12 x 160 + 4 x
+// 24 <= 16 x 128), longer ones for 8 of 232 (168: 8 x 232 + 4 x 24 <= 12 x 168).
+constexpr int kCoopSync = 4, kCoopSyncRegs = 24;
+template <int NW>
+constexpr int kCoopRegs = NW == 12 ? 160 : 232;
+template <typename T>
+__host__ __device__ constexpr int coop_nw(int kk) { return coop_warps(kk, sizeof(T) == 8); }
 constexpr int kCoopShared = 128;   // largest table kept in shared memory
 constexpr long long kCoopSpinLimit = 1LL << 28;   // polls of a shared-memory mbarrier (see kBarSpinLimit in dscf_pers.cu)
 
@@ -419,8 +461,8 @@ __device__ __forceinline__ void cbar_wait(unsigned long long* bar, unsigned pari
 }
 
 template <typename T, int KK>
-__global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(const CoopCtl ctl) {
-    constexpr int NW = kCoopWarps;
+__global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_coop(const CoopCtl ctl) {
+    constexpr int NW = coop_nw<T>(KK);
     // the table in shared memory: the levels' acquire loads keep invalidating its cached copy
     __shared__ CoopRep tab[kCoopShared];
     __shared__ __align__(8) unsigned long long done[2], go[2];   // per chain: level computed here; computed everywhere
@@ -477,10 +519,19 @@ __global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(
         return;
     }
     // ---- compute warps ----
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kCoopRegs));
-    // neighbouring runs (the same row, then the next rows) go to one CTA: their rows meet in its L1
-    const int p = blockIdx.x * NW + w, P = ncta * NW;
-    int nact = ctl.nrep + 1, b0 = 0, b1 = 0;   // active replicas; this warp's share of their cost
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kCoopRegs<NW>));
+    const int p = blockIdx.x * NW + w;
+    int nact = ctl.nrep + 1;        // active replicas
+    CoopCut cut = {};
+    if (ctl.runs > 0) {
+        const CoopRep& R = reps[0];
+        const int i = blockIdx.x * ctl.per + w, k = i % ctl.runs;
+        cut.row = i / ctl.runs;
+        if (w < ctl.per && cut.row * R.nz < R.units) {
+            cut.za = (int)((long long)R.nz * k / ctl.runs);
+            cut.ze = (int)((long long)R.nz * (k + 1) / ctl.runs);
+        }
+    }
     if (ctl.j0 == 0) {   // shares of Q of replicas this warp has none of
         for (int r = lane; r < ctl.nrep; r += 32)
             if (!reps[r].qrow) reps[r].pq[p] = 0.0;
@@ -492,9 +543,12 @@ __global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(
         while (nact > 0 && reps[nact - 1].N <= j) --nact;
         if (nact != before) {
             const CoopRep& last = reps[nact - 1];
-            const long long total = last.cost0 + last.units * (last.layout & 15);
-            b0 = (int)(total * p / P);
-            b1 = (int)(total * (p + 1) / P);
+            const long long total = last.cost0 + last.units / last.strip * last.wgt;
+            const long long P = ncta * NW, pa = blockIdx.x * NW;
+            cut.b0 = (int)(total * p / P);
+            cut.b1 = (int)(total * (p + 1) / P);
+            cut.a0 = (int)(total * pa / P);
+            cut.a1 = (int)(total * (pa + NW) / P);
         }
         const int d = j - ctl.j0;            // levels of this launch before this one
         const unsigned par = (unsigned)((d - 1) & 1);
@@ -505,14 +559,14 @@ __global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(
             if (nact != before) cbar_wait(&go[1], par, ctl, dead);
             __syncwarp();
         }
-        coop_level<T, KK, 0>(reps, nact, j, p, b0, b1);
+        coop_level<T, KK, 0>(reps, nact, ctl.runs, j, p, cut);
         if (sync) {
             __syncwarp();
             if (lane == 0) cbar_arrive(&done[0]);
             if (d > 0) cbar_wait(&go[1], par, ctl, dead);
             __syncwarp();
         }
-        coop_level<T, KK, 1>(reps, nact, j, p, b0, b1);
+        coop_level<T, KK, 1>(reps, nact, ctl.runs, j, p, cut);
         if (sync) {
             __syncwarp();
             if (lane == 0) cbar_arrive(&done[1]);
@@ -526,7 +580,7 @@ __global__ void __launch_bounds__(32 * (kCoopWarps + kCoopSync), 1) k_prop_coop(
         for (int r = 0; r < ctl.nrep; ++r) {
             const CoopRep& R = reps[r];
             const int units = R.units;
-            for (int g = p; 32 * g < units; g += P) {
+            for (int g = p; 32 * g < units; g += ncta * NW) {
                 const int u = 32 * g + lane;
                 const double t = warp_sum(u < units ? R.qrow[u] : 0.0);
                 if (lane == 0) R.pq[g] = t;
@@ -568,9 +622,10 @@ const void* coop_kernel(int kk) {
 // ever if they did not).
 template <typename T>
 int coop_prepare(int kk) {
+    const int nw = coop_nw<T>(kk);
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, coop_kernel<T>(kk));
-    if (e == cudaSuccess && fa.numRegs * (kCoopWarps + kCoopSync) < kCoopRegs * kCoopWarps + kCoopSyncRegs * kCoopSync)
+    if (e == cudaSuccess && fa.numRegs * (nw + kCoopSync) < (nw == 12 ? kCoopRegs<12> : kCoopRegs<8>) * nw + kCoopSyncRegs * kCoopSync)
         e = cudaErrorInvalidConfiguration;
     return (int)e;
 }
@@ -586,9 +641,11 @@ int launch_prop_coop(const Launch& L, const CoopPlan& c, int j0, int j1, int lim
     ctl.abort = c.abort;
     ctl.status = L.status;
     ctl.limit = limit;
+    ctl.runs = c.runs;
+    ctl.per = c.per;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c.ncta);
-    cfg.blockDim = dim3(32 * (kCoopWarps + kCoopSync));
+    cfg.blockDim = dim3(32 * (coop_nw<T>(c.kk) + kCoopSync));
     cfg.stream = L.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -1,24 +1,57 @@
 // General contour sweeps (dscf_coop.cuh), FP32, and what the host needs to know of them.
 #include "dscf_coop.cuh"
 
+#include <algorithm>
+
 namespace dscf {
 
 long long coop_units(const Rep& R) { return (long long)R.ny * R.nz * (R.nx <= 256 ? 1 : (R.nx + kCoopTile - 1) / kCoopTile); }
 
-// CTAs of a launch: one per SM, fewer where that would leave a warp less than two row planes.
-int coop_ctas(long long units, int nsm) {
-    const long long w = 2LL * kCoopWarps;
-    const long long n = (units + w - 1) / w;
-    return (int)(n < 1 ? 1 : (n < nsm ? n : nsm));
-}
-int coop_warps_per_cta() { return kCoopWarps; }
+// Strips of 8 rows where a field exceeds the L2, so that a CTA's warps share rows at about the same time
+// (256^3, N = 64: 7.93 -> 7.56 ms); in smaller grids sharing gains nothing.
+static int strip_rows(const Rep& R) { return R.V >= (1LL << 23) && R.ny % 8 == 0 && coop_warps(coop_layout(R.nx), false) == 8 ? 8 : 1; }
+static int x_tiles(int nx) { return nx <= 256 ? 1 : (nx + kCoopTile - 1) / kCoopTile; }
 
-CoopRep coop_rep(const Rep& R, int cost0) {
+// Cut of a launch's work.  One replica whose rows can be cut into equal runs gives every warp one run
+// (runs > 0): a warp of an even cut of all row planes mostly ends one row and begins another, which costs two
+// more planes of the y and x passes and, in FP32, the loads' latency once more, and the slowest warp makes
+// the level's time.  Density evaluations with the even cut and with runs: 100 x 90 x 75, N = 48, FP32 364 and
+// 281 us; 64^3, N = 64, FP32 331 and 241; 32^3, N = 32, FP64 265 and 132.  The runs are spread over all SMs.
+// Where whole runs would leave too many warps idle (estimated below in planes), and in batches, the cut is
+// even, at least two row planes a warp.
+void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm) {
+    const int nw = coop_warps(c.kk, fp64), P = nsm * nw;
+    c.runs = c.per = 0;
+    if (c.nrep == 1) {
+        const long long rows = (long long)x_tiles(R.nx) * R.ny;
+        if (rows <= P) {
+            int r = std::min((int)(P / rows), R.nz);
+            const int n = (R.nz + r - 1) / r;
+            r = (R.nz + n - 1) / n;
+            const double even = (double)((work + P - 1) / P) + (fp64 ? 2.0 + 2.0 * rows / P : 8.0);
+            if (n + (fp64 ? 2 : 4) <= even) {
+                c.runs = r;
+                c.per = (int)((rows * r + nsm - 1) / nsm);
+                c.ncta = (int)((rows * r + c.per - 1) / c.per);
+                return;
+            }
+        }
+    }
+    const long long w = 2LL * nw, n = (work + w - 1) / w;
+    c.ncta = (int)(n < 1 ? 1 : (n < nsm ? n : nsm));
+}
+
+// a row plane's time: FP32 mostly the latency of its loads, FP64 mostly its operations
+int coop_cost(const Rep& R, bool fp64) { return fp64 ? 1 + 2 * coop_sites(R.nx) : 4 + coop_sites(R.nx); }
+
+CoopRep coop_rep(const Rep& R, int cost, int cost0) {
     CoopRep c = {};
     c.nx = R.nx; c.ny = R.ny; c.nz = R.nz; c.N = R.N; c.nA = R.nA;
     c.layout = coop_layout(R.nx);
     c.cost0 = cost0;
     c.units = (int)coop_units(R);
+    c.strip = strip_rows(R);
+    c.wgt = cost * c.strip;
     c.V = R.V;
     c.E = R.E; c.G = R.G; c.Gp0 = R.Gp0; c.Gp1 = R.Gp1; c.q = R.q;
     c.qrow = R.qrow;

@@ -416,8 +416,9 @@ __device__ __forceinline__ float bexp(float x) { return expf(-x); }
 struct CoopRep {
     int nx, ny, nz, N, nA;
     int layout;          // coop_layout(nx)
-    int cost0;           // cost (row planes x sites per lane) of the entries before
     int units;           // row planes
+    int strip;           // rows cut together: 8 (a CTA's warps side by side) or 1
+    int wgt, cost0;      // cost of a plane of a strip, of all entries before
     long long V;
     void *E, *G, *Gp0, *Gp1, *q;
     double *qrow, *pq;   // sums of G_N per row plane (or nullptr), the P_Q slot
@@ -430,6 +431,7 @@ struct CoopPlan {
     int* cnt;            // device: barrier counters (3 lines), zero between launches
     int* abort;
     int kk, ncta;
+    int runs, per;       // runs > 0: one replica, each row cut into this many, one per warp, `per` in a CTA
 };
 // Row layout of a grid: sites per lane + 16 (1 + mode), mode 0 blocked, 1 strided, 2 tiled.  Blocked
 // where some K of 1, 2, 3, 4, 6, 8 divides nx into at most 32 lanes without leaving more than about
@@ -442,11 +444,13 @@ __host__ __device__ constexpr int coop_layout(int nx) {
     return k + 32;
 }
 __host__ __device__ constexpr int coop_sites(int nx) { return coop_layout(nx) & 15; }
+// Compute warps of a CTA of the general sweeps (kk: the row layout of all replicas, or 0).
+__host__ __device__ constexpr int coop_warps(int kk, bool fp64) { return kk > 0 && (kk & 15) * (fp64 ? 8 : 4) <= 16 ? 12 : 8; }
 constexpr int kCoopMaxCtas = 152;
 long long coop_units(const Rep& R);   // row planes (of x tiles beyond 256 sites)
-int coop_ctas(long long units, int nsm);
-int coop_warps_per_cta();
-CoopRep coop_rep(const Rep& R, int cost0);
+int coop_cost(const Rep& R, bool fp64);   // of a row plane
+void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm);   // ncta, runs, per
+CoopRep coop_rep(const Rep& R, int cost, int cost0);   // cost: of a row plane
 template <typename T> int coop_prepare(int kk);   // cudaError_t
 template <typename T> int launch_prop_coop(const Launch& L, const CoopPlan& c, int j0, int j1, int limit);   // cudaError_t
 // mode: 0 exp(-U), 1 trial exp(-(U + a1 d)), 2 commit U += a d then exp(-U), 3 exp(-Uext)

@@ -109,9 +109,11 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
         return DSCF_ERR_CUDA;
     }
     if (nsm > kCoopMaxCtas) nsm = kCoopMaxCtas;
-    const long long units = coop_units(R);
-    const int ncta = coop_ctas(units, nsm);
-    R.nq = ncta * coop_warps_per_cta();
+    CoopPlan plan;
+    plan.nrep = 1;
+    plan.kk = coop_layout(R.nx);
+    coop_cut(plan, R, coop_units(R), precision == DSCF_FP64, nsm);
+    R.nq = plan.ncta * coop_warps(plan.kk, precision == DSCF_FP64);
     R.part_stride = R.nq > R.nblk ? R.nq : R.nblk;
 
     // Scratch layout: replica table, maps, Boltzmann factors, propagators, quadratures,
@@ -160,8 +162,7 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     R.ext_off = 0;
     R.vbase = 0;
 
-    const int kk = coop_layout(R.nx);
-    if ((precision == DSCF_FP64 ? coop_prepare<double>(kk) : coop_prepare<float>(kk)) != 0) {
+    if ((precision == DSCF_FP64 ? coop_prepare<double>(plan.kk) : coop_prepare<float>(plan.kk)) != 0) {
         set_thread_error("dscf_densities_static: the contour kernels do not load");
         return DSCF_ERR_CUDA;
     }
@@ -176,19 +177,15 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     L.nlb_total = R.lb_nblk;
     L.nrep = 1;
     L.stream = s;
-    CoopPlan plan;
     plan.reps = (const CoopRep*)(base + o_coop);
-    plan.nrep = 1;
     plan.cnt = plan.abort = nullptr;   // one level per launch: no barrier inside a launch
-    plan.kk = kk;
-    plan.ncta = ncta;
     // the only state that must start at zero: the block map (one replica, index 0)
     cudaError_t e = cudaMemsetAsync(base + o_b2r, 0, sizeof(int) * R.nblk, s);
     if (e != cudaSuccess) {
         set_thread_error("dscf_densities_static: cudaMemsetAsync failed");
         return DSCF_ERR_CUDA;
     }
-    k_put_rep<<<1, 1, 0, s>>>((Rep*)(base + o_rep), R, (CoopRep*)(base + o_coop), coop_rep(R, 0));
+    k_put_rep<<<1, 1, 0, s>>>((Rep*)(base + o_rep), R, (CoopRep*)(base + o_coop), coop_rep(R, 1, 0));
     if (precision == DSCF_FP64) {
         launch_exp<double>(L, 3, 0, U_in);
         for (int j = 0; j < R.N; ++j) launch_prop_coop<double>(L, plan, j, j + 1, 1);

@@ -44,6 +44,25 @@ def test_general_sweeps_where_the_chains_meet(N, precision):
         check_densities(melt((34, 7, 6), N, nA), precision, 30 + N, tuning=(8, 1))
 
 
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("tile,reps", [((32, 16, 8), (8, 16, 16)),      # even cut of strips of 8 rows
+                                       ((32, 16, 8), (8, 8, 32)),       # wide field, one run per warp
+                                       ((8, 10, 3), (1, 200, 1)),       # more rows than warps: even cut
+                                       ((9, 7, 37), (1, 1, 1))],        # one row plane per warp, uneven CTAs
+                         ids=["strips", "runs-wide", "even", "runs-small"])
+def test_general_sweeps_cuts(tile, reps, precision):
+    """A periodic field of any period has the densities of one period."""
+    cfg, big = (melt(g, 4, 1) for g in (tile, tuple(t * r for t, r in zip(tile, reps))))
+    U = inputs.random_field(ncomp_shape(cfg), seed=60, scale=0.5)
+    ref, _, _ = oracle.densities(cfg, U)
+    up = lambda a: np.tile(a, (1,) + reps[::-1])
+    ctx = dscf.Context(big, precision, tuning=(8, 1))
+    got = t2n(ctx.densities(torch.from_numpy(up(U))))
+    ctx.status()
+    ctx.close()
+    assert rel(got, up(ref)) < (1e-12 if precision == dscf.FP64 else 1e-5)
+
+
 @pytest.mark.parametrize("N", [2, 3, 4, 5, 8, 9])
 @pytest.mark.parametrize("grid,zc", [((128, 16, 16), 16), ((64, 8, 8), 8), ((48, 16, 32), 16)])
 def test_brick_sweeps_where_the_chains_meet(N, grid, zc):
