@@ -358,7 +358,7 @@ def learned_form(cfg, dev, phi0, timed, world, tuning, steps):
 def learned256_form(dev, timed, rank, world, steps=40):
     """The learned predictor on its own workload: the 256^3 symmetric melt (f = 0.5, chi N = 20,
     N = 64), corrector every 10 steps; the exact FP32 step at the same size beside it (these rows
-    of 256 sites take the multi-launch contour kernels: a persistent sweep cannot hold 16.8 M sites).
+    of 256 sites take the general sweeps: bricks cannot hold 16.8 M sites).
     The network is trained as in the 128^3 form, on 32^3 boxes of this physics, and fine-tuned on
     ten exact steps of the run."""
     import numpy as np
@@ -722,9 +722,8 @@ def run_ours(a):
         forms["net_forward"] = net_forward_form(dev, timed)
 
     hbm, peak_kind = peaks()
-    # Dominant kernel: the propagator sweeps.  The unit is one contour step (the autotuner runs
-    # N of them per launch in the persistent kernel, K per launch in the fused one, one in the
-    # single-step kernels).  Algorithmic bytes per contour step: the store-forward propagator
+    # Dominant kernel: the propagator sweeps.  The unit is one contour step of one chain (a launch
+    # runs all N of both).  Algorithmic bytes per contour step: the store-forward propagator
     # solve must write G_s once and read it once per density evaluation plus read U and write
     # phi: (8N + 16) B per site per evaluation over its 2N contour steps, i.e. (4 + 8/N) B per
     # site per step (FP32).
@@ -734,8 +733,8 @@ def run_ours(a):
     traffic = ncu_traffic(os.path.join(ROOT, "paper_1204_2088_gb300", "csrc", "dscf_pers.cu"), N)
     roof = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
             "traffic": traffic,
-            "kernel": {0: "k_prop_pers (persistent sweep)", 1: "k_prop (single step)"}.get(
-                diag["kfuse"], f"k_prop_fused (K={diag['kfuse']})") + "; unit = one contour step",
+            "kernel": ("k_prop_pers (brick sweeps)" if diag["kfuse"] == 0 else "k_prop_coop (general sweeps)")
+            + "; unit = one contour step",
             "alg_bytes_per_launch": alg_bytes, "ms_per_launch": per_launch_s * 1e3, "peak_kind": peak_kind}
     lb_alg = 180.0 * V
     bstep = step_bytes_per_site(N, cfg["ncg_iters"], cfg["cn_sweeps"], cfg["hydro"])

@@ -286,8 +286,8 @@ int dscf_inject_lag(dscf_ctx* ctx, int32_t brick);
 int dscf_fma_peak(int32_t precision, void* stream, double* tflops);
 
 /* Timing probe.  enable != 0 makes the next dscf_step capture CUDA events (created by the
- * library) into the step graph: around the 2N contour-sweep launches of the first gradient
- * evaluation of the step, around the LB collide-stream launch, and around the whole step.
+ * library) into the step graph: around the contour sweeps (N contour steps of each
+ * chain) of the first gradient evaluation of the step, around the LB collide-stream launch, and around the whole step.
  * dscf_probe_ms synchronises the stream and returns, for the most recent step, the elapsed
  * milliseconds of those three regions (ms[0] sweeps, ms[1] LB, ms[2] step); regions that did
  * not run read 0.  DSCF_ERR_STATE if the probe is off or no step ran since enabling it. */

@@ -20,8 +20,8 @@
 // (c + r (a + d), r = alpha / (1 - 2 alpha), the centre weights folded into the Boltzmann factors and the
 // normalisation): 7 operations a site and contour step forward, 8 with the quadrature.
 //
-// FP64 at 128^3 is bound by the FP64 pipe (31 us of operations in a level's 33 us), 256^3 by HBM (13 fields
-// of 67 MB a pair of levels), the rest by the latency of loads and of the barrier: hence loads several planes
+// FP64 at 128^3 is bound by the FP64 pipe (31 us of operations in a level's 33 us), 256^3 by HBM (592 MB
+// a pair of levels at 77% of the copy rate), the rest by the latency of loads and of the barrier: hence loads several planes
 // ahead, 12 warps where the registers allow it (128^3 FP32: 750 us with 8, 689 with 12) and one run per warp.
 // A density evaluation, one launch per contour step and direction, and so: 32^3, N = 32, FP64 539 -> 127 us;
 // 100 x 90 x 75, N = 48, FP32 1013 -> 276 us; 128^3, N = 64, FP64 8.9 -> 4.2 ms; 256^3, N = 64, FP32 8.07

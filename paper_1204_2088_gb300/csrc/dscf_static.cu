@@ -113,23 +113,29 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     plan.nrep = 1;
     plan.kk = coop_layout(R.nx);
     coop_cut(plan, R, coop_units(R), precision == DSCF_FP64, nsm);
-    R.nq = plan.ncta * coop_warps(plan.kk, precision == DSCF_FP64);
-    R.part_stride = R.nq > R.nblk ? R.nq : R.nblk;
-
     // Scratch layout: replica table, maps, Boltzmann factors, propagators, quadratures,
     // partial sums, scalars.
     const size_t V = (size_t)R.V;
-    size_t off = 0;
-    const size_t o_rep = off; off = up256(off + sizeof(Rep));
-    const size_t o_coop = off; off = up256(off + sizeof(CoopRep));
-    const size_t o_b2r = off; off = up256(off + sizeof(int) * R.nblk);
-    const size_t o_E = off; off = up256(off + (size_t)R.ns * V * es);
-    const size_t o_G = off; off = up256(off + (size_t)R.N * V * es);
-    const size_t o_Gp0 = off; off = up256(off + V * es);
-    const size_t o_Gp1 = off; off = up256(off + V * es);
-    const size_t o_q = off; off = up256(off + 2 * V * es);
-    const size_t o_part = off; off = up256(off + sizeof(double) * 2 * (size_t)R.part_stride);   // P_Q, P_ES
-    const size_t o_scal = off; off = up256(off + sizeof(double) * kScalStride);
+    size_t off, o_rep, o_coop, o_b2r, o_E, o_G, o_Gp0, o_Gp1, o_q, o_part, o_scal;
+    for (;;) {
+        R.nq = plan.ncta * coop_warps(plan.kk, precision == DSCF_FP64);
+        R.part_stride = R.nq > R.nblk ? R.nq : R.nblk;
+        off = 0;
+        auto take = [&](size_t bytes) { const size_t o = off; off = up256(off + bytes); return o; };
+        o_rep = take(sizeof(Rep));
+        o_coop = take(sizeof(CoopRep));
+        o_b2r = take(sizeof(int) * R.nblk);
+        o_E = take((size_t)R.ns * V * es);
+        o_G = take((size_t)R.N * V * es);
+        o_Gp0 = take(V * es);
+        o_Gp1 = take(V * es);
+        o_q = take(2 * V * es);
+        o_part = take(sizeof(double) * 2 * (size_t)R.part_stride);   // P_Q, P_ES
+        o_scal = take(sizeof(double) * kScalStride);
+        if (off <= (size_t)DSCF_STATIC_SCRATCH_BYTES || plan.ncta == 1) break;
+        plan.ncta = (plan.ncta + 1) / 2;   // near the limit: fewer warps' partial sums, an even cut
+        plan.runs = plan.per = 0;
+    }
     if (off > (size_t)DSCF_STATIC_SCRATCH_BYTES) {
         set_thread_error("dscf_densities_static: the problem needs more scratch than DSCF_STATIC_SCRATCH_BYTES");
         return DSCF_ERR_OOM;

@@ -92,6 +92,17 @@ def test_general_sweeps_of_unlike_replicas_equal_solo_runs(precision):
         off += p.size
 
 
+def test_static_density_map_at_its_scratch_limit():
+    """A small grid with the longest chain that fits: few warps, an even cut."""
+    grid = (16, 8, 16)
+    cfg = melt(grid, 64 * 1024 * 1024 // (2048 * 8) - 7, 1000)   # 2048 sites of 8 bytes: N + 6 fields and tables
+    U = inputs.random_field(ncomp_shape(cfg), seed=70, scale=0.01)
+    ref, _, _ = oracle.densities(cfg, U)
+    U = torch.from_numpy(U).cuda()
+    got = t2n(dscf.densities_static(cfg, U, torch.empty_like(U)))
+    assert rel(got, ref) < 1e-10      # the bound of a coupled FP64 step: 4089 contour steps
+
+
 def test_bricks_that_do_not_run_together_take_the_general_sweeps():
     """256 shallow bricks: the tuning stays valid, the densities are those of the deep bricks."""
     cfg = melt((128, 128, 128), 3, 2)
