@@ -170,7 +170,7 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
     // rings of rows and of operands (the widest FP64 rows have registers for one operand plane only); FP64, bound by
     // its pipe, loses more to the instruction cache in a longer loop than it gains (128^3, N = 64: 4.46 ms
     // unrolled by 6, 4.18 by 2)
-    constexpr int RU = sizeof(T) == 8 ? (B <= 16 ? 3 : 2) : B <= 8 ? 6 : B <= 12 ? 4 : 3, D = RU - 1;
+    constexpr int RU = sizeof(T) == 8 ? (B <= 16 ? 3 : 2) : B <= 8 ? 6 : B <= 12 ? 4 : B <= 16 || B > 24 ? 3 : 2, D = RU - 1;
     constexpr int EU = RU == 6 ? 3 : RU > 2 ? RU : B < 48 + 16 * (MODE == BLOCKED) ? 2 : 1, DE = EU > 2 ? 2 : EU - 1;
     constexpr int UN = RU;
     constexpr bool SHIFT = UN % 3 != 0;   // the planes of the z pass move by copies
@@ -421,8 +421,10 @@ __device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int ru
 }
 
 // Warps of a CTA, one CTA per SM: compute warps, and one warpgroup for the barriers, one warp per chain.
-// Rows of at most 16 bytes a lane leave room for 12 compute warps of 160 registers a thread (the launch has 128: 12 x 160 + 4 x
-// 24 <= 16 x 128), longer ones for 8 of 232 (168: 8 x 232 + 4 x 24 <= 12 x 168).
+// Rows of at most 16 bytes a lane (FP32: 24) leave room for 12 compute warps of 160 registers a thread (the
+// launch has 128: 12 x 160 + 4 x 24 <= 16 x 128), longer ones for 8 of 232 (168: 8 x 232 + 4 x 24 <= 12 x
+// 168).  N = 32, FP32, 8 and 12 warps: 140 x 80 x 80 274 and 265 us, 163 x 80 x 80 303 and 291, but 200 x
+// 100 x 64 323 and 371, 256^3 3.92 and 4.08 ms.
 constexpr int kCoopSync = 4, kCoopSyncRegs = 24;
 template <int NW>
 constexpr int kCoopRegs = NW == 12 ? 160 : 232;

@@ -445,7 +445,7 @@ __host__ __device__ constexpr int coop_layout(int nx) {
 }
 __host__ __device__ constexpr int coop_sites(int nx) { return coop_layout(nx) & 15; }
 // Compute warps of a CTA of the general sweeps (kk: the row layout of all replicas, or 0).
-__host__ __device__ constexpr int coop_warps(int kk, bool fp64) { return kk > 0 && (kk & 15) * (fp64 ? 8 : 4) <= 16 ? 12 : 8; }
+__host__ __device__ constexpr int coop_warps(int kk, bool fp64) { return kk > 0 && (kk & 15) * (fp64 ? 8 : 4) <= (fp64 ? 16 : 24) ? 12 : 8; }
 constexpr int kCoopMaxCtas = 152;
 long long coop_units(const Rep& R);   // row planes (of x tiles beyond 256 sites)
 int coop_cost(const Rep& R, bool fp64);   // of a row plane
