@@ -2,6 +2,7 @@
 // dscf_pers.cu, bricks.)
 #include "dscf_internal.cuh"
 
+#include <cstdint>
 #include <type_traits>
 
 namespace dscf {
@@ -65,7 +66,8 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
     const T ta = ta_sh, be3 = pars<T>(R).be3;
     T es = T(0);
     bool vec = false;
-    if constexpr (sizeof(T) == 4) vec = (V & 3) == 0 && (mode != 3 || (R.ext_off & 3) == 0);
+    // (the caller's field may begin at any element: 16-byte accesses only where its blocks are aligned)
+    if constexpr (sizeof(T) == 4) vec = (V & 3) == 0 && (mode != 3 || ((uintptr_t)(Uext + R.ext_off) & 15) == 0);
     if (vec) {   // FP32, 4 consecutive sites per thread and iteration (16-byte accesses)
         const float fa = (float)ta;
         float es4 = 0.f;

@@ -157,3 +157,18 @@ def test_weight_gradients_on_ragged_tiles(grid):
     for got, ref, a in ((gW2, dW2, aW2), (gW1, dW1, aW1)):
         assert np.all(np.abs(got - ref) <= B * V * 2.0 ** -22 * a)
         assert np.abs(ref).max() > 0
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_potentials_at_any_element_of_an_allocation(shift):
+    """A contiguous view may begin 4, 8 or 12 bytes into its allocation: same densities, bit for bit
+    (a melt: per-site factors, no sum that the order of the threads' sites could change)."""
+    cfg = melt((36, 6, 5), 5, 2)
+    U = torch.from_numpy(inputs.random_field(ncomp_shape(cfg), seed=90, scale=0.5)).float().cuda()
+    view = torch.empty(U.numel() + shift, device="cuda")[shift:].view(U.shape).copy_(U)
+    assert view.is_contiguous() and view.data_ptr() % 16 == 4 * shift
+    ctx = dscf.Context(cfg, dscf.FP32)
+    assert torch.equal(ctx.densities(view), ctx.densities(U))
+    ctx.status()
+    out = [dscf.densities_static(cfg, u, torch.empty_like(U), dscf.FP32) for u in (view, U)]
+    assert torch.equal(out[0], out[1])
