@@ -111,7 +111,7 @@ void assign_tiles(Layout& L, const dscf_params* p, int n, int prec) {
     int cost = 0;
     for (int k = 0; k < n; ++k) {
         const Rep& R = L.reps[order[k]];
-        L.coop.push_back(coop_rep(R, all <= INT32_MAX ? coop_cost(R, prec == DSCF_FP64) : 1, cost));
+        L.coop.push_back(coop_rep(R, prec == DSCF_FP64, all <= INT32_MAX ? coop_cost(R, prec == DSCF_FP64) : 1, cost));
         L.work += L.coop.back().units;
         cost += L.coop.back().units / L.coop.back().strip * L.coop.back().wgt;
         if (L.coop.back().layout != L.kk) L.kk = 0;

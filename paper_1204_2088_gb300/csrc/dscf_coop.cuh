@@ -17,7 +17,7 @@
 // L + 32, ... of the row, so any row length and alignment has coalesced accesses), and combines three
 // planes in registers.  No pass is computed twice but the y and x passes of the two planes beside a
 // run, no shared memory and no barrier inside a level, and each pass is one add and one fma
-// (c + r (a + d), r = alpha / (1 - 2 alpha), the centre weights folded into the Boltzmann factors and the
+// (c + r (a + d), r = alpha / (1 - 2 alpha), the centre weights made up for by the Boltzmann factors and the
 // normalisation): 7 operations a site and contour step forward, 8 with the quadrature.
 //
 // FP64 at 128^3 is bound by the FP64 pipe (31 us of operations in a level's 33 us), 256^3 by HBM (592 MB
@@ -599,10 +599,18 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
             __threadfence();
             for (int r = w; r < ctl.nrep; r += NW) {
                 const CoopRep& R = reps[r];
-                double s = 0.0;
-                for (int g = lane; 32 * g < R.units; g += 32) s += __ldcg(R.pq + g);
-                s = warp_sum(s);
-                if (lane == 0) *R.qsum = s;
+                if constexpr (sizeof(T) == 8) {
+                    const Two s = total_of(R.pq, (R.units + 31) / 32);
+                    if (lane == 0) {
+                        R.qsum[0] = s.hi;
+                        R.qsum[S_QLO - S_QSUM] = s.lo;
+                    }
+                } else {
+                    double s = 0.0;
+                    for (int g = lane; 32 * g < R.units; g += 32) s += __ldcg(R.pq + g);
+                    s = warp_sum(s);
+                    if (lane == 0) *R.qsum = s;
+                }
             }
         }
     }

@@ -44,7 +44,7 @@ void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm) {
 // a row plane's time: FP32 mostly the latency of its loads, FP64 mostly its operations
 int coop_cost(const Rep& R, bool fp64) { return fp64 ? 1 + 2 * coop_sites(R.nx) : 4 + coop_sites(R.nx); }
 
-CoopRep coop_rep(const Rep& R, int cost, int cost0) {
+CoopRep coop_rep(const Rep& R, bool fp64, int cost, int cost0) {
     CoopRep c = {};
     c.nx = R.nx; c.ny = R.ny; c.nz = R.nz; c.N = R.N; c.nA = R.nA;
     c.layout = coop_layout(R.nx);
@@ -57,7 +57,7 @@ CoopRep coop_rep(const Rep& R, int cost, int cost0) {
     c.qrow = R.qrow;
     c.pq = R.part + (size_t)P_Q * R.part_stride;
     c.qsum = R.scal + S_QSUM;
-    c.rr = R.alpha / (1.0 - 2.0 * R.alpha);
+    c.rr = fp64 ? R.pd.rr : (double)R.pf.rr;
     return c;
 }
 

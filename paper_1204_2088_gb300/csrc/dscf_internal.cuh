@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 namespace dscf {
 
 constexpr int kFlatThreads = 256;     // threads of every site-parallel ("flat") kernel
@@ -41,7 +43,7 @@ enum ScalSlot {
     S_H0S, S_CDS, S_H1S,         // line search: <g,d>, <d, phi_m d>, h1
     S_GGS0, S_GGS1,              // <g,g> in the parity slots of the iterations
     S_TOT0, S_TOT1, S_TOT2,      // sum_r phi_I before the mass correction
-    S_QSUM, S_ESS,               // sum_r G_N(r) and sum_r exp(-U_S) of the last evaluation
+    S_QSUM, S_QLO, S_ESS, S_ESLO,   // sum_r G_N(r) and sum_r exp(-U_S) of the last evaluation (FP64: two parts)
     S_SHF0, S_SHF1, S_SHF2,      // mass correction per site
     S_QFIN,                      // finished-brick count of the sweeps (an unsigned)
     S_WARM,                      // steps whose starting potentials Uprev holds (0, 1, 2 = enough)
@@ -69,7 +71,11 @@ constexpr size_t kStatusInts = (size_t)kFlagBase + (size_t)kMaxBricks * kFlagStr
 // at 48^3, N = 16, FP32 fell from 1.29 to 1.02 ms, one of four at 128^3, N = 64 from 4.00 to 3.71 ms.
 template <typename T>
 struct Par {
-    T al, be, be3;             // stencil: alpha, 1 - 2 alpha and its cube
+    T al, be;                  // stencil: alpha, 1 - 2 alpha
+    T rr;                      // the sweeps' passes: c + rr (a + d), rr = alpha / (1 - 2 alpha)
+    T ew;                      // weight of the copolymer's Boltzmann factors, near 1 / (1 + 2 rr)^3
+    T s1;                      // the three passes of the constant field 1, rounded as the sweeps round it
+    double qn;                 // Q from the sweeps' mean of G_N, which holds N weights
     T rho0, gs, gb, dt2;       // LB: density, 1 - 1/tau, dt^2
     T dtM, c, kappa, floor;    // diffusion: dt M, dt M / 2, compressibility, floor of phi
     T chi[9];
@@ -130,7 +136,18 @@ __host__ __device__ __forceinline__ const Par<T>& pars(const Rep& R) {
 template <typename T>
 inline void set_par(const Rep& R, Par<T>& p) {
     const double be = 1.0 - 2.0 * R.alpha;
-    p.al = (T)R.alpha; p.be = (T)be; p.be3 = (T)(be * be * be);
+    p.al = (T)R.alpha; p.be = (T)be;
+    p.rr = (T)(R.alpha / be);
+    // The passes leave out their centre weights, so a level grows by w3 = (1 + 2 rr)^3 and the factors carry
+    // a weight against it.  Any weight will do (it cancels in the densities); a power of two adds no
+    // rounding to the factors, which are the same at every bead of a block: with 1 / w3 the potentials of a
+    // 128^3 FP64 step were 3 times as far off.  The nearest power leaves a level a drift of at most sqrt 2,
+    // which short chains hold easily (2^32 in FP32, 2^128 in FP64); longer ones take 1 / w3.
+    const long double w = 1.0L + 2.0L * (long double)p.rr, w3 = w * w * w;
+    p.ew = R.N <= (sizeof(T) == 4 ? 64 : 256) ? (T)std::exp2(-std::round(std::log2((double)w3))) : (T)(1.0L / w3);
+    const T t = std::fma(p.rr, T(2), T(1)), u = std::fma(p.rr, t + t, t);
+    p.s1 = std::fma(p.rr, u + u, u);
+    p.qn = (double)(std::pow((long double)p.ew * w3, (long double)-R.N) * (w3 / (long double)p.s1));
     p.rho0 = (T)R.rho0; p.gs = (T)R.gs; p.gb = (T)R.gb; p.dt2 = (T)(R.dt * R.dt);
     p.dtM = (T)(R.dt * R.M); p.c = (T)(0.5 * R.dt * R.M); p.kappa = (T)R.kappa; p.floor = (T)R.phi_floor;
     for (int i = 0; i < 9; ++i) p.chi[i] = (T)R.chi[i];
@@ -287,6 +304,29 @@ __device__ __forceinline__ double block_max(double v, double* sh) {
 
 __device__ __forceinline__ double block_top(double v, double* sh) { return block_max(v, sh); }
 
+// A sum carried with its rounding errors (Knuth's two-sum).  The totals of Q and of exp(-U_S) in FP64 end in
+// a few additions of numbers as large as themselves, whose roundings nothing averages out: up to 2e-16 of
+// the total and so of every density.
+struct Two {
+    double hi, lo;
+};
+__device__ __forceinline__ Two operator+(const Two& a, const Two& b) {
+    const double s = a.hi + b.hi, z = s - a.hi;
+    return {s, ((a.hi - (s - z)) + (b.hi - z)) + (a.lo + b.lo)};
+}
+__device__ __forceinline__ Two warp_sum(Two v) {   // in every lane
+    for (int o = 16; o > 0; o >>= 1)
+        v = v + Two{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+    return v;
+}
+// Total of n partials read through L2, by a warp.  Only the last additions carry their errors: a lane's own
+// are of parts of the total, and their roundings average out.
+__device__ __forceinline__ Two total_of(const double* p, int n) {
+    double s = 0.0;
+    for (int i = threadIdx.x & 31; i < n; i += 32) s += __ldcg(p + i);
+    return warp_sum(Two{s, 0.0});
+}
+
 // Total of n partials, same fixed order in every block.
 __device__ __forceinline__ double reduce_parts(const double* __restrict__ p, int n, double* sh) {
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
@@ -423,7 +463,7 @@ struct CoopRep {
     void *E, *G, *Gp0, *Gp1, *q;
     double *qrow, *pq;   // sums of G_N per row plane (or nullptr), the P_Q slot
     double* qsum;        // where their total goes
-    double rr;           // alpha / (1 - 2 alpha)
+    double rr;           // Par<T>::rr
 };
 struct CoopPlan {
     const CoopRep* reps; // device table
@@ -450,7 +490,7 @@ constexpr int kCoopMaxCtas = 152;
 long long coop_units(const Rep& R);   // row planes (of x tiles beyond 256 sites)
 int coop_cost(const Rep& R, bool fp64);   // of a row plane
 void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm);   // ncta, runs, per
-CoopRep coop_rep(const Rep& R, int cost, int cost0);   // cost: of a row plane
+CoopRep coop_rep(const Rep& R, bool fp64, int cost, int cost0);   // cost: of a row plane
 template <typename T> int coop_prepare(int kk);   // cudaError_t
 template <typename T> int launch_prop_coop(const Launch& L, const CoopPlan& c, int j0, int j1, int limit);   // cudaError_t
 // mode: 0 exp(-U), 1 trial exp(-(U + a1 d)), 2 commit U += a d then exp(-U), 3 exp(-Uext)

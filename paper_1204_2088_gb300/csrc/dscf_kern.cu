@@ -32,61 +32,61 @@ __device__ __forceinline__ void site_xyz(int i, int nx, int ny, int& x, int& y, 
 // Normalisation of the quadrature (Eq. 2 prefactor):  phi_I = phi_p/(N Q) q_I,
 // phi_S = phi_s exp(-U_S)/<exp(-U_S)>.
 // ---------------------------------------------------------------------------------------------
-// A factor of the model densities in the field precision: two parts for FP32, whose rounded factor alone
-// would shift every density the same way (up to 6e-8 of it, which the inversion turns into a shift of
-// the potentials).
+// A factor of the model densities in two parts of the field precision: one rounded factor alone would shift
+// every density the same way (by up to 6e-8 of it in FP32, 1e-16 in FP64), and the inversion turns that into
+// a shift of the potentials ten times as large.
 template <typename T>
 struct Fac {
     T hi, lo;
-    __device__ __forceinline__ T operator()(T q) const {
-        if constexpr (sizeof(T) == 8) return hi * q;
-        else return fma(hi, q, lo * q);
-    }
+    __device__ __forceinline__ T operator()(T q) const { return fma(hi, q, lo * q); }
+    __device__ __forceinline__ T from(T p, T q) const { return fma(-lo, q, fma(-hi, q, p)); }   // p - f q
 };
+// n V / (a b c), the products' and the quotient's remainders included
 template <typename T>
-__device__ __forceinline__ Fac<T> fac(double v) {
-    const T hi = (T)v;
-    return {hi, (T)(v - (double)hi)};
+__device__ __forceinline__ Fac<T> fac(double n, double V, double a, const Two& b, double c) {
+    const double m = n * V, me = fma(n, V, -m);
+    const double p = a * b.hi, pe = fma(a, b.hi, -p) + a * b.lo, q = p * c, qe = fma(p, c, -q) + pe * c;
+    const double iq = 1.0 / q, v = m * iq;
+    const double r = ((fma(-v, q, m) + me) - v * qe) * iq;
+    const T hi = (T)v, lo = (T)((v - (double)hi) + r);
+    return {hi, isfinite(lo) ? lo : T(0)};   // (no finite factor: hi alone says so)
 }
 template <typename T>
 struct Norm {
     Fac<T> f[2];       // of q_I, of E_S
-    double Q, qs;      // in thread 0 only
+    double Q, qs;      // in thread 0 only, where asked for
 };
-// One thread forms the factors for its block; sh: >= 33 doubles.  net: the learned predictor's output is
-// already normalised.
+// One thread forms a factor for its block; sh: >= 33 doubles.  net: the learned predictor's output is
+// already normalised.  want: Q and qs too (two more divisions in a row).
+// The sweeps apply each pass of the stencil divided by its centre weight, c + r (a + d).  A quadrature has as
+// many Boltzmann factors as G_N, whose weights cancel, and one stencil more, so its factor divides by the
+// stencil's value on the constant field, s1: with r and every pass rounded as in the sweeps, because both
+// chains begin there (G_0 = G+_{N+1} = 1), q holds its rounding twice and Q once.  Only so do the densities
+// keep their means (FP64, with (1 + 2 r)^3 and one rounded factor in its place: off by up to 3e-16).
 template <typename T>
-__device__ __forceinline__ Norm<T> norm_of(const Rep& R, double* sh, int net = 0) {
+__device__ __forceinline__ Norm<T> norm_of(const Rep& R, double* sh, int net = 0, bool want = false) {
     __shared__ Fac<T> f[2];
     Norm<T> n;
     n.Q = 0.0;
     n.qs = 1.0;
-    double qt = 0.0, et = 0.0;
+    Two qt = {0.0, 0.0}, et = {0.0, 0.0};
     if (!net && R.nq > 0) {   // partial sums, no total (the allocation-free path)
-        qt = reduce_parts(slot(R, P_Q), R.nq, sh);
-        if (R.ns == 3) et = reduce_parts(slot(R, P_ES), R.nblk, sh);
+        qt.hi = reduce_parts(slot(R, P_Q), R.nq, sh);
+        if (R.ns == 3) et.hi = reduce_parts(slot(R, P_ES), R.nblk, sh);
+    }
+    const double V = (double)R.V;
+    if (!net && R.nq == 0) {
+        qt = {R.scal[S_QSUM], sizeof(T) == 8 ? R.scal[S_QLO] : 0.0};
+        if (R.ns == 3) et = {R.scal[S_ESS], sizeof(T) == 8 ? R.scal[S_ESLO] : 0.0};
     }
     if (threadIdx.x == 0) {
-        f[0] = {T(1), T(0)};
-        if (!net) {
-            if (R.nq == 0) {
-                qt = R.scal[S_QSUM];
-                et = R.ns == 3 ? R.scal[S_ESS] : 0.0;
-            }
-            // the sweeps apply each pass of the stencil divided by its centre weight, c + r (a + d), and
-            // the Boltzmann factors of the copolymer carry the weight's cube; a quadrature has one stencil
-            // more than Boltzmann factors, so it lacks 1 / (1 + 2 r)^3, with r as rounded in the sweeps:
-            // only so do the densities keep their means (with be^3 instead they are off by up to 4e-8 in
-            // FP32)
-            const double w = 1.0 + 2.0 * (double)(T)(R.alpha / (1.0 - 2.0 * R.alpha));
-            n.Q = qt / (double)R.V;
-            if (R.ns == 3) n.qs = et / (double)R.V;
-            const double coef = R.phi_p / ((double)R.N * n.Q * (w * w * w));
-            f[0] = fac<T>(coef);
-            n.Q = coef > 0.0 ? n.Q : 0.0;
+        f[0] = net ? Fac<T>{T(1), T(0)} : fac<T>(R.phi_p, V, (double)R.N, qt, (double)pars<T>(R).s1);
+        if (!net && want) {
+            n.Q = qt.hi > 0.0 && isfinite(qt.hi) ? qt.hi / V * pars<T>(R).qn : 0.0;
+            if (R.ns == 3) n.qs = et.hi / V;
         }
-        f[1] = fac<T>((1.0 - R.phi_p) / n.qs);
     }
+    if (threadIdx.x == 32 && R.ns == 3) f[1] = fac<T>(1.0 - R.phi_p, V, 1.0, et, 1.0);   // (a predictor has no solvent)
     __syncthreads();
     n.f[0] = f[0];
     n.f[1] = f[1];
@@ -94,9 +94,12 @@ __device__ __forceinline__ Norm<T> norm_of(const Rep& R, double* sh, int net = 0
 }
 // phi_I[U] at one site in the field precision (FP64 only in the normalisation constants).
 template <typename T>
+__device__ __forceinline__ T model_q(const Rep& R, int I, int i) {
+    return I < 2 ? ((const T*)R.q)[(size_t)I * R.V + i] : ((const T*)R.E)[2 * (size_t)R.V + i];
+}
+template <typename T>
 __device__ __forceinline__ T model_phi(const Rep& R, const Norm<T>& n, int I, int i) {
-    if (I < 2) return n.f[0](((const T*)R.q)[(size_t)I * R.V + i]);
-    return n.f[1](((const T*)R.E)[2 * (size_t)R.V + i]);
+    return n.f[I < 2 ? 0 : 1](model_q<T>(R, I, i));
 }
 
 // FP32 fields with V a multiple of 4 are also walked as float4 (4 consecutive sites per thread and
@@ -139,15 +142,15 @@ __global__ void __launch_bounds__(kFlatThreads) k_trial(const Rep* __restrict__ 
                 if (I >= ns) break;
                 const size_t o = (size_t)I * V + i;
                 const float4 p = ld4((const float*)phi + o), dd = ld4((const float*)d + o), q = ld4(src[I] + i);
-                h1 += (T)((p.x - sc[I](q.x)) * dd.x + (p.y - sc[I](q.y)) * dd.y + (p.z - sc[I](q.z)) * dd.z +
-                          (p.w - sc[I](q.w)) * dd.w);
+                h1 += (T)(sc[I].from(p.x, q.x) * dd.x + sc[I].from(p.y, q.y) * dd.y + sc[I].from(p.z, q.z) * dd.z +
+                          sc[I].from(p.w, q.w) * dd.w);
             }
         }
     } else {
         for (int I = 0; I < R.ns; ++I)
             _Pragma("unroll 4") for (int i = i0 + threadIdx.x; i < i1; i += kFlatThreads) {
                 const size_t o = (size_t)I * V + i;
-                h1 += (phi[o] - model_phi<T>(R, n, I, i)) * d[o];
+                h1 += n.f[I < 2 ? 0 : 1].from(phi[o], model_q<T>(R, I, i)) * d[o];
             }
     }
     const T v[1] = {h1};
@@ -168,7 +171,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_grad(const Rep* __restrict__ r
                                                        int k, int net) {
     __shared__ double sh[33];
     FLAT_PROLOGUE
-    const Norm<T> n = norm_of<T>(R, sh, net);
+    const Norm<T> n = norm_of<T>(R, sh, net, lb == 0);
     if (lb == 0 && threadIdx.x == 0 && !net) {
         R.scal[S_Q] = n.Q;
         R.scal[S_QS] = n.qs;

@@ -11,8 +11,8 @@ namespace dscf {
 //   mode 0: U' = U;  mode 1 (trial): U' = U + a1 d with a1 = -<g,d>/<d,phi_m d>;
 //   mode 2 (commit): secant step a = a1 (-h0)/(h1 - h0), U <- U + a d, U' = U;
 //   mode 3: U' = external potential (forward density map alone).
-// The copolymer's factors carry be^3, the centre weight of the stencil (be = 1 - 2 alpha), which the
-// sweeps leave out of their passes.  Also the FP64 partial sums of exp(-U'_S) for the solvent
+// The copolymer's factors carry a weight against the growth of the sweeps' passes, which leave out their
+// centre weights (Par::ew).  Also the FP64 partial sums of exp(-U'_S) for the solvent
 // normalisation.
 template <typename T>
 __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ reps, const int* __restrict__ blk2rep,
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
     T* __restrict__ U = (T*)R.U;
     const T* __restrict__ d = (const T*)R.d;
     T* __restrict__ E = (T*)R.E;
-    const T ta = ta_sh, be3 = pars<T>(R).be3;
+    const T ta = ta_sh, ew = pars<T>(R).ew;
     T es = T(0);
     bool vec = false;
     // (the caller's field may begin at any element: 16-byte accesses only where its blocks are aligned)
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
                                 u.w += fa * dd.w;
                                 if (mode == 2) *(float4*)((float*)U + o) = u;
                             }
-                            const float w = I == 2 ? 1.f : (float)be3;   // the solvent has no stencil
+                            const float w = I == 2 ? 1.f : (float)ew;   // the solvent has no stencil
                             const float4 e =
                                 write_u ? u : make_float4(w * bexp(u.x), w * bexp(u.y), w * bexp(u.z), w * bexp(u.w));
                             *(float4*)((float*)E + o) = e;
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
             } else {
                 u = Uext[R.ext_off + o];
             }
-            const T e = write_u ? u : (I == 2 ? bexp(u) : be3 * bexp(u));   // write_u: the learned predictor takes U' itself
+            const T e = write_u ? u : (I == 2 ? bexp(u) : ew * bexp(u));   // write_u: the learned predictor takes U' itself
             E[o] = e;
             if (I == 2) es += e;
         }
@@ -146,8 +146,18 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
         if (threadIdx.x == 0) slot(R, P_ES)[lb] = t[0];
         __shared__ int fin;
         if (R.nq == 0 && last_block_of(R, &fin)) {   // (nq: the allocation-free path sums in norm_of)
-            const double s = reduce_parts_cg(slot(R, P_ES), R.nblk, sh);
-            if (threadIdx.x == 0) R.scal[S_ESS] = s;
+            if constexpr (sizeof(T) == 8) {
+                if (threadIdx.x < 32) {
+                    const Two s = total_of(slot(R, P_ES), R.nblk);
+                    if (threadIdx.x == 0) {
+                        R.scal[S_ESS] = s.hi;
+                        R.scal[S_ESLO] = s.lo;
+                    }
+                }
+            } else {
+                const double s = reduce_parts_cg(slot(R, P_ES), R.nblk, sh);
+                if (threadIdx.x == 0) R.scal[S_ESS] = s;
+            }
         }
     }
 }

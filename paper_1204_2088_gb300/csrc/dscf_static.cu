@@ -191,7 +191,7 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
         set_thread_error("dscf_densities_static: cudaMemsetAsync failed");
         return DSCF_ERR_CUDA;
     }
-    k_put_rep<<<1, 1, 0, s>>>((Rep*)(base + o_rep), R, (CoopRep*)(base + o_coop), coop_rep(R, 1, 0));
+    k_put_rep<<<1, 1, 0, s>>>((Rep*)(base + o_rep), R, (CoopRep*)(base + o_coop), coop_rep(R, precision == DSCF_FP64, 1, 0));
     if (precision == DSCF_FP64) {
         launch_exp<double>(L, 3, 0, U_in);
         for (int j = 0; j < R.N; ++j) launch_prop_coop<double>(L, plan, j, j + 1, 1);

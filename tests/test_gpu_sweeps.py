@@ -2,6 +2,9 @@
 sweeps, chain lengths around the place where the two chains meet, batches of unlike replicas, and
 ragged blocks of the network's mma.sync kernels.  Tolerances as in test_gpu_parity.py (FP64 1e-12,
 FP32 1e-5 of the largest value) and test_gpu_net_exact.py (exact, or the FP32 accumulation bound)."""
+import itertools
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -172,3 +175,24 @@ def test_potentials_at_any_element_of_an_allocation(shift):
     ctx.status()
     out = [dscf.densities_static(cfg, u, torch.empty_like(U), dscf.FP32) for u in (view, U)]
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("a", [0.6, 1.1543, 1.5, 1.68])
+@pytest.mark.parametrize("grid,ns", [((32, 32, 32), 2), ((30, 31, 33), 2), ((36, 28, 32), 3)], ids=["32", "odd", "solution"])
+def test_densities_keep_their_means(grid, ns, a, precision):
+    """The densities of a chain sum to phi_p whatever the Boltzmann factors.  Per site the sweeps' and the
+    factor's roundings add up to some ulps of either sign, whose mean over 3e4 sites is below a tenth of an
+    ulp; the bound, half an ulp of 1, leaves no room for a factor that is itself off by a rounding."""
+    cfg = dict(melt(grid, 16, 7) if ns == 2 else solution(grid, 16, 7), a=a)
+    U = torch.from_numpy(inputs.random_field(ncomp_shape(cfg), seed=95, scale=0.1))
+    ctx = dscf.Context(cfg, precision, tuning=(8, 1))
+    phi = t2n(ctx.densities(U))
+    ctx.status()
+    ctx.close()
+    V = grid[0] * grid[1] * grid[2]
+    ulp = 2.0 ** (-53 if precision == dscf.FP64 else -24)
+    off = lambda f, mean: math.fsum(itertools.chain(f.ravel(), itertools.repeat(-mean, V))) / V   # one rounding
+    assert abs(off(phi[:2], cfg["phi_p"])) < 0.5 * ulp
+    if ns == 3:
+        assert abs(off(phi[2], 1.0 - cfg["phi_p"])) < 0.5 * ulp
