@@ -40,7 +40,8 @@
 // the row layouts that coop_layout() gives: (sites per lane, mode)
 #define DSCF_COOP_LAYOUTS(X)                                                                                \
     X(1, BLOCKED) X(2, BLOCKED) X(3, BLOCKED) X(4, BLOCKED) X(6, BLOCKED) X(8, BLOCKED) X(1, STRIDED) X(2, STRIDED) \
-    X(3, STRIDED) X(4, STRIDED) X(5, STRIDED) X(6, STRIDED) X(7, STRIDED) X(8, STRIDED) X(8, TILE)
+    X(3, STRIDED) X(4, STRIDED) X(5, STRIDED) X(6, STRIDED) X(7, STRIDED) X(8, STRIDED) X(4, TILE) X(5, TILE) \
+    X(4, BTILE)
 
 namespace dscf {
 
@@ -115,8 +116,13 @@ __device__ __forceinline__ CoopOps<T> coop_ops(const CoopRep& R, int j) {
 //   blocked: lane L holds sites K L .. K L + K - 1 (K divides nx, nx / K <= 32 lanes): vector
 //            accesses, two shuffles for the x pass;
 //   strided: lane L holds sites L, L + 32, ... (any nx <= 256): scalar accesses, 2 K + 2 shuffles;
-//   tile:    like strided, of columns x0 - 1 .. x0 + 254 of which the outer two are halo (nx > 256).
-enum { BLOCKED = 0, STRIDED = 1, TILE = 2 };
+//   tile:    like strided, of columns x0 - 1 .. x0 + tile of which the outer two are neighbours (nx > 256);
+//   btile:   like blocked, the first and the last lane hold the neighbours' sites (nx > 256, 4 | nx).
+// Rows of more than 256 sites, density evaluations of N = 24, us, by the kernels before these (a launch per
+// level), in whole strided tiles of 254 columns (300 columns then cost 512), and in equal tiles:
+//   512 x 128 x 128 FP32 2570, 4713, 1794, FP64 11608, 14301, 7656;  300 x 300 x 100 FP32 2650, 5330, 1921;
+//   1024 x 64 x 64 FP32 1408, 2652, 795;  257 x 40 x 40 FP32 446, 510, 216, FP64 1064, 1156, 652.
+enum { BLOCKED = 0, STRIDED = 1, TILE = 2, BTILE = 3 };
 
 // K values of a lane at p: one access of 16, 8 or 4 bytes each where their size allows.
 template <typename T, int K>
@@ -171,35 +177,42 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
     // its pipe, loses more to the instruction cache in a longer loop than it gains (128^3, N = 64: 4.46 ms
     // unrolled by 6, 4.18 by 2)
     constexpr int RU = sizeof(T) == 8 ? (B <= 16 ? 3 : 2) : B <= 8 ? 6 : B <= 12 ? 4 : B <= 16 || B > 24 ? 3 : 2, D = RU - 1;
-    constexpr int EU = RU == 6 ? 3 : RU > 2 ? RU : B < 48 + 16 * (MODE == BLOCKED) ? 2 : 1, DE = EU > 2 ? 2 : EU - 1;
+    constexpr int EU = RU == 6 ? 3 : RU > 2 ? RU : B < 48 + 16 * (MODE == BLOCKED || MODE == BTILE) ? 2 : 1, DE = EU > 2 ? 2 : EU - 1;
     constexpr int UN = RU;
     constexpr bool SHIFT = UN % 3 != 0;   // the planes of the z pass move by copies
     const int lane = threadIdx.x & 31;
     const int nx = R.nx, ny = R.ny, nz = R.nz;
     const int plane = nx * ny;
     const int dm = (y == 0 ? ny - 1 : -1) * nx, dp = (y == ny - 1 ? 1 - ny : 1) * nx;   // to the y neighbours
+    constexpr bool VEC = MODE == BLOCKED || MODE == BTILE;
+    const int x1 = MODE == TILE || MODE == BTILE ? min(nx, x0 + R.tile) : nx;   // end of the outputs
     // lane's first column, its other columns, which of them exist
-    const int LL = MODE == BLOCKED ? nx / K - 1 : 31;   // blocked: last lane
-    const int xl = MODE == BLOCKED ? K * min(lane, LL) : lane;
+    const int LL = MODE == BLOCKED ? nx / K - 1 : MODE == BTILE ? (x1 - x0) / K + 1 : 31;   // vectors: last lane
+    int xl = VEC ? K * min(lane, LL) : lane;
+    if (MODE == BTILE) {
+        xl += x0 - K;
+        xl = xl < 0 ? xl + nx : (xl >= nx ? xl - nx : xl);
+    }
     auto col = [&](int k) {   // relative to xl
         if (MODE != TILE) return 32 * k;
         int x = x0 - 1 + 32 * k + lane;
         return (x < 0 ? x + nx : (x >= nx ? x - nx : x)) - xl;
     };
     auto there = [&](int k) {   // loads: columns of the row (tile: up to the halo column of a ragged last tile)
-        if (MODE == BLOCKED) return true;
+        if (VEC) return true;
         if (MODE == STRIDED) return k < K - 1 || 32 * (K - 1) + lane < nx;
-        return x0 - 1 + 32 * k + lane <= nx;
+        return x0 - 1 + 32 * k + lane <= x1;
     };
     auto mine = [&](int k) {    // outputs
         if (MODE == BLOCKED) return lane <= LL;
+        if (MODE == BTILE) return lane >= 1 && lane < LL;
         if (MODE == STRIDED) return k < K - 1 || 32 * (K - 1) + lane < nx;
         const int c = 32 * k + lane;
-        return c >= 1 && c <= 32 * K - 2 && x0 - 1 + c < nx;
+        return c >= 1 && x0 - 1 + c < x1;
     };
     auto get = [&](const T* p, T (&v)[K], bool outs) {
-        if constexpr (MODE == BLOCKED) {
-            ldk<T, K>(p, v);
+        if constexpr (VEC) {
+            if (MODE == BLOCKED || !outs || mine(0)) ldk<T, K>(p, v);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k)
@@ -207,8 +220,8 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
         }
     };
     auto put = [&](T* p, const T (&v)[K]) {
-        if constexpr (MODE == BLOCKED) {
-            if (lane <= LL) stk<T, K>(p, v);
+        if constexpr (VEC) {
+            if (mine(0)) stk<T, K>(p, v);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k)
@@ -251,8 +264,8 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
 #pragma unroll
     for (int d = 0; d < D; ++d)
         if (d < last) load(raw[d]);
-    const int lsrc = MODE == BLOCKED ? (lane == 0 ? LL : lane - 1) : ((lane + 31) & 31);
-    const int rsrc = MODE == BLOCKED ? (lane >= LL ? 0 : lane + 1) : ((lane + 1) & 31);
+    const int lsrc = VEC ? (lane == 0 ? LL : lane - 1) : ((lane + 31) & 31);
+    const int rsrc = VEC ? (lane >= LL ? 0 : lane + 1) : ((lane + 1) & 31);
     for (int i0 = 0; i0 < last; i0 += UN) {
 #pragma unroll
         for (int d = 0; d < UN; ++d) {
@@ -265,7 +278,7 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
             T(&uc)[K] = u[SHIFT ? 2 : d % 3];
 #pragma unroll
             for (int k = 0; k < K; ++k) t[k] = fma(rr, raw[d % RU][0][k] + raw[d % RU][2][k], raw[d % RU][1][k]);
-            if constexpr (MODE == BLOCKED) {
+            if constexpr (VEC) {   // (btile: wrong in the outer lanes, whose results are not used)
                 const T lv = __shfl_sync(0xffffffffu, t[K - 1], lsrc), rv = __shfl_sync(0xffffffffu, t[0], rsrc);
 #pragma unroll
                 for (int k = 0; k < K; ++k)
@@ -333,7 +346,7 @@ template <typename T, int K, int MODE>
 __device__ __forceinline__ void coop_run_first(const CoopRep& R, const CoopOps<T>& o, int x0, int y, int za, int n, T rr) {
     const int lane = threadIdx.x & 31, nx = R.nx, plane = nx * R.ny;
     const T t = fma(rr, T(2), T(1)), u = fma(rr, t + t, t), sg = fma(rr, u + u, u);
-    const int xe = MODE == TILE ? min(nx, x0 + 32 * K - 2) : nx;
+    const int xe = MODE == TILE || MODE == BTILE ? min(nx, x0 + R.tile) : nx;
     for (int z = za; z < za + n; ++z)
         for (int x = x0 + lane; x < xe; x += 32) {
             const int i = z * plane + y * nx + x;
@@ -341,16 +354,14 @@ __device__ __forceinline__ void coop_run_first(const CoopRep& R, const CoopOps<T
         }
 }
 
-// Rows of the x tiling: one whole row up to 256 sites, tiles of 254 columns beyond.
-constexpr int kCoopTile = 32 * 8 - 2;
-
 // n planes from za of row y of x tile xt, at level j of chain C.
 template <typename T, int K, int MODE, int C>
 __device__ __forceinline__ void coop_rows(const CoopRep& R, const CoopOps<T>& o, int j, int xt, int y, int za, int n, double& qs) {
     const T rr = (T)R.rr;
-    if (j == 0) coop_run_first<T, K, MODE>(R, o, xt * kCoopTile, y, za, n, rr);
-    else if (o.st) coop_run<T, K, MODE, true>(R, o, xt * kCoopTile, y, za, n, rr, (xt * R.ny + y) * R.nz + za, qs);
-    else coop_run<T, K, MODE, false>(R, o, xt * kCoopTile, y, za, n, rr, 0, qs);
+    const int x0 = xt * R.tile;
+    if (j == 0) coop_run_first<T, K, MODE>(R, o, x0, y, za, n, rr);
+    else if (o.st) coop_run<T, K, MODE, true>(R, o, x0, y, za, n, rr, (xt * R.ny + y) * R.nz + za, qs);
+    else coop_run<T, K, MODE, false>(R, o, x0, y, za, n, rr, 0, qs);
 }
 
 // Planes u0 .. u1 - 1 of the strips (strip-major) of a replica; of strips of 8 rows this warp's row.
@@ -361,7 +372,7 @@ __device__ __forceinline__ void coop_segment(const CoopRep& R, int j, int u0, in
     for (int u = u0; u < u1;) {
         const int g = u / nz, z = u - g * nz, n = min(nz - z, u1 - u);
         const int row = R.strip == 8 ? 8 * g + w : g;
-        const int xt = MODE == TILE ? row / R.ny : 0;
+        const int xt = MODE == TILE || MODE == BTILE ? row / R.ny : 0;
         coop_rows<T, K, MODE, C>(R, o, j, xt, row - xt * R.ny, z, n, qs);
         u += n;
     }
@@ -381,7 +392,7 @@ __device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int ru
             constexpr int MODE = (KK >> 4) - 1;
             double qs = 0.0;
             if (cut.za < cut.ze) {
-                const int xt = MODE == TILE ? cut.row / R.ny : 0;
+                const int xt = MODE == TILE || MODE == BTILE ? cut.row / R.ny : 0;
                 coop_rows<T, (KK & 15), MODE, C>(R, coop_ops<T, C>(R, j), j, xt, cut.row - xt * R.ny, cut.za, cut.ze - cut.za, qs);
             }
             if (C == 0 && j == R.N - 1 && !R.qrow) {   // s = N: this warp's share of Q

@@ -5,12 +5,11 @@
 
 namespace dscf {
 
-long long coop_units(const Rep& R) { return (long long)R.ny * R.nz * (R.nx <= 256 ? 1 : (R.nx + kCoopTile - 1) / kCoopTile); }
+long long coop_units(const Rep& R) { return (long long)R.ny * R.nz * coop_tiles(R.nx); }
 
 // Strips of 8 rows where a field exceeds the L2, so that a CTA's warps share rows at about the same time
 // (256^3, N = 64: 7.93 -> 7.56 ms); in smaller grids sharing gains nothing.
 static int strip_rows(const Rep& R) { return R.V >= (1LL << 23) && R.ny % 8 == 0 && coop_warps(coop_layout(R.nx), false) == 8 ? 8 : 1; }
-static int x_tiles(int nx) { return nx <= 256 ? 1 : (nx + kCoopTile - 1) / kCoopTile; }
 
 // Cut of a launch's work.  One replica whose rows can be cut into equal runs gives every warp one run
 // (runs > 0): a warp of an even cut of all row planes mostly ends one row and begins another, which costs two
@@ -23,7 +22,7 @@ void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm) {
     const int nw = coop_warps(c.kk, fp64), P = nsm * nw;
     c.runs = c.per = 0;
     if (c.nrep == 1) {
-        const long long rows = (long long)x_tiles(R.nx) * R.ny;
+        const long long rows = (long long)coop_tiles(R.nx) * R.ny;
         if (rows <= P) {
             int r = std::min((int)(P / rows), R.nz);
             const int n = (R.nz + r - 1) / r;
@@ -47,10 +46,11 @@ int coop_cost(const Rep& R, bool fp64) { return fp64 ? 1 + 2 * coop_sites(R.nx) 
 CoopRep coop_rep(const Rep& R, bool fp64, int cost, int cost0) {
     CoopRep c = {};
     c.nx = R.nx; c.ny = R.ny; c.nz = R.nz; c.N = R.N; c.nA = R.nA;
-    c.layout = coop_layout(R.nx);
+    c.layout = (short)coop_layout(R.nx);
     c.cost0 = cost0;
     c.units = (int)coop_units(R);
-    c.strip = strip_rows(R);
+    c.tile = coop_tile(R.nx);
+    c.strip = (short)strip_rows(R);
     c.wgt = cost * c.strip;
     c.V = R.V;
     c.E = R.E; c.G = R.G; c.Gp0 = R.Gp0; c.Gp1 = R.Gp1; c.q = R.q;

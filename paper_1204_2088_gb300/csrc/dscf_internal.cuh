@@ -452,12 +452,15 @@ __device__ __forceinline__ float bexp(float x) { return expf(-x); }
 // ---------------------------------------------------------------------------------------------
 // General sweeps of both chains (dscf_coop.cu), levels j0 .. j1 - 1: a cooperative launch for several
 // levels, a plain one for one.  kk: row layout of every replica, 0 if they differ.
-// A replica as the general sweeps see it; their table holds the replicas by decreasing chain length.
+// A replica as the general sweeps see it; their table holds the replicas by decreasing chain length.  (120
+// bytes: with 128 the kernel's table would pass 16 KB of shared memory, whose next size takes 16 KB from the
+// L1 cache; 256^3, N = 64: 7.43 and 7.51 ms.)
 struct CoopRep {
     int nx, ny, nz, N, nA;
-    int layout;          // coop_layout(nx)
+    short layout;        // coop_layout(nx)
+    short strip;         // rows cut together: 8 (a CTA's warps side by side) or 1
     int units;           // row planes
-    int strip;           // rows cut together: 8 (a CTA's warps side by side) or 1
+    int tile;            // sites of an x tile (coop_tile)
     int wgt, cost0;      // cost of a plane of a strip, of all entries before
     long long V;
     void *E, *G, *Gp0, *Gp1, *q;
@@ -465,6 +468,7 @@ struct CoopRep {
     double* qsum;        // where their total goes
     double rr;           // Par<T>::rr
 };
+static_assert(sizeof(CoopRep) <= 120, "the general sweeps' table");
 struct CoopPlan {
     const CoopRep* reps; // device table
     int nrep;
@@ -473,11 +477,25 @@ struct CoopPlan {
     int kk, ncta;
     int runs, per;       // runs > 0: one replica, each row cut into this many, one per warp, `per` in a CTA
 };
-// Row layout of a grid: sites per lane + 16 (1 + mode), mode 0 blocked, 1 strided, 2 tiled.  Blocked
-// where some K of 1, 2, 3, 4, 6, 8 divides nx into at most 32 lanes without leaving more than about
-// a third of them idle.
+// Row layout of a grid: sites per lane + 16 (1 + mode), mode 0 blocked, 1 strided, 2 and 3 the same in x
+// tiles (rows of more than 256 sites).  Blocked for the smallest K of 1, 2, 3, 4, 6, 8 that divides nx into
+// at most 32 lanes, up to one and a half times what 32 full lanes would need.
+constexpr int kCoopRow = 256;   // longest untiled row
+// Tiles of a longer row: of up to 30 groups of 4 sites where they divide it, else of up to 126 or 158 sites
+// (4 or 5 a lane, the fewer lanes in all; 6 a lane lose: 511 x 255 x 63 FP32), two lanes or columns more
+// being the neighbours' on either side (coop_run).
+__host__ __device__ constexpr int coop_tile_k(int nx) {   // sites per lane
+    return nx % 4 == 0 || 4 * ((nx + 125) / 126) <= 5 * ((nx + 157) / 158) ? 4 : 5;
+}
+__host__ __device__ constexpr int coop_tiles(int nx) {
+    return nx <= kCoopRow ? 1 : nx % 4 == 0 ? (nx / 4 + 29) / 30 : coop_tile_k(nx) == 4 ? (nx + 125) / 126 : (nx + 157) / 158;
+}
+__host__ __device__ constexpr int coop_tile(int nx) {   // sites of a tile; the last may have fewer
+    const int t = coop_tiles(nx), u = nx <= kCoopRow || nx % 4 ? 1 : 4;
+    return u * ((nx / u + t - 1) / t);
+}
 __host__ __device__ constexpr int coop_layout(int nx) {
-    if (nx > 256) return 8 + 48;
+    if (nx > kCoopRow) return coop_tile_k(nx) + (nx % 4 == 0 ? 64 : 48);
     const int k = (nx + 31) / 32;
     for (int K = k; K <= 8 && 2 * K <= 3 * k + 1; ++K)
         if (K != 5 && K != 7 && nx % K == 0) return K + 16;

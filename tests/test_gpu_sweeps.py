@@ -40,6 +40,13 @@ def test_general_sweeps_row_layouts(nx, precision):
     check_densities(melt((nx, 3, 5), 5, 2), precision, 20, tuning=(8, 1))
 
 
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("nx", [259, 260, 264, 380, 381, 382, 480, 484, 570, 573, 764, 1000, 1021])
+def test_general_sweeps_tiles_of_long_rows(nx, precision):
+    """Two to nine tiles a row, of equal and of unequal length, either kind; more planes than one."""
+    check_densities(melt((nx, 2, 6), 5, 3), precision, 25, tuning=(8, 1))
+
+
 @pytest.mark.parametrize("N", [2, 3, 4, 5, 8, 9])
 @pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
 def test_general_sweeps_where_the_chains_meet(N, precision):
