@@ -64,13 +64,13 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
     const T* __restrict__ d = (const T*)R.d;
     T* __restrict__ E = (T*)R.E;
     const T ta = ta_sh, ew = pars<T>(R).ew;
-    T es = T(0);
+    double es = 0.0;   // sum of exp(-U_S) of the scalar loop
+    float es4 = 0.f;   // and of the vector loop
     bool vec = false;
     // (the caller's field may begin at any element: 16-byte accesses only where its blocks are aligned)
     if constexpr (sizeof(T) == 4) vec = (V & 3) == 0 && (mode != 3 || ((uintptr_t)(Uext + R.ext_off) & 15) == 0);
     if (vec) {   // FP32, 4 consecutive sites per thread and iteration (16-byte accesses)
         const float fa = (float)ta;
-        float es4 = 0.f;
         const int j0 = (int)i0, j1 = (int)i1;
         constexpr int S = 4 * kFlatThreads;   // sites per block-wide iteration
         // UB iterations of NS species at a time: every load of the batch is issued before the
@@ -118,7 +118,6 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
         };
         if (ns == 2) run(std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{});
         else run(std::integral_constant<int, 3>{}, std::integral_constant<int, 1>{});
-        es += (T)es4;
     }
     for (int I = 0; I < ns && !vec; ++I) {
         for (long long i = i0 + threadIdx.x; i < i1; i += kFlatThreads) {
@@ -136,13 +135,17 @@ __global__ void __launch_bounds__(kFlatThreads) k_exp(const Rep* __restrict__ re
             }
             const T e = write_u ? u : (I == 2 ? bexp(u) : ew * bexp(u));   // write_u: the learned predictor takes U' itself
             E[o] = e;
-            if (I == 2) es += e;
+            if (I == 2) es += (double)e;
         }
     }
     if (ns == 3) {
-        const T v[1] = {es};
-        double t[1];
-        block_total<1>(v, sh, t);
+        double t[1] = {es};
+        if (vec) {
+            const float v[1] = {es4};
+            block_total<1>(v, sh, t);
+        } else {
+            block_sum_n<1>(t, sh);
+        }
         if (threadIdx.x == 0) slot(R, P_ES)[lb] = t[0];
         __shared__ int fin;
         if (R.nq == 0 && last_block_of(R, &fin)) {   // (nq: the allocation-free path sums in norm_of)

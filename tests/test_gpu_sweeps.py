@@ -203,3 +203,16 @@ def test_densities_keep_their_means(grid, ns, a, precision):
     assert abs(off(phi[:2], cfg["phi_p"])) < 0.5 * ulp
     if ns == 3:
         assert abs(off(phi[2], 1.0 - cfg["phi_p"])) < 0.5 * ulp
+
+
+@pytest.mark.parametrize("grid", [(127, 127, 127), (33, 17, 9)], ids=["14 a thread", "1 a thread"])
+def test_solvent_sum_keeps_every_term(grid):
+    """Site counts that no vector access divides are summed in FP64, term by term: the mean of V equal
+    FP32 factors is that factor."""
+    cfg = solution(grid, 2, 1)
+    ctx = dscf.Context(cfg, dscf.FP32, tuning=(8, 1))
+    ctx.set(dscf.U, torch.full(ncomp_shape(cfg), 0.37))
+    ctx.observables()               # evaluates the densities at U
+    qs = ctx.diagnostics()["QS"]
+    assert abs(qs - math.exp(-0.37)) < 1e-6
+    assert abs(qs - float(np.float32(qs))) < 1e-12 * qs
