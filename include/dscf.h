@@ -262,18 +262,20 @@ int dscf_set_inversion_tol(dscf_ctx* ctx, double tol);
  * re-captures the step graph.  DSCF_ERR_ARG for another mode. */
 int dscf_set_warm_start(dscf_ctx* ctx, int32_t mode);
 
-/* Failure detection of the persistent sweeps.  Every wait of a persistent sweep on a
- * neighbouring brick is bounded by `polls` polls (default 4194304, several seconds; each poll is
- * an acquire load of the neighbour's step counter followed by a short sleep).  A CTA that runs out
- * sets the status bit and a global abort flag; every other CTA then stops waiting, all launches
+/* Failure detection of the contour sweeps.  Every wait of a sweep, on a neighbouring brick or at the
+ * general sweeps' barrier between contour steps, is bounded by `polls` polls (default 4194304, several
+ * seconds; each poll is an acquire load of a counter followed by a short sleep, and the bound is looked at
+ * every 32 polls, some tens of microseconds: a wait may need as long as one CTA can fall behind
+ * another, so a bound of less than about 2000 polls can end sweeps that nothing holds up).  A CTA that
+ * runs out sets the status bit and a global abort flag; every other CTA then stops waiting, all launches
  * finish, and dscf_status reports DSCF_ERR_TIMEOUT.  That call also re-arms the step counters, so
  * the context stays usable once the caller has restored its fields (they are invalid after a
  * timeout).  dscf_set_wait_limit synchronises and re-captures the step graph.
- * dscf_inject_lag (test hook, host side: one 4-byte copy) sets brick `brick`'s step counter far
- * behind the others, so that during the next persistent sweep its neighbours wait for values it
- * never publishes and run out of polls.  Bricks are numbered replica by replica (in the order
- * of the replicas), y fastest, then z.  DSCF_ERR_STATE unless the context uses persistent sweeps
- * (kfuse 0), DSCF_ERR_ARG for a brick outside 0 .. bricks-1 (all replicas) or polls < 1. */
+ * dscf_inject_lag (test hook, host side: one 4-byte copy) sets a counter far behind, so that the next
+ * sweep runs out of polls.  Brick sweeps: brick `brick`'s step counter, whose neighbours then wait for
+ * values it never publishes (bricks are numbered replica by replica, in the order of the replicas, y
+ * fastest, then z).  General sweeps: the barrier counter of chain `brick`, 0 forward, 1 backward.
+ * DSCF_ERR_ARG for a brick outside 0 .. bricks-1 (all replicas), another chain, or polls < 1. */
 int dscf_set_wait_limit(dscf_ctx* ctx, int32_t polls);
 int dscf_inject_lag(dscf_ctx* ctx, int32_t brick);
 

@@ -1247,15 +1247,14 @@ int dscf_set_wait_limit(dscf_ctx* c, int32_t polls) {
 
 int dscf_inject_lag(dscf_ctx* c, int32_t brick) {
     if (!c) return DSCF_ERR_ARG;
-    if (!c->bricks) return fail(c, DSCF_ERR_STATE, "the context does not run persistent sweeps");
-    const int nb = pers_total_bricks(c);
-    if (brick < 0 || brick >= nb) return fail(c, DSCF_ERR_ARG, "brick index out of range");
+    if (brick < 0 || brick >= (c->bricks ? pers_total_bricks(c) : 2)) return fail(c, DSCF_ERR_ARG, "brick or chain index out of range");
     if (int rc = set_dev(c)) return rc;
-    // a counter far behind the others: the brick's neighbours wait for step values it never
-    // publishes during the next sweep, the brick itself sees its neighbours ahead and runs through
+    // A counter far behind the others.  Bricks: the brick's neighbours wait for step values it never
+    // publishes during the next sweep, the brick itself sees its neighbours ahead and runs through.
+    // General sweeps: the chain's barrier never reaches its count.
     const int lag = -(1 << 24);
-    cudaError_t e = cudaMemcpyAsync(c->d_status + kFlagBase + (size_t)brick * kFlagStride, &lag, sizeof(int),
-                                    cudaMemcpyHostToDevice, c->stream);
+    const size_t at = c->bricks ? kFlagBase + (size_t)brick * kFlagStride : kCoopBase + (size_t)brick * kFlagStride;
+    cudaError_t e = cudaMemcpyAsync(c->d_status + at, &lag, sizeof(int), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     return cuda_check(c, e, "inject lag");
 }

@@ -354,11 +354,12 @@ class Context:
         self._net = net
 
     def set_wait_limit(self, polls):
-        """Polls a persistent sweep spends on a neighbour before it reports DSCF_ERR_TIMEOUT."""
+        """Polls a contour sweep spends on one wait before it reports DSCF_ERR_TIMEOUT."""
         self._check(self.lib.dscf_set_wait_limit(self.h, int(polls)))
 
     def inject_lag(self, brick):
-        """Test hook: make brick's step counter lag so the next persistent sweep times out."""
+        """Test hook: make a counter lag so that the next sweep times out, of a brick or, in a context on
+        the general sweeps, of chain 0 (forward) or 1 (backward)."""
         self._check(self.lib.dscf_inject_lag(self.h, int(brick)))
 
     def set_noise(self, omega, lb_noise=True, seed=0):

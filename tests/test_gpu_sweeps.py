@@ -216,3 +216,43 @@ def test_solvent_sum_keeps_every_term(grid):
     qs = ctx.diagnostics()["QS"]
     assert abs(qs - math.exp(-0.37)) < 1e-6
     assert abs(qs - float(np.float32(qs))) < 1e-12 * qs
+
+
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("batch", [False, True], ids=["solo", "batch"])
+@pytest.mark.parametrize("chain", [0, 1])
+def test_general_sweeps_timeout_is_reported_and_the_context_recovers(chain, batch, precision):
+    """Failure detection without a GPU fault: a chain's barrier counter is set far behind (host side), so
+    no CTA ever sees the barrier complete; the bounded waits run out, the launch finishes, the host reads
+    DSCF_ERR_TIMEOUT, and the counters are as before the launch."""
+    cfgs = [melt((40, 30, 20), 9, 4), solution((33, 12, 10), 6, 3)] if batch else [melt((40, 30, 20), 9, 4)]
+    U = np.concatenate([inputs.random_field(ncomp_shape(c), seed=97 + i, scale=0.5).ravel() for i, c in enumerate(cfgs)])
+    ctx = dscf.Context(cfgs, precision, tuning=(8, 1))
+    U = torch.from_numpy(U).to(ctx.dtype).cuda()
+    good = ctx.densities(U)
+    ctx.status()
+    ctx.set_wait_limit(2000)
+    ctx.inject_lag(chain)
+    ctx.densities(U)
+    with pytest.raises(dscf.DSCFError) as err:
+        ctx.status()
+    assert err.value.code == -4
+    ctx.status()                    # re-armed by the call that reported the timeout
+    for _ in range(2):
+        assert torch.equal(ctx.densities(U), good)
+    ctx.status()
+    with pytest.raises(dscf.DSCFError):
+        ctx.inject_lag(2)
+
+
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+def test_general_sweeps_of_more_replicas_than_the_shared_table(precision):
+    """130 replicas: the kernel reads its table from global memory.  Equal chains and two row layouts."""
+    cfgs = [melt((6 + 27 * (i % 2), 5, 4), 3 + i % 3, 1 + i % 2) for i in range(130)]
+    U = [inputs.random_field(ncomp_shape(c), seed=200 + i, scale=0.5) for i, c in enumerate(cfgs)]
+    ref = np.concatenate([oracle.densities(c, u)[0].ravel() for c, u in zip(cfgs, U)])
+    ctx = dscf.Context(cfgs, precision)
+    for _ in range(2):
+        got = t2n(ctx.densities(torch.from_numpy(np.concatenate([u.ravel() for u in U]))))
+        ctx.status()
+        assert rel(got, ref) < (1e-12 if precision == dscf.FP64 else 1e-5)
