@@ -219,7 +219,8 @@ int64_t dscf_launches_per_step(const dscf_ctx* ctx);
  * warps, or of nx x 8 x 8 (nx x 16 x 8) on 8, one CTA per SM; nz a multiple of the brick depth; at
  * most one brick of 16 planes, or two of 8, of a replica per SM; replicas share cooperative launches
  * while their bricks fit the SMs together, so a batch takes a few launches per density evaluation;
- * a context whose shallow bricks do not run together, one per SM, takes the general sweeps).  With
+ * a context with more bricks of 8 planes than SMs takes bricks of 16, the uppermost of 8 where 16 does not
+ * divide nz, and the general sweeps if these do not run together either).  With
  * kfuse = 0, zc = 16 or 8 selects the brick depth (DSCF_ERR_ARG if the grids do not allow it),
  * any other zc keeps the current depth.  Synchronises the stream; the
  * next dscf_step re-captures its graph.  Results do not depend on either value beyond rounding. */

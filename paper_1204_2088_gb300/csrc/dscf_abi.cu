@@ -235,8 +235,9 @@ struct dscf_ctx {
     cudaGraphExec_t exec_pred = nullptr;
     int kfuse = 1;          // as chosen or asked for: 0 persistent brick sweeps, 1..4 general sweeps
     bool bricks = false;    // the brick sweeps run (kfuse 0, and all bricks of a replica fit the SMs together)
-    int pers_bz = 0;        // brick depth of the persistent sweeps (0 = not available)
-    int pers_nw = 16;       // warps per CTA of the persistent sweeps
+    int pers_bz = 0;        // brick depth asked for or chosen (0 = no bricks)
+    int run_bz = 0;         // brick depth that runs, on as many warps (pers_fit)
+    bool run_rag = false;   // the uppermost bricks may have 8 planes of its 16
     struct PersGroup { int width, pby, first, nbricks; };   // one cooperative launch
     std::vector<PersGroup> pgroups;                    // brick table entries [first, first + nbricks)
     int wait_limit = kPersSpinLimit;   // polls before a persistent sweep gives up on a neighbour
@@ -293,7 +294,7 @@ int* pers_flags(dscf_ctx* c) { return c->d_status + kFlagBase; }
 int4* pers_table(dscf_ctx* c) { return (int4*)(c->d_status + kFlagBase + (size_t)kMaxBricks * kFlagStride); }
 int pers_total_bricks(const dscf_ctx* c) {
     int t = 0;
-    for (const Rep& R : c->L.reps) t += pers_bricks(R, c->pers_bz);
+    for (const Rep& R : c->L.reps) t += pers_bricks(R, c->run_bz);
     return t;
 }
 
@@ -303,7 +304,7 @@ int pers_total_bricks(const dscf_ctx* c) {
 // (which lasts as long as its longest chain) mostly holds chains of equal length.  A launch whose
 // replicas share one row width and brick height runs that width's kernel, any other the
 // mixed-width kernel (rows of 32 to 96 sites; 128-wide replicas share launches only with each
-// other).  Each brick's step counter is at its replica's flag base (the replicas'
+// other, and so does every width where uppermost bricks have 8 planes).  Each brick's step counter is at its replica's flag base (the replicas'
 // bricks in index order).
 // Placement: the CTAs of a sweep-shaped cooperative launch land on SMs in a fixed pattern that
 // scatters consecutive CTA indices over the GPCs (and both dies); within a launch the bricks are
@@ -312,7 +313,7 @@ int pers_total_bricks(const dscf_ctx* c) {
 // GPCs.  The table is a permutation: correctness does not depend on the placement repeating.
 int place_bricks(dscf_ctx* c) {
     c->pgroups.clear();
-    const int n = c->nrep, bz = c->pers_bz;
+    const int n = c->nrep, bz = c->run_bz;
     const int cap = std::min(c->nsm, kMaxBricks);
     std::vector<int> fbase(n), nbr(n), order(n);
     int tot = 0;
@@ -331,10 +332,13 @@ int place_bricks(dscf_ctx* c) {
     });
     std::vector<std::vector<int>> bins;
     std::vector<int> load;
-    auto wide = [&](int r) { return c->L.reps[r].nx == 128; };   // 128-wide replicas share launches only with each other
+    auto apart = [&](int a, int b) {
+        const Rep &A = c->L.reps[a], &B = c->L.reps[b];
+        return c->run_rag ? A.nx != B.nx || pers_pby(A) != pers_pby(B) : (A.nx == 128) != (B.nx == 128);
+    };
     for (int r : order) {
         size_t k = 0;
-        while (k < bins.size() && (load[k] + nbr[r] > cap || wide(bins[k][0]) != wide(r))) ++k;
+        while (k < bins.size() && (load[k] + nbr[r] > cap || apart(bins[k][0], r))) ++k;
         if (k == bins.size()) { bins.emplace_back(); load.push_back(0); }
         bins[k].push_back(r);
         load[k] += nbr[r];
@@ -352,7 +356,7 @@ int place_bricks(dscf_ctx* c) {
         }
         const int nb = (int)ent.size();
         std::vector<int> smid(nb), ord(nb);
-        int rc = cuda_check(c, (cudaError_t)pers_placement(bz, c->pers_nw, nb, d_smid, c->stream), "placement probe");
+        int rc = cuda_check(c, (cudaError_t)pers_placement(bz, bz, nb, d_smid, c->stream), "placement probe");
         if (!rc) rc = cuda_check(c, cudaMemcpyAsync(smid.data(), d_smid, sizeof(int) * nb, cudaMemcpyDeviceToHost, c->stream),
                                  "placement probe");
         if (!rc) rc = cuda_check(c, cudaStreamSynchronize(c->stream), "placement probe");
@@ -373,7 +377,7 @@ int place_bricks(dscf_ctx* c) {
 // The persistent sweeps of every replica, both chains: one cooperative launch per group.
 int64_t launch_pers_sweeps(dscf_ctx* c, const Launch& L, int limit) {
     for (const auto& g : c->pgroups)
-        launch_prop_pers(L, g.width, g.pby, c->pers_bz, c->pers_nw, g.nbricks, pers_table(c) + g.first,
+        launch_prop_pers(L, g.width, g.pby, c->run_bz, c->run_bz, c->run_rag, g.nbricks, pers_table(c) + g.first,
                          pers_flags(c), c->d_status + 2, limit);
     return (int64_t)c->pgroups.size();
 }
@@ -638,31 +642,37 @@ bool pers_all_supported(const dscf_ctx* c, int bz, int nw) {
     return tot <= kMaxBricks;
 }
 
-// Every replica's bricks at the context's depth run together, one per SM.
-bool pers_fit(const dscf_ctx* c) {
+// The bricks that run for a depth of bz: those, if every replica's run together, one per SM; else (8 planes)
+// bricks of 16, the uppermost of 8 planes where 16 does not divide nz; else none.  128^3, N = 48: 16 planes
+// 327 us, the general sweeps 564; 64 x 256 x 136: 359 and 691; 32 x 256 x 120: 239 and 572.
+bool pers_fit(dscf_ctx* c, int bz) {
+    for (int b = bz; b <= 16; b += 8) {
+        bool fit = true, rag = false;
+        for (const Rep& R : c->L.reps) {
+            fit = fit && pers_bricks(R, b) <= c->nsm;
+            rag = rag || R.nz % b;
+        }
+        if (!fit) continue;
+        c->run_bz = b;
+        c->run_rag = rag;
+        return true;
+    }
+    return false;
+}
+// Their kernels' attributes.
+int pers_ready(dscf_ctx* c, int bz, bool rag) {
     for (const Rep& R : c->L.reps)
-        if (pers_bricks(R, c->pers_bz) > c->nsm) return false;
-    return true;
+        if (int rc = cuda_check(c, (cudaError_t)pers_prepare(R.nx, pers_pby(R), bz, bz, rag), "persistent sweep set-up"))
+            return rc;
+    return rag ? DSCF_OK : cuda_check(c, (cudaError_t)pers_prepare(0, 0, bz, bz, false), "persistent sweep set-up");
 }
 
-int pers_select(dscf_ctx* c, std::vector<std::pair<int, int>>& pcand) {
-    c->pers_bz = 0;
+// Brick depths that can be asked for; the first becomes the context's.
+void pers_select(dscf_ctx* c, std::vector<int>& pcand) {
     pcand.clear();
-    if (pers_all_supported(c, 16, 16)) pcand.push_back({16, 16});
-    if (pers_all_supported(c, 8, 8)) pcand.push_back({8, 8});
-    for (auto& pc : pcand) {
-        for (const Rep& R : c->L.reps)
-            if (int rc = cuda_check(c, (cudaError_t)pers_prepare(R.nx, pers_pby(R), pc.first, pc.second),
-                                    "persistent sweep set-up"))
-                return rc;
-        if (int rc = cuda_check(c, (cudaError_t)pers_prepare(0, 0, pc.first, pc.second), "persistent sweep set-up"))
-            return rc;
-    }
-    if (!pcand.empty()) {
-        c->pers_bz = pcand[0].first;
-        c->pers_nw = pcand[0].second;
-    }
-    return DSCF_OK;
+    for (int bz : {16, 8})
+        if (pers_all_supported(c, bz, bz)) pcand.push_back(bz);
+    c->pers_bz = pcand.empty() ? 0 : pcand[0];
 }
 
 // Grids for which contour fusion can be asked for (kfuse 2..4).  Those kernels are gone (the general
@@ -684,8 +694,8 @@ bool fusable(const dscf_ctx* c, int kfuse) {
 int autotune_zc(dscf_ctx* c) {
     long long Vtot = 0;
     for (const Rep& R : c->L.reps) Vtot += R.V;
-    std::vector<std::pair<int, int>> pcand;
-    if (int rc = pers_select(c, pcand)) return rc;
+    std::vector<int> pcand;
+    pers_select(c, pcand);
     c->kfuse = 1;
     c->bricks = false;
     if (Vtot >= 32 * 32 * 32 && !pcand.empty()) {
@@ -707,23 +717,23 @@ int autotune_zc(dscf_ctx* c) {
         };
         const float t = sweep_ms();
         float tp = 1e30f;
-        std::pair<int, int> pbest = pcand[0];
-        for (auto& pc : pcand) {   // the first candidate (bricks of 16 planes) unless another is 2% faster
-            c->pers_bz = pc.first;
-            c->pers_nw = pc.second;
-            if (!pers_fit(c)) continue;
-            int rc = reset_pers_flags(c);
+        int pbest = pcand[0], last = 0;
+        for (int bz : pcand) {   // the first candidate (bricks of 16 planes) unless another is 2% faster
+            if (!pers_fit(c, bz) || c->run_bz == last) continue;   // (8 planes may stand for 16)
+            last = c->run_bz;
+            int rc = pers_ready(c, c->run_bz, c->run_rag);
+            if (!rc) rc = reset_pers_flags(c);
             if (!rc) rc = place_bricks(c);
             if (rc) return leave(rc);
             c->bricks = true;
             const float ti = sweep_ms();
-            if (ti < (tp < 1e29f ? 0.98f * tp : tp)) { tp = ti; pbest = pc; }
+            if (ti < (tp < 1e29f ? 0.98f * tp : tp)) { tp = ti; pbest = bz; }
         }
-        c->pers_bz = pbest.first;
-        c->pers_nw = pbest.second;
+        c->pers_bz = pbest;
         c->bricks = tp < t;
         if (c->bricks) {
             c->kfuse = 0;
+            pers_fit(c, pbest);
             int rc = reset_pers_flags(c);
             if (!rc) rc = place_bricks(c);
             if (rc) return leave(rc);
@@ -738,8 +748,8 @@ int autotune_zc(dscf_ctx* c) {
 }
 // A tuning chosen earlier (for instance cached from an autotuner run) instead of the autotuner.
 int apply_tuning(dscf_ctx* c, int zc, int kfuse) {
-    std::vector<std::pair<int, int>> pcand;
-    if (int rc = pers_select(c, pcand)) return rc;
+    std::vector<int> pcand;
+    pers_select(c, pcand);
     if (int rc = dscf_set_tuning(c, zc, kfuse)) return rc;
     return DSCF_OK;
 }
@@ -1330,10 +1340,9 @@ int dscf_set_tuning(dscf_ctx* c, int32_t zc, int32_t kfuse) {
         return fail(c, DSCF_ERR_ARG,
                     "persistent sweeps need FP32 replicas with nx in {32, 48, 64, 96, 128}, ny %% 8 = 0 and nz a "
                     "multiple of the brick depth (16, or 8), and all bricks co-resident");
-    int pbz = c->pers_bz, pnw = c->pers_nw;
+    int pbz = c->pers_bz;
     if (kfuse == 0 && (zc == 8 || zc == 16)) {   // brick depth requested
-        if (zc == 16 && pers_all_supported(c, 16, 16)) { pbz = 16; pnw = 16; }
-        else if (zc == 8 && pers_all_supported(c, 8, 8)) { pbz = 8; pnw = 8; }
+        if (pers_all_supported(c, zc, zc)) pbz = zc;
         else return fail(c, DSCF_ERR_ARG, "no persistent sweep with bricks of %d planes for these grids", zc);
     }
     for (const Rep& R : c->L.reps)
@@ -1350,13 +1359,9 @@ int dscf_set_tuning(dscf_ctx* c, int32_t zc, int32_t kfuse) {
     }
     c->bricks = false;
     if (kfuse == 0) {
-        for (const Rep& R : c->L.reps)
-            if (int rc = cuda_check(c, (cudaError_t)pers_prepare(R.nx, pers_pby(R), pbz, pnw), "persistent sweep set-up"))
-                return rc;
-        if (int rc = cuda_check(c, (cudaError_t)pers_prepare(0, 0, pbz, pnw), "persistent sweep set-up")) return rc;
         c->pers_bz = pbz;
-        c->pers_nw = pnw;
-        if (pers_fit(c)) {   // otherwise the general sweeps
+        if (pers_fit(c, pbz)) {   // otherwise the general sweeps
+            if (int rc = pers_ready(c, c->run_bz, c->run_rag)) return rc;
             if (int rc = reset_pers_flags(c)) return rc;
             if (int rc = place_bricks(c)) return rc;
             c->bricks = true;

@@ -556,11 +556,11 @@ size_t pers_smem_bytes(int width, int pby, int bz);
 size_t pers_mix_smem_bytes(int bz);                            // the mixed-width launches (width 0)
 bool pers_width_ok(int nx);
 int pers_pby(const Rep& R);                                    // brick rows of a replica (8 or 16)
-bool pers_supported(const Rep& R, int bz, int nw, int nsm);   // nw: warps per CTA (16, or 8 with 2 CTAs per SM)
-int pers_bricks(const Rep& R, int bz);
-int pers_prepare(int width, int pby, int bz, int nw);   // cudaError_t; width 0: the mixed-width kernel
-// width 0: bricks of several widths in one launch (bricks of 16 planes)
-int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, int nbricks, const int4* table,
+bool pers_supported(const Rep& R, int bz, int nw, int nsm);   // nw: warps per CTA
+int pers_bricks(const Rep& R, int bz);   // the uppermost may have fewer planes
+// width 0: bricks of several widths in one launch; rag (16 planes, one width): fewer planes in the uppermost
+int pers_prepare(int width, int pby, int bz, int nw, bool rag);   // cudaError_t
+int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, bool rag, int nbricks, const int4* table,
                      int* flags, int* abortf, int limit);  // cudaError_t
 // SM id of each CTA of a sweep-shaped cooperative launch (cudaError_t)
 int pers_placement(int bz, int nw, int nbricks, int* d_smid, cudaStream_t stream);

@@ -11,7 +11,7 @@
 // levels near the middle are read back while still in L2), but a chain's halo exchange (release,
 // neighbours' counters, copies: L2 round trips of 5 to 6 thousand cycles) runs while the SM
 // computes the other chain's unit.  128^3, N = 64: 540 us for the two sweeps one after the other
-// (4.2 us a contour step, the exchange in the open), 345 us so (2.7 us).
+// (4.2 us a contour step, the exchange in the open), 362 us so (2.8 us).
 //
 // The lattice is cut into bricks of nx x PBY x BZ sites, one brick per CTA and one CTA per SM (the
 // launch is cooperative, so all CTAs are resident together), one compute warp per plane of the
@@ -40,8 +40,8 @@
 // sweep: the registers let one CTA of 16 compute warps (all 512 columns) or one of 8 (256) on an
 // SM, whatever context or stream they belong to.
 // Each 1-D pass of the separable stencil is one add and one fma per site, as packed f32x2 pairs
-// (a scalar tail for three sites per lane), with the centre weight folded into the Boltzmann
-// factors.  Every wait is bounded: on timeout the CTA sets a status bit and a global abort flag
+// (a scalar tail for three sites per lane), with the centre weight left out and made up for by the
+// Boltzmann factors.  Every wait is bounded: on timeout the CTA sets a status bit and a global abort flag
 // that makes every other CTA stop waiting, so the launch always finishes.
 #include "dscf_internal.cuh"
 
@@ -285,6 +285,8 @@ struct PersWarp {
     size_t own;            // lane's first site of its first row in a field
     size_t slab;           // lane's 128-byte line of the plane's run in a field (past its end: none)
     int N, nA, hm, w, lane, hf, xo, lsrc, rsrc;
+    int planes;            // of the brick
+    bool act;              // the warp has one of them
     bool face_plane;
     float rr;
     unsigned long long rr2;
@@ -336,7 +338,7 @@ __device__ __forceinline__ int halo_row(int r, int pl) {
 }
 
 // One unit: contour step j of chain C (0 forward, s = j + 1; 1 backward, s = N - j).
-template <int W, int PBY, int BZ, int NW, int C>
+template <int W, int PBY, int BZ, int NW, bool RAG, int C>
 __device__ __forceinline__ void pers_unit(PersWarp& k, float (&xf)[PRow<W, PBY>::RPL][PRow<W, PBY>::VEC], const int j) {
     using RG = PRow<W, PBY>;
     constexpr int VEC = RG::VEC, LPR = RG::LPR, RPL = RG::RPL;
@@ -347,6 +349,8 @@ __device__ __forceinline__ void pers_unit(PersWarp& k, float (&xf)[PRow<W, PBY>:
     const unsigned long long rr2 = k.rr2;
     float* ysl = k.YS + (w * PBY + k.hf * RPL) * W + xo;   // plane w - 1 (YS holds planes -1..BZ)
     const float* hs = k.HS + C * NH * W + xo;
+    const bool act = !RAG || k.act;
+    const int top = RAG ? k.planes : BZ;   // planes of the brick
     const int s = C ? N - j : j + 1;
     const int sp = s <= k.nA ? 0 : 1;
     const bool acc = C ? j >= N - hm : j >= hm;
@@ -385,7 +389,7 @@ __device__ __forceinline__ void pers_unit(PersWarp& k, float (&xf)[PRow<W, PBY>:
         ldv<VEC>(hs + halo_row<PBY, BZ>(r + 1, pl) * W, d);
         mixv<VEC>(a, c, d, rr, rr2, m);
         xpassv<VEC>(k, m, o);
-        stv<VEC>(k.YS + ((pl + 1) * PBY + r) * W + xo, o);
+        stv<VEC>(k.YS + ((side ? top + 1 : 0) * PBY + r) * W + xo, o);
     }
     {
         float* yw = ysl + PBY * W;
@@ -404,7 +408,7 @@ __device__ __forceinline__ void pers_unit(PersWarp& k, float (&xf)[PRow<W, PBY>:
                 prev[i] = cur[i];
                 xf[p][i] = yv[i];   // xf now holds the y-filtered rows
             }
-            stv<VEC>(yw + p * W, yv);
+            if (act) stv<VEC>(yw + p * W, yv);   // (an idle warp's place may be the upper halo plane's)
         }
     }
     compute_sync(32 * NW);
@@ -445,8 +449,8 @@ __device__ __forceinline__ void pers_unit(PersWarp& k, float (&xf)[PRow<W, PBY>:
             for (int i = 0; i < VEC; ++i) q2[p & 1][i] = q[i];
             tm_st<VS>(ta + p * VS, q2[p & 1]);
         }
-        if (edge_row(p) && !last) stg<VEC>(dst + p * W, out);
-        if (C == 0 && last) {
+        if (edge_row(p) && !last && act) stg<VEC>(dst + p * W, out);
+        if (C == 0 && last && act) {
             float t = out[0] + out[1];
             if constexpr (VEC == 3) t = t + out[2];
             if constexpr (VEC == 4) t = t + (out[2] + out[3]);
@@ -461,14 +465,14 @@ __device__ __forceinline__ void pers_unit(PersWarp& k, float (&xf)[PRow<W, PBY>:
     if (!acc) {
 #pragma unroll
         for (int p = 0; p < RPL; ++p)
-            if (!edge_row(p)) stg<VEC>(dst + p * W, xf[p]);
+            if (!edge_row(p) && act) stg<VEC>(dst + p * W, xf[p]);
     }
     // The next unit's stack level (the other chain's), if that unit accumulates: every thread copies
     // the values of its own sites, which it stored itself, and brings the line that the chain after
     // it takes next into L2 meanwhile.
     {
         const int jn = C ? j + 1 : j;
-        if ((C ? jn >= hm : jn >= N - hm) && jn < N) {
+        if ((C ? jn >= hm : jn >= N - hm) && jn < N && act) {
             const float* src = k.A.stack + (size_t)(C ? jn : N - jn - 1) * k.A.V;
 #pragma unroll
             for (int p = 0; p < RPL; ++p) cpv<VEC>(k.GS + p * W, src + k.own + p * W);
@@ -499,7 +503,13 @@ size_t pers_smem_bytes(int width, int pby, int bz) {
 // 6000 cycles): the shared-memory pipe (y-filtered rows written once and read twice, halo and stack
 // rows, shuffles: about 2500 cycles of it before the middle and 3700 past it) and the latencies
 // between the barriers.
-template <int W, int PBY, int BZ, int NW>
+//
+// RAG: the planes need not be a multiple of BZ; the uppermost bricks then have the remainder (a multiple of
+// 8), and the warps beyond it only take part in the halo planes and the barriers.  For grids with more
+// bricks of 8 planes than SMs, two of which do not fit one (the tensor memory).  Density evaluations, N = 48,
+// two bricks per SM (the kernels before these), the general sweeps, and so: 128 x 128 x 136 527, 573 and 342 us;
+// 64 x 256 x 136 520, 691, 359; 32 x 256 x 120 407, 572, 239; 96 x 128 x 120 475, 486, 367.
+template <int W, int PBY, int BZ, int NW, bool RAG>
 __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const PersCtl& ctl) {
     static_assert(NW == BZ, "one warp per plane");
     using RG = PRow<W, PBY>;
@@ -523,9 +533,10 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
     const int ny = R.ny, nz = R.nz, N = R.N, nA = R.nA;
     const int plane = W * ny;
     const size_t V = (size_t)R.V;
-    const int nby = ny / PBY, nbz = nz / BZ;
+    const int nby = ny / PBY, nbz = RAG ? (nz + BZ - 1) / BZ : nz / BZ;
     const int by = b % nby, bz = b / nby;
     const int y0 = by * PBY, z0 = bz * BZ;
+    const int planes = RAG ? min(BZ, nz - z0) : BZ;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int* fown = ctl.flags + (size_t)(tb.z + tb.y) * kFlagStride;   // own step counters: +0 forward, +kFlagChain
     if (threadIdx.x < 8) {
@@ -570,7 +581,7 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
         const int lr = lane / CH, lc = 4 * (lane - lr * CH);
         float* hdst = HS + (c * NH + part * (NH / 2) + lr) * W + lc;
         const int yrow = (part ? (y0 + PBY == ny ? 0 : y0 + PBY) : (y0 == 0 ? ny - 1 : y0 - 1)) * W + lc;
-        const int zpl = (part ? (z0 + BZ == nz ? 0 : z0 + BZ) : (z0 == 0 ? nz - 1 : z0 - 1)) * plane + y0 * W + lc;
+        const int zpl = (part ? (z0 + planes == nz ? 0 : z0 + planes) : (z0 == 0 ? nz - 1 : z0 - 1)) * plane + y0 * W + lc;
         for (int j = 0; j < N; ++j) {
             bar_wait(&pub[c], (unsigned)(j & 1), ctl, dead);
             // pub orders every warp's boundary stores before this release store, and release is
@@ -602,9 +613,10 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
             if (lr < RPI) {
 #pragma unroll 3
                 for (int i0 = 0; i0 < BZ + 2; i0 += RPI) {   // row -1 (PBY) of planes -1..BZ
-                    const int i = i0 + lr;
-                    int z = z0 - 1 + i;
+                    const int i = i0 + lr;                  // (slot BZ + 1: the plane above the brick)
+                    int z = RAG && i == BZ + 1 ? z0 + planes : z0 - 1 + i;
                     z = z < 0 ? z + nz : (z >= nz ? z - nz : z);
+                    if (RAG && i > planes && i <= BZ) continue;
                     if ((BZ + 2) % RPI == 0 || i < BZ + 2) cp16(hdst + i0 * W, src + z * plane + yrow);
                 }
 #pragma unroll 2
@@ -621,15 +633,14 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
         const int seg = lane - li;
         const int lsrc = seg + ((li + LPR - 1) & (LPR - 1)), rsrc = seg + ((li + 1) & (LPR - 1));
         // Each 1-D pass is applied as c + r (a + d) with r = alpha / (1 - 2 alpha), i.e. the
-        // stencil's pass divided by its centre weight be = 1 - 2 alpha; the three passes then give
-        // sigma / be^3; the Boltzmann factors carry be^3, the normalisation gives it back to q.
-        const double be_d = 1.0 - 2.0 * R.alpha;
-        const float rr = (float)(R.alpha / be_d);
+        // stencil's pass divided by its centre weight; the Boltzmann factors carry a weight against the
+        // growth (Par::ew), and the normalisation takes both into account.
+        const float rr = R.pf.rr;
         // own plane never wraps: (row r, plane w) is own0 + r * W
         const size_t own0 = (size_t)(z0 + w) * plane + (size_t)(y0 + hf * RPL) * W + xo;
         PersWarp k = {arr, ctl, full, pub, YS, HS, GS + (w * PBY + hf * RPL) * W + xo, own0,
                       (size_t)(z0 + w) * plane + (size_t)y0 * W + 32 * lane,
-                      N, nA, (N + 1) / 2, w, lane, hf, xo, lsrc, rsrc, w == 0 || w == BZ - 1, rr, pk2(rr, rr),
+                      N, nA, (N + 1) / 2, w, lane, hf, xo, lsrc, rsrc, planes, w < planes, w == 0 || w == planes - 1, rr, pk2(rr, rr),
                       tmem_slot + ((unsigned)((w & 3) * 32) << 16) + (unsigned)((w >> 2) * 128), 0.f, false};
         const unsigned tbase = k.tbase;
 
@@ -639,8 +650,8 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
             const float* E = (const float*)R.E + (size_t)I * V;
 #pragma unroll
             for (int p = 0; p < RPL; ++p) {
-                float t[VS], zero[VS], e[VEC];
-                ldv<VEC>(E + own0 + (size_t)p * W, e);
+                float t[VS], zero[VS], e[VEC] = {};
+                if (!RAG || k.act) ldv<VEC>(E + own0 + (size_t)p * W, e);
 #pragma unroll
                 for (int i = 0; i < VS; ++i) {
                     t[i] = i < VEC ? e[i < VEC ? i : 0] : 0.f;
@@ -661,8 +672,8 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
 
 #pragma unroll 1
         for (int j = 0; j < N; ++j) {
-            pers_unit<W, PBY, BZ, NW, 0>(k, xF, j);
-            pers_unit<W, PBY, BZ, NW, 1>(k, xB, j);
+            pers_unit<W, PBY, BZ, NW, RAG, 0>(k, xF, j);
+            pers_unit<W, PBY, BZ, NW, RAG, 1>(k, xB, j);
         }
         // both quadratures
 #pragma unroll
@@ -675,7 +686,7 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
                 tm_wait_ld<VS>(t);
 #pragma unroll
                 for (int i = 0; i < VEC; ++i) o[i] = t[i];
-                stv<VEC>(q + own0 + (size_t)p * W, o);
+                if (!RAG || k.act) stv<VEC>(q + own0 + (size_t)p * W, o);
             }
         }
         // the brick's share of Q, the end of the tensor memory's use (compute warps only: the
@@ -707,9 +718,9 @@ __device__ __forceinline__ void pers_sweep(const Rep* __restrict__ reps, const P
     }
 }
 
-template <int W, int PBY, int BZ, int NW>
+template <int W, int PBY, int BZ, int NW, bool RAG = false>
 __global__ void __launch_bounds__(32 * (NW + kXWarps), 1) k_prop_pers(const Rep* __restrict__ reps, PersCtl ctl) {
-    pers_sweep<W, PBY, BZ, NW>(reps, ctl);
+    pers_sweep<W, PBY, BZ, NW, RAG>(reps, ctl);
 }
 
 // Bricks of several row widths (32 to 96 sites) in one launch (batches): each CTA runs the sweep of
@@ -720,13 +731,13 @@ __global__ void __launch_bounds__(32 * (NW + kXWarps), 1) k_prop_pers_mix(const 
     const Rep& R = reps[ctl.table[blockIdx.x].x];
     const int pby = pers_pby_of(R.nx, R.ny);
     switch (R.nx * 32 + pby) {
-        case 32 * 32 + 8: pers_sweep<32, 8, BZ, NW>(reps, ctl); break;
-        case 32 * 32 + 16: pers_sweep<32, 16, BZ, NW>(reps, ctl); break;
-        case 48 * 32 + 8: pers_sweep<48, 8, BZ, NW>(reps, ctl); break;
-        case 48 * 32 + 16: pers_sweep<48, 16, BZ, NW>(reps, ctl); break;
-        case 64 * 32 + 8: pers_sweep<64, 8, BZ, NW>(reps, ctl); break;
-        case 64 * 32 + 16: pers_sweep<64, 16, BZ, NW>(reps, ctl); break;
-        case 96 * 32 + 8: pers_sweep<96, 8, BZ, NW>(reps, ctl); break;
+        case 32 * 32 + 8: pers_sweep<32, 8, BZ, NW, false>(reps, ctl); break;
+        case 32 * 32 + 16: pers_sweep<32, 16, BZ, NW, false>(reps, ctl); break;
+        case 48 * 32 + 8: pers_sweep<48, 8, BZ, NW, false>(reps, ctl); break;
+        case 48 * 32 + 16: pers_sweep<48, 16, BZ, NW, false>(reps, ctl); break;
+        case 64 * 32 + 8: pers_sweep<64, 8, BZ, NW, false>(reps, ctl); break;
+        case 64 * 32 + 16: pers_sweep<64, 16, BZ, NW, false>(reps, ctl); break;
+        case 96 * 32 + 8: pers_sweep<96, 8, BZ, NW, false>(reps, ctl); break;
         default: break;   // not reached: the host builds mixed launches of these widths only
     }
 }
@@ -745,7 +756,8 @@ size_t pers_mix_smem_bytes(int bz) {
 }
 
 // Brick depths: 16 planes on 16 warps or 8 planes on 8 warps.  (Grids of up to two shallow bricks per SM
-// are accepted; more than one do not run together, and such grids take the general sweeps.)
+// are accepted; more than one do not run together, and such grids take bricks of 16 planes, the uppermost
+// of 8 where 16 does not divide nz, or the general sweeps.)
 bool pers_supported(const Rep& R, int bz, int nw, int nsm) {
     if (!pers_width_ok(R.nx) || R.ny % 8 || R.nz % bz) return false;
     if (!((bz == 16 && nw == 16) || (bz == 8 && nw == 8))) return false;   // one warp per plane
@@ -753,7 +765,7 @@ bool pers_supported(const Rep& R, int bz, int nw, int nsm) {
     return nb >= 1 && nb <= nsm * (nw == 8 ? 2 : 1);   // all bricks co-resident
 }
 
-int pers_bricks(const Rep& R, int bz) { return (R.ny / pers_pby(R)) * (R.nz / bz); }
+int pers_bricks(const Rep& R, int bz) { return (R.ny / pers_pby(R)) * ((R.nz + bz - 1) / bz); }
 
 namespace {
 // Also checks that the registers the kernel launches with cover the shares its warps take
@@ -769,9 +781,9 @@ cudaError_t pers_attr_of(K kernel, size_t smem) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     return e;
 }
-template <int W, int PBY, int BZ, int NW>
+template <int W, int PBY, int BZ, int NW, bool RAG = false>
 cudaError_t pers_attr() {
-    return pers_attr_of<NW>(k_prop_pers<W, PBY, BZ, NW>, pers_smem_bytes(W, PBY, BZ));
+    return pers_attr_of<NW>(k_prop_pers<W, PBY, BZ, NW, RAG>, pers_smem_bytes(W, PBY, BZ));
 }
 template <int BZ, int NW>
 cudaError_t pers_mix_attr() {
@@ -793,10 +805,13 @@ cudaError_t pers_mix_attr() {
         default: break;                                          \
     }
 
-int pers_prepare(int width, int pby, int bz, int nw) {
+int pers_prepare(int width, int pby, int bz, int nw, bool rag) {
     cudaError_t e = cudaErrorInvalidValue;
 #define DSCF_PERS_ATTR(WW, PP, BB, NN) e = pers_attr<WW, PP, BB, NN>()
-    if (bz == 16 && nw == 16) {
+#define DSCF_PERS_ATTR_RAG(WW, PP, BB, NN) e = pers_attr<WW, PP, BB, NN, true>()
+    if (rag) {
+        DSCF_PERS_SWITCH(16, 16, DSCF_PERS_ATTR_RAG)
+    } else if (bz == 16 && nw == 16) {
         if (width == 0) e = pers_mix_attr<16, 16>();
         else DSCF_PERS_SWITCH(16, 16, DSCF_PERS_ATTR)
     } else if (bz == 8 && nw == 8) {
@@ -804,6 +819,7 @@ int pers_prepare(int width, int pby, int bz, int nw) {
         else DSCF_PERS_SWITCH(8, 8, DSCF_PERS_ATTR)
     }
 #undef DSCF_PERS_ATTR
+#undef DSCF_PERS_ATTR_RAG
     return (int)e;
 }
 
@@ -843,7 +859,7 @@ int pers_placement(int bz, int nw, int nbricks, int* d_smid, cudaStream_t stream
     return (int)e;
 }
 
-int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, int nbricks, const int4* table,
+int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, bool rag, int nbricks, const int4* table,
                      int* flags, int* abortf, int limit) {
     PersCtl ctl;
     ctl.flags = flags;
@@ -863,7 +879,10 @@ int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, int nb
     cfg.numAttrs = 1;
     cudaError_t e = cudaErrorInvalidValue;
 #define DSCF_PERS_LAUNCH(WW, PP, BB, NN) e = cudaLaunchKernelEx(&cfg, k_prop_pers<WW, PP, BB, NN>, L.reps, ctl)
-    if (bz == 16 && nw == 16) {
+#define DSCF_PERS_LAUNCH_RAG(WW, PP, BB, NN) e = cudaLaunchKernelEx(&cfg, k_prop_pers<WW, PP, BB, NN, true>, L.reps, ctl)
+    if (rag) {
+        DSCF_PERS_SWITCH(16, 16, DSCF_PERS_LAUNCH_RAG)
+    } else if (bz == 16 && nw == 16) {
         if (width == 0) e = cudaLaunchKernelEx(&cfg, k_prop_pers_mix<16, 16>, L.reps, ctl);
         else DSCF_PERS_SWITCH(16, 16, DSCF_PERS_LAUNCH)
     } else if (bz == 8 && nw == 8) {
@@ -871,6 +890,7 @@ int launch_prop_pers(const Launch& L, int width, int pby, int bz, int nw, int nb
         else DSCF_PERS_SWITCH(8, 8, DSCF_PERS_LAUNCH)
     }
 #undef DSCF_PERS_LAUNCH
+#undef DSCF_PERS_LAUNCH_RAG
     return (int)e;
 }
 #undef DSCF_PERS_SWITCH

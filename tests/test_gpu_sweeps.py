@@ -256,3 +256,38 @@ def test_general_sweeps_of_more_replicas_than_the_shared_table(precision):
         got = t2n(ctx.densities(torch.from_numpy(np.concatenate([u.ravel() for u in U]))))
         ctx.status()
         assert rel(got, ref) < (1e-12 if precision == dscf.FP64 else 1e-5)
+
+
+@pytest.mark.parametrize("grid", [(32, 256, 120), (64, 256, 136), (128, 128, 136), (96, 128, 120), (48, 128, 168), (64, 72, 136)],
+                         ids=lambda g: "x".join(map(str, g)))
+def test_bricks_of_eight_planes_beyond_the_sms(grid):
+    """More bricks of 8 planes than SMs and nz an odd multiple of 8: bricks of 16, the uppermost of 8; the
+    halo rows of every brick against the oracle, and the same bits every time."""
+    for N, nA in ((2, 1), (5, 3)):
+        cfg = melt(grid, N, nA)
+        U = inputs.random_field(ncomp_shape(cfg), seed=98, scale=0.5)
+        ref, _, _ = oracle.densities(cfg, U)
+        ctx = dscf.Context(cfg, dscf.FP32, tuning=(8, 0))
+        U = torch.from_numpy(U).float().cuda()
+        first = ctx.densities(U)
+        ctx.status()
+        assert rel(t2n(first), ref) < 1e-5
+        for _ in range(10):
+            assert torch.equal(ctx.densities(U), first)
+        ctx.status()
+        ctx.close()
+
+
+def test_bricks_of_eight_planes_beyond_the_sms_in_a_batch():
+    """Replicas of several widths, heights and depths: each as alone."""
+    cfgs = [melt((64, 256, 136), 4, 2), melt((48, 128, 24), 5, 2), melt((64, 64, 40), 4, 1), solution((128, 16, 16), 6, 3)]
+    U = [torch.from_numpy(inputs.random_field(ncomp_shape(c), seed=300 + i, scale=0.5)).float().cuda() for i, c in enumerate(cfgs)]
+    ctx = dscf.Context(cfgs, dscf.FP32, tuning=(8, 0))
+    got = t2n(ctx.densities(torch.cat([u.reshape(-1) for u in U])))
+    ctx.status()
+    off = 0
+    for c, u in zip(cfgs, U):
+        solo = dscf.Context(c, dscf.FP32, tuning=(8, 0))
+        assert rel(got[off:off + u.numel()], t2n(solo.densities(u)).ravel()) < 1e-6
+        off += u.numel()
+        solo.close()
