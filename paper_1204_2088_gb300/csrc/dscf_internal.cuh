@@ -137,7 +137,10 @@ template <typename T>
 inline void set_par(const Rep& R, Par<T>& p) {
     const double be = 1.0 - 2.0 * R.alpha;
     p.al = (T)R.alpha; p.be = (T)be;
-    p.rr = (T)(R.alpha / be);
+    // (FP32: 1 - 2 alpha no smaller than 2^-25, a change of alpha below its own rounding, so that a level grows
+    // by at most 2^75 within the passes; alpha may be as close to 1/2 as FP64 holds it, and (1 / be)^3 then
+    // passes 1e38)
+    p.rr = (T)(R.alpha / (sizeof(T) == 4 && be < 0x1p-25 ? 0x1p-25 : be));
     // The passes leave out their centre weights, so a level grows by w3 = (1 + 2 rr)^3 and the factors carry
     // a weight against it.  Any weight will do (it cancels in the densities); a power of two adds no
     // rounding to the factors, which are the same at every bead of a block: with 1 / w3 the potentials of a

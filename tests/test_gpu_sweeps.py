@@ -291,3 +291,13 @@ def test_bricks_of_eight_planes_beyond_the_sms_in_a_batch():
         assert rel(got[off:off + u.numel()], t2n(solo.densities(u)).ravel()) < 1e-6
         off += u.numel()
         solo.close()
+
+
+@pytest.mark.parametrize("short", [1e-15, 1e-13, 1e-11, 1e-8, 1e-4])
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+def test_segments_up_to_the_longest(short, precision):
+    """alpha = a^2 / 6 just below 1/2, where the stencil's centre weight vanishes."""
+    a = math.sqrt(3.0) * (1.0 - short)
+    for cfg, tunings in ((melt((34, 7, 6), 6, 2), [(8, 1)]), (melt((32, 16, 16), 70, 30), [(8, 1), (16, 0)])):
+        for tuning in tunings[:1 if precision == dscf.FP64 else 2]:
+            check_densities(dict(cfg, a=a), precision, 99, tuning=tuning)
