@@ -104,10 +104,10 @@ void assign_tiles(Layout& L, const dscf_params* p, int n, int prec) {
     }
     L.coop.clear();
     L.work = 0;
-    L.kk = coop_layout(L.reps[0].nx);
+    L.kk = coop_layout(L.reps[0].nx, L.reps[0].V, prec == DSCF_FP64);
     // costs in 32 bits: not weighted where they would not fit
     long long all = 0;
-    for (const Rep& R : L.reps) all += coop_units(R) * coop_cost(R, prec == DSCF_FP64);
+    for (const Rep& R : L.reps) all += coop_units(R, prec == DSCF_FP64) * coop_cost(R, prec == DSCF_FP64);
     int cost = 0;
     for (int k = 0; k < n; ++k) {
         const Rep& R = L.reps[order[k]];
@@ -137,7 +137,7 @@ Layout make_layout(const dscf_params* p, int n, int prec, char* base) {
         tile_replica(R);
         max_blk_total += R.nblk;
         R.part_stride = std::max(R.nblk, R.lb_nblk);
-        R.nq_units = (int)coop_units(R);
+        R.nq_units = (int)coop_units(R, prec == DSCF_FP64);
         R.part_stride = std::max(R.part_stride, (R.nq_units + 31) / 32);
         R.hydro = q.hydro;
         R.cn_sweeps = q.cn_sweeps;

@@ -31,7 +31,8 @@
 // Every wait is bounded as in dscf_pers.cu: a CTA that runs out sets the status bit and the abort flag
 // and waits no more; arrivals do not depend on waits, so the launch always finishes and leaves its
 // counters at zero.
-// Included by dscf_coop32.cu and dscf_coop64.cu, one per precision (they compile in parallel).
+// Included by dscf_coop32.cu and dscf_coop64.cu, one per precision, and by dscf_coop32m.cu and dscf_coop64m.cu
+// for the kernels that hold every row layout (they compile in parallel).
 #pragma once
 #include "dscf_internal.cuh"
 
@@ -42,6 +43,7 @@
     X(1, BLOCKED) X(2, BLOCKED) X(3, BLOCKED) X(4, BLOCKED) X(6, BLOCKED) X(8, BLOCKED) X(1, STRIDED) X(2, STRIDED) \
     X(3, STRIDED) X(4, STRIDED) X(5, STRIDED) X(6, STRIDED) X(7, STRIDED) X(8, STRIDED) X(4, TILE) X(5, TILE) \
     X(4, BTILE)
+#define DSCF_COOP_LAYOUTS32(X) X(2, ROWS) X(4, ROWS)   // in FP32 only
 
 namespace dscf {
 
@@ -122,7 +124,8 @@ __device__ __forceinline__ CoopOps<T> coop_ops(const CoopRep& R, int j) {
 // level), in whole strided tiles of 254 columns (300 columns then cost 512), and in equal tiles:
 //   512 x 128 x 128 FP32 2570, 4713, 1794, FP64 11608, 14301, 7656;  300 x 300 x 100 FP32 2650, 5330, 1921;
 //   1024 x 64 x 64 FP32 1408, 2652, 795;  257 x 40 x 40 FP32 446, 510, 216, FP64 1064, 1156, 652.
-enum { BLOCKED = 0, STRIDED = 1, TILE = 2, BTILE = 3 };
+//   rows:    blocked, several adjacent rows side by side (nx <= 32, large FP32 fields).
+enum { BLOCKED = 0, STRIDED = 1, TILE = 2, BTILE = 3, ROWS = 4 };
 
 // K values of a lane at p: one access of 16, 8 or 4 bytes each where their size allows.
 template <typename T, int K>
@@ -183,12 +186,18 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
     const int lane = threadIdx.x & 31;
     const int nx = R.nx, ny = R.ny, nz = R.nz;
     const int plane = nx * ny;
+    constexpr bool VEC = MODE == BLOCKED || MODE == BTILE || MODE == ROWS;
+    // rows: this lane's row of the group (y), its place there; lanes past the group or past the last row idle
+    const int lr = nx / K, grp = MODE == ROWS ? min(lane / lr, R.tile - 1) : 0, seg = grp * lr;
+    const int yl = MODE == ROWS ? y * R.tile + grp : y;
+    const bool on = MODE != ROWS || (yl < ny && lane < R.tile * lr);
+    y = MODE == ROWS ? min(yl, ny - 1) : y;
     const int dm = (y == 0 ? ny - 1 : -1) * nx, dp = (y == ny - 1 ? 1 - ny : 1) * nx;   // to the y neighbours
-    constexpr bool VEC = MODE == BLOCKED || MODE == BTILE;
     const int x1 = MODE == TILE || MODE == BTILE ? min(nx, x0 + R.tile) : nx;   // end of the outputs
     // lane's first column, its other columns, which of them exist
-    const int LL = MODE == BLOCKED ? nx / K - 1 : MODE == BTILE ? (x1 - x0) / K + 1 : 31;   // vectors: last lane
-    int xl = VEC ? K * min(lane, LL) : lane;
+    const int LL = MODE == BLOCKED || MODE == ROWS ? lr - 1 : MODE == BTILE ? (x1 - x0) / K + 1 : 31;   // vectors: last lane
+    const int li = min(lane - seg, LL);   // (only of VEC)
+    int xl = VEC ? K * li : lane;
     if (MODE == BTILE) {
         xl += x0 - K;
         xl = xl < 0 ? xl + nx : (xl >= nx ? xl - nx : xl);
@@ -205,6 +214,7 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
     };
     auto mine = [&](int k) {    // outputs
         if (MODE == BLOCKED) return lane <= LL;
+        if (MODE == ROWS) return on;
         if (MODE == BTILE) return lane >= 1 && lane < LL;
         if (MODE == STRIDED) return k < K - 1 || 32 * (K - 1) + lane < nx;
         const int c = 32 * k + lane;
@@ -212,7 +222,7 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
     };
     auto get = [&](const T* p, T (&v)[K], bool outs) {
         if constexpr (VEC) {
-            if (MODE == BLOCKED || !outs || mine(0)) ldk<T, K>(p, v);
+            if (MODE != BTILE || !outs || mine(0)) ldk<T, K>(p, v);
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k)
@@ -264,8 +274,8 @@ __device__ __forceinline__ void coop_run(const CoopRep& R, const CoopOps<T>& o, 
 #pragma unroll
     for (int d = 0; d < D; ++d)
         if (d < last) load(raw[d]);
-    const int lsrc = VEC ? (lane == 0 ? LL : lane - 1) : ((lane + 31) & 31);
-    const int rsrc = VEC ? (lane >= LL ? 0 : lane + 1) : ((lane + 1) & 31);
+    const int lsrc = VEC ? seg + (li == 0 ? LL : li - 1) : ((lane + 31) & 31);
+    const int rsrc = VEC ? seg + (li >= LL ? 0 : li + 1) : ((lane + 1) & 31);
     for (int i0 = 0; i0 < last; i0 += UN) {
 #pragma unroll
         for (int d = 0; d < UN; ++d) {
@@ -346,7 +356,8 @@ template <typename T, int K, int MODE>
 __device__ __forceinline__ void coop_run_first(const CoopRep& R, const CoopOps<T>& o, int x0, int y, int za, int n, T rr) {
     const int lane = threadIdx.x & 31, nx = R.nx, plane = nx * R.ny;
     const T t = fma(rr, T(2), T(1)), u = fma(rr, t + t, t), sg = fma(rr, u + u, u);
-    const int xe = MODE == TILE || MODE == BTILE ? min(nx, x0 + R.tile) : nx;
+    const int xe = MODE == TILE || MODE == BTILE ? min(nx, x0 + R.tile) : MODE == ROWS ? min(R.tile, R.ny - y * R.tile) * nx : nx;
+    if (MODE == ROWS) y *= R.tile;   // (adjacent rows: one run of sites)
     for (int z = za; z < za + n; ++z)
         for (int x = x0 + lane; x < xe; x += 32) {
             const int i = z * plane + y * nx + x;
@@ -358,7 +369,7 @@ __device__ __forceinline__ void coop_run_first(const CoopRep& R, const CoopOps<T
 template <typename T, int K, int MODE, int C>
 __device__ __forceinline__ void coop_rows(const CoopRep& R, const CoopOps<T>& o, int j, int xt, int y, int za, int n, double& qs) {
     const T rr = (T)R.rr;
-    const int x0 = xt * R.tile;
+    const int x0 = MODE == ROWS ? 0 : xt * R.tile;
     if (j == 0) coop_run_first<T, K, MODE>(R, o, x0, y, za, n, rr);
     else if (o.st) coop_run<T, K, MODE, true>(R, o, x0, y, za, n, rr, (xt * R.ny + y) * R.nz + za, qs);
     else coop_run<T, K, MODE, false>(R, o, x0, y, za, n, rr, 0, qs);
@@ -420,6 +431,10 @@ __device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int ru
 #define DSCF_COOP_CASE(KV, MV) case KV + 16 * (MV + 1): coop_segment<T, KV, MV, C>(R, j, u0, u1, w, qs); break;
             switch (lay) {
                 DSCF_COOP_LAYOUTS(DSCF_COOP_CASE)
+                default: break;
+            }
+            if constexpr (sizeof(T) == 4) switch (lay) {
+                DSCF_COOP_LAYOUTS32(DSCF_COOP_CASE)
                 default: break;
             }
 #undef DSCF_COOP_CASE
@@ -630,9 +645,13 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
 template <typename T>
 const void* coop_kernel(int kk) {
 #define DSCF_COOP_KERNEL(KV, MV) case KV + 16 * (MV + 1): return (const void*)k_prop_coop<T, KV + 16 * (MV + 1)>;
+    if constexpr (sizeof(T) == 4) switch (kk) {
+        DSCF_COOP_LAYOUTS32(DSCF_COOP_KERNEL)
+        default: break;
+    }
     switch (kk) {
         DSCF_COOP_LAYOUTS(DSCF_COOP_KERNEL)
-        default: return (const void*)k_prop_coop<T, 0>;
+        default: return coop_mixed<T>();
     }
 #undef DSCF_COOP_KERNEL
 }

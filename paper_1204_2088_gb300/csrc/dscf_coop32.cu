@@ -5,11 +5,16 @@
 
 namespace dscf {
 
-long long coop_units(const Rep& R) { return (long long)R.ny * R.nz * coop_tiles(R.nx); }
+static int layout_of(const Rep& R, bool fp64) { return coop_layout(R.nx, R.V, fp64); }
+static long long rows_of(const Rep& R, bool fp64) {
+    const int g = coop_group(R.nx, R.V, fp64);
+    return (long long)coop_tiles(R.nx) * ((R.ny + g - 1) / g);
+}
+long long coop_units(const Rep& R, bool fp64) { return rows_of(R, fp64) * R.nz; }
 
 // Strips of 8 rows where a field exceeds the L2, so that a CTA's warps share rows at about the same time
 // (256^3, N = 64: 7.93 -> 7.56 ms); in smaller grids sharing gains nothing.
-static int strip_rows(const Rep& R) { return R.V >= (1LL << 23) && R.ny % 8 == 0 && coop_warps(coop_layout(R.nx), false) == 8 ? 8 : 1; }
+static int strip_rows(const Rep& R) { return R.V >= (1LL << 23) && R.ny % 8 == 0 && coop_warps(layout_of(R, false), false) == 8 ? 8 : 1; }
 
 // Cut of a launch's work.  One replica whose rows can be cut into equal runs gives every warp one run
 // (runs > 0): a warp of an even cut of all row planes mostly ends one row and begins another, which costs two
@@ -22,7 +27,7 @@ void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm) {
     const int nw = coop_warps(c.kk, fp64), P = nsm * nw;
     c.runs = c.per = 0;
     if (c.nrep == 1) {
-        const long long rows = (long long)coop_tiles(R.nx) * R.ny;
+        const long long rows = rows_of(R, fp64);
         if (rows <= P) {
             int r = std::min((int)(P / rows), R.nz);
             const int n = (R.nz + r - 1) / r;
@@ -41,15 +46,15 @@ void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm) {
 }
 
 // a row plane's time: FP32 mostly the latency of its loads, FP64 mostly its operations
-int coop_cost(const Rep& R, bool fp64) { return fp64 ? 1 + 2 * coop_sites(R.nx) : 4 + coop_sites(R.nx); }
+int coop_cost(const Rep& R, bool fp64) { return fp64 ? 1 + 2 * (layout_of(R, true) & 15) : 4 + (layout_of(R, false) & 15); }
 
 CoopRep coop_rep(const Rep& R, bool fp64, int cost, int cost0) {
     CoopRep c = {};
     c.nx = R.nx; c.ny = R.ny; c.nz = R.nz; c.N = R.N; c.nA = R.nA;
-    c.layout = (short)coop_layout(R.nx);
+    c.layout = (short)layout_of(R, fp64);
     c.cost0 = cost0;
-    c.units = (int)coop_units(R);
-    c.tile = coop_tile(R.nx);
+    c.units = (int)coop_units(R, fp64);
+    c.tile = coop_narrow(R.nx, R.V, fp64) ? coop_group(R.nx, R.V, fp64) : coop_tile(R.nx);
     c.strip = (short)strip_rows(R);
     c.wgt = cost * c.strip;
     c.V = R.V;

@@ -453,17 +453,17 @@ __device__ __forceinline__ float bexp(float x) { return expf(-x); }
 // ---------------------------------------------------------------------------------------------
 // Host launchers (defined in the kernel translation units, explicit per precision).
 // ---------------------------------------------------------------------------------------------
-// General sweeps of both chains (dscf_coop.cu), levels j0 .. j1 - 1: a cooperative launch for several
+// General sweeps of both chains (dscf_coop.cuh), levels j0 .. j1 - 1: a cooperative launch for several
 // levels, a plain one for one.  kk: row layout of every replica, 0 if they differ.
 // A replica as the general sweeps see it; their table holds the replicas by decreasing chain length.  (120
 // bytes: with 128 the kernel's table would pass 16 KB of shared memory, whose next size takes 16 KB from the
 // L1 cache; 256^3, N = 64: 7.43 and 7.51 ms.)
 struct CoopRep {
     int nx, ny, nz, N, nA;
-    short layout;        // coop_layout(nx)
+    short layout;        // coop_layout
     short strip;         // rows cut together: 8 (a CTA's warps side by side) or 1
     int units;           // row planes
-    int tile;            // sites of an x tile (coop_tile)
+    int tile;            // sites of an x tile (coop_tile); mode 4: rows of a group
     int wgt, cost0;      // cost of a plane of a strip, of all entries before
     long long V;
     void *E, *G, *Gp0, *Gp1, *q;
@@ -497,21 +497,34 @@ __host__ __device__ constexpr int coop_tile(int nx) {   // sites of a tile; the 
     const int t = coop_tiles(nx), u = nx <= kCoopRow || nx % 4 ? 1 : 4;
     return u * ((nx / u + t - 1) / t);
 }
-__host__ __device__ constexpr int coop_layout(int nx) {
+// Short rows of FP32 fields that hold many of them: a warp takes as many adjacent rows as its lanes hold, with
+// 4 or 2 sites a lane, mode 4.  One row a warp has a quarter of the bytes in flight or less; small fields,
+// whose rows are to fill all warps, take one, and FP64, bound by its pipe.  Density evaluations, N = 24, us, one
+// row a warp and groups: 16^3 100, 110; 32^3 103, 110; 32 x 64 x 64 122, 119; 24 x 100 x 100 160, 136; 16 x 128 x
+// 128 198, 131; 32 x 512 x 512 2662, 1541 (a launch per level, before these sweeps: 2433); 24 x 600 x 600 3636,
+// 1667 (3087); 8 x 1000 x 1000 8365, 1498 (7384).
+__host__ __device__ constexpr bool coop_narrow(int nx, long long V, bool fp64) {
+    return !fp64 && nx <= 32 && nx % 2 == 0 && V >= (1LL << 17);
+}
+__host__ __device__ constexpr int coop_group(int nx, long long V, bool fp64) {   // rows of a warp
+    return coop_narrow(nx, V, fp64) ? 32 / (nx / (nx % 4 == 0 ? 4 : 2)) : 1;
+}
+__host__ __device__ constexpr int coop_layout(int nx, long long V, bool fp64) {
+    if (coop_narrow(nx, V, fp64)) return (nx % 4 == 0 ? 4 : 2) + 80;
     if (nx > kCoopRow) return coop_tile_k(nx) + (nx % 4 == 0 ? 64 : 48);
     const int k = (nx + 31) / 32;
     for (int K = k; K <= 8 && 2 * K <= 3 * k + 1; ++K)
         if (K != 5 && K != 7 && nx % K == 0) return K + 16;
     return k + 32;
 }
-__host__ __device__ constexpr int coop_sites(int nx) { return coop_layout(nx) & 15; }
 // Compute warps of a CTA of the general sweeps (kk: the row layout of all replicas, or 0).
 __host__ __device__ constexpr int coop_warps(int kk, bool fp64) { return kk > 0 && (kk & 15) * (fp64 ? 8 : 4) <= (fp64 ? 16 : 24) ? 12 : 8; }
 constexpr int kCoopMaxCtas = 152;
-long long coop_units(const Rep& R);   // row planes (of x tiles beyond 256 sites)
+long long coop_units(const Rep& R, bool fp64);   // planes of rows, of x tiles or of groups of rows
 int coop_cost(const Rep& R, bool fp64);   // of a row plane
 void coop_cut(CoopPlan& c, const Rep& R, long long work, bool fp64, int nsm);   // ncta, runs, per
 CoopRep coop_rep(const Rep& R, bool fp64, int cost, int cost0);   // cost: of a row plane
+template <typename T> const void* coop_mixed();   // the kernel of replicas of unlike row layouts
 template <typename T> int coop_prepare(int kk);   // cudaError_t
 template <typename T> int launch_prop_coop(const Launch& L, const CoopPlan& c, int j0, int j1, int limit);   // cudaError_t
 // mode: 0 exp(-U), 1 trial exp(-(U + a1 d)), 2 commit U += a d then exp(-U), 3 exp(-Uext)

@@ -111,8 +111,8 @@ int densities_static_on(const dscf_params* p, int32_t precision, const void* U_i
     if (nsm > kCoopMaxCtas) nsm = kCoopMaxCtas;
     CoopPlan plan;
     plan.nrep = 1;
-    plan.kk = coop_layout(R.nx);
-    coop_cut(plan, R, coop_units(R), precision == DSCF_FP64, nsm);
+    plan.kk = coop_layout(R.nx, R.V, precision == DSCF_FP64);
+    coop_cut(plan, R, coop_units(R, precision == DSCF_FP64), precision == DSCF_FP64, nsm);
     // Scratch layout: replica table, maps, Boltzmann factors, propagators, quadratures,
     // partial sums, scalars.
     const size_t V = (size_t)R.V;

@@ -47,6 +47,25 @@ def test_general_sweeps_tiles_of_long_rows(nx, precision):
     check_densities(melt((nx, 2, 6), 5, 3), precision, 25, tuning=(8, 1))
 
 
+@pytest.mark.parametrize("nx,ny,nz", [(2, 1025, 256), (6, 307, 301), (8, 257, 256), (12, 211, 210), (20, 173, 155), (22, 161, 151),
+                                      (24, 149, 151), (30, 125, 141), (32, 130, 127),
+                                      (32, 61, 68), (16, 99, 83)])
+def test_general_sweeps_groups_of_short_rows(nx, ny, nz):
+    """Several rows a warp, the last group of fewer; also in a batch beside another layout, bit for bit."""
+    cfg = melt((nx, ny, nz), 5, 3)
+    assert nx * ny * nz >= 1 << 17 and ny % (32 // (nx // (4 if nx % 4 == 0 else 2)))
+    U = inputs.random_field(ncomp_shape(cfg), seed=26, scale=0.5)
+    ref, _, _ = oracle.densities(cfg, U)
+    other = melt((33, 5, 4), 7, 2)
+    V = inputs.random_field(ncomp_shape(other), seed=27, scale=0.5)
+    solo = dscf.Context(cfg, dscf.FP32, tuning=(8, 1)).densities(torch.from_numpy(U))
+    assert rel(t2n(solo), ref) < 1e-5
+    ctx = dscf.Context([cfg, other], dscf.FP32)
+    both = ctx.densities(torch.from_numpy(np.concatenate([U.ravel(), V.ravel()])))
+    ctx.status()
+    assert torch.equal(both[:U.size], solo.reshape(-1))
+
+
 @pytest.mark.parametrize("N", [2, 3, 4, 5, 8, 9])
 @pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
 def test_general_sweeps_where_the_chains_meet(N, precision):
