@@ -67,7 +67,7 @@ bool validate(const dscf_params* p, int n, std::string& why) {
 
 // Flat blocks of the replicas and the general sweeps' table (replicas by decreasing chain length, so that
 // those still active at a contour step are a prefix).
-void assign_tiles(Layout& L, const dscf_params* p, int n, int prec) {
+void assign_work(Layout& L, const dscf_params* p, int n, int prec) {
     // Flat kernels: about kMaxFlatBlocks blocks over the whole batch (one wave of four per SM).  A
     // replica whose own tiling would give it smaller chunks takes the batch's common chunk, so a
     // batch of many replicas does not launch tens of thousands of short blocks.  (A single
@@ -155,7 +155,7 @@ Layout make_layout(const dscf_params* p, int n, int prec, char* base) {
         vb += R.V;
         L.Nmax = std::max(L.Nmax, q.N);
     }
-    assign_tiles(L, p, n, prec);
+    assign_work(L, p, n, prec);
     // workspace
     size_t off = 0;
     auto take = [&](size_t bytes) -> void* {
@@ -619,14 +619,14 @@ int check_predictor(dscf_ctx* c, bool after_pred) {
 
 int set_dev(dscf_ctx* c) { return cuda_check(c, cudaSetDevice(c->device), "cudaSetDevice"); }
 
-int upload_tiles(dscf_ctx* c) {
+int upload_tables(dscf_ctx* c) {
     int rc = cuda_check(c, cudaMemcpyAsync(c->d_reps, c->L.reps.data(), sizeof(Rep) * c->nrep, cudaMemcpyHostToDevice,
                                            c->stream), "reps");
     if (rc) return rc;
     rc = cuda_check(c, cudaMemcpyAsync(c->d_b2r, c->L.blk2rep.data(), sizeof(int) * c->L.nblk, cudaMemcpyHostToDevice,
                                        c->stream), "block map");
     if (rc) return rc;
-    return cuda_check(c, cudaStreamSynchronize(c->stream), "tile upload");
+    return cuda_check(c, cudaStreamSynchronize(c->stream), "table upload");
 }
 
 // Persistent-sweep candidates (one warp per plane of the brick): bricks of 16 planes and bricks of 8
@@ -691,7 +691,7 @@ bool fusable(const dscf_ctx* c, int kfuse) {
 // Autotuner: one density evaluation of each kind of sweeps, timed on the context's own buffers: the
 // general sweeps, and the persistent brick sweeps where the grids allow them (both brick depths).  Small
 // problems and grids without bricks take the general sweeps untimed.
-int autotune_zc(dscf_ctx* c) {
+int autotune(dscf_ctx* c) {
     long long Vtot = 0;
     for (const Rep& R : c->L.reps) Vtot += R.V;
     std::vector<int> pcand;
@@ -704,7 +704,7 @@ int autotune_zc(dscf_ctx* c) {
         if (int rc = cuda_check(c, cudaEventCreate(&e1), "tune event")) { cudaEventDestroy(e0); return rc; }
         auto leave = [&](int rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; };
         auto sweep_ms = [&]() -> float {   // (bricks exist in FP32 only)
-            if (upload_tiles(c)) return 1e30f;
+            if (upload_tables(c)) return 1e30f;
             const Launch L = launch_of(c, c->stream);
             enqueue_sweeps<float>(c, L);
             cudaEventRecord(e0, c->stream);
@@ -744,7 +744,7 @@ int autotune_zc(dscf_ctx* c) {
         if (st & ST_TIMEOUT) return fail(c, DSCF_ERR_TIMEOUT, "a contour sweep timed out during tuning");
     }
     c->zc = c->bricks ? c->pers_bz : std::min(c->L.reps[0].nz, 8);
-    return upload_tiles(c);
+    return upload_tables(c);
 }
 // A tuning chosen earlier (for instance cached from an autotuner run) instead of the autotuner.
 int apply_tuning(dscf_ctx* c, int zc, int kfuse) {
@@ -809,7 +809,7 @@ int dscf_init_tuned(const dscf_params* p, int32_t n, int32_t precision, void* wo
     rc = rc ? rc : chk(cudaStreamCreateWithFlags(&c->cap_body, cudaStreamNonBlocking), "capture stream");
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_reps, c->L.reps.data(), sizeof(Rep) * n, cudaMemcpyHostToDevice, c->stream), "reps");
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_b2r, c->L.blk2rep.data(), sizeof(int) * c->L.nblk, cudaMemcpyHostToDevice, c->stream), "b2r");
-    assign_tiles(c->L, c->params.data(), n, precision);   // (the sweeps' table with the final pointers)
+    assign_work(c->L, c->params.data(), n, precision);   // (the sweeps' table with the final pointers)
     rc = rc ? rc : chk(cudaMemcpyAsync(c->d_coop, c->L.coop.data(), sizeof(CoopRep) * n, cudaMemcpyHostToDevice, c->stream), "sweep table");
     rc = rc ? rc : chk(cudaMemsetAsync(c->d_status, 0, sizeof(int) * kStatusInts, c->stream), "status");
     const size_t es = precision == DSCF_FP64 ? 8 : 4;
@@ -836,7 +836,7 @@ int dscf_init_tuned(const dscf_params* p, int32_t n, int32_t precision, void* wo
     rc = rc ? rc : chk(cudaGetLastError(), "fill");
     rc = rc ? rc : chk(cudaStreamSynchronize(c->stream), "init sync");
     rc = rc ? rc : chk((cudaError_t)(precision == DSCF_FP64 ? coop_prepare<double>(c->L.kk) : coop_prepare<float>(c->L.kk)), "contour sweeps");
-    if (!rc) rc = (zc < 0) ? autotune_zc(c) : apply_tuning(c, zc, kfuse);
+    if (!rc) rc = (zc < 0) ? autotune(c) : apply_tuning(c, zc, kfuse);
     if (rc) {
         g_init_error = c->err;
         if (c->cap) cudaStreamDestroy(c->cap);
@@ -1369,7 +1369,7 @@ int dscf_set_tuning(dscf_ctx* c, int32_t zc, int32_t kfuse) {
     }
     c->zc = kfuse == 0 ? c->pers_bz : zc;
     c->kfuse = kfuse;
-    return upload_tiles(c);
+    return upload_tables(c);
 }
 
 int dscf_free(dscf_ctx* c) {

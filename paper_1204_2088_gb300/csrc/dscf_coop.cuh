@@ -40,7 +40,7 @@
 
 // the row layouts that coop_layout() gives: (sites per lane, mode)
 #define DSCF_COOP_LAYOUTS(X)                                                                                \
-    X(1, BLOCKED) X(2, BLOCKED) X(3, BLOCKED) X(4, BLOCKED) X(6, BLOCKED) X(8, BLOCKED) X(1, STRIDED) X(2, STRIDED) \
+    X(1, BLOCKED) X(2, BLOCKED) X(3, BLOCKED) X(4, BLOCKED) X(6, BLOCKED) X(8, BLOCKED) X(2, STRIDED) \
     X(3, STRIDED) X(4, STRIDED) X(5, STRIDED) X(6, STRIDED) X(7, STRIDED) X(8, STRIDED) X(4, TILE) X(5, TILE) \
     X(4, BTILE)
 #define DSCF_COOP_LAYOUTS32(X) X(2, ROWS) X(4, ROWS)   // in FP32 only
@@ -60,12 +60,7 @@ struct CoopCtl {
     int runs, per;               // runs > 0: one replica, one run of a row per warp, `per` warps of a CTA
 };
 
-__device__ __forceinline__ int cld_acquire(const int* p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void cred_release(int* p) {
+__device__ __forceinline__ void red_release(int* p) {
     asm volatile("red.release.gpu.global.add.s32 [%0], 1;\n" ::"l"(p) : "memory");
 }
 
@@ -457,30 +452,11 @@ constexpr int kCoopRegs = NW == 12 ? 160 : 232;
 template <typename T>
 __host__ __device__ constexpr int coop_nw(int kk) { return coop_warps(kk, sizeof(T) == 8); }
 constexpr int kCoopShared = 128;   // largest table kept in shared memory
-constexpr long long kCoopSpinLimit = 1LL << 28;   // polls of a shared-memory mbarrier (see kBarSpinLimit in dscf_pers.cu)
 
-__device__ __forceinline__ unsigned csaddr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cbar_init(unsigned long long* bar, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(csaddr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void cbar_arrive(unsigned long long* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(csaddr(bar)) : "memory");
-}
-__device__ __forceinline__ bool cbar_test(unsigned long long* bar, unsigned parity) {
-    unsigned done;
-    asm volatile(
-        "{\n\t.reg .pred P1;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, P1;\n\t}\n"
-        : "=r"(done)
-        : "r"(csaddr(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-__device__ __forceinline__ void cbar_wait(unsigned long long* bar, unsigned parity, const CoopCtl& ctl, bool& dead) {
+__device__ __forceinline__ void bar_wait(unsigned long long* bar, unsigned parity, const CoopCtl& ctl, bool& dead) {
     if (dead) return;
-    for (long long spins = 0; !cbar_test(bar, parity); ++spins)
-        if (spins > kCoopSpinLimit) {
+    for (long long spins = 0; !bar_test(bar, parity); ++spins)
+        if (spins > kBarSpinLimit) {
             atomicOr(ctl.status, (int)ST_TIMEOUT);
             atomicExch(ctl.abort, 1);
             dead = true;
@@ -504,8 +480,8 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
     }
     if (threadIdx.x == 0) {
         for (int c = 0; c < 2; ++c) {
-            cbar_init(&done[c], NW);
-            cbar_init(&go[c], 1);
+            bar_init(&done[c], NW);
+            bar_init(&go[c], 1);
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -516,17 +492,17 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kCoopSyncRegs));
         const int c = w - NW;
         if (!sync || c >= 2 || lane != 0) return;
-        bool aborted = cld_acquire(ctl.abort) != 0;
+        bool aborted = ld_acquire(ctl.abort) != 0;
         int* f = ctl.cnt + c * kFlagStride;
         for (int d = 0; d < ctl.j1 - ctl.j0; ++d) {
-            cbar_wait(&done[c], (unsigned)(d & 1), ctl, dead);
+            bar_wait(&done[c], (unsigned)(d & 1), ctl, dead);
             // `done` orders the compute warps' stores before this release; release is cumulative
-            cred_release(f);
+            red_release(f);
             const int target = (d + 1) * ncta;
             int spins = 0;
-            while (!aborted && cld_acquire(f) < target) {
+            while (!aborted && ld_acquire(f) < target) {
                 if ((++spins & 31) == 0) {
-                    if (cld_acquire(ctl.abort) != 0) {
+                    if (ld_acquire(ctl.abort) != 0) {
                         aborted = true;
                     } else if (spins > ctl.limit) {
                         atomicOr(ctl.status, (int)ST_TIMEOUT);
@@ -536,7 +512,7 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
                 }
                 __nanosleep(20);
             }
-            cbar_arrive(&go[c]);
+            bar_arrive(&go[c]);
         }
         // the last of all barrier warps leaves the counters at zero
         __threadfence();
@@ -581,29 +557,29 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
         const int d = j - ctl.j0;            // levels of this launch before this one
         const unsigned par = (unsigned)((d - 1) & 1);
         if (sync && d > 0) {
-            cbar_wait(&go[0], par, ctl, dead);
+            bar_wait(&go[0], par, ctl, dead);
             // another cut of the work when chains end: what a warp has written itself so far may now
             // be another warp's, so both chains' levels must be complete
-            if (nact != before) cbar_wait(&go[1], par, ctl, dead);
+            if (nact != before) bar_wait(&go[1], par, ctl, dead);
             __syncwarp();
         }
         coop_level<T, KK, 0>(reps, nact, ctl.runs, j, p, cut);
         if (sync) {
             __syncwarp();
-            if (lane == 0) cbar_arrive(&done[0]);
-            if (d > 0) cbar_wait(&go[1], par, ctl, dead);
+            if (lane == 0) bar_arrive(&done[0]);
+            if (d > 0) bar_wait(&go[1], par, ctl, dead);
             __syncwarp();
         }
         coop_level<T, KK, 1>(reps, nact, ctl.runs, j, p, cut);
         if (sync) {
             __syncwarp();
-            if (lane == 0) cbar_arrive(&done[1]);
+            if (lane == 0) bar_arrive(&done[1]);
         }
     }
     if (sync) {
         // Q: every 32 row planes of a replica make one partial sum, whatever the cut of the work, so a
         // replica's Q is the same alone and in any batch
-        cbar_wait(&go[0], (unsigned)((ctl.j1 - ctl.j0 - 1) & 1), ctl, dead);
+        bar_wait(&go[0], (unsigned)((ctl.j1 - ctl.j0 - 1) & 1), ctl, dead);
         __syncwarp();
         for (int r = 0; r < ctl.nrep; ++r) {
             const CoopRep& R = reps[r];

@@ -12,8 +12,9 @@ static long long rows_of(const Rep& R, bool fp64) {
 }
 long long coop_units(const Rep& R, bool fp64) { return rows_of(R, fp64) * R.nz; }
 
-// Strips of 8 rows where a field exceeds the L2, so that a CTA's warps share rows at about the same time
-// (256^3, N = 64: 7.93 -> 7.56 ms); in smaller grids sharing gains nothing.
+// Strips of 8 rows in fields of 2^23 sites and more, so that a CTA's warps share rows in the L1 at about the same
+// time (256^3, N = 64: 7.93 -> 7.56 ms; levels of that size, FP32 or FP64, pass through the L2); up to 128^3
+// sharing gains nothing (924 -> 984 us).
 static int strip_rows(const Rep& R) { return R.V >= (1LL << 23) && R.ny % 8 == 0 && coop_warps(layout_of(R, false), false) == 8 ? 8 : 1; }
 
 // Cut of a launch's work.  One replica whose rows can be cut into equal runs gives every warp one run

@@ -107,13 +107,13 @@ struct Rep {
     void* q;     // [2][V]  contour quadratures
     void* E;     // [ns][V] Boltzmann factors exp(-U)
     void* G;     // [N][V]  forward propagators G_1..G_N
-    void* Gp0;   // [V]     backward propagator ping
-    void* Gp1;   // [V]     backward propagator pong
+    void* Gp0;   // [V]     general sweeps: a chain's first level past the middle, forward
+    void* Gp1;   // [V]     and backward; bricks: the backward chain's boundary rows past the middle
     void* u;     // [3][V]  LB velocity (lattice units)
     void* pop0;  // [19][V] LB population deviations (post-collision), even steps
     void* pop1;  // [19][V] odd steps
-    void* del0;  // [ns][V] Jacobi iterate ping
-    void* del1;  // [ns][V] Jacobi iterate pong
+    void* del0;  // [ns][V] Jacobi iterates; bricks: the forward chain's boundary rows past the middle
+    void* del1;  // [ns][V]
     void* rhs;   // [ns][V] right-hand side of the Crank-Nicolson system
     void* Uprev; // [ns][V] potentials the previous step's inversion started from
     // thermal noise (dscf_set_noise): composition flux variance 2 M dt / Omega per unit phi,
@@ -402,10 +402,35 @@ __device__ __forceinline__ bool last_block_of(const Rep& R, int* flag_sh) {
     return last;
 }
 
-__device__ __forceinline__ int wrapi(int v, int n) {
-    v %= n;
-    return v < 0 ? v + n : v;
+// Waits of the contour sweeps: acquire loads of other CTAs' counters, mbarriers in shared memory.
+__device__ __forceinline__ unsigned saddr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ int ld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
+__device__ __forceinline__ void bar_init(unsigned long long* bar, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(saddr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(unsigned long long* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(saddr(bar)) : "memory");
+}
+__device__ __forceinline__ bool bar_test(unsigned long long* bar, unsigned parity) {
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred P1;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, P1;\n\t}\n"
+        : "=r"(done)
+        : "r"(saddr(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+// Polls of a shared-memory mbarrier before giving up.  What completes them (a CTA's own copies, its compute
+// warps, its exchange or barrier warps, whose waits on other CTAs are bounded by the context's limit)
+// depends on no unbounded wait, so this bound is fixed and far above any real time (a shorter limit set for
+// failure tests must not abandon a copy that is still landing in this CTA's shared memory).
+constexpr long long kBarSpinLimit = 1LL << 28;
 
 // Boltzmann factor exp(-x) in the field precision (CUDA's exp / expf, not re-implemented).
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds; each multiplies counter words 0

@@ -52,12 +52,6 @@ namespace dscf {
 
 namespace {
 
-// Polls of a shared-memory mbarrier before giving up.  What completes them (this CTA's copies, its
-// compute warps, its exchange warp, whose own waits on neighbours are bounded by the context's
-// limit) depends on no unbounded wait, so this bound is fixed and far above any real time (a
-// shorter neighbour-wait limit set for failure tests must not abandon a copy that is still landing
-// in this CTA's shared memory).
-constexpr long long kBarSpinLimit = 1LL << 28;
 // Compute warps per CTA: 16 for bricks of 16 planes, 8 for bricks of 8 planes; one CTA per SM.
 // Beside them one warpgroup of four warps does the exchange (two per chain): a whole warpgroup, so that
 // it can hand most of its registers to the compute warps (setmaxnreg).  Launched registers a thread
@@ -70,7 +64,6 @@ struct PersRegs {
     static constexpr int exchange = NW == 16 ? 32 : 24;
 };
 
-__device__ __forceinline__ unsigned saddr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp16(void* s, const void* g) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(saddr(s)), "l"(g));
 }
@@ -87,30 +80,8 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 __device__ __forceinline__ void cp_arrive(unsigned long long* bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(saddr(bar)) : "memory");
 }
-__device__ __forceinline__ int ld_acquire(const int* p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ void st_release(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ void bar_init(unsigned long long* bar, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(saddr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(unsigned long long* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(saddr(bar)) : "memory");
-}
-__device__ __forceinline__ bool bar_test(unsigned long long* bar, unsigned parity) {
-    unsigned done;
-    asm volatile(
-        "{\n\t.reg .pred P1;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, P1;\n\t}\n"
-        : "=r"(done)
-        : "r"(saddr(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
 }
 
 // Packed FP32 pairs (sm_100+ f32x2 arithmetic): two lanes of a float4 per instruction.
