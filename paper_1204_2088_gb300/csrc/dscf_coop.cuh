@@ -21,11 +21,11 @@
 // normalisation): 7 operations a site and contour step forward, 8 with the quadrature.
 //
 // FP64 at 128^3 is bound by the FP64 pipe (31 us of operations in a level's 33 us), 256^3 by HBM (592 MB
-// a pair of levels at 77% of the copy rate), the rest by the latency of loads and of the barrier: hence loads several planes
-// ahead, 12 warps where the registers allow it (128^3 FP32: 750 us with 8, 689 with 12) and one run per warp.
-// A density evaluation, one launch per contour step and direction, and so: 32^3, N = 32, FP64 539 -> 127 us;
-// 100 x 90 x 75, N = 48, FP32 1013 -> 276 us; 128^3, N = 64, FP64 8.9 -> 4.2 ms; 256^3, N = 64, FP32 8.07
-// (fused pairs of steps) -> 7.40 ms.  Against the brick sweeps (dscf_pers.cu): 48^3, N = 16 71 us (bricks 137),
+// a pair of levels at 77% of the copy rate), the rest by the latency of loads and of the barrier: hence loads
+// several planes ahead, 12 warps where the registers allow it (128^3 FP32: 750 us with 8, 689 with 12) and one run per warp.
+// A density evaluation, one launch per contour step and direction, and so: 32^3, N = 32, FP64 539 -> 126 us;
+// 100 x 90 x 75, N = 48, FP32 1013 -> 274 us; 128^3, N = 64, FP64 8.9 -> 4.2 ms; 256^3, N = 64, FP32 8.07
+// (fused pairs of steps) -> 7.25 ms.  Against the brick sweeps (dscf_pers.cu): 48^3, N = 16 71 us (bricks 137),
 // 64^3, N = 64 241 (361), 96^3, N = 48 347 (227), 128^3, N = 64 689 (386).
 //
 // Every wait is bounded as in dscf_pers.cu: a CTA that runs out sets the status bit and the abort flag
@@ -114,12 +114,12 @@ __device__ __forceinline__ CoopOps<T> coop_ops(const CoopRep& R, int j) {
 //            accesses, two shuffles for the x pass;
 //   strided: lane L holds sites L, L + 32, ... (any nx <= 256): scalar accesses, 2 K + 2 shuffles;
 //   tile:    like strided, of columns x0 - 1 .. x0 + tile of which the outer two are neighbours (nx > 256);
-//   btile:   like blocked, the first and the last lane hold the neighbours' sites (nx > 256, 4 | nx).
+//   btile:   like blocked, the first and the last lane hold the neighbours' sites (nx > 256, 4 | nx);
+//   rows:    blocked, several adjacent rows side by side (even nx <= 32 in FP32 fields of many rows).
 // Rows of more than 256 sites, density evaluations of N = 24, us, by the kernels before these (a launch per
 // level), in whole strided tiles of 254 columns (300 columns then cost 512), and in equal tiles:
 //   512 x 128 x 128 FP32 2570, 4713, 1794, FP64 11608, 14301, 7656;  300 x 300 x 100 FP32 2650, 5330, 1921;
 //   1024 x 64 x 64 FP32 1408, 2652, 795;  257 x 40 x 40 FP32 446, 510, 216, FP64 1064, 1156, 652.
-//   rows:    blocked, several adjacent rows side by side (nx <= 32, large FP32 fields).
 enum { BLOCKED = 0, STRIDED = 1, TILE = 2, BTILE = 3, ROWS = 4 };
 
 // K values of a lane at p: one access of 16, 8 or 4 bytes each where their size allows.
