@@ -384,17 +384,29 @@ __device__ __forceinline__ void coop_segment(const CoopRep& R, int j, int u0, in
     }
 }
 
+// The replicas' table in shared memory (the levels' acquire loads keep invalidating its cached copy): all of it,
+// or, of more replicas than it holds, those from the first of the CTA's share on.
+constexpr int kCoopShared = 128;
+struct CoopTable {
+    const CoopRep *loc, *all;   // shared, device
+    int first;                  // the replica of loc[0]
+    __device__ __forceinline__ const CoopRep& operator[](int i) const {
+        return i - first < kCoopShared ? loc[i - first] : all[i];
+    }
+};
+
 // This warp's share of a level.  KK: row layout of every replica of the launch, or 0: a switch per replica.
 // cut: its run of the one replica (row; first plane, end), or the cost bounds of the warp and of its CTA.
 struct CoopCut {
     int row, za, ze;
     int b0, b1, a0, a1;
+    int r0;   // first replica of the CTA's share
 };
 template <typename T, int KK, int C>
-__device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int runs, int j, int p, const CoopCut& cut) {
+__device__ __forceinline__ void coop_level(const CoopTable& tab, int nact, int runs, int j, int p, const CoopCut& cut) {
     if constexpr (KK > 0) {
         if (runs > 0) {
-            const CoopRep& R = reps[0];
+            const CoopRep& R = tab.loc[0];
             constexpr int MODE = (KK >> 4) - 1;
             double qs = 0.0;
             if (cut.za < cut.ze) {
@@ -409,8 +421,8 @@ __device__ __forceinline__ void coop_level(const CoopRep* reps, int nact, int ru
         }
     }
     const int w = threadIdx.x >> 5;
-    for (int i = 0; i < nact; ++i) {
-        const CoopRep& R = reps[i];
+    for (int i = cut.r0; i < nact; ++i) {
+        const CoopRep& R = tab[i];
         const int lay = KK > 0 ? KK : R.layout, wgt = R.wgt, planes = R.units / R.strip;
         const int b0 = R.strip == 8 ? cut.a0 : cut.b0, b1 = R.strip == 8 ? cut.a1 : cut.b1;
         const int c0 = R.cost0, c1 = c0 + planes * wgt;
@@ -451,7 +463,6 @@ template <int NW>
 constexpr int kCoopRegs = NW == 12 ? 160 : 232;
 template <typename T>
 __host__ __device__ constexpr int coop_nw(int kk) { return coop_warps(kk, sizeof(T) == 8); }
-constexpr int kCoopShared = 128;   // largest table kept in shared memory
 
 __device__ __forceinline__ void bar_wait(unsigned long long* bar, unsigned parity, const CoopCtl& ctl, bool& dead) {
     if (dead) return;
@@ -467,15 +478,14 @@ __device__ __forceinline__ void bar_wait(unsigned long long* bar, unsigned parit
 template <typename T, int KK>
 __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_coop(const CoopCtl ctl) {
     constexpr int NW = coop_nw<T>(KK);
-    // the table in shared memory: the levels' acquire loads keep invalidating its cached copy
     __shared__ CoopRep tab[kCoopShared];
     __shared__ __align__(8) unsigned long long done[2], go[2];   // per chain: level computed here; computed everywhere
     __shared__ bool fin;
     const int ncta = (int)gridDim.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool sync = ctl.j1 - ctl.j0 > 1;   // one level per launch: the launches are the barriers
     const CoopRep* reps = ctl.nrep <= kCoopShared ? tab : ctl.reps;
+    constexpr int WORDS = sizeof(CoopRep) / sizeof(int);
     if (ctl.nrep <= kCoopShared) {
-        constexpr int WORDS = sizeof(CoopRep) / sizeof(int);
         for (int i = threadIdx.x; i < ctl.nrep * WORDS; i += blockDim.x) ((int*)tab)[i] = ((const int*)ctl.reps)[i];
     }
     if (threadIdx.x == 0) {
@@ -526,6 +536,8 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kCoopRegs<NW>));
     const int p = blockIdx.x * NW + w;
     int nact = ctl.nrep + 1;        // active replicas
+    int ends = 0;                   // the level after the shortest active chain's last
+    CoopTable table = {tab, ctl.reps, 0};
     CoopCut cut = {};
     if (ctl.runs > 0) {
         const CoopRep& R = reps[0];
@@ -543,8 +555,11 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
     }
     for (int j = ctl.j0; j < ctl.j1; ++j) {
         const int before = nact;
-        nact = min(nact, ctl.nrep);
-        while (nact > 0 && reps[nact - 1].N <= j) --nact;
+        if (j >= ends) {
+            nact = min(nact, ctl.nrep);
+            while (reps[nact - 1].N <= j) --nact;   // (the longest chain has more levels)
+            ends = reps[nact - 1].N;
+        }
         if (nact != before) {
             const CoopRep& last = reps[nact - 1];
             const long long total = last.cost0 + last.units / last.strip * last.wgt;
@@ -553,6 +568,23 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
             cut.b1 = (int)(total * (p + 1) / P);
             cut.a0 = (int)(total * pa / P);
             cut.a1 = (int)(total * (pa + NW) / P);
+            // the last replica that begins at a0 or before (all of them at every level, and their sums of Q all
+            // in the first CTAs below: a step of five evaluations of 200 replicas of 8^3 sites, N = 8, FP32 4241
+            // us, 557 so, 602 with a launch per level; 40 of 20^3, N = 16, 1438, 804, 1106)
+            int lo = 0, hi = nact - 1;
+            while (lo < hi) {
+                const int m = (lo + hi + 1) >> 1;
+                if (reps[m].cost0 <= cut.a0) lo = m;
+                else hi = m - 1;
+            }
+            cut.r0 = lo;
+            if (ctl.nrep > kCoopShared) {
+                asm volatile("bar.sync 1, %0;\n" ::"r"(32 * NW) : "memory");   // every warp is done with the table's last part
+                const int n = min(kCoopShared, nact - lo) * WORDS;
+                for (int i = threadIdx.x; i < n; i += 32 * NW) ((int*)tab)[i] = ((const int*)(ctl.reps + lo))[i];
+                asm volatile("bar.sync 1, %0;\n" ::"r"(32 * NW) : "memory");
+                table.first = lo;
+            }
         }
         const int d = j - ctl.j0;            // levels of this launch before this one
         const unsigned par = (unsigned)((d - 1) & 1);
@@ -563,14 +595,14 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
             if (nact != before) bar_wait(&go[1], par, ctl, dead);
             __syncwarp();
         }
-        coop_level<T, KK, 0>(reps, nact, ctl.runs, j, p, cut);
+        coop_level<T, KK, 0>(table, nact, ctl.runs, j, p, cut);
         if (sync) {
             __syncwarp();
             if (lane == 0) bar_arrive(&done[0]);
             if (d > 0) bar_wait(&go[1], par, ctl, dead);
             __syncwarp();
         }
-        coop_level<T, KK, 1>(reps, nact, ctl.runs, j, p, cut);
+        coop_level<T, KK, 1>(table, nact, ctl.runs, j, p, cut);
         if (sync) {
             __syncwarp();
             if (lane == 0) bar_arrive(&done[1]);
@@ -581,13 +613,26 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
         // replica's Q is the same alone and in any batch
         bar_wait(&go[0], (unsigned)((ctl.j1 - ctl.j0 - 1) & 1), ctl, dead);
         __syncwarp();
-        for (int r = 0; r < ctl.nrep; ++r) {
-            const CoopRep& R = reps[r];
-            const int units = R.units;
-            for (int g = p; 32 * g < units; g += ncta * NW) {
-                const int u = 32 * g + lane;
-                const double t = warp_sum(u < units ? R.qrow[u] : 0.0);
-                if (lane == 0) R.pq[g] = t;
+        // (replica r's from the r-th CTA on, so that many small replicas do not all meet in the first)
+        const int P = ncta * NW;
+        for (int rb = 0; rb < ctl.nrep; rb += 32) {
+            const int r = rb + lane;
+            int g0 = 0;
+            bool some = false;
+            if (r < ctl.nrep) {
+                g0 = p - r % ncta * NW;
+                g0 += g0 < 0 ? P : 0;
+                some = 32LL * g0 < reps[r].units;
+            }
+            for (unsigned m = __ballot_sync(0xffffffffu, some); m; m &= m - 1) {
+                const int k = __ffs(m) - 1;
+                const CoopRep& R = reps[rb + k];
+                const int units = R.units;
+                for (int g = __shfl_sync(0xffffffffu, g0, k); 32LL * g < units; g += P) {
+                    const int u = 32 * g + lane;
+                    const double t = warp_sum(u < units ? R.qrow[u] : 0.0);
+                    if (lane == 0) R.pq[g] = t;
+                }
             }
         }
         // the last CTA adds up the partial sums, in order
@@ -599,19 +644,30 @@ __global__ void __launch_bounds__(32 * (coop_nw<T>(KK) + kCoopSync), 1) k_prop_c
         asm volatile("bar.sync 1, %0;\n" ::"r"(32 * NW) : "memory");
         if (fin) {
             __threadfence();
-            for (int r = w; r < ctl.nrep; r += NW) {
-                const CoopRep& R = reps[r];
-                if constexpr (sizeof(T) == 8) {
-                    const Two s = total_of(R.pq, (R.units + 31) / 32);
-                    if (lane == 0) {
-                        R.qsum[0] = s.hi;
-                        R.qsum[S_QLO - S_QSUM] = s.lo;
+            constexpr int U = 4;   // replicas of a warp side by side: their loads' latencies overlap
+            for (int r = w; r < ctl.nrep; r += U * NW) {
+                double s[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    s[u] = 0.0;
+                    if (r + u * NW >= ctl.nrep) continue;
+                    const CoopRep& R = reps[r + u * NW];
+                    for (int g = lane; 32LL * g < R.units; g += 32) s[u] += __ldcg(R.pq + g);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (r + u * NW >= ctl.nrep) break;
+                    double* q = reps[r + u * NW].qsum;
+                    if constexpr (sizeof(T) == 8) {
+                        const Two t = warp_sum(Two{s[u], 0.0});
+                        if (lane == 0) {
+                            q[0] = t.hi;
+                            q[S_QLO - S_QSUM] = t.lo;
+                        }
+                    } else {
+                        const double t = warp_sum(s[u]);
+                        if (lane == 0) *q = t;
                     }
-                } else {
-                    double s = 0.0;
-                    for (int g = lane; 32 * g < R.units; g += 32) s += __ldcg(R.pq + g);
-                    s = warp_sum(s);
-                    if (lane == 0) *R.qsum = s;
                 }
             }
         }

@@ -150,7 +150,10 @@ inline void set_par(const Rep& R, Par<T>& p) {
     p.ew = R.N <= (sizeof(T) == 4 ? 64 : 256) ? (T)std::exp2(-std::round(std::log2((double)w3))) : (T)(1.0L / w3);
     const T t = std::fma(p.rr, T(2), T(1)), u = std::fma(p.rr, t + t, t);
     p.s1 = std::fma(p.rr, u + u, u);
-    p.qn = (double)(std::pow((long double)p.ew * w3, (long double)-R.N) * (w3 / (long double)p.s1));
+    long double qn = w3 / (long double)p.s1, f = 1.0L / ((long double)p.ew * w3);
+    for (int n = R.N; n; n >>= 1, f *= f)   // (a call of pow in long double takes some microseconds on the host)
+        if (n & 1) qn *= f;
+    p.qn = (double)qn;
     p.rho0 = (T)R.rho0; p.gs = (T)R.gs; p.gb = (T)R.gb; p.dt2 = (T)(R.dt * R.dt);
     p.dtM = (T)(R.dt * R.M); p.c = (T)(0.5 * R.dt * R.M); p.kappa = (T)R.kappa; p.floor = (T)R.phi_floor;
     for (int i = 0; i < 9; ++i) p.chi[i] = (T)R.chi[i];

@@ -320,3 +320,21 @@ def test_segments_up_to_the_longest(short, precision):
     for cfg, tunings in ((melt((34, 7, 6), 6, 2), [(8, 1)]), (melt((32, 16, 16), 70, 30), [(8, 1), (16, 0)])):
         for tuning in tunings[:1 if precision == dscf.FP64 else 2]:
             check_densities(dict(cfg, a=a), precision, 99, tuning=tuning)
+
+
+@pytest.mark.parametrize("precision", [dscf.FP64, dscf.FP32], ids=["fp64", "fp32"])
+def test_general_sweeps_of_hundreds_of_replicas(precision):
+    """Chains of five lengths: the CTAs' parts of the table move as chains end.  Sampled replicas bit for bit as
+    alone."""
+    cfgs = [melt((3 + 7 * (i % 5), 2 + i % 3, 3 + i % 4), 2 + i % 5, 1 + i % 2 * (i % 5 > 0)) for i in range(330)]
+    U = [inputs.random_field(ncomp_shape(c), seed=400 + i, scale=0.5) for i, c in enumerate(cfgs)]
+    ref = np.concatenate([oracle.densities(c, u)[0].ravel() for c, u in zip(cfgs, U)])
+    ctx = dscf.Context(cfgs, precision)
+    flat = torch.from_numpy(np.concatenate([u.ravel() for u in U])).to(ctx.dtype).cuda()
+    got = ctx.densities(flat)
+    ctx.status()
+    assert rel(t2n(got), ref) < (1e-12 if precision == dscf.FP64 else 1e-5)
+    at = np.cumsum([0] + [u.size for u in U])
+    for i in (0, 1, 4, 127, 128, 200, 329):
+        solo = dscf.Context(cfgs[i], precision).densities(torch.from_numpy(U[i]))
+        assert torch.equal(got[at[i]:at[i + 1]], solo.reshape(-1))
