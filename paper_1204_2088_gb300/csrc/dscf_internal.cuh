@@ -144,10 +144,12 @@ inline void set_par(const Rep& R, Par<T>& p) {
     // The passes leave out their centre weights, so a level grows by w3 = (1 + 2 rr)^3 and the factors carry
     // a weight against it.  Any weight will do (it cancels in the densities); a power of two adds no
     // rounding to the factors, which are the same at every bead of a block: with 1 / w3 the potentials of a
-    // 128^3 FP64 step were 3 times as far off.  The nearest power leaves a level a drift of at most sqrt 2,
-    // which short chains hold easily (2^32 in FP32, 2^128 in FP64); longer ones take 1 / w3.
+    // 128^3 FP64 step were 3 times as far off.  The nearest power leaves a level a drift of up to sqrt 2, so
+    // it is taken only where the whole chain drifts by less than a twelfth of the exponents' range (2^10 in
+    // FP32, 2^80 in FP64); other chains take 1 / w3.
     const long double w = 1.0L + 2.0L * (long double)p.rr, w3 = w * w * w;
-    p.ew = R.N <= (sizeof(T) == 4 ? 64 : 256) ? (T)std::exp2(-std::round(std::log2((double)w3))) : (T)(1.0L / w3);
+    const double lw = std::log2((double)w3), drift = R.N * std::fabs(lw - std::round(lw));
+    p.ew = drift <= (sizeof(T) == 4 ? 10 : 80) ? (T)std::exp2(-std::round(lw)) : (T)(1.0L / w3);
     const T t = std::fma(p.rr, T(2), T(1)), u = std::fma(p.rr, t + t, t);
     p.s1 = std::fma(p.rr, u + u, u);
     long double qn = w3 / (long double)p.s1, f = 1.0L / ((long double)p.ew * w3);

@@ -338,3 +338,19 @@ def test_general_sweeps_of_hundreds_of_replicas(precision):
     for i in (0, 1, 4, 127, 128, 200, 329):
         solo = dscf.Context(cfgs[i], precision).densities(torch.from_numpy(U[i]))
         assert torch.equal(got[at[i]:at[i + 1]], solo.reshape(-1))
+
+
+@pytest.mark.parametrize("a", [0.6, 1.0, 1.1543, 1.5])
+@pytest.mark.parametrize("N", [8, 20, 64])
+@pytest.mark.parametrize("total", [-78.0, 78.0])
+def test_fp32_potentials_of_any_gauge(total, N, a):
+    """A constant added to both potentials does not change the densities, also where exp(-N U) comes within a few
+    units of FP32's limits: the sweeps' own scale takes little of the range.  The bound allows for the rounding
+    of the shifted potentials: N half ulps of |total| / N + |U|."""
+    cfg = dict(melt((34, 10, 9), N, N // 3), a=a)
+    U = inputs.random_field(ncomp_shape(cfg), seed=96, scale=0.5 / N)
+    ref, _, _ = oracle.densities(cfg, U)
+    ctx = dscf.Context(cfg, dscf.FP32, tuning=(8, 1))
+    got = t2n(ctx.densities(torch.from_numpy(U + total / N)))
+    ctx.status()
+    assert rel(got, ref) < 1e-5 + abs(total) * 2.0 ** -23
